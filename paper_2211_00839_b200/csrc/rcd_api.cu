@@ -66,7 +66,7 @@ size_t layout_workspace(void *base, rcd_feat_dtype dtype, const Sizes &sz, Works
     const size_t L = (size_t)std::max<int32_t>(sz.L, 1), W = (size_t)std::max<int32_t>(sz.W, 1);
     const size_t N = (size_t)std::max<int64_t>(sz.N, 1);
     const size_t sElem = 4;                                     // int32 / fp32
-    const size_t gElem = (sz.floatArith && !sz.graphCut) ? 4 : 8;   // fp32 gains / int64 gains, or 8-byte ties
+    const size_t gElem = 8;                                     // int64 gains (fp32 ones use half of it), or 8-byte ties
     Workspace w{};
     // the head does not depend on the class sizes: it is used before they are known
     w.status = c.take<int32_t>(4);
@@ -116,6 +116,7 @@ size_t layout_workspace(void *base, rcd_feat_dtype dtype, const Sizes &sz, Works
     w.stepBytes = c.take<unsigned long long>((size_t)sz.maxM + 1);
     w.stepOps = c.take<unsigned long long>((size_t)sz.maxM + 1);
     w.phaseNs = c.take<unsigned long long>(kPhaseWords);   // phase clocks, the grid-barrier counter, threshold-pass and row-skipping counters
+    w.g0 = c.take<long long>(N);
     w.bytes = align_up(c.off);
     if (ws) *ws = w;
     return w.bytes;
@@ -671,6 +672,7 @@ rcd_status rcd_partition(rcd_ctx *ctx, const void *features_dev, rcd_feat_dtype 
     RCD_CUDA(ctx, cudaMemcpyAsync(P.ws.quota, quota.data(), quota.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
 
     if (P.sz.graphCut) rs = launch_cut(ctx, P.sz, P.ws, assignment_dev, order_dev_or_null, st);
+    else if (cluster_form_takes(ctx, P.sz) && P.sz.maxM > 0) rs = launch_greedy_cluster(ctx, P.sz, P.ws, P.desc, assignment_dev, order_dev_or_null, st);
     else rs = launch_greedy(ctx, P.sz.floatArith ? RCD_FEAT_BF16 : RCD_FEAT_I8, P.sz, P.ws, P.desc, assignment_dev, order_dev_or_null, st);
     if (rs != RCD_OK) return rs;
     if (prof) RCD_CUDA(ctx, cudaEventRecord(ctx->evPhase[3], st));

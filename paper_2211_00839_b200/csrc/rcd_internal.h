@@ -127,6 +127,7 @@ struct Workspace {
     unsigned long long *stepBytes;   // [steps+1] bytes the sweep of step t has to read
     unsigned long long *stepOps;     // [steps+1] element x block pairs of that sweep
     unsigned long long *phaseNs;     // [6] sweep-/pick-phase ns of the persistent kernel, barrier counter, threshold-pass hits / elements / max blocks
+    long long *g0;          // [N] cluster form: gain of every sample for an empty block
     int32_t *status;        // [1]
     size_t bytes;           // total bytes laid out
 };
@@ -189,6 +190,7 @@ struct rcd_ctx {
     const unsigned long long *stepOpsDev = nullptr;
     const unsigned long long *phaseNsDev = nullptr;
     const int32_t *statusDev = nullptr;
+    int maxClusters[5]{};               // clusters of 1, 2, 4, 8, 16 CTAs of the cluster form resident at once (0: not asked yet)
 };
 
 namespace rcd {
@@ -225,6 +227,11 @@ size_t gaussian_scratch_bytes(int64_t N, int32_t L, int64_t maxM);
 rcd_status launch_greedy(rcd_ctx *ctx, rcd_feat_dtype dtype, const Sizes &sz, const Workspace &ws,
                          const std::vector<ClassDesc> &descHost, int32_t *assignment, int32_t *order,
                          cudaStream_t st);
+
+// greedy loop, one thread-block cluster per class
+bool cluster_form_takes(const rcd_ctx *ctx, const Sizes &sz);
+rcd_status launch_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, const std::vector<ClassDesc> &descHost,
+                                 int32_t *assignment, int32_t *order, cudaStream_t st);
 
 rcd_status launch_bounded_wait_selftest(rcd_ctx *ctx, unsigned *counter, int32_t *status, cudaStream_t st);
 
