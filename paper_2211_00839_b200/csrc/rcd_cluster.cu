@@ -28,13 +28,15 @@ namespace {
 constexpr int kMaxWarps = 16;             // team warps per CTA (one more warp leads in the cluster's first CTA)
 constexpr int kRaisedPerWarp = 64;        // raised columns a team lists at a time, per warp
 constexpr int kClusterBlocks = 128;       // blocks a cluster can lead (their notes sit in one CTA's shared memory)
-constexpr int kEntries = 32;              // candidates per note
-constexpr uint32_t kScanCmd = 0u;         // (a command's low word: 0 = look again, else sample + 1)
+constexpr int kEntries = 16;              // candidates per note
+constexpr uint32_t kScanCmd = 0u;         // a command's low word: look again;
+constexpr uint32_t kStopCmd = ~0u;        //   the class is done;  anything else: sample + 1 joins the block
 constexpr unsigned kPollLimit = 1u << 25;
 
+// What a team tells the leader about a block: the key of its best candidate (0: none), and for the case that other
+// blocks took that one: [1, 17) keys of leading candidates, [17, 17 + T) per team warp a key that no other exceeds.
 struct Note {
-    unsigned long long entry[kEntries];   // keys of exact candidates (0: none)
-    unsigned long long bound[kMaxWarps];  // per team warp: no candidate outside the entries has a key above it
+    unsigned long long word[1 + kEntries + kMaxWarps];
 };
 
 struct __align__(16) Raised {
@@ -45,10 +47,7 @@ struct __align__(16) Raised {
 
 struct Team {
     unsigned long long best[kMaxWarps];
-    int32_t count;                        // raised columns of the update in hand
-    int32_t slot;                         // what warp 0 of the team decided to do next
-    uint32_t what;
-    int32_t pad_;
+    int32_t count[4];                     // lengths of its lists: foreseen samples (in turn), others
 };
 
 }  // namespace
@@ -75,7 +74,7 @@ struct ClusterParams {
     int32_t maxLd;
     uint32_t one;              // the value 1, opaque to the compiler
     // byte offsets into dynamic shared memory
-    int32_t offTeams, offLists, offRows, offCmd, offSeen, offBits, offNotes, offBars, offCover, offGains;
+    int32_t offTeams, offLists, offRows, offCmd, offBits, offNotes, offBars, offCover, offKeys;
 };
 
 namespace {
@@ -88,11 +87,11 @@ __device__ __forceinline__ uint32_t remote(uint32_t addr, uint32_t rank)
 }
 __device__ __forceinline__ void st_remote(uint32_t addr, unsigned long long v)
 {
-    asm volatile("st.relaxed.cluster.shared::cluster.u64 [%0], %1;" :: "r"(addr), "l"(v) : "memory");
+    asm volatile("st.volatile.shared::cluster.u64 [%0], %1;" :: "r"(addr), "l"(v) : "memory");
 }
 __device__ __forceinline__ void st_remote32(uint32_t addr, uint32_t v)
 {
-    asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" :: "r"(addr), "r"(v) : "memory");
+    asm volatile("st.volatile.shared::cluster.u32 [%0], %1;" :: "r"(addr), "r"(v) : "memory");
 }
 // Asynchronous store to a CTA of the cluster; its 8 bytes count towards the phase of that CTA's mbarrier.
 __device__ __forceinline__ void st_async(uint32_t addr, unsigned long long v, uint32_t bar)
@@ -102,7 +101,7 @@ __device__ __forceinline__ void st_async(uint32_t addr, unsigned long long v, ui
 __device__ __forceinline__ unsigned long long ld_relaxed(uint32_t addr)      // (own shared memory)
 {
     unsigned long long v;
-    asm volatile("ld.relaxed.cluster.shared::cta.u64 %0, [%1];" : "=l"(v) : "r"(addr) : "memory");
+    asm volatile("ld.volatile.shared::cta.u64 %0, [%1];" : "=l"(v) : "r"(addr) : "memory");
     return v;
 }
 __device__ __forceinline__ void cluster_fence() { asm volatile("fence.acq_rel.cluster;" ::: "memory"); }
@@ -114,7 +113,7 @@ __device__ __forceinline__ void bar_expect(uint32_t bar, uint32_t bytes)
 __device__ __forceinline__ bool bar_done(uint32_t bar, uint32_t parity)
 {
     uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
                  : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
@@ -143,6 +142,14 @@ __device__ __forceinline__ unsigned long long add_wide(int x, uint32_t one, unsi
 {
     unsigned long long r;
     asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(r) : "r"((uint32_t)x), "r"(one), "l"(acc));
+    return r;
+}
+
+// key with a loss of l taken off its gain (one multiply-add)
+__device__ __forceinline__ unsigned long long take_off(unsigned long long key, int l)
+{
+    unsigned long long r;
+    asm("mad.wide.s32 %0, %1, -65536, %2;" : "=l"(r) : "r"(l), "l"(key));
     return r;
 }
 
@@ -181,17 +188,15 @@ __device__ __forceinline__ unsigned long long row_value(const int4 *row, int ld4
     return warp_sum(acc);
 }
 
-// What a team knows while it works on a class.
+// The team of a warp, and what it knows while it works on a class.
 struct TeamView {
     const int4 *S4;            // the class's similarity matrix
     int ld4;
     int warpIn, lane, T, team; // warp inside the team
     Team *tm;
     Raised *list;              // columns the update in hand raised
-    int4 *rowBuf;              // row of sample bufV (each thread reads only the pieces it copied itself)
-    int bufV;
+    int4 *rowBuf;              // a sample's row (each thread reads only the pieces it copied itself)
     const uint32_t *bits;      // assigned samples (and everything from M on)
-    uint32_t one;
 };
 
 // 16 bytes global -> shared without passing through registers
@@ -199,135 +204,354 @@ __device__ __forceinline__ void copy16(int4 *dst, const int4 *src)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(smem32(dst)), "l"(src) : "memory");
 }
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_group %0;" :: "n"(N) : "memory"); }
 
 // Starts copying the team's pieces of row v into its row buffer.
-__device__ __forceinline__ void fetch_row(TeamView &t, int v)
+__device__ __forceinline__ void fetch_row(const TeamView &t, int v)
 {
     const int4 *row = t.S4 + (int64_t)v * t.ld4;
-    asm volatile("cp.async.wait_group 0;" ::: "memory");    // (an earlier fetch into the same buffer may be under way)
     for (int q = t.warpIn * 32 + t.lane; q < t.ld4; q += t.T * 32) copy16(t.rowBuf + q, row + q);
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    t.bufV = v;
+    copies_commit();
 }
 
-// The block's leading candidates go to the leader: the bests of the team's 32 T threads merge into 32 candidates, and
-// what they leave out is bounded.  Then the row of the first candidate is fetched: it is, as a rule, the sample the
-// block receives next.
-__device__ __forceinline__ void post_candidates(TeamView &t, const long long *gains, uint32_t noteAddr, uint32_t barAddr)
+// What a candidate loses for one raised column: min(max(x, old), new) - old, as one instruction.  Similarities stay
+// below 2^30 either way, so x - old does not wrap, and two losses fit an int.
+__device__ __forceinline__ int loss(int x, const Raised &e) { return __viaddmin_s32_relu(x, e.minusOld, e.by); }
+
+__device__ __forceinline__ unsigned long long tile_max(uint32_t mask, unsigned long long k)
 {
-    const int T = t.T, lane = t.lane;
-    unsigned long long e = 0, o = 0;
-    for (int q = t.warpIn * 32 + lane; q < t.ld4; q += T * 32) {
+    const uint32_t hi = (uint32_t)(k >> 32), lo = (uint32_t)k;
+    const uint32_t mhi = __reduce_max_sync(mask, hi);
+    const uint32_t mlo = __reduce_max_sync(mask, hi == mhi ? lo : 0u);
+    return ((unsigned long long)mhi << 32) | mlo;
+}
+
+// A warp's part of a note from its threads' best and second-best keys: entries (one per tile of 2 T lanes, at the tile's
+// first lane), a bound on everything else, and the best of all.
+struct Summary {
+    unsigned long long entry, bound, top;
+};
+__device__ __forceinline__ Summary summarize(unsigned long long e, unsigned long long o, int T, int lane)
+{
+    Summary s;
+    if (T <= 2) {
+        for (int off = 1; off < 2 * T; off <<= 1) {
+            const unsigned long long e2 = __shfl_xor_sync(0xffffffffu, e, off), o2 = __shfl_xor_sync(0xffffffffu, o, off);
+            o = umax(umax(o, o2), umin(e, e2));
+            e = umax(e, e2);
+        }
+        s.entry = e;
+        s.bound = warp_max_u64(o);
+    } else {
+        const int tile = 2 * T;
+        const uint32_t mask = tile == 32 ? 0xffffffffu : ((1u << tile) - 1u) << (lane & ~(tile - 1));
+        s.entry = tile_max(mask, e);
+        s.bound = warp_max_u64(e == s.entry ? o : e);
+    }
+    s.top = warp_max_u64(s.entry);
+    return s;
+}
+__device__ __forceinline__ void post(const TeamView &t, const Summary &s, uint32_t noteAddr, uint32_t barAddr)
+{
+    const int tile = 2 * t.T;
+    if ((t.lane & (tile - 1)) == 0) st_async(noteAddr + (uint32_t)(1 + (t.warpIn * 32 + t.lane) / tile) * 8, s.entry, barAddr);
+    if (t.lane == 1) st_async(noteAddr + (uint32_t)(1 + kEntries + t.warpIn) * 8, s.bound, barAddr);
+}
+
+// Columns of one piece that rose join the list, as far as it has room.  Returns which did.
+__device__ __forceinline__ int list_raised(const TeamView &t, int32_t *count, int q, const int4 &r, const int4 &m)
+{
+    int up = (r.x > m.x ? 1 : 0) | (r.y > m.y ? 2 : 0) | (r.z > m.z ? 4 : 0) | (r.w > m.w ? 8 : 0);
+    if (up) {
+        const int room = t.T * kRaisedPerWarp;
+        int at = atomicAdd(count, __popc(up));
+        const int row = 4 * q * t.ld4;
+        const int took = min(room - at, __popc(up));
+        if (took < __popc(up)) {                                          // the list is full: these wait for the next one
+            for (int k = 0; k < took; ++k) t.list[at + k] = Raised{0, 0, 0, 0};
+            return 0;
+        }
+        if (up & 1) t.list[at++] = Raised{row, -m.x, r.x - m.x, 0};
+        if (up & 2) t.list[at++] = Raised{row + t.ld4, -m.y, r.y - m.y, 0};
+        if (up & 4) t.list[at++] = Raised{row + 2 * t.ld4, -m.z, r.z - m.z, 0};
+        if (up & 8) t.list[at++] = Raised{row + 3 * t.ld4, -m.w, r.w - m.w, 0};
+    }
+    return up;
+}
+
+// Takes the listed columns' losses off the keys (gain << 16 | tie-break) of one piece, U rows of S in flight.
+template <int U>
+__device__ __forceinline__ int correct_batch(const int4 *S4q, const Raised *list, int left, unsigned long long (&key)[4])
+{
+    int4 x[U];
+    int changed = 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) x[u] = ld_row_once(S4q + list[min(u, left - 1)].row);
+#pragma unroll
+    for (int u = 0; u < U; u += 2) {
+        const Raised a = list[min(u, left - 1)];
+        Raised b = list[min(u + 1, left - 1)];
+        if (u + 1 >= left) b.minusOld = b.by = 0;
+        if (u < left) {
+            const int l0 = loss(x[u].x, a) + loss(x[u + 1].x, b), l1 = loss(x[u].y, a) + loss(x[u + 1].y, b);
+            const int l2 = loss(x[u].z, a) + loss(x[u + 1].z, b), l3 = loss(x[u].w, a) + loss(x[u + 1].w, b);
+            changed |= l0 | l1 | l2 | l3;
+            key[0] = take_off(key[0], l0);
+            key[1] = take_off(key[1], l1);
+            key[2] = take_off(key[2], l2);
+            key[3] = take_off(key[3], l3);
+        }
+    }
+    return changed;
+}
+__device__ __forceinline__ int correct_full(const int4 *S4q, const Raised *list, unsigned long long (&key)[4])
+{
+    int4 x[8];
+    int changed = 0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) x[u] = ld_row_once(S4q + list[u].row);
+#pragma unroll
+    for (int u = 0; u < 8; u += 2) {
+        const Raised a = list[u], b = list[u + 1];
+        const int l0 = loss(x[u].x, a) + loss(x[u + 1].x, b), l1 = loss(x[u].y, a) + loss(x[u + 1].y, b);
+        const int l2 = loss(x[u].z, a) + loss(x[u + 1].z, b), l3 = loss(x[u].w, a) + loss(x[u + 1].w, b);
+        changed |= l0 | l1 | l2 | l3;
+        key[0] = take_off(key[0], l0);
+        key[1] = take_off(key[1], l1);
+        key[2] = take_off(key[2], l2);
+        key[3] = take_off(key[3], l3);
+    }
+    return changed;
+}
+__device__ __forceinline__ int correct(const TeamView &t, int n, int q, unsigned long long (&key)[4])
+{
+    const int4 *S4q = t.S4 + q;
+    int changed = 0, e0 = 0;
+    for (; e0 + 8 <= n; e0 += 8) changed |= correct_full(S4q, t.list + e0, key);
+    if (e0 + 4 < n) changed |= correct_batch<8>(S4q, t.list + e0, n - e0, key);
+    else if (e0 + 2 < n) changed |= correct_batch<4>(S4q, t.list + e0, n - e0, key);
+    else if (e0 < n) changed |= correct_batch<2>(S4q, t.list + e0, n - e0, key);
+    return changed;
+}
+
+// A thread's best and second-best key among its pieces of a block's stored gains.
+__device__ __forceinline__ void scan_keys(const TeamView &t, const unsigned long long *keys, unsigned long long &e, unsigned long long &o)
+{
+    e = o = 0;
+    for (int q = t.warpIn * 32 + t.lane; q < t.ld4; q += t.T * 32) {
         const uint32_t nib = t.bits[q >> 3] >> ((q & 7) * 4);
-        const ulonglong2 a0 = reinterpret_cast<const ulonglong2 *>(gains)[2 * q], a1 = reinterpret_cast<const ulonglong2 *>(gains)[2 * q + 1];
+        const ulonglong2 a0 = reinterpret_cast<const ulonglong2 *>(keys)[2 * q], a1 = reinterpret_cast<const ulonglong2 *>(keys)[2 * q + 1];
         const unsigned long long g[4] = {a0.x, a0.y, a1.x, a1.y};
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const unsigned long long k = (nib >> c & 1) ? 0ull : make_key(g[c], 4 * q + c);
+        for (int u = 0; u < 4; ++u) {
+            const unsigned long long k = (nib >> u & 1) ? 0ull : g[u];
             o = umax(o, umin(e, k));
             e = umax(e, k);
         }
     }
-    for (int off = 1; off < T; off <<= 1) {
-        const unsigned long long e2 = __shfl_xor_sync(0xffffffffu, e, off), o2 = __shfl_xor_sync(0xffffffffu, o, off);
-        o = umax(umax(o, o2), umin(e, e2));
-        e = umax(e, e2);
-    }
-    if ((lane & (T - 1)) == 0) st_async(noteAddr + (uint32_t)((t.warpIn * 32 + lane) / T) * 8, e, barAddr);
-    o = warp_max_u64(o);
-    if (lane == 0) st_async(noteAddr + (kEntries + t.warpIn) * 8, o, barAddr);
-    unsigned long long top = warp_max_u64(e);
-    if (T > 1) {
-        if (lane == 0) t.tm->best[t.warpIn] = top;
-        team_barrier(t.team, T);
-        top = warp_max_u64(lane < T ? t.tm->best[lane] : 0ull);
-    }
-    if (top) fetch_row(t, key_sample(top));
 }
 
-// What a candidate loses for one raised column: min(max(x, old), new) - old, as one instruction.  Similarities stay
-// within 2^30 either way, so x - old does not wrap.
-__device__ __forceinline__ uint32_t loss(int x, const Raised &e) { return (uint32_t)__viaddmin_s32_relu(x, e.minusOld, e.by); }
-
-// One batch of U raised columns applied to a thread's four columns q.
-template <int U>
-__device__ __forceinline__ void correct_batch(const int4 *base, const Raised *list, uint32_t one, unsigned long long (&d)[4])
+// Applies the n listed columns to the thread's pieces of a block's keys.  Returns whether any moved.
+__device__ __forceinline__ bool correct_keys(const TeamView &t, int n, unsigned long long *keys)
 {
-    int4 x[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) x[u] = ld_row_once(base + list[u].row);
-#pragma unroll
-    for (int u = 0; u < U; u += 2) {
-        const Raised a = list[u], b = list[u + 1];
-        d[0] = add_wide(loss(x[u].x, a) + loss(x[u + 1].x, b), one, d[0]);       // (each below 2^31)
-        d[1] = add_wide(loss(x[u].y, a) + loss(x[u + 1].y, b), one, d[1]);
-        d[2] = add_wide(loss(x[u].z, a) + loss(x[u + 1].z, b), one, d[2]);
-        d[3] = add_wide(loss(x[u].w, a) + loss(x[u + 1].w, b), one, d[3]);
+    bool moved = false;
+    for (int q = t.warpIn * 32 + t.lane; q < t.ld4; q += t.T * 32) {
+        ulonglong2 *p = reinterpret_cast<ulonglong2 *>(keys) + 2 * q;
+        ulonglong2 a = p[0], b = p[1];
+        unsigned long long k[4] = {a.x, a.y, b.x, b.y};
+        if (correct(t, n, q, k)) {
+            moved = true;
+            p[0] = make_ulonglong2(k[0], k[1]);
+            p[1] = make_ulonglong2(k[2], k[3]);
+        }
     }
+    return moved;
 }
 
-// A sample joins a block: its row is folded into the coverage and the stored gains follow, one row of S per column that
-// rose (S is symmetric): g(v) falls by min(max(S[v][i], old), new) - old.  The list of raised columns has a fixed room;
-// when more rise, the fold stops there and is taken up again after the correction.
-__device__ __forceinline__ void take_sample(TeamView &t, int v, int4 *cov, long long *gains, unsigned &rows)
+// Folds a row into the coverage and corrects the keys, list by list.  The row: in the team's buffer (each thread's own
+// pieces) or in S.
+__device__ __forceinline__ void take_in_lists(const TeamView &t, const int4 *row, int4 *cov, unsigned long long *keys, unsigned &rows)
 {
-    const int first = t.warpIn * 32 + t.lane, step = t.T * 32;
+    const int tid = t.warpIn * 32 + t.lane, step = t.T * 32;
     const int room = t.T * kRaisedPerWarp;
-    if (t.bufV != v) fetch_row(t, v);
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    int32_t *count = &t.tm->count[2];
     for (;;) {
-        for (int q = first; q < t.ld4; q += step) {
-            const int4 r = t.rowBuf[q];
-            const int4 m = cov[q];
-            const int up = (r.x > m.x ? 1 : 0) | (r.y > m.y ? 2 : 0) | (r.z > m.z ? 4 : 0) | (r.w > m.w ? 8 : 0);
-            if (up) {
-                const int n = __popc(up);
-                int at = atomicAdd(&t.tm->count, n);
-                if (at + n <= room) {
-                    const int row = 4 * q * t.ld4;
-                    if (up & 1) t.list[at++] = Raised{row, -m.x, r.x - m.x, 0};
-                    if (up & 2) t.list[at++] = Raised{row + t.ld4, -m.y, r.y - m.y, 0};
-                    if (up & 4) t.list[at++] = Raised{row + 2 * t.ld4, -m.z, r.z - m.z, 0};
-                    if (up & 8) t.list[at++] = Raised{row + 3 * t.ld4, -m.w, r.w - m.w, 0};
-                    cov[q] = make_int4(max(r.x, m.x), max(r.y, m.y), max(r.z, m.z), max(r.w, m.w));
-                } else {
-                    for (; at < room; ++at) t.list[at] = Raised{0, 0, 0, 0};     // (room that stays unused: no loss)
-                }
-            }
+        team_barrier(t.team, t.T);                         // (the list's last readers are done)
+        if (tid == 0) *count = 0;
+        team_barrier(t.team, t.T);
+        for (int q = tid; q < t.ld4; q += step) {
+            const int4 r = row[q], m = cov[q];
+            if (list_raised(t, count, q, r, m)) cov[q] = make_int4(max(r.x, m.x), max(r.y, m.y), max(r.z, m.z), max(r.w, m.w));
         }
         team_barrier(t.team, t.T);
-        const int all = *(volatile int32_t *)&t.tm->count;
+        const int all = *(volatile int32_t *)count;
         const int n = min(all, room);
         rows += n;
-        // the list is read in batches: entries without effect fill the last one
-        if (first < 8 && n + first < room + 8) t.list[n + first] = Raised{0, 0, 0, 0};
-        team_barrier(t.team, t.T);
-        if (n > 0) {
-            const bool own = n == 1 && t.list[0].row == v * t.ld4;           // (most picks: the sample itself is all that rose)
-            for (int q = first; q < t.ld4; q += step) {
-                unsigned long long d[4] = {0, 0, 0, 0};
-                if (own) {
-                    const int4 x = t.rowBuf[q];
-                    const Raised e = t.list[0];
-                    d[0] = loss(x.x, e); d[1] = loss(x.y, e); d[2] = loss(x.z, e); d[3] = loss(x.w, e);
-                } else {
-                    int e0 = 0;
-                    for (; e0 + 4 < n; e0 += 8) correct_batch<8>(t.S4 + q, t.list + e0, t.one, d);
-                    if (e0 + 2 < n) correct_batch<4>(t.S4 + q, t.list + e0, t.one, d);
-                    else if (e0 < n) correct_batch<2>(t.S4 + q, t.list + e0, t.one, d);
-                }
-                if (d[0] | d[1] | d[2] | d[3]) {
-                    ulonglong2 *p = reinterpret_cast<ulonglong2 *>(gains) + 2 * q;
-                    ulonglong2 a = p[0], b = p[1];
-                    a.x -= d[0]; a.y -= d[1]; b.x -= d[2]; b.y -= d[3];
-                    p[0] = a; p[1] = b;
+        if (n > 0) correct_keys(t, n, keys);
+        if (all <= room) break;
+    }
+}
+
+// Keys of an empty block and its coverage.
+__device__ __forceinline__ void start_block(const ClusterParams &prm, const ClassDesc &c, const TeamView &t, int4 *cov, unsigned long long *keys)
+{
+    for (int q = t.warpIn * 32 + t.lane; q < t.ld4; q += t.T * 32) {
+        cov[q] = make_int4(0, 0, 0, 0);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int v = 4 * q + u;
+            keys[v] = v < c.M ? make_key((unsigned long long)__ldcg(prm.g0 + c.row0 + v), v) : 0ull;
+        }
+    }
+}
+
+// A team with one block.
+__device__ __forceinline__ void team_of_one(const ClusterParams &prm, const ClassDesc &c, const TeamView &t, int4 *cov, unsigned long long *keys,
+                                            uint32_t cmdAddr, uint32_t noteAddr, uint32_t barAddr, unsigned &corrected, unsigned &rows)
+{
+    const int T = t.T, tid = t.warpIn * 32 + t.lane, step = T * 32, lane = t.lane;
+    const int room = T * kRaisedPerWarp;
+    start_block(prm, c, t, cov, keys);
+    if (tid == 0) t.tm->count[0] = t.tm->count[1] = 0;
+    unsigned long long e = 0, o = 0;
+    Summary sum{0, 0, 0};
+    bool dirty = true;
+    uint32_t had = 0;
+    for (int par = 0;; par ^= 1) {
+        // candidates: a thread looks again when its gains changed or its best has been assigned
+        if (!dirty && e != 0) {
+            const int s = key_sample(e);
+            dirty = t.bits[s >> 5] >> (s & 31) & 1;
+        }
+        if (__any_sync(0xffffffffu, dirty)) {
+            if (dirty) scan_keys(t, keys, e, o);
+            __syncwarp();
+            sum = summarize(e, o, T, lane);
+            dirty = false;
+            // (the warp's best may be the block's best some picks from now: its row comes to L2 meanwhile)
+            if (T > 1 && sum.top) {
+                const char *row = reinterpret_cast<const char *>(t.S4 + (int64_t)key_sample(sum.top) * t.ld4);
+                for (int at = lane * 128; at < t.ld4 * 16; at += 32 * 128) asm volatile("prefetch.global.L2 [%0];" :: "l"(row + at));
+            }
+        }
+        post(t, sum, noteAddr, barAddr);
+        unsigned long long top = sum.top;
+        if (T > 1) {
+            if (lane == 0) t.tm->best[t.warpIn] = top;
+            team_barrier(t.team, T);
+            top = warp_max_u64(lane < T ? t.tm->best[lane] : 0ull);
+        }
+        if (tid == 0) st_async(noteAddr, top, barAddr);
+        // until the command comes: the row of the best candidate, which is, as a rule, the sample the block receives
+        // next, and the columns it would raise
+        int v = top ? key_sample(top) : -1;
+        int32_t *count = &t.tm->count[par];
+        int all = 0;
+        if (v >= 0) {
+            fetch_row(t, v);
+            copies_wait<0>();
+            for (int q = tid; q < t.ld4; q += step) list_raised(t, count, q, t.rowBuf[q], cov[q]);
+            team_barrier(t.team, T);
+            all = *(volatile int32_t *)count;
+        }
+        if (tid == 0) t.tm->count[par ^ 1] = 0;
+        unsigned long long cmd = 0;
+        unsigned spin = 0;
+        while ((uint32_t)((cmd = ld_relaxed(cmdAddr)) >> 32) == had && ++spin < kPollLimit) { }
+        if (spin >= kPollLimit) {
+            if (lane == 0) atomicOr(prm.status, kDevTimeout);
+            break;
+        }
+        had = (uint32_t)(cmd >> 32);
+        const uint32_t what = (uint32_t)cmd;
+        if (what == kStopCmd) break;
+        if (what == kScanCmd) {
+            cluster_fence();
+            dirty = true;
+            continue;
+        }
+        ++corrected;
+        if ((int)what - 1 != v || all > room) {
+            // another sample than foreseen, or more raised columns than one list holds
+            if ((int)what - 1 != v) {
+                fetch_row(t, (int)what - 1);
+                copies_wait<0>();
+            }
+            take_in_lists(t, t.rowBuf, cov, keys, rows);
+            dirty = true;
+            continue;
+        }
+        rows += all;
+        const bool own = all == 1 && t.list[0].row == v * t.ld4;         // (most picks: the sample itself is all that rose)
+        const Raised mine = t.list[0];
+        for (int q = tid; q < t.ld4 && all > 0; q += step) {
+            const int4 r = t.rowBuf[q], m = cov[q];
+            if (r.x > m.x || r.y > m.y || r.z > m.z || r.w > m.w) cov[q] = make_int4(max(r.x, m.x), max(r.y, m.y), max(r.z, m.z), max(r.w, m.w));
+            if (own) {
+                const int l0 = loss(r.x, mine), l1 = loss(r.y, mine), l2 = loss(r.z, mine), l3 = loss(r.w, mine);
+                if (l0 | l1 | l2 | l3) {
+                    dirty = true;
+                    ulonglong2 *p = reinterpret_cast<ulonglong2 *>(keys) + 2 * q;
+                    const ulonglong2 a = p[0], b = p[1];
+                    p[0] = make_ulonglong2(take_off(a.x, l0), take_off(a.y, l1));
+                    p[1] = make_ulonglong2(take_off(b.x, l2), take_off(b.y, l3));
                 }
             }
         }
-        if (all <= room) break;
-        team_barrier(t.team, t.T);
-        if (first == 0) t.tm->count = 0;
-        team_barrier(t.team, t.T);
+        if (!own && all > 0) dirty = correct_keys(t, all, keys);         // (the sample's own gain is 0 now)
+    }
+    copies_wait<0>();
+}
+
+// A one-warp team with several blocks: it serves whichever has a command.
+template <typename Where>
+__device__ __forceinline__ void team_of_many(const ClusterParams &prm, int l, const ClassDesc &c, const TeamView &t, int mine, uint32_t cmd0,
+                                             int cmdStride, Where where, unsigned &corrected, unsigned &rows)
+{
+    const int lane = t.lane;
+    int4 *cov;
+    unsigned long long *keys;
+    uint32_t noteAddr, barAddr;
+    auto tell = [&] {
+        unsigned long long e, o;
+        scan_keys(t, keys, e, o);
+        const Summary sum = summarize(e, o, 1, lane);
+        post(t, sum, noteAddr, barAddr);
+        if (lane == 0) st_async(noteAddr, sum.top, barAddr);
+    };
+    for (int i = 0; i < mine; ++i) {
+        const int j = where(i, cov, keys, noteAddr, barAddr);
+        start_block(prm, c, t, cov, keys);
+        if (prm.quota[(int64_t)l * prm.W + j] > 0) tell();
+    }
+    // lane i watches the command of the team's i-th block
+    const uint32_t at = cmd0 + (uint32_t)(min(lane, mine - 1) * cmdStride);
+    uint32_t had = 0;
+    for (;;) {
+        unsigned long long cmd = 0;
+        unsigned pending = 0, spin = 0;
+        do {
+            cmd = ld_relaxed(at);
+            pending = __ballot_sync(0xffffffffu, lane < mine && (uint32_t)(cmd >> 32) != had);
+        } while (pending == 0 && ++spin < kPollLimit);
+        if (pending == 0) {
+            if (lane == 0) atomicOr(prm.status, kDevTimeout);
+            break;
+        }
+        const int who = __ffs(pending) - 1;
+        const uint32_t what = __shfl_sync(0xffffffffu, (uint32_t)cmd, who);
+        if (lane == who) had = (uint32_t)(cmd >> 32);
+        if (what == kStopCmd) break;
+        where(who, cov, keys, noteAddr, barAddr);
+        if (what == kScanCmd) {
+            cluster_fence();
+        } else {
+            ++corrected;
+            take_in_lists(t, t.S4 + (int64_t)((int)what - 1) * t.ld4, cov, keys, rows);
+        }
+        __syncwarp();
+        tell();
     }
 }
 
@@ -336,22 +560,24 @@ __device__ __forceinline__ void take_sample(TeamView &t, int v, int4 *cov, long 
 template <int KW>
 __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsigned char *shared, uint32_t C, uint32_t &parities)
 {
-    const int lane = threadIdx.x & 31, W = prm.W;
-    const uint32_t noteBytes = (kEntries + prm.teamWarps) * 8;
+    const int lane = threadIdx.x & 31, W = prm.W, T = prm.teamWarps;
+    const uint32_t noteBytes = (1 + kEntries + T) * 8;
     const uint32_t base = smem32(shared);
     volatile uint32_t *bits = reinterpret_cast<uint32_t *>(shared + prm.offBits);
-    const Note *notes = reinterpret_cast<const Note *>(shared + prm.offNotes);
+    const uint32_t myBits = remote(base + prm.offBits, (uint32_t)lane < C ? lane : 0);
+    volatile const Note *notes = reinterpret_cast<const Note *>(shared + prm.offNotes);
     const uint32_t bars = base + prm.offBars;
-    unsigned long long f[KW];
+    unsigned long long f[KW];              // value << 7 | block
     int room[KW];
-    uint32_t seq[KW];
+    uint32_t seq[KW], cmdAddr[KW];
     uint32_t awaited = 0;                  // bit k: block lane + 32 k owes a note
 #pragma unroll
     for (int k = 0; k < KW; ++k) {
         const int p = lane + 32 * k;
-        f[k] = 0;
+        f[k] = p;
         seq[k] = 0;
         room[k] = p < W ? prm.quota[(int64_t)l * W + p] : 0;
+        cmdAddr[k] = remote(base + prm.offCmd + (uint32_t)((p < W ? p : 0) / C) * 8, (uint32_t)(p < W ? p : 0) % C);
         if (room[k] > 0) {
             bar_expect(bars + p * 8, noteBytes);
             awaited |= 1u << k;
@@ -360,11 +586,10 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
     __syncwarp();
     unsigned rescans = 0;
     bool ok = true;
-    for (int t = 0; t < c.M && ok; ++t) {
+    for (int t = 0; t < c.M; ++t) {
         unsigned long long least = ~0ull;
 #pragma unroll
-        for (int k = 0; k < KW; ++k)
-            if (room[k] > 0) least = umin(least, (f[k] << 7) | (unsigned long long)(lane + 32 * k));
+        for (int k = 0; k < KW; ++k) least = room[k] > 0 ? umin(least, f[k]) : least;
         least = ~warp_max_u64(~least);
         if (least == ~0ull) {
             if (lane == 0) atomicOr(prm.status, kDevNoCandidate);
@@ -372,14 +597,12 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
             break;
         }
         const int j = (int)(least & 127);
-        const int jk = j >> 5, jl = j & 31;
-        const uint32_t cmd = base + prm.offCmd + (uint32_t)(j / C) * 8;
-        const uint32_t owner = (uint32_t)(j % C);
+        const int jk = KW == 1 ? 0 : j >> 5, jl = j & 31;
+        const uint32_t state = __shfl_sync(0xffffffffu, awaited | parities << 16, jl) >> jk;
+        uint32_t waits = state & 1, parity = state >> 16 & 1;
         unsigned long long best = 0;
         for (;;) {
-            const uint32_t waits = __shfl_sync(0xffffffffu, awaited, jl) >> jk & 1;
             if (waits) {
-                const uint32_t parity = __shfl_sync(0xffffffffu, parities, jl) >> jk & 1;
                 unsigned spin = 0;
                 while (!bar_done(bars + j * 8, parity) && ++spin < kPollLimit) { }
                 if (spin >= kPollLimit) {
@@ -387,65 +610,75 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
                     ok = false;
                     break;
                 }
+                parity ^= 1;
                 if (lane == jl) { awaited &= ~(1u << jk); parities ^= 1u << jk; }
             }
-            const unsigned long long k = notes[j].entry[lane];
-            const unsigned long long bound = lane < prm.teamWarps ? notes[j].bound[lane] : 0ull;
-            const int v = key_sample(k);
-            const bool free = k != 0 && !(bits[v >> 5] >> (v & 31) & 1);
+            best = notes[j].word[0];
+            {
+                const int s = key_sample(best);
+                if (best != 0 && !(bits[s >> 5] >> (s & 31) & 1)) break;
+            }
+            // the best one has been taken: the best of those left, if none that the note leaves out can lead
+            const unsigned long long k = lane < kEntries + T ? notes[j].word[1 + lane] : 0ull;
+            const int s = key_sample(k);
+            const bool free = lane < kEntries && k != 0 && !(bits[s >> 5] >> (s & 31) & 1);
             best = warp_max_u64(free ? k : 0ull);
-            if (best != 0 && __ballot_sync(0xffffffffu, bound >= best) == 0) break;
+            if (best != 0 && __ballot_sync(0xffffffffu, lane >= kEntries && k >= best) == 0) break;
             // every candidate that is sure to lead has been taken by other blocks: look again
             ++rescans;
+            waits = 1;
             cluster_fence();                               // (the team must see which samples are taken)
             if (lane == jl) {
                 bar_expect(bars + j * 8, noteBytes);
                 awaited |= 1u << jk;
 #pragma unroll
-                for (int q = 0; q < KW; ++q) if (q == jk) st_remote(remote(cmd, owner), ((unsigned long long)++seq[q] << 32) | kScanCmd);
+                for (int q = 0; q < KW; ++q) if (q == jk) st_remote(cmdAddr[q], ((unsigned long long)++seq[q] << 32) | kScanCmd);
             }
         }
         if (!ok) break;
         const int v = key_sample(best);
+        if (lane == jl) {
+#pragma unroll
+            for (int k = 0; k < KW; ++k)
+                if (k == jk) {
+                    f[k] += best >> 16 << 7;
+                    if (--room[k] > 0) {                   // (a full block needs no gains any more)
+                        bar_expect(bars + j * 8, noteBytes);
+                        awaited |= 1u << k;
+                        st_remote(cmdAddr[k], ((unsigned long long)++seq[k] << 32) | (unsigned long long)(v + 1));
+                    }
+                }
+        }
         const uint32_t word = bits[v >> 5] | (1u << (v & 31));
         __syncwarp();
-        if (lane == 0) bits[v >> 5] = word;
-        else if (lane < (int)C) st_remote32(remote(base + prm.offBits + (uint32_t)(v >> 5) * 4, lane), word);
-        if (lane == jl) {
-            const int left = [&] {
-                int r = 0;
-#pragma unroll
-                for (int k = 0; k < KW; ++k) if (k == jk) { f[k] += best >> 16; r = --room[k]; }
-                return r;
-            }();
-            if (left > 0) {                                // (a full block needs no gains any more)
-                bar_expect(bars + j * 8, noteBytes);
-                awaited |= 1u << jk;
-#pragma unroll
-                for (int k = 0; k < KW; ++k) if (k == jk) st_remote(remote(cmd, owner), ((unsigned long long)++seq[k] << 32) | (unsigned long long)(v + 1));
-            }
+        if (lane == 0) {
+            bits[v >> 5] = word;
+            prm.picks[c.row0 + t] = (uint32_t)v | ((uint32_t)j << 16);
+        } else if (lane < (int)C) {
+            st_remote32(myBits + (uint32_t)(v >> 5) * 4, word);
         }
-        if (lane == 0) prm.picks[c.row0 + t] = (uint32_t)v | ((uint32_t)j << 16);
         __syncwarp();
     }
-    // notes still under way land before the class ends
-    if (ok)
-        for (int k = 0; k < KW; ++k)
-            if (awaited >> k & 1) {
-                unsigned spin = 0;
-                while (!bar_done(bars + (lane + 32 * k) * 8, parities >> k & 1) && ++spin < kPollLimit) { }
-                if (spin >= kPollLimit) atomicOr(prm.status, kDevTimeout);
-                parities ^= 1u << k;
-            }
-    __syncwarp();
-    if (lane < (int)C) st_remote(remote(base + prm.offCmd + (uint32_t)prm.slots * 8, lane), 1ull);
+    // notes still under way land before the class ends; then every team is sent home
 #pragma unroll
-    for (int k = 0; k < KW; ++k)
-        if (lane + 32 * k < W) prm.fval[(int64_t)l * W + lane + 32 * k] = (long long)f[k];
+    for (int k = 0; k < KW; ++k) {
+        const int p = lane + 32 * k;
+        if (ok && (awaited >> k & 1)) {
+            unsigned spin = 0;
+            while (!bar_done(bars + p * 8, parities >> k & 1) && ++spin < kPollLimit) { }
+            if (spin >= kPollLimit) atomicOr(prm.status, kDevTimeout);
+            parities ^= 1u << k;
+        }
+        if (p < W) {
+            st_remote(cmdAddr[k], ((unsigned long long)++seq[k] << 32) | kStopCmd);
+            prm.fval[(int64_t)l * W + p] = (long long)(f[k] >> 7);
+        }
+    }
     if (lane == 0 && rescans) atomicAdd(prm.stats + 9, (unsigned long long)rescans);
 }
 
-template <int KW, bool kSmemState>
+// kSmemState: coverage and stored gains fit the CTAs' shared memory.  kManyBlocks: teams of one warp with several blocks.
+template <int KW, bool kSmemState, bool kManyBlocks>
 __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) greedy_cluster_kernel(const __grid_constant__ ClusterParams prm)
 {
     extern __shared__ __align__(128) unsigned char shared[];
@@ -456,7 +689,6 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) greedy_cluster_kernel
     const uint32_t base = smem32(shared);
     uint32_t *bits = reinterpret_cast<uint32_t *>(shared + prm.offBits);
     volatile unsigned long long *cmds = reinterpret_cast<volatile unsigned long long *>(shared + prm.offCmd);
-    uint32_t *seen = reinterpret_cast<uint32_t *>(shared + prm.offSeen);
     const int W = prm.W;
     uint32_t parities = 0;
 
@@ -489,10 +721,7 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) greedy_cluster_kernel
             }
         for (int i = threadIdx.x; i < (c.ld + 31) / 32; i += blockDim.x)
             bits[i] = 32 * i + 32 <= c.M ? 0u : (32 * i >= c.M ? ~0u : ~0u << (c.M - 32 * i));
-        for (int i = threadIdx.x; i <= prm.slots; i += blockDim.x) {
-            cmds[i] = 0;
-            if (i < prm.slots) seen[i] = 0;
-        }
+        for (int i = threadIdx.x; i < prm.slots; i += blockDim.x) cmds[i] = 0;
         cluster_barrier();
 
         if (warp == NW) {
@@ -503,73 +732,37 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) greedy_cluster_kernel
             t.S4 = S4; t.ld4 = ld4;
             t.warpIn = warp - team * T; t.lane = lane; t.T = T; t.team = team;
             t.tm = reinterpret_cast<Team *>(shared + prm.offTeams) + team;
-            t.list = reinterpret_cast<Raised *>(shared + prm.offLists) + team * (T * kRaisedPerWarp + 8);
+            t.list = reinterpret_cast<Raised *>(shared + prm.offLists) + team * (T * kRaisedPerWarp + 1);
             t.rowBuf = reinterpret_cast<int4 *>(shared + prm.offRows) + (size_t)team * (prm.maxLd >> 2);
-            t.bufV = -1;
             t.bits = bits;
-            t.one = prm.one;
             unsigned corrected = 0, rows = 0;
-            auto cover_of = [&](int slot) -> int4 * {
-                if (kSmemState) return reinterpret_cast<int4 *>(shared + prm.offCover) + (size_t)slot * (prm.maxLd >> 2);
-                return reinterpret_cast<int4 *>(prm.cover + c.vOff) + (size_t)(slot * C + rank) * ld4;
+            const uint32_t notes0 = remote(base + prm.offNotes, 0), bars0 = remote(base + prm.offBars, 0);
+            // the i-th block of the team
+            auto where = [&](int i, int4 *&cov, unsigned long long *&keys, uint32_t &noteAddr, uint32_t &barAddr) -> int {
+                const int slot = team + i * nTeams, j = slot * (int)C + (int)rank;
+                if (kSmemState) {
+                    cov = reinterpret_cast<int4 *>(shared + prm.offCover) + (size_t)slot * (prm.maxLd >> 2);
+                    keys = reinterpret_cast<unsigned long long *>(shared + prm.offKeys) + (size_t)slot * prm.maxLd;
+                } else {
+                    cov = reinterpret_cast<int4 *>(prm.cover + c.vOff) + (size_t)j * ld4;
+                    keys = reinterpret_cast<unsigned long long *>(prm.gains + c.vOff) + (size_t)j * c.ld;
+                }
+                noteAddr = notes0 + j * (uint32_t)sizeof(Note);
+                barAddr = bars0 + j * 8;
+                return j;
             };
-            auto gains_of = [&](int slot) -> long long * {
-                if (kSmemState) return reinterpret_cast<long long *>(shared + prm.offGains) + (size_t)slot * prm.maxLd;
-                return prm.gains + c.vOff + (size_t)(slot * C + rank) * c.ld;
-            };
-            const uint32_t notes0 = remote(base + prm.offNotes, 0);
-            const uint32_t bars0 = remote(base + prm.offBars, 0);
             int mine = 0;
-            for (int slot = team; slot < prm.slots; slot += nTeams) {
-                const int j = slot * (int)C + (int)rank;
-                if (j >= W) break;
-                ++mine;
-                if (prm.quota[(int64_t)l * W + j] == 0) continue;
-                int4 *cov = cover_of(slot);
-                long long *gains = gains_of(slot);
-                for (int q = t.warpIn * 32 + lane; q < ld4; q += T * 32) {
-                    cov[q] = make_int4(0, 0, 0, 0);
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) gains[4 * q + u] = 4 * q + u < c.M ? __ldcg(prm.g0 + c.row0 + 4 * q + u) : 0;
-                }
-                post_candidates(t, gains, notes0 + j * (uint32_t)sizeof(Note), bars0 + j * 8);
+            while (team + mine * nTeams < prm.slots && (team + mine * nTeams) * (int)C + (int)rank < W) ++mine;
+            if (mine == 1 && !kManyBlocks) {
+                int4 *cov;
+                unsigned long long *keys;
+                uint32_t noteAddr, barAddr;
+                const int j = where(0, cov, keys, noteAddr, barAddr);
+                if (prm.quota[(int64_t)l * W + j] > 0)
+                    team_of_one(prm, c, t, cov, keys, base + prm.offCmd + team * 8, noteAddr, barAddr, corrected, rows);
+            } else if (mine >= 1 && kManyBlocks) {
+                team_of_many(prm, l, c, t, mine, base + prm.offCmd + team * 8, nTeams * 8, where, corrected, rows);
             }
-            for (;;) {
-                if (t.warpIn == 0) {
-                    // lane i watches the command of the team's i-th block, lane 31 the end of the class
-                    const uint32_t at = base + prm.offCmd + (uint32_t)(lane == 31 ? prm.slots : team + lane * nTeams) * 8;
-                    const uint32_t had = lane < mine ? seen[team + lane * nTeams] : 0u;
-                    unsigned pending = 0;
-                    unsigned long long cmd = 0;
-                    for (unsigned spin = 0; spin < kPollLimit; ++spin) {
-                        if (lane < mine || lane == 31) cmd = ld_relaxed(at);
-                        pending = __ballot_sync(0xffffffffu, lane == 31 ? cmd != 0 : (lane < mine && (uint32_t)(cmd >> 32) != had));
-                        if (pending) break;
-                    }
-                    if (pending == 0 && lane == 0) atomicOr(prm.status, kDevTimeout);
-                    const int who = pending ? __ffs(pending) - 1 : 31;
-                    if (lane == who) {
-                        t.tm->count = 0;
-                        t.tm->slot = who == 31 ? -1 : team + who * nTeams;
-                        t.tm->what = (uint32_t)cmd;
-                        if (who != 31) seen[team + who * nTeams] = (uint32_t)(cmd >> 32);
-                        if ((uint32_t)cmd == kScanCmd) cluster_fence();
-                    }
-                }
-                team_barrier(team, T);
-                const int slot = *(volatile int32_t *)&t.tm->slot;
-                if (slot < 0) break;
-                const uint32_t what = *(volatile uint32_t *)&t.tm->what;
-                const int j = slot * (int)C + (int)rank;
-                int4 *cov = cover_of(slot);
-                long long *gains = gains_of(slot);
-                if (what != kScanCmd) {
-                    ++corrected;
-                    take_sample(t, (int)what - 1, cov, gains, rows);
-                }
-                post_candidates(t, gains, notes0 + j * (uint32_t)sizeof(Note), bars0 + j * 8);
-            }
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
             if (lane == 0 && t.warpIn == 0 && corrected) {
                 atomicAdd(prm.stats + 15, (unsigned long long)corrected);
                 atomicAdd(prm.stats + 16, (unsigned long long)rows);
@@ -595,10 +788,17 @@ static int pow2_at_least(int x)
     return p;
 }
 
-template <int KW, bool kSmemState>
-static rcd_status launch_cluster(rcd_ctx *ctx, const ClusterParams &prm, int C, int clusters, size_t smem, cudaStream_t st, bool query, int *active)
+typedef void (*ClusterKernel)(ClusterParams);
+
+template <int KW>
+static ClusterKernel pick_kernel(bool smemState, bool many)
 {
-    auto kernel = greedy_cluster_kernel<KW, kSmemState>;
+    if (many) return smemState ? greedy_cluster_kernel<KW, true, true> : greedy_cluster_kernel<KW, false, true>;
+    return smemState ? greedy_cluster_kernel<KW, true, false> : greedy_cluster_kernel<KW, false, false>;
+}
+
+static rcd_status launch_cluster(rcd_ctx *ctx, ClusterKernel kernel, const ClusterParams &prm, int C, int clusters, size_t smem, cudaStream_t st, int *active)
+{
     RCD_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     RCD_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     cudaLaunchConfig_t cfg = {};
@@ -612,7 +812,7 @@ static rcd_status launch_cluster(rcd_ctx *ctx, const ClusterParams &prm, int C, 
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (query) {
+    if (active) {                                          // how many such clusters are resident at once
         RCD_CUDA(ctx, cudaOccupancyMaxActiveClusters(active, kernel, &cfg));
         return RCD_OK;
     }
@@ -628,7 +828,7 @@ bool cluster_form_takes(const rcd_ctx *ctx, const Sizes &sz)
     const rcd_config &c = ctx->cfg;
     return c.greedy_path == 0 && c.profile < 2 && c.sweep_batch_max == 0 && c.sweep_mode == 0 && c.async_group == 0 && c.async_help_min == 0 &&
            c.threshold_from == 0 && c.threshold_hit_shift == 0 && c.lazy_mode == 0 && c.lazy_from == 0 && c.dense_ring == 0 &&
-           c.incremental == 0 && c.incremental_max == 0 && sz.W <= kClusterBlocks && sz.maxM <= 65535 && !sz.graphCut && !sz.floatArith;
+           c.incremental == 0 && c.incremental_max == 0 && sz.W <= kClusterBlocks && sz.maxM <= 65535 && sz.d <= 65535 && !sz.graphCut && !sz.floatArith;
 }
 
 rcd_status launch_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, const std::vector<ClassDesc> &descHost,
@@ -669,35 +869,35 @@ rcd_status launch_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const Workspace 
     prm.warps = kMaxWarps;
 
     const size_t cap = (size_t)ctx->maxSmemOptin - 1024;
+    bool many = false;
     auto layout = [&](int C, bool state) -> size_t {
         prm.slots = (sz.W + C - 1) / C;
-        int teams = std::min(kMaxWarps, pow2_at_least(prm.slots));
-        // no more warps per team than a row has work for
-        teams = std::max(teams, kMaxWarps / std::min(kMaxWarps, pow2_at_least((maxLd / 4 + 15) / 16)));
-        prm.teamWarps = kMaxWarps / teams;
+        // a team per block, of as many warps as a row has work for
+        const int most = kMaxWarps / std::min(kMaxWarps, pow2_at_least(prm.slots));
+        prm.teamWarps = std::min(most, pow2_at_least((maxLd / 4 + 31) / 32));
+        many = prm.slots > kMaxWarps;
+        const int teams = kMaxWarps / prm.teamWarps;
         size_t off = 0;
         auto take = [&](size_t bytes) { const size_t at = off; off = (off + bytes + 15) / 16 * 16; return (int32_t)at; };
         prm.offTeams = take(sizeof(Team) * (size_t)teams);
-        prm.offCmd = take(8 * (size_t)(prm.slots + 1));
-        prm.offSeen = take(4 * (size_t)(prm.slots + 1));
+        prm.offCmd = take(8 * (size_t)prm.slots);
         prm.offBits = take((size_t)(maxLd + 31) / 32 * 4);
-        prm.offLists = take(sizeof(Raised) * (size_t)kMaxWarps * (kRaisedPerWarp + 8));
-        prm.offRows = take((size_t)std::min(teams, prm.slots) * maxLd * 4);
+        prm.offLists = take(sizeof(Raised) * (size_t)(kMaxWarps * kRaisedPerWarp + teams));
         prm.offNotes = take(sizeof(Note) * (size_t)sz.W);
         prm.offBars = take(8 * (size_t)sz.W);
+        prm.offRows = take(many ? 0 : (size_t)prm.slots * maxLd * 4);
         prm.offCover = take(state ? (size_t)prm.slots * maxLd * 4 : 0);
-        prm.offGains = take(state ? (size_t)prm.slots * maxLd * 8 : 0);
+        prm.offKeys = take(state ? (size_t)prm.slots * maxLd * 8 : 0);
         return off;
     };
     // Cluster size: as many CTAs per class as there are blocks for and as all classes find room for at once; with more
-    // classes than that, the fewest whose shared memory holds the state.
+    // classes than that, the fewest that keep the state on the chip.
     const int most = std::min(16, pow2_at_least(sz.W));
     int C = 0;
     for (int i = 4; i >= 0; --i) {
         const int size = 1 << i;
         if (ctx->maxClusters[i] == 0) {
-            layout(size, false);
-            rcd_status rs = launch_cluster<4, true>(ctx, prm, size, 1, cap, st, true, &ctx->maxClusters[i]);
+            rcd_status rs = launch_cluster(ctx, pick_kernel<1>(true, false), prm, size, 1, cap, st, &ctx->maxClusters[i]);
             if (rs != RCD_OK) return rs;
         }
         if (size <= most && ctx->maxClusters[i] >= nonEmpty && C == 0) C = size;
@@ -713,12 +913,8 @@ rcd_status launch_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const Workspace 
     const bool state = smem <= cap;
     if (!state) smem = layout(C, false);
     const int clusters = std::max(1, std::min(nonEmpty, ctx->maxClusters[idx]));
-    const int kw = sz.W <= 32 ? 1 : (sz.W <= 64 ? 2 : 4);
-    rcd_status rs;
-    if (state) rs = kw == 1 ? launch_cluster<1, true>(ctx, prm, C, clusters, smem, st, false, nullptr)
-                 : kw == 2 ? launch_cluster<2, true>(ctx, prm, C, clusters, smem, st, false, nullptr)
-                           : launch_cluster<4, true>(ctx, prm, C, clusters, smem, st, false, nullptr);
-    else rs = launch_cluster<4, false>(ctx, prm, C, clusters, smem, st, false, nullptr);
+    ClusterKernel kernel = sz.W <= 32 ? pick_kernel<1>(state, many) : sz.W <= 64 ? pick_kernel<2>(state, many) : pick_kernel<4>(state, many);
+    const rcd_status rs = launch_cluster(ctx, kernel, prm, C, clusters, smem, st, nullptr);
     if (rs != RCD_OK) return rs;
     ctx->steps = sz.maxM;
     ctx->phaseNsDev = ws.phaseNs;
