@@ -117,6 +117,7 @@ size_t layout_workspace(void *base, rcd_feat_dtype dtype, const Sizes &sz, Works
     w.stepOps = c.take<unsigned long long>((size_t)sz.maxM + 1);
     w.phaseNs = c.take<unsigned long long>(kPhaseWords);   // phase clocks, the grid-barrier counter, threshold-pass and row-skipping counters
     w.g0 = c.take<long long>(N);
+    w.fixedExp = c.take<int32_t>(L);
     w.bytes = align_up(c.off);
     if (ws) *ws = w;
     return w.bytes;

@@ -63,6 +63,7 @@ struct ClusterParams {
     const int32_t *quota;
     long long *fval;           // [L][W]
     int32_t *assignment, *order;
+    const int32_t *fixedExp;   // [L] floating-point similarities: S = round(sim * 2^fixedExp) (null: integers)
     const int32_t *classOrder;
     int32_t *counter;
     int32_t *status;
@@ -671,7 +672,8 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
         }
         if (p < W) {
             st_remote(cmdAddr[k], ((unsigned long long)++seq[k] << 32) | kStopCmd);
-            prm.fval[(int64_t)l * W + p] = (long long)(f[k] >> 7);
+            const long long value = (long long)(f[k] >> 7);
+            prm.fval[(int64_t)l * W + p] = prm.fixedExp ? __double_as_longlong(ldexp((double)value, -prm.fixedExp[l])) : value;
         }
     }
     if (lane == 0 && rescans) atomicAdd(prm.stats + 9, (unsigned long long)rescans);
@@ -781,6 +783,40 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) greedy_cluster_kernel
 
 }  // namespace
 
+// Floating-point similarities as fixed-point integers, so that sums of them are exact.  The largest similarity of a class
+// is the largest squared norm (Cauchy-Schwarz), i.e. on the diagonal; it lands in [2^29, 2^30), which leaves every entry
+// an absolute precision of 2^-30 of it: finer than the fp32 dot products themselves (2^-24 of the products they add up).
+__global__ void __launch_bounds__(256, 8) fixed_exponent_kernel(const ClassDesc *__restrict__ desc, const float *__restrict__ S, int32_t *__restrict__ fixedExp)
+{
+    __shared__ float shMax[8];
+    const ClassDesc c = desc[blockIdx.x];
+    float m = 0.f;
+    for (int v = threadIdx.x; v < c.M; v += 256) m = fmaxf(m, S[c.sOff + (int64_t)v * c.ld + v]);
+    for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+    if ((threadIdx.x & 31) == 0) shMax[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) m = fmaxf(m, shMax[w]);
+        int e = 0;
+        if (m > 0.f && m <= 3.4e38f) frexpf(m, &e);         // m = x 2^e, x in [0.5, 1)
+        fixedExp[blockIdx.x] = 30 - e;
+    }
+}
+__global__ void __launch_bounds__(256, 8) fixed_point_kernel(const ClassDesc *__restrict__ desc, const int32_t *__restrict__ fixedExp, float *__restrict__ S)
+{
+    const ClassDesc c = desc[blockIdx.y];
+    const float scale = ldexpf(1.f, fixedExp[blockIdx.y]);
+    float4 *p = reinterpret_cast<float4 *>(S + c.sOff);
+    const int64_t n = (int64_t)c.M * (c.ld >> 2);
+    constexpr int kMost = (1 << 30) - 1;
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
+        const float4 x = p[i];
+        const int4 y = make_int4(min(max(__float2int_rn(x.x * scale), -kMost), kMost), min(max(__float2int_rn(x.y * scale), -kMost), kMost),
+                                 min(max(__float2int_rn(x.z * scale), -kMost), kMost), min(max(__float2int_rn(x.w * scale), -kMost), kMost));
+        reinterpret_cast<int4 *>(p)[i] = y;
+    }
+}
+
 static int pow2_at_least(int x)
 {
     int p = 1;
@@ -828,7 +864,7 @@ bool cluster_form_takes(const rcd_ctx *ctx, const Sizes &sz)
     const rcd_config &c = ctx->cfg;
     return c.greedy_path == 0 && c.profile < 2 && c.sweep_batch_max == 0 && c.sweep_mode == 0 && c.async_group == 0 && c.async_help_min == 0 &&
            c.threshold_from == 0 && c.threshold_hit_shift == 0 && c.lazy_mode == 0 && c.lazy_from == 0 && c.dense_ring == 0 &&
-           c.incremental == 0 && c.incremental_max == 0 && sz.W <= kClusterBlocks && sz.maxM <= 65535 && sz.d <= 65535 && !sz.graphCut && !sz.floatArith;
+           c.incremental == 0 && c.incremental_max == 0 && sz.W <= kClusterBlocks && sz.maxM <= 65535 && sz.d <= 65535 && !sz.graphCut && sz.L <= 65535;
 }
 
 rcd_status launch_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, const std::vector<ClassDesc> &descHost,
@@ -858,6 +894,15 @@ rcd_status launch_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const Workspace 
     prm.fval = (long long *)ws.fval;
     prm.assignment = assignment;
     prm.order = order;
+    prm.fixedExp = sz.floatArith ? ws.fixedExp : nullptr;
+    if (sz.floatArith) {
+        fixed_exponent_kernel<<<sz.L, 256, 0, st>>>(ws.desc, (const float *)ws.S, ws.fixedExp);
+        const int64_t pieces = sz.maxM * (int64_t)(maxLd / 4);
+        const dim3 grid((unsigned)std::min<int64_t>((pieces + 1023) / 1024, std::max(1, 16 * ctx->smCount / sz.L)), (unsigned)sz.L);
+        fixed_point_kernel<<<grid, 256, 0, st>>>(ws.desc, ws.fixedExp, (float *)ws.S);
+        ctx->kernelLaunches += 2;
+        RCD_CUDA(ctx, cudaGetLastError());
+    }
     prm.classOrder = ws.classOrder;
     prm.counter = ws.nSweep;
     prm.status = ws.status;

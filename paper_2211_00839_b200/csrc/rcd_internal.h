@@ -128,6 +128,7 @@ struct Workspace {
     unsigned long long *stepOps;     // [steps+1] element x block pairs of that sweep
     unsigned long long *phaseNs;     // [6] sweep-/pick-phase ns of the persistent kernel, barrier counter, threshold-pass hits / elements / max blocks
     long long *g0;          // [N] cluster form: gain of every sample for an empty block
+    int32_t *fixedExp;      // [L] cluster form, floating-point similarities: S holds round(sim * 2^fixedExp)
     int32_t *status;        // [1]
     size_t bytes;           // total bytes laid out
 };
