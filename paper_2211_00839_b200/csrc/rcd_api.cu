@@ -30,21 +30,29 @@ rcd_status cuda_fail(rcd_ctx *ctx, cudaError_t e, const char *what)
     return fail(ctx, RCD_ERR_CUDA, "CUDA error %d (%s) in %s", (int)e, cudaGetErrorString(e), what);
 }
 
-// Device-side errors of a call are collected in a status word inside the caller's workspace (the kernels'
-// target, ctx->statusDev) and copied into the context's own word when the call has enqueued its last kernel:
-// rcd_sync_status reads only the context's word, so it never touches a workspace the caller may have freed.
+// Device-side errors of a call are collected in a status word of the context (the kernels' target, ctx->statusDev), so
+// rcd_sync_status never touches a workspace the caller may have freed.
 static cudaError_t status_begin(rcd_ctx *ctx, cudaStream_t st)
 {
     ctx->statusDev = ctx->statusOwn;
     return cudaMemsetAsync(ctx->statusOwn, 0, sizeof(int32_t), st);
 }
-static cudaError_t status_publish(rcd_ctx *ctx, cudaStream_t st)
+
+// Pinned memory for what a call's host side hands to the device.  Grows to the largest call; the wait is for the last
+// copy out of it (done long ago unless the context changed streams).
+static rcd_status blob_begin(rcd_ctx *ctx, size_t bytes)
 {
-    cudaError_t e = cudaSuccess;
-    if (ctx->statusDev && ctx->statusDev != ctx->statusOwn)
-        e = cudaMemcpyAsync(ctx->statusOwn, ctx->statusDev, sizeof(int32_t), cudaMemcpyDeviceToDevice, st);
-    ctx->statusDev = ctx->statusOwn;
-    return e;
+    if (ctx->evBlob) RCD_CUDA(ctx, cudaEventSynchronize(ctx->evBlob));
+    else RCD_CUDA(ctx, cudaEventCreateWithFlags(&ctx->evBlob, cudaEventDisableTiming));
+    if (bytes > ctx->hostBlobBytes) {
+        if (ctx->hostBlob) cudaFreeHost(ctx->hostBlob);
+        ctx->hostBlob = nullptr;
+        ctx->hostBlobBytes = 0;
+        const size_t want = align_up(bytes + bytes / 2, 65536);
+        RCD_CUDA(ctx, cudaMallocHost((void **)&ctx->hostBlob, want));
+        ctx->hostBlobBytes = want;
+    }
+    return RCD_OK;
 }
 
 // Bump allocator over the caller's workspace.
@@ -69,15 +77,21 @@ size_t layout_workspace(void *base, rcd_feat_dtype dtype, const Sizes &sz, Works
     const size_t gElem = 8;                                     // int64 gains (fp32 ones use half of it), or 8-byte ties
     Workspace w{};
     // the head does not depend on the class sizes: it is used before they are known
-    w.status = c.take<int32_t>(4);
+    w.status = c.take<int32_t>(4);           // (from here to counts: zeroed by one memset at the start of a call)
+    w.counter = c.take<int32_t>(4);
+    w.phaseNs = c.take<unsigned long long>(kPhaseWords);   // phase clocks, the grid-barrier counter, threshold-pass and row-skipping counters
     w.counts = c.take<int32_t>(L);
     w.nSweep = c.take<int32_t>(4);
-    // everything below is placed once the class sizes are known
+    // what the host computes from the class sizes, copied in one piece
     w.desc = c.take<ClassDesc>(L);
     w.tilePrefix = c.take<int32_t>(L + 1);
+    w.classOrder = c.take<int32_t>(L);
+    w.sizesSorted = c.take<int32_t>(L);
+    w.quota = c.take<int32_t>(L * W);
     w.chunkHist = c.take<int32_t>((size_t)std::max<int32_t>(sz.nChunks, 1) * L);
     w.perm = c.take<int32_t>(N);
-    w.Xs = c.take<unsigned char>(N * (size_t)sz.d * feat_bytes(dtype));
+    // (the head ends here: everything above is placed before the class sizes are known)
+    w.Xs = c.take<unsigned char>(N * (size_t)sz.pitch);
     w.S = c.take<unsigned char>((size_t)std::max<int64_t>(sz.sElems, 1) * sElem);
     w.gaussNorms = c.take<int32_t>(N);
     w.gaussPartial = c.take<double>(L * (size_t)((sz.maxM + 63) / 64 + 1));
@@ -88,7 +102,6 @@ size_t layout_workspace(void *base, rcd_feat_dtype dtype, const Sizes &sz, Works
     w.gains = c.take<unsigned char>((size_t)std::max<int64_t>(sz.vElems, 1) * gElem);
     w.fval = c.take<unsigned char>(L * W * 8);
     w.cnt = c.take<int32_t>(L * W);
-    w.quota = c.take<int32_t>(L * W);
     w.valid = c.take<uint8_t>(L * W);
     w.cand = c.take<int32_t>(N);
     w.pos = c.take<int32_t>(N);
@@ -107,15 +120,12 @@ size_t layout_workspace(void *base, rcd_feat_dtype dtype, const Sizes &sz, Works
     w.sync = c.take<ClassSync>(L);
     w.tickets = c.take<int32_t>(N + L);
     w.sweepF = c.take<long long>(L * 8);
-    w.sizesSorted = c.take<int32_t>(L);
-    w.classOrder = c.take<int32_t>(L);
     w.floorv = c.take<unsigned char>(L * kLazyBlocks * 8);
     w.theta = c.take<unsigned char>(L * kLazyBlocks * 8);
     w.sweepTheta = c.take<unsigned char>(L * kLazyBlocks * 8);
     w.lazyStat = c.take<int32_t>(L * 4);
     w.stepBytes = c.take<unsigned long long>((size_t)sz.maxM + 1);
     w.stepOps = c.take<unsigned long long>((size_t)sz.maxM + 1);
-    w.phaseNs = c.take<unsigned long long>(kPhaseWords);   // phase clocks, the grid-barrier counter, threshold-pass and row-skipping counters
     w.g0 = c.take<long long>(N);
     w.fixedExp = c.take<int32_t>(L);
     w.bytes = align_up(c.off);
@@ -123,12 +133,19 @@ size_t layout_workspace(void *base, rcd_feat_dtype dtype, const Sizes &sz, Works
     return w.bytes;
 }
 
-static int32_t chunks_for(int64_t N) { return (int32_t)((N + kGroupChunk - 1) / kGroupChunk); }
+static int32_t chunks_for(int64_t N) { return (int32_t)((N + group_chunk(N) - 1) / group_chunk(N)); }
 
 // Sizes for the promise "no class larger than Mmax".
 static bool float_arith(const rcd_ctx *ctx, rcd_feat_dtype dtype)
 {
     return dtype == RCD_FEAT_BF16 || ctx->cfg.similarity_kind == RCD_SIM_GAUSSIAN;
+}
+
+// (rows keep their own pitch when the caller asked for the generic similarity kernel)
+static int64_t features_pitch(const rcd_ctx *ctx, rcd_feat_dtype dtype, int64_t d)
+{
+    const int64_t rowBytes = d * (int64_t)feat_bytes(dtype);
+    return ctx->cfg.similarity_path == 2 ? rowBytes : row_pitch(rowBytes);
 }
 
 static Sizes bound_sizes(const rcd_ctx *ctx, rcd_feat_dtype dtype, int64_t N, int64_t d, int32_t L, int64_t Mmax, int32_t W)
@@ -142,6 +159,7 @@ static Sizes bound_sizes(const rcd_ctx *ctx, rcd_feat_dtype dtype, int64_t N, in
     sz.sElems = N * (int64_t)pad_row(Mmax);               // sum M_l * ld_l <= N * pad_row(Mmax)
     sz.vElems = (int64_t)W * (N + 7LL * L);               // sum W * ld_l,  ld_l <= M_l + 7
     sz.nChunks = chunks_for(N);
+    sz.pitch = features_pitch(ctx, dtype, d);
     return sz;
 }
 
@@ -178,8 +196,12 @@ static void quotas_host(int64_t M, const double *r, int32_t W, int32_t *out)
 {
     volatile double sum = 0.0;
     for (int32_t j = 0; j < W; ++j) sum = sum + r[j];
-    std::vector<double> frac((size_t)W);
-    std::vector<int32_t> rank((size_t)W);
+    double fracFew[1024];                                  // (up to 1024 blocks without an allocation)
+    int32_t rankFew[1024];
+    std::vector<double> fracMany(W > 1024 ? (size_t)W : 0);
+    std::vector<int32_t> rankMany(W > 1024 ? (size_t)W : 0);
+    double *frac = W > 1024 ? fracMany.data() : fracFew;
+    int32_t *rank = W > 1024 ? rankMany.data() : rankFew;
     int64_t placed = 0;
     for (int32_t j = 0; j < W; ++j) {
         volatile double numerator = (double)M * r[j];
@@ -190,7 +212,7 @@ static void quotas_host(int64_t M, const double *r, int32_t W, int32_t *out)
         placed += (int64_t)whole;
         rank[(size_t)j] = j;
     }
-    std::stable_sort(rank.begin(), rank.end(), [&](int32_t a, int32_t b) { return frac[(size_t)a] > frac[(size_t)b]; });
+    std::stable_sort(rank, rank + W, [&](int32_t a, int32_t b) { return frac[(size_t)a] > frac[(size_t)b]; });
     int64_t left = M - placed;
     for (size_t k = 0; left > 0; k = (k + 1) % (size_t)W, --left) out[rank[k]] += 1;
     for (size_t k = (size_t)W; left < 0 && k-- > 0;)
@@ -205,31 +227,40 @@ struct Prepared {
     std::vector<ClassDesc> desc;
 };
 
+// capacities null: no quotas wanted.
 static rcd_status prepare(rcd_ctx *ctx, const void *features, rcd_feat_dtype dtype, int64_t N, int64_t d,
-                          const int32_t *labels, int32_t L, int32_t W, void *workspace, size_t workspaceBytes,
+                          const int32_t *labels, int32_t L, int32_t W, const double *capacities, void *workspace, size_t workspaceBytes,
                           cudaStream_t st, Prepared *out)
 {
     if (((uintptr_t)workspace) % kAlign != 0) return fail(ctx, RCD_ERR_INVALID_ARG, "workspace must be 256-byte aligned");
-    // head of the workspace: status, counts
+    // head of the workspace: status, counts, what the host will send, the split's tables
     Sizes head{};
     head.N = N; head.d = d; head.L = L; head.W = W; head.nChunks = chunks_for(N);
     head.floatArith = float_arith(ctx, dtype);
     head.graphCut = ctx->cfg.objective == RCD_OBJ_GRAPH_CUT;
+    head.pitch = features_pitch(ctx, dtype, d);
     Workspace hw{};
-    Sizes tiny = head;
-    layout_workspace(workspace, dtype, tiny, &hw);
-    size_t headBytes = (size_t)((unsigned char *)hw.desc - (unsigned char *)workspace);
+    layout_workspace(workspace, dtype, head, &hw);
+    const size_t headBytes = (size_t)((unsigned char *)hw.Xs - (unsigned char *)workspace);
     if (workspaceBytes < headBytes) return fail(ctx, RCD_ERR_WORKSPACE_TOO_SMALL, "workspace smaller than its %zu-byte head", headBytes);
     if ((size_t)L > ctx->hostStageInts) return fail(ctx, RCD_ERR_UNSUPPORTED, "L=%d exceeds the %zu classes the context can stage", L, ctx->hostStageInts);
 
-    RCD_CUDA(ctx, cudaMemsetAsync(hw.status, 0, 4 * sizeof(int32_t), st));
-    RCD_CUDA(ctx, cudaMemsetAsync(hw.counts, 0, (size_t)L * sizeof(int32_t), st));
-    rcd_status rs = launch_count_labels(ctx, labels, N, L, hw.counts, hw.status, st);
+    const size_t zeroBytes = (size_t)((unsigned char *)(hw.counts + L) - (unsigned char *)hw.status);
+    RCD_CUDA(ctx, cudaMemsetAsync(hw.status, 0, zeroBytes, st));
+    rcd_status rs = launch_label_hist(ctx, labels, N, L, hw.chunkHist, hw.counts, hw.status, ctx->statusOwn, st);
     if (rs != RCD_OK) return rs;
-    RCD_CUDA(ctx, cudaMemcpyAsync(ctx->hostStage, hw.counts, (size_t)L * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-    RCD_CUDA(ctx, cudaMemcpyAsync(ctx->hostStage + L, hw.status, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-    RCD_CUDA(ctx, cudaStreamSynchronize(st));
-    if (ctx->hostStage[L] & kDevBadLabel) return fail(ctx, RCD_ERR_INVALID_ARG, "a label lies outside [0, %d)", L);
+    ctx->statusDev = ctx->statusOwn;
+    // the class sizes come back together with the words before them (the label check's verdict is the first)
+    const size_t statusInts = (size_t)(hw.counts - hw.status);
+    RCD_CUDA(ctx, cudaMemcpyAsync(ctx->hostStage, hw.status, zeroBytes, cudaMemcpyDeviceToHost, st));
+    if (!ctx->evCounts) RCD_CUDA(ctx, cudaEventCreateWithFlags(&ctx->evCounts, cudaEventDisableTiming));
+    RCD_CUDA(ctx, cudaEventRecord(ctx->evCounts, st));
+    const size_t blobBytes = (size_t)((unsigned char *)(hw.quota + (size_t)L * W) - (unsigned char *)hw.desc);
+    rs = blob_begin(ctx, blobBytes);
+    if (rs != RCD_OK) return rs;
+    RCD_CUDA(ctx, cudaEventSynchronize(ctx->evCounts));
+    if (ctx->hostStage[0] & kDevBadLabel) return fail(ctx, RCD_ERR_INVALID_ARG, "a label lies outside [0, %d)", L);
+    const int32_t *counts = ctx->hostStage + statusInts;
 
     Prepared &P = *out;
     P.desc.resize((size_t)L);
@@ -237,7 +268,7 @@ static rcd_status prepare(rcd_ctx *ctx, const void *features, rcd_feat_dtype dty
     int64_t row = 0, sOff = 0, vOff = 0, maxM = 0;
     for (int32_t l = 0; l < L; ++l) {
         ClassDesc c{};
-        c.M = ctx->hostStage[l];
+        c.M = counts[l];
         c.ld = pad_row(c.M);
         c.row0 = (int32_t)row;
         c.sOff = sOff;
@@ -254,38 +285,57 @@ static rcd_status prepare(rcd_ctx *ctx, const void *features, rcd_feat_dtype dty
     if (need > workspaceBytes)
         return fail(ctx, RCD_ERR_WORKSPACE_TOO_SMALL, "workspace has %zu bytes, the class sizes found need %zu", workspaceBytes, need);
     P.sz = sz;
-    ctx->statusDev = P.ws.status;
 
-    RCD_CUDA(ctx, cudaMemcpyAsync(P.ws.desc, P.desc.data(), (size_t)L * sizeof(ClassDesc), cudaMemcpyHostToDevice, st));
-    rs = launch_stable_split(ctx, labels, N, L, sz.nChunks, P.ws.chunkHist, P.ws.desc, P.ws.perm, st);
-    if (rs != RCD_OK) return rs;
-    rs = launch_gather_rows(ctx, features, P.ws.perm, N, d * (int64_t)feat_bytes(dtype), P.ws.Xs, st);
-    if (rs != RCD_OK) return rs;
-    if (ctx->cfg.profile >= 1) RCD_CUDA(ctx, cudaEventRecord(ctx->evPhase[1], st));
+    // descriptors, tile prefixes, classes by size and quotas: one copy from pinned memory
+    auto at = [&](void *dev) { return ctx->hostBlob + ((unsigned char *)dev - (unsigned char *)hw.desc); };
+    memcpy(at(hw.desc), P.desc.data(), (size_t)L * sizeof(ClassDesc));
+    int32_t *prefix = (int32_t *)at(hw.tilePrefix), *order = (int32_t *)at(hw.classOrder), *sorted = (int32_t *)at(hw.sizesSorted);
     SimClasses cls{};
     cls.src.table = P.ws.desc;
     cls.L = L;
     cls.maxM = maxM;
-    {
-        std::vector<int32_t> prefix((size_t)L + 1);
-        int64_t run = 0;
-        for (int32_t l = 0; l < L; ++l) {
-            prefix[(size_t)l] = (int32_t)run;
-            run += sim_tiles(P.desc[(size_t)l].M);
-            if (run > 0x7fffffffLL) return fail(ctx, RCD_ERR_UNSUPPORTED, "too many similarity tiles");
-        }
-        prefix[(size_t)L] = (int32_t)run;
-        cls.upperTiles = run;
-        cls.tilePrefixDev = P.ws.tilePrefix;
-        RCD_CUDA(ctx, cudaMemcpyAsync(P.ws.tilePrefix, prefix.data(), prefix.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+    cls.tilePrefixDev = P.ws.tilePrefix;
+    for (int32_t l = 0; l < L; ++l) {
+        prefix[l] = (int32_t)cls.upperTiles;
+        cls.upperTiles += sim_tiles(P.desc[(size_t)l].M);
+        if (cls.upperTiles > 0x7fffffffLL) return fail(ctx, RCD_ERR_UNSUPPORTED, "too many similarity tiles");
+        order[l] = l;
+        sorted[l] = P.desc[(size_t)l].M;
     }
-    rs = launch_similarity(ctx, P.ws.Xs, dtype, N, d, cls, P.ws.S, st);
+    prefix[L] = (int32_t)cls.upperTiles;
+    auto quotas = [&] {
+        int32_t *quota = (int32_t *)at(hw.quota);
+        for (int32_t l = 0; l < L; ++l) {
+            // (classes of one size have one set of quotas)
+            if (l > 0 && P.desc[(size_t)l].M == P.desc[(size_t)l - 1].M) memcpy(quota + (size_t)l * W, quota + (size_t)(l - 1) * W, (size_t)W * 4);
+            else quotas_host(P.desc[(size_t)l].M, capacities, W, quota + (size_t)l * W);
+        }
+    };
+    if (capacities) {
+        std::sort(sorted, sorted + L);
+        std::stable_sort(order, order + L, [&](int32_t a, int32_t b) { return P.desc[(size_t)a].M > P.desc[(size_t)b].M; });
+    }
+    const bool early = capacities && L <= 64;               // (few quotas: not worth a copy of their own behind the similarity kernel)
+    if (early) quotas();
+    const size_t firstBytes = early ? blobBytes : (size_t)((unsigned char *)hw.quota - (unsigned char *)hw.desc);
+    RCD_CUDA(ctx, cudaMemcpyAsync(P.ws.desc, ctx->hostBlob, firstBytes, cudaMemcpyHostToDevice, st));
+    rs = launch_stable_split(ctx, labels, N, L, P.ws.chunkHist, P.ws.desc, nullptr, nullptr, nullptr, P.ws.perm,
+                             features, d * (int64_t)feat_bytes(dtype), sz.pitch, P.ws.Xs, st);
+    if (rs != RCD_OK) return rs;
+    if (ctx->cfg.profile >= 1) RCD_CUDA(ctx, cudaEventRecord(ctx->evPhase[1], st));
+    const int64_t dPitch = sz.pitch / (int64_t)feat_bytes(dtype);
+    rs = launch_similarity(ctx, P.ws.Xs, dtype, N, dPitch, cls, P.ws.S, st);
     if (rs != RCD_OK) return rs;
     if (ctx->cfg.similarity_kind == RCD_SIM_GAUSSIAN) {
-        rs = launch_gaussian(ctx, P.ws.Xs, dtype, N, d, cls, P.ws.S, P.ws.gaussNorms, P.ws.gaussPartial, P.ws.gaussSigma,
+        rs = launch_gaussian(ctx, P.ws.Xs, dtype, N, dPitch, cls, P.ws.S, P.ws.gaussNorms, P.ws.gaussPartial, P.ws.gaussSigma,
                              P.ws.gaussScale, st);
         if (rs != RCD_OK) return rs;
     }
+    if (capacities && !early) {
+        quotas();
+        RCD_CUDA(ctx, cudaMemcpyAsync(P.ws.quota, at(hw.quota), (size_t)L * W * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+    }
+    RCD_CUDA(ctx, cudaEventRecord(ctx->evBlob, st));
     if (ctx->cfg.profile >= 1) RCD_CUDA(ctx, cudaEventRecord(ctx->evPhase[2], st));
     return RCD_OK;
 }
@@ -340,7 +390,7 @@ rcd_status rcd_create(rcd_ctx **out, int cuda_device, const rcd_config *cfg)
     ctx->cooperative = prop.cooperativeLaunch != 0;
     if (cfg) ctx->cfg = *cfg;
     ctx->hostStageInts = 1 << 20;
-    if (cudaMallocHost((void **)&ctx->hostStage, (ctx->hostStageInts + 16) * sizeof(int32_t)) != cudaSuccess) {
+    if (cudaMallocHost((void **)&ctx->hostStage, (ctx->hostStageInts + 512) * sizeof(int32_t)) != cudaSuccess) {
         delete ctx;
         return RCD_ERR_CUDA;
     }
@@ -361,6 +411,9 @@ void rcd_destroy(rcd_ctx *ctx)
     for (auto &e : ctx->evPhase) if (e) cudaEventDestroy(e);
     for (auto &e : ctx->evSweep) cudaEventDestroy(e);
     if (ctx->hostStage) cudaFreeHost(ctx->hostStage);
+    if (ctx->hostBlob) cudaFreeHost(ctx->hostBlob);
+    if (ctx->evBlob) cudaEventDestroy(ctx->evBlob);
+    if (ctx->evCounts) cudaEventDestroy(ctx->evCounts);
     if (ctx->statusOwn) cudaFree(ctx->statusOwn);
     delete ctx;
 }
@@ -458,7 +511,6 @@ rcd_status rcd_quotas(int64_t M, const double *capacities_host, int32_t W, int32
 struct ListsWorkspace {
     int32_t *status;      // [4]
     int32_t *counts;      // [W]
-    ClassDesc *desc;      // [W] (only row0 is used: where a worker's list starts)
     int32_t *chunkHist;   // [nChunks][W]
     size_t bytes;
 };
@@ -470,7 +522,6 @@ static size_t layout_lists(void *base, int64_t N, int32_t W, ListsWorkspace *out
     const size_t Wn = (size_t)std::max<int32_t>(W, 1);
     w.status = c.take<int32_t>(4);
     w.counts = c.take<int32_t>(Wn);
-    w.desc = c.take<ClassDesc>(Wn);
     w.chunkHist = c.take<int32_t>((size_t)std::max<int32_t>(chunks_for(N), 1) * Wn);
     w.bytes = align_up(c.off);
     if (out) *out = w;
@@ -499,37 +550,19 @@ rcd_status rcd_worker_lists(rcd_ctx *ctx, const int32_t *assignment_dev, int64_t
     cudaStream_t st = (cudaStream_t)cuda_stream;
     RCD_CUDA(ctx, cudaSetDevice(ctx->device));
     ctx->kernelLaunches = 0;
-    RCD_CUDA(ctx, status_begin(ctx, st));
-    ctx->statusDev = ws.status;
-    RCD_CUDA(ctx, cudaMemsetAsync(ws.status, 0, 4 * sizeof(int32_t), st));
-    RCD_CUDA(ctx, cudaMemsetAsync(ws.counts, 0, (size_t)W * sizeof(int32_t), st));
-    // sizes of the lists (a histogram of the block numbers), read back: they fix where each list starts
-    rcd_status rs = launch_count_labels(ctx, assignment_dev, N, W, ws.counts, ws.status, st);
+    ctx->statusDev = ctx->statusOwn;
+    RCD_CUDA(ctx, cudaMemsetAsync(ws.status, 0, (size_t)((unsigned char *)(ws.counts + W) - (unsigned char *)ws.status), st));
+    rcd_status rs = launch_label_hist(ctx, assignment_dev, N, W, ws.chunkHist, ws.counts, ws.status, ctx->statusOwn, st);
     if (rs != RCD_OK) return rs;
-    RCD_CUDA(ctx, cudaMemcpyAsync(ctx->hostStage, ws.counts, (size_t)W * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-    RCD_CUDA(ctx, cudaMemcpyAsync(ctx->hostStage + W, ws.status, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-    RCD_CUDA(ctx, cudaStreamSynchronize(st));
-    if (ctx->hostStage[W] & kDevBadLabel) return fail(ctx, RCD_ERR_INVALID_ARG, "an assignment entry lies outside [0, %d)", W);
-    std::vector<ClassDesc> desc((size_t)W);
-    std::vector<int64_t> offsets((size_t)W + 1);
-    int64_t run = 0;
-    for (int32_t j = 0; j < W; ++j) {
-        ClassDesc c{};
-        c.M = ctx->hostStage[j];
-        c.row0 = (int32_t)run;
-        desc[(size_t)j] = c;
-        offsets[(size_t)j] = run;
-        run += c.M;
-    }
-    offsets[(size_t)W] = run;
-    if (run != N) return fail(ctx, RCD_ERR_INTERNAL, "list sizes sum to %lld, expected %lld", (long long)run, (long long)N);
-    // (pageable host memory: the runtime stages these copies before it returns)
-    RCD_CUDA(ctx, cudaMemcpyAsync(offsets_dev, offsets.data(), offsets.size() * sizeof(int64_t), cudaMemcpyHostToDevice, st));
-    RCD_CUDA(ctx, cudaMemcpyAsync(ws.desc, desc.data(), desc.size() * sizeof(ClassDesc), cudaMemcpyHostToDevice, st));
-    // a stable split by block number: inside a list the dataset indices ascend
-    rs = launch_stable_split(ctx, assignment_dev, N, W, chunks_for(N), ws.chunkHist, ws.desc, indices_dev, st);
+    RCD_CUDA(ctx, cudaMemcpyAsync(ctx->hostStage, ws.status, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    if (!ctx->evCounts) RCD_CUDA(ctx, cudaEventCreateWithFlags(&ctx->evCounts, cudaEventDisableTiming));
+    RCD_CUDA(ctx, cudaEventRecord(ctx->evCounts, st));
+    // the list boundaries are sums of the sizes, and a stable split by block number fills the lists (inside a list the
+    // dataset indices ascend): enqueued behind the check of the entries, whose verdict they read themselves
+    rs = launch_stable_split(ctx, assignment_dev, N, W, ws.chunkHist, nullptr, ws.counts, offsets_dev, ws.status, indices_dev, nullptr, 0, 0, nullptr, st);
     if (rs != RCD_OK) return rs;
-    RCD_CUDA(ctx, status_publish(ctx, st));
+    RCD_CUDA(ctx, cudaEventSynchronize(ctx->evCounts));
+    if (ctx->hostStage[0] & kDevBadLabel) return fail(ctx, RCD_ERR_INVALID_ARG, "an assignment entry lies outside [0, %d)", W);
     return RCD_OK;
 }
 
@@ -661,27 +694,27 @@ rcd_status rcd_partition(rcd_ctx *ctx, const void *features_dev, rcd_feat_dtype 
     ctx->phaseNsDev = nullptr;
     ctx->sweepEventsUsed = 0;
     const bool prof = ctx->cfg.profile >= 1;
-    RCD_CUDA(ctx, status_begin(ctx, st));
     if (prof) RCD_CUDA(ctx, cudaEventRecord(ctx->evPhase[0], st));
 
     Prepared P;
-    rs = prepare(ctx, features_dev, dtype, N, d, labels_dev, L, W, workspace_dev, workspace_bytes, st, &P);
+    rs = prepare(ctx, features_dev, dtype, N, d, labels_dev, L, W, capacities_host, workspace_dev, workspace_bytes, st, &P);
     if (rs != RCD_OK) return rs;
 
-    std::vector<int32_t> quota((size_t)L * W);
-    for (int32_t l = 0; l < L; ++l) quotas_host(P.desc[(size_t)l].M, capacities_host, W, quota.data() + (size_t)l * W);
-    RCD_CUDA(ctx, cudaMemcpyAsync(P.ws.quota, quota.data(), quota.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-
-    if (P.sz.graphCut) rs = launch_cut(ctx, P.sz, P.ws, assignment_dev, order_dev_or_null, st);
-    else if (cluster_form_takes(ctx, P.sz) && P.sz.maxM > 0) rs = launch_greedy_cluster(ctx, P.sz, P.ws, P.desc, assignment_dev, order_dev_or_null, st);
-    else rs = launch_greedy(ctx, P.sz.floatArith ? RCD_FEAT_BF16 : RCD_FEAT_I8, P.sz, P.ws, P.desc, assignment_dev, order_dev_or_null, st);
+    bool valuesWritten = false;
+    if (P.sz.graphCut) {
+        rs = launch_cut(ctx, P.sz, P.ws, assignment_dev, order_dev_or_null, st);
+    } else if (P.sz.maxM > 0 && cluster_form_takes(ctx, P.sz, P.desc)) {
+        valuesWritten = true;
+        rs = launch_greedy_cluster(ctx, P.sz, P.ws, P.desc, assignment_dev, order_dev_or_null, part_values_dev_or_null, st);
+    } else {
+        rs = launch_greedy(ctx, P.sz.floatArith ? RCD_FEAT_BF16 : RCD_FEAT_I8, P.sz, P.ws, P.desc, assignment_dev, order_dev_or_null, st);
+    }
     if (rs != RCD_OK) return rs;
     if (prof) RCD_CUDA(ctx, cudaEventRecord(ctx->evPhase[3], st));
-    if (part_values_dev_or_null) {
+    if (part_values_dev_or_null && !valuesWritten) {
         if (P.sz.maxM == 0) RCD_CUDA(ctx, cudaMemsetAsync(part_values_dev_or_null, 0, (size_t)L * W * 8, st));
         else RCD_CUDA(ctx, cudaMemcpyAsync(part_values_dev_or_null, P.ws.fval, (size_t)L * W * 8, cudaMemcpyDeviceToDevice, st));
     }
-    RCD_CUDA(ctx, status_publish(ctx, st));
     if (prof) {
         RCD_CUDA(ctx, cudaEventRecord(ctx->evPhase[4], st));
         ctx->phaseValid = true;
@@ -782,11 +815,10 @@ rcd_status rcd_objective(rcd_ctx *ctx, const void *features_dev, rcd_feat_dtype 
     if (!workspace_dev) return fail(ctx, RCD_ERR_INVALID_ARG, "workspace is null");
     cudaStream_t st = (cudaStream_t)cuda_stream;
     RCD_CUDA(ctx, cudaSetDevice(ctx->device));
-    RCD_CUDA(ctx, status_begin(ctx, st));
     const int savedProfile = ctx->cfg.profile;
     ctx->cfg.profile = 0;
     Prepared P;
-    rs = prepare(ctx, features_dev, dtype, N, d, labels_dev, L, W, workspace_dev, workspace_bytes, st, &P);
+    rs = prepare(ctx, features_dev, dtype, N, d, labels_dev, L, W, nullptr, workspace_dev, workspace_bytes, st, &P);
     ctx->cfg.profile = savedProfile;
     if (rs != RCD_OK) return rs;
     size_t scratchB = objective_scratch_bytes(L, P.sz.maxM, W);
@@ -798,9 +830,7 @@ rcd_status rcd_objective(rcd_ctx *ctx, const void *features_dev, rcd_feat_dtype 
     else
         rs = launch_objective(ctx, P.sz.floatArith ? RCD_FEAT_BF16 : RCD_FEAT_I8, P.sz, P.ws.desc, P.desc, P.ws.S, P.ws.perm, assignment_dev,
                               part_values_dev, total_dev, scratch, st);
-    if (rs != RCD_OK) return rs;
-    RCD_CUDA(ctx, status_publish(ctx, st));
-    return RCD_OK;
+    return rs;
 }
 
 }  // extern "C"

@@ -859,28 +859,23 @@ static rcd_status launch_cluster(rcd_ctx *ctx, ClusterKernel kernel, const Clust
 
 // Whether the cluster form takes a problem: chosen by the library (no pass-based form or option asked for), samples of
 // a class and blocks within the packed keys' range.
-bool cluster_form_takes(const rcd_ctx *ctx, const Sizes &sz)
+bool cluster_form_takes(const rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &)
 {
     const rcd_config &c = ctx->cfg;
     return c.greedy_path == 0 && c.profile < 2 && c.sweep_batch_max == 0 && c.sweep_mode == 0 && c.async_group == 0 && c.async_help_min == 0 &&
            c.threshold_from == 0 && c.threshold_hit_shift == 0 && c.lazy_mode == 0 && c.lazy_from == 0 && c.dense_ring == 0 &&
-           c.incremental == 0 && c.incremental_max == 0 && sz.W <= kClusterBlocks && sz.maxM <= 65535 && sz.d <= 65535 && !sz.graphCut && sz.L <= 65535;
+           c.incremental == 0 && c.incremental_max == 0 && sz.W <= kClusterBlocks && sz.maxM <= 65535 && sz.d <= 65535 && !sz.graphCut && sz.L <= 65535 &&
+           (sz.L <= ctx->smCount || sz.maxM <= 512);
 }
 
 rcd_status launch_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, const std::vector<ClassDesc> &descHost,
-                                 int32_t *assignment, int32_t *order, cudaStream_t st)
+                                 int32_t *assignment, int32_t *order, void *partValues, cudaStream_t st)
 {
     int nonEmpty = 0, maxLd = 8;
-    std::vector<int32_t> bySize(descHost.size());
-    for (size_t i = 0; i < bySize.size(); ++i) {
-        bySize[i] = (int32_t)i;
-        if (descHost[i].M > 0) ++nonEmpty;
-        maxLd = std::max(maxLd, (int)descHost[i].ld);
+    for (const ClassDesc &c : descHost) {
+        if (c.M > 0) ++nonEmpty;
+        maxLd = std::max(maxLd, (int)c.ld);
     }
-    std::stable_sort(bySize.begin(), bySize.end(), [&](int32_t a, int32_t b) { return descHost[(size_t)a].M > descHost[(size_t)b].M; });
-    RCD_CUDA(ctx, cudaMemcpyAsync(ws.classOrder, bySize.data(), bySize.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-    RCD_CUDA(ctx, cudaMemsetAsync(ws.nSweep, 0, 4 * sizeof(int32_t), st));
-    RCD_CUDA(ctx, cudaMemsetAsync(ws.phaseNs, 0, kPhaseWords * sizeof(unsigned long long), st));
 
     ClusterParams prm{};
     prm.desc = ws.desc;
@@ -891,7 +886,7 @@ rcd_status launch_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const Workspace 
     prm.picks = (uint32_t *)ws.cand;
     prm.perm = ws.perm;
     prm.quota = ws.quota;
-    prm.fval = (long long *)ws.fval;
+    prm.fval = (long long *)(partValues ? partValues : ws.fval);
     prm.assignment = assignment;
     prm.order = order;
     prm.fixedExp = sz.floatArith ? ws.fixedExp : nullptr;
@@ -904,8 +899,8 @@ rcd_status launch_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const Workspace 
         RCD_CUDA(ctx, cudaGetLastError());
     }
     prm.classOrder = ws.classOrder;
-    prm.counter = ws.nSweep;
-    prm.status = ws.status;
+    prm.counter = ws.counter;
+    prm.status = ctx->statusOwn;
     prm.stats = ws.phaseNs;
     prm.L = sz.L;
     prm.W = sz.W;

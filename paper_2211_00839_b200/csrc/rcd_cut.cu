@@ -230,7 +230,7 @@ static rcd_status run_cut(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, in
     prm.perm = ws.perm;
     prm.assignment = assignment;
     prm.order = order;
-    prm.status = ws.status;
+    prm.status = ctx->statusOwn;
     prm.L = sz.L;
     prm.W = sz.W;
     cut_chain_kernel<SV><<<sz.L, kCutThreads, 0, st>>>(prm);

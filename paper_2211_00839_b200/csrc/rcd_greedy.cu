@@ -2405,7 +2405,7 @@ static rcd_status run_greedy(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws,
     prm.stepOps = ws.stepOps;
     prm.phaseNs = ws.phaseNs;
     prm.barrier = (unsigned *)(ws.phaseNs + 2);
-    prm.status = ws.status;
+    prm.status = ctx->statusOwn;
     prm.perm = ws.perm;
     prm.assignment = assignment;
     prm.order = order;
@@ -2433,26 +2433,15 @@ static rcd_status run_greedy(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws,
     prm.asyncGroup = 1;
     prm.helpMin = 1;
     {
-        std::vector<int32_t> sorted;
-        sorted.reserve(descHost.size());
-        for (const auto &c : descHost) sorted.push_back(c.M);
-        std::sort(sorted.begin(), sorted.end());
         prm.sizesSorted = ws.sizesSorted;
         prm.classOrder = ws.classOrder;
-        {
-            std::vector<int32_t> order(descHost.size());
-            for (size_t i = 0; i < order.size(); ++i) order[i] = (int32_t)i;
-            std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) { return descHost[(size_t)a].M > descHost[(size_t)b].M; });
-            RCD_CUDA(ctx, cudaMemcpyAsync(ws.classOrder, order.data(), order.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-        }
         prm.nonEmpty = 0;
         prm.minM = 0;
-        for (int32_t m : sorted) {
-            if (m <= 0) continue;
-            if (prm.nonEmpty == 0) prm.minM = m;
+        for (const auto &c : descHost) {
+            if (c.M <= 0) continue;
+            prm.minM = prm.nonEmpty == 0 ? c.M : std::min<int32_t>(prm.minM, c.M);
             ++prm.nonEmpty;
         }
-        RCD_CUDA(ctx, cudaMemcpyAsync(ws.sizesSorted, sorted.data(), sorted.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     }
     int maxLd = 0;
     for (const auto &c : descHost) if (c.ld > maxLd) maxLd = c.ld;

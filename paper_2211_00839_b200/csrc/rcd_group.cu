@@ -4,14 +4,179 @@
 // dataset order, which is what fixes the lowest-index tie-breaks downstream.
 #include "rcd_internal.h"
 
+#include <algorithm>
+
 namespace rcd {
 
-// ---- label histogram ------------------------------------------------------------------------
+// ---- stable split ---------------------------------------------------------------------------
+// Chunks of consecutive samples (group_chunk(N) of them).  Three launches:
+//   histogram  a CTA per chunk counts its labels in shared memory, writes chunkHist[chunk][label] and adds to counts[label];
+//   scan       per label, exclusive running sum over the chunks, started at the class offset;
+//   place      position = chunk base + rank inside the chunk; the CTA then copies its feature rows to their places.
+// Up to kMaxSharedLabels labels the counters of a chunk sit in shared memory (a sample costs one shared-memory atomic
+// and one warp match, against 1024 comparisons per sample and one global atomic before: 1.3 M samples over 64 labels
+// 1155 -> 40 us).  More labels than that take the kernels at the end of this section.
+constexpr int kGroupThreads = 256;
+constexpr int kGroupWarps = kGroupThreads / 32;
+constexpr int kMaxSharedLabels = 6000;      // kGroupWarps counters per label: 192 KB
+
+__global__ void __launch_bounds__(kGroupThreads) label_hist_kernel(const int32_t *__restrict__ labels, int64_t N, int32_t L, int32_t chunk,
+                                                                  int32_t *__restrict__ chunkHist, int32_t *__restrict__ counts,
+                                                                  int32_t *__restrict__ status, int32_t *__restrict__ callStatus)
+{
+    extern __shared__ int32_t shCount[];
+    if (callStatus && blockIdx.x == 0 && threadIdx.x == 0) *callStatus = 0;       // (the word the later kernels report to)
+    for (int l = threadIdx.x; l < L; l += kGroupThreads) shCount[l] = 0;
+    __syncthreads();
+    const int64_t base = (int64_t)blockIdx.x * chunk;
+    const int n = (int)min((int64_t)chunk, N - base);
+    bool bad = false;
+    for (int i = threadIdx.x; i < n; i += kGroupThreads) {
+        const int32_t lab = labels[base + i];
+        if (lab < 0 || lab >= L) bad = true;
+        else atomicAdd(&shCount[lab], 1);
+    }
+    if (bad) atomicOr(status, kDevBadLabel);
+    __syncthreads();
+    for (int l = threadIdx.x; l < L; l += kGroupThreads) {
+        const int32_t c = shCount[l];
+        chunkHist[(int64_t)blockIdx.x * L + l] = c;
+        if (c) atomicAdd(&counts[l], c);
+    }
+}
+
+// Exclusive sums over the chunks for 32 labels per CTA: thread (x, y) takes label x and the y-th of 32 runs of chunks.
+// start: where label l begins (desc[l].row0), or null: after the counts of the labels below it.
+__global__ void __launch_bounds__(1024) label_scan_kernel(int32_t *__restrict__ chunkHist, int32_t nChunks, int32_t L,
+                                                         const ClassDesc *__restrict__ desc, const int32_t *__restrict__ counts,
+                                                         int64_t *__restrict__ offsets, const int32_t *__restrict__ status)
+{
+    __shared__ int32_t shRun[32][33];
+    __shared__ int32_t shStart[33];
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+    const int l = blockIdx.x * 32 + x;
+    const int per = (nChunks + 31) / 32;
+    const int c0 = min(nChunks, y * per), c1 = min(nChunks, c0 + per);
+    int32_t sum = 0;
+    if (l < L)
+        for (int c = c0; c < c1; ++c) sum += chunkHist[(int64_t)c * L + l];
+    shRun[y][x] = sum;
+    if (!desc) {
+        // labels below this CTA's, by its first warp; then the 32 of its own
+        if (y == 0) {
+            int32_t below = 0;
+            for (int i = x; i < (int)blockIdx.x * 32; i += 32) below += counts[i];
+            below = __reduce_add_sync(0xffffffffu, below);
+            int32_t run = l < L ? counts[l] : 0;
+            const int32_t own = run;
+            for (int off = 1; off < 32; off <<= 1) {
+                const int32_t up = __shfl_up_sync(0xffffffffu, run, off);
+                if (x >= off) run += up;
+            }
+            shStart[x] = below + run - own;
+            if (offsets && !(*status & kDevBadLabel)) {
+                if (l < L) offsets[l] = below + run - own;
+                if (l == L - 1) offsets[L] = below + run;
+            }
+        }
+    } else if (y == 0) {
+        shStart[x] = l < L ? desc[l].row0 : 0;
+    }
+    __syncthreads();
+    if (y == 0) {
+        int32_t run = shStart[x];
+        for (int k = 0; k < 32; ++k) {
+            const int32_t h = shRun[k][x];
+            shRun[k][x] = run;
+            run += h;
+        }
+    }
+    __syncthreads();
+    if (l < L) {
+        int32_t run = shRun[y][x];
+        for (int c = c0; c < c1; ++c) {
+            const int64_t at = (int64_t)c * L + l;
+            const int32_t h = chunkHist[at];
+            chunkHist[at] = run;
+            run += h;
+        }
+    }
+}
+
+// Copies one row of `bytes` to a row of `pitch` >= bytes (the rest zeros) by one warp.
+__device__ __forceinline__ void copy_row(const uint8_t *__restrict__ src, uint8_t *__restrict__ dst, int64_t bytes, int64_t pitch, bool vec, int lane)
+{
+    if (vec) {
+        const int4 *s = reinterpret_cast<const int4 *>(src);
+        int4 *d = reinterpret_cast<int4 *>(dst);
+        const int n = (int)(bytes >> 4), np = (int)(pitch >> 4);
+        int i = lane;
+        for (; i + 96 < n; i += 128) {
+            const int4 a = __ldg(s + i), b = __ldg(s + i + 32), c = __ldg(s + i + 64), e = __ldg(s + i + 96);
+            d[i] = a; d[i + 32] = b; d[i + 64] = c; d[i + 96] = e;
+        }
+        for (; i < np; i += 32) d[i] = i < n ? __ldg(s + i) : make_int4(0, 0, 0, 0);
+    } else {
+        for (int64_t i = lane; i < pitch; i += 32) dst[i] = i < bytes ? src[i] : (uint8_t)0;
+    }
+}
+
+__global__ void __launch_bounds__(kGroupThreads) label_place_kernel(const int32_t *__restrict__ labels, int64_t N, int32_t L, int32_t chunk,
+                                                                   const int32_t *__restrict__ chunkBase, int32_t *__restrict__ perm,
+                                                                   const uint8_t *__restrict__ X, int64_t rowBytes, int64_t pitch,
+                                                                   uint8_t *__restrict__ Xs, const int32_t *__restrict__ status)
+{
+    extern __shared__ int32_t shWarp[];                 // [kGroupWarps][L] counters, then [chunk] positions
+    if (status && (*status & kDevBadLabel)) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int32_t *mine = shWarp + (size_t)warp * L;
+    int32_t *shPos = shWarp + (size_t)kGroupWarps * L;
+    const int64_t base = (int64_t)blockIdx.x * chunk;
+    const int n = (int)min((int64_t)chunk, N - base);
+    const int per = chunk / kGroupWarps;                // a warp's run of consecutive samples (a multiple of 32)
+    for (int l = lane; l < L; l += 32) mine[l] = 0;
+    __syncwarp();
+    const int i0 = warp * per, i1 = min(n, i0 + per);
+    for (int i = i0 + lane; i < i1; i += 32) atomicAdd(&mine[labels[base + i]], 1);
+    __syncthreads();
+    for (int l = threadIdx.x; l < L; l += kGroupThreads) {
+        int32_t run = chunkBase[(int64_t)blockIdx.x * L + l];
+        for (int w = 0; w < kGroupWarps; ++w) {
+            const int32_t c = shWarp[(size_t)w * L + l];
+            shWarp[(size_t)w * L + l] = run;
+            run += c;
+        }
+    }
+    __syncthreads();
+    for (int i = i0; i < i1; i += 32) {
+        const bool in = i + lane < i1;
+        const int32_t lab = in ? labels[base + i + lane] : -1;
+        const unsigned same = __match_any_sync(0xffffffffu, lab);
+        const int rank = __popc(same & ((1u << lane) - 1u));
+        int32_t pos = 0;
+        if (in) pos = mine[lab] + rank;
+        __syncwarp();
+        if (in && rank == 0) mine[lab] = pos + __popc(same);
+        __syncwarp();
+        if (in) {
+            perm[pos] = (int32_t)(base + i + lane);
+            if (Xs) shPos[i + lane] = pos;
+        }
+    }
+    if (!Xs) return;
+    __syncthreads();
+    const bool vec = rowBytes % 16 == 0 && pitch % 16 == 0 && ((uintptr_t)X) % 16 == 0 && ((uintptr_t)Xs) % 16 == 0;
+    for (int i = warp; i < n; i += kGroupWarps)
+        copy_row(X + (base + i) * rowBytes, Xs + (int64_t)shPos[i] * pitch, rowBytes, pitch, vec, lane);
+}
+
+// ---- more labels than fit shared memory ------------------------------------------------------
 __global__ void count_labels_kernel(const int32_t *__restrict__ labels, int64_t N, int32_t L,
-                                    int32_t *__restrict__ counts, int32_t *__restrict__ status)
+                                    int32_t *__restrict__ counts, int32_t *__restrict__ status, int32_t *__restrict__ callStatus)
 {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     bool bad = false;
+    if (callStatus && blockIdx.x == 0 && threadIdx.x == 0) *callStatus = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += stride) {
         int32_t lab = labels[i];
         if (lab < 0 || lab >= L) { bad = true; continue; }
@@ -19,25 +184,6 @@ __global__ void count_labels_kernel(const int32_t *__restrict__ labels, int64_t 
     }
     if (bad) atomicOr(status, kDevBadLabel);
 }
-
-rcd_status launch_count_labels(rcd_ctx *ctx, const int32_t *labels, int64_t N, int32_t L, int32_t *counts,
-                               int32_t *status, cudaStream_t st)
-{
-    if (N == 0) return RCD_OK;
-    int threads = 256;
-    int64_t blocks = (N + threads - 1) / threads;
-    if (blocks > 4LL * ctx->smCount) blocks = 4LL * ctx->smCount;
-    count_labels_kernel<<<(unsigned)blocks, threads, 0, st>>>(labels, N, L, counts, status);
-    ctx->kernelLaunches++;
-    RCD_CUDA(ctx, cudaGetLastError());
-    return RCD_OK;
-}
-
-// ---- stable split ---------------------------------------------------------------------------
-// Chunks of kGroupChunk consecutive samples.  Pass A: per chunk and label, how many samples of
-// that label the chunk holds (written by the chunk's last sample of the label).  Pass B: per
-// label, exclusive running sum over chunks, started at the class offset.  Pass C: position =
-// chunk base + rank inside the chunk.
 
 __device__ __forceinline__ void chunk_rank(const int32_t *sh, int n, int t, int lab, int &rank, bool &last)
 {
@@ -52,12 +198,15 @@ __device__ __forceinline__ void chunk_rank(const int32_t *sh, int n, int t, int 
     }
 }
 
-__global__ void __launch_bounds__(kGroupChunk, 1) chunk_hist_kernel(const int32_t *__restrict__ labels, int64_t N,
-                                                                int32_t L, int32_t *__restrict__ chunkHist)
+// hist: writes how many samples of the label the chunk holds (by the chunk's last sample of the label); else: places
+template <bool kHist>
+__global__ void __launch_bounds__(1024, 1) chunk_rank_kernel(const int32_t *__restrict__ labels, int64_t N, int32_t L, int32_t chunk,
+                                                            int32_t *__restrict__ chunkHist, int32_t *__restrict__ perm, const int32_t *__restrict__ status)
 {
-    __shared__ int32_t sh[kGroupChunk];
-    int64_t base = (int64_t)blockIdx.x * kGroupChunk;
-    int n = (int)min((int64_t)kGroupChunk, N - base);
+    __shared__ int32_t sh[1024];
+    if (!kHist && status && (*status & kDevBadLabel)) return;
+    int64_t base = (int64_t)blockIdx.x * chunk;
+    int n = (int)min((int64_t)chunk, N - base);
     int t = threadIdx.x;
     int lab = -1;
     if (t < n) lab = labels[base + t];
@@ -66,94 +215,78 @@ __global__ void __launch_bounds__(kGroupChunk, 1) chunk_hist_kernel(const int32_
     if (t < n && lab >= 0 && lab < L) {
         int rank; bool last;
         chunk_rank(sh, n, t, lab, rank, last);
-        if (last) chunkHist[(int64_t)blockIdx.x * L + lab] = rank + 1;
+        const int64_t at = (int64_t)blockIdx.x * L + lab;
+        if (!kHist) perm[chunkHist[at] + rank] = (int32_t)(base + t);
+        else if (last) chunkHist[at] = rank + 1;
     }
 }
 
-__global__ void chunk_scan_kernel(int32_t *__restrict__ chunkHist, int32_t nChunks, int32_t L,
-                                  const ClassDesc *__restrict__ desc)
+__global__ void __launch_bounds__(256) gather_rows_kernel(const uint8_t *__restrict__ X, const int32_t *__restrict__ perm, int64_t N,
+                                                          int64_t rowBytes, int64_t pitch, uint8_t *__restrict__ Xs)
 {
-    int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= L) return;
-    int32_t run = desc[l].row0;
-    for (int c = 0; c < nChunks; ++c) {
-        int64_t at = (int64_t)c * L + l;
-        int32_t h = chunkHist[at];
-        chunkHist[at] = run;
-        run += h;
-    }
+    const int lane = threadIdx.x & 31;
+    const bool vec = rowBytes % 16 == 0 && pitch % 16 == 0 && ((uintptr_t)X) % 16 == 0 && ((uintptr_t)Xs) % 16 == 0;
+    for (int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); r < N; r += (int64_t)gridDim.x * 8)
+        copy_row(X + (int64_t)perm[r] * rowBytes, Xs + r * pitch, rowBytes, pitch, vec, lane);
 }
 
-__global__ void __launch_bounds__(kGroupChunk, 1) chunk_place_kernel(const int32_t *__restrict__ labels, int64_t N,
-                                                                 int32_t L, const int32_t *__restrict__ chunkBase,
-                                                                 int32_t *__restrict__ perm)
-{
-    __shared__ int32_t sh[kGroupChunk];
-    int64_t base = (int64_t)blockIdx.x * kGroupChunk;
-    int n = (int)min((int64_t)kGroupChunk, N - base);
-    int t = threadIdx.x;
-    int lab = -1;
-    if (t < n) lab = labels[base + t];
-    sh[t] = lab;
-    __syncthreads();
-    if (t < n && lab >= 0 && lab < L) {
-        int rank; bool last;
-        chunk_rank(sh, n, t, lab, rank, last);
-        perm[chunkBase[(int64_t)blockIdx.x * L + lab] + rank] = (int32_t)(base + t);
-    }
-}
+static bool shared_labels(int32_t L) { return L <= kMaxSharedLabels; }
 
-rcd_status launch_stable_split(rcd_ctx *ctx, const int32_t *labels, int64_t N, int32_t L, int32_t nChunks,
-                               int32_t *chunkHist, const ClassDesc *descDev, int32_t *perm, cudaStream_t st)
+// Histogram of the labels: counts[L] (zeroed by the caller, like *status), and per chunk.
+rcd_status launch_label_hist(rcd_ctx *ctx, const int32_t *labels, int64_t N, int32_t L, int32_t *chunkHist, int32_t *counts,
+                             int32_t *status, int32_t *callStatus, cudaStream_t st)
 {
-    if (N == 0) return RCD_OK;
-    RCD_CUDA(ctx, cudaMemsetAsync(chunkHist, 0, (size_t)nChunks * L * sizeof(int32_t), st));
-    chunk_hist_kernel<<<nChunks, kGroupChunk, 0, st>>>(labels, N, L, chunkHist);
-    chunk_scan_kernel<<<(L + 127) / 128, 128, 0, st>>>(chunkHist, nChunks, L, descDev);
-    chunk_place_kernel<<<nChunks, kGroupChunk, 0, st>>>(labels, N, L, chunkHist, perm);
-    ctx->kernelLaunches += 3;
+    if (N == 0) {
+        if (callStatus) RCD_CUDA(ctx, cudaMemsetAsync(callStatus, 0, sizeof(int32_t), st));
+        return RCD_OK;
+    }
+    const int chunk = group_chunk(N);
+    const unsigned nChunks = (unsigned)((N + chunk - 1) / chunk);
+    if (shared_labels(L)) {
+        const size_t smem = (size_t)L * 4;
+        if (smem > 48 * 1024) RCD_CUDA(ctx, cudaFuncSetAttribute(label_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        label_hist_kernel<<<nChunks, kGroupThreads, smem, st>>>(labels, N, L, chunk, chunkHist, counts, status, callStatus);
+        ctx->kernelLaunches++;
+    } else {
+        const unsigned blocks = (unsigned)std::min<int64_t>((N + 255) / 256, 4LL * ctx->smCount);
+        count_labels_kernel<<<blocks, 256, 0, st>>>(labels, N, L, counts, status, callStatus);
+        RCD_CUDA(ctx, cudaMemsetAsync(chunkHist, 0, (size_t)nChunks * L * sizeof(int32_t), st));
+        chunk_rank_kernel<true><<<nChunks, 1024, 0, st>>>(labels, N, L, chunk, chunkHist, nullptr, nullptr);
+        ctx->kernelLaunches += 2;
+    }
     RCD_CUDA(ctx, cudaGetLastError());
     return RCD_OK;
 }
 
-// ---- feature gather -------------------------------------------------------------------------
-__global__ void gather_rows16_kernel(const int4 *__restrict__ X, const int32_t *__restrict__ perm, int64_t N,
-                                     int64_t row16, int4 *__restrict__ Xs)
+// Stable split after launch_label_hist: perm, and with X the rows in split order (Xs, `pitch` bytes apart, zero-filled
+// beyond rowBytes).  desc null: label l starts after the counts of the labels below it; the starts go to offsets[L + 1].
+rcd_status launch_stable_split(rcd_ctx *ctx, const int32_t *labels, int64_t N, int32_t L, int32_t *chunkHist, const ClassDesc *descDev,
+                               const int32_t *counts, int64_t *offsets, const int32_t *status, int32_t *perm,
+                               const void *X, int64_t rowBytes, int64_t pitch, void *Xs, cudaStream_t st)
 {
-    int64_t total = N * row16;
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
-        int64_t r = i / row16, c = i - r * row16;
-        Xs[i] = X[(int64_t)perm[r] * row16 + c];
+    if (N == 0) {
+        if (offsets) RCD_CUDA(ctx, cudaMemsetAsync(offsets, 0, (size_t)(L + 1) * sizeof(int64_t), st));
+        return RCD_OK;
     }
-}
-
-__global__ void gather_rows1_kernel(const uint8_t *__restrict__ X, const int32_t *__restrict__ perm, int64_t N,
-                                    int64_t rowBytes, uint8_t *__restrict__ Xs)
-{
-    int64_t total = N * rowBytes;
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
-        int64_t r = i / rowBytes, c = i - r * rowBytes;
-        Xs[i] = X[(int64_t)perm[r] * rowBytes + c];
-    }
-}
-
-rcd_status launch_gather_rows(rcd_ctx *ctx, const void *X, const int32_t *perm, int64_t N, int64_t rowBytes,
-                              void *Xs, cudaStream_t st)
-{
-    if (N == 0 || rowBytes == 0) return RCD_OK;
-    int threads = 256;
-    bool vec = (rowBytes % 16 == 0) && (((uintptr_t)X) % 16 == 0) && (((uintptr_t)Xs) % 16 == 0);
-    int64_t total = vec ? N * (rowBytes / 16) : N * rowBytes;
-    int64_t blocks = (total + threads - 1) / threads;
-    int64_t cap = 32LL * ctx->smCount;
-    if (blocks > cap) blocks = cap;
-    if (vec)
-        gather_rows16_kernel<<<(unsigned)blocks, threads, 0, st>>>((const int4 *)X, perm, N, rowBytes / 16, (int4 *)Xs);
-    else
-        gather_rows1_kernel<<<(unsigned)blocks, threads, 0, st>>>((const uint8_t *)X, perm, N, rowBytes, (uint8_t *)Xs);
+    const int chunk = group_chunk(N);
+    const int nChunks = (int)((N + chunk - 1) / chunk);
+    label_scan_kernel<<<(L + 31) / 32, 1024, 0, st>>>(chunkHist, nChunks, L, descDev, counts, offsets, status);
     ctx->kernelLaunches++;
+    if (shared_labels(L)) {
+        const size_t smem = ((size_t)kGroupWarps * L + (Xs ? chunk : 0)) * 4;
+        if (smem > 48 * 1024) RCD_CUDA(ctx, cudaFuncSetAttribute(label_place_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        label_place_kernel<<<nChunks, kGroupThreads, smem, st>>>(labels, N, L, chunk, chunkHist, perm, (const uint8_t *)X, rowBytes, pitch,
+                                                                (uint8_t *)Xs, status);
+        ctx->kernelLaunches++;
+    } else {
+        chunk_rank_kernel<false><<<nChunks, 1024, 0, st>>>(labels, N, L, chunk, chunkHist, perm, status);
+        ctx->kernelLaunches++;
+        if (Xs) {
+            const unsigned blocks = (unsigned)std::min<int64_t>((N + 7) / 8, 32LL * ctx->smCount);
+            gather_rows_kernel<<<blocks, 256, 0, st>>>((const uint8_t *)X, perm, N, rowBytes, pitch, (uint8_t *)Xs);
+            ctx->kernelLaunches++;
+        }
+    }
     RCD_CUDA(ctx, cudaGetLastError());
     return RCD_OK;
 }

@@ -81,10 +81,11 @@ struct SimClasses {
 // Pointers into the caller's workspace for one rcd_partition call.
 struct Workspace {
     // grouping
+    int32_t *counter;       // [4] zero when the call starts (classes drawn by the cluster form)
     int32_t *counts;        // [L]
     int32_t *chunkHist;     // [nChunks][L]
     int32_t *perm;          // [N] class-sorted position -> dataset index
-    void *Xs;               // [N][d] features in class-sorted order
+    void *Xs;               // [N][pitch] features in class-sorted order
     // per class
     ClassDesc *desc;        // [L]
     int32_t *tilePrefix;    // [L+1] first upper-triangle tile of every class (tensor-core similarity)
@@ -140,11 +141,17 @@ struct Sizes {
     int64_t vElems;         // sum W * ld_l
     int64_t maxM;
     int32_t nChunks;
+    int64_t pitch;          // bytes between rows of Xs
     bool floatArith;        // fp32 S / fp32 gains / double f (bf16 features, or the Gaussian kernel)
     bool graphCut;          // graph-cut objective: the gains array holds 8-byte ties
 };
 
-constexpr int kGroupChunk = 1024;           // samples per chunk of the stable class split
+// Samples per chunk of the stable class split: small chunks while that is what fills the SMs, large ones where the
+// per-chunk tables (chunks x labels) would grow.
+inline int group_chunk(int64_t N) { return N <= 131072 ? 256 : 1024; }
+// Bytes between the class-sorted feature rows: whole 16-byte pieces, at least one 128-byte slab, so that every width can
+// be loaded by the tensor-core kernel (the padding is zeros and adds nothing to a dot product).
+inline int64_t row_pitch(int64_t rowBytes) { return rowBytes <= 128 ? 128 : (rowBytes + 15) / 16 * 16; }
 
 inline size_t feat_bytes(rcd_feat_dtype t) { return t == RCD_FEAT_I8 ? 1 : 2; }
 inline size_t align_up(size_t x, size_t a = kAlign) { return (x + a - 1) / a * a; }
@@ -179,6 +186,10 @@ struct rcd_ctx {
     int32_t *hostStage = nullptr;       // pinned, counts / status read-back
     int32_t *statusOwn = nullptr;       // device status word for calls that take no workspace
     size_t hostStageInts = 0;
+    unsigned char *hostBlob = nullptr;  // pinned, what a call's host side hands to its kernels
+    size_t hostBlobBytes = 0;
+    cudaEvent_t evBlob = nullptr;       // the last copy out of hostBlob
+    cudaEvent_t evCounts = nullptr;     // the class sizes have arrived
     // profiling
     cudaEvent_t evPhase[5]{};           // start, after group, after similarity, after greedy, end
     bool phaseValid = false;
@@ -208,12 +219,11 @@ rcd_status cuda_fail(rcd_ctx *ctx, cudaError_t e, const char *what);
 // ---- launchers implemented in the .cu files (all asynchronous on `st`) ----
 
 // class split
-rcd_status launch_count_labels(rcd_ctx *ctx, const int32_t *labels, int64_t N, int32_t L, int32_t *counts,
-                               int32_t *status, cudaStream_t st);
-rcd_status launch_stable_split(rcd_ctx *ctx, const int32_t *labels, int64_t N, int32_t L, int32_t nChunks,
-                               int32_t *chunkHist, const ClassDesc *descDev, int32_t *perm, cudaStream_t st);
-rcd_status launch_gather_rows(rcd_ctx *ctx, const void *X, const int32_t *perm, int64_t N, int64_t rowBytes,
-                              void *Xs, cudaStream_t st);
+rcd_status launch_label_hist(rcd_ctx *ctx, const int32_t *labels, int64_t N, int32_t L, int32_t *chunkHist, int32_t *counts,
+                             int32_t *status, int32_t *callStatus, cudaStream_t st);
+rcd_status launch_stable_split(rcd_ctx *ctx, const int32_t *labels, int64_t N, int32_t L, int32_t *chunkHist, const ClassDesc *descDev,
+                               const int32_t *counts, int64_t *offsets, const int32_t *status, int32_t *perm,
+                               const void *X, int64_t rowBytes, int64_t pitch, void *Xs, cudaStream_t st);
 
 // similarity: S_l = Xs_l Xs_l^T for every class described by desc
 rcd_status launch_similarity(rcd_ctx *ctx, const void *Xs, rcd_feat_dtype dtype, int64_t Ntot, int64_t d,
@@ -230,9 +240,9 @@ rcd_status launch_greedy(rcd_ctx *ctx, rcd_feat_dtype dtype, const Sizes &sz, co
                          cudaStream_t st);
 
 // greedy loop, one thread-block cluster per class
-bool cluster_form_takes(const rcd_ctx *ctx, const Sizes &sz);
+bool cluster_form_takes(const rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost);
 rcd_status launch_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, const std::vector<ClassDesc> &descHost,
-                                 int32_t *assignment, int32_t *order, cudaStream_t st);
+                                 int32_t *assignment, int32_t *order, void *partValues, cudaStream_t st);
 
 rcd_status launch_bounded_wait_selftest(rcd_ctx *ctx, unsigned *counter, int32_t *status, cudaStream_t st);
 
