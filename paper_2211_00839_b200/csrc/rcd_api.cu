@@ -77,7 +77,8 @@ size_t layout_workspace(void *base, rcd_feat_dtype dtype, const Sizes &sz, Works
     const size_t gElem = 8;                                     // int64 gains (fp32 ones use half of it), or 8-byte ties
     Workspace w{};
     // the head does not depend on the class sizes: it is used before they are known
-    w.status = c.take<int32_t>(4);           // (from here to counts: zeroed by one memset at the start of a call)
+    w.topGain = c.take<unsigned long long>(L);             // (from here to counts: zeroed by one memset at the start of a call)
+    w.status = c.take<int32_t>(4);
     w.counter = c.take<int32_t>(4);
     w.phaseNs = c.take<unsigned long long>(kPhaseWords);   // phase clocks, the grid-barrier counter, threshold-pass and row-skipping counters
     w.counts = c.take<int32_t>(L);
@@ -245,14 +246,13 @@ static rcd_status prepare(rcd_ctx *ctx, const void *features, rcd_feat_dtype dty
     if (workspaceBytes < headBytes) return fail(ctx, RCD_ERR_WORKSPACE_TOO_SMALL, "workspace smaller than its %zu-byte head", headBytes);
     if ((size_t)L > ctx->hostStageInts) return fail(ctx, RCD_ERR_UNSUPPORTED, "L=%d exceeds the %zu classes the context can stage", L, ctx->hostStageInts);
 
-    const size_t zeroBytes = (size_t)((unsigned char *)(hw.counts + L) - (unsigned char *)hw.status);
-    RCD_CUDA(ctx, cudaMemsetAsync(hw.status, 0, zeroBytes, st));
+    RCD_CUDA(ctx, cudaMemsetAsync(hw.topGain, 0, (size_t)((unsigned char *)(hw.counts + L) - (unsigned char *)hw.topGain), st));
     rcd_status rs = launch_label_hist(ctx, labels, N, L, hw.chunkHist, hw.counts, hw.status, ctx->statusOwn, st);
     if (rs != RCD_OK) return rs;
     ctx->statusDev = ctx->statusOwn;
     // the class sizes come back together with the words before them (the label check's verdict is the first)
     const size_t statusInts = (size_t)(hw.counts - hw.status);
-    RCD_CUDA(ctx, cudaMemcpyAsync(ctx->hostStage, hw.status, zeroBytes, cudaMemcpyDeviceToHost, st));
+    RCD_CUDA(ctx, cudaMemcpyAsync(ctx->hostStage, hw.status, (statusInts + L) * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     if (!ctx->evCounts) RCD_CUDA(ctx, cudaEventCreateWithFlags(&ctx->evCounts, cudaEventDisableTiming));
     RCD_CUDA(ctx, cudaEventRecord(ctx->evCounts, st));
     const size_t blobBytes = (size_t)((unsigned char *)(hw.quota + (size_t)L * W) - (unsigned char *)hw.desc);
@@ -260,7 +260,7 @@ static rcd_status prepare(rcd_ctx *ctx, const void *features, rcd_feat_dtype dty
     if (rs != RCD_OK) return rs;
     RCD_CUDA(ctx, cudaEventSynchronize(ctx->evCounts));
     if (ctx->hostStage[0] & kDevBadLabel) return fail(ctx, RCD_ERR_INVALID_ARG, "a label lies outside [0, %d)", L);
-    const int32_t *counts = ctx->hostStage + statusInts;
+    const int32_t *counts = ctx->hostStage + statusInts;      // (behind the zeroed words that came along)
 
     Prepared &P = *out;
     P.desc.resize((size_t)L);
@@ -390,7 +390,7 @@ rcd_status rcd_create(rcd_ctx **out, int cuda_device, const rcd_config *cfg)
     ctx->cooperative = prop.cooperativeLaunch != 0;
     if (cfg) ctx->cfg = *cfg;
     ctx->hostStageInts = 1 << 20;
-    if (cudaMallocHost((void **)&ctx->hostStage, (ctx->hostStageInts + 512) * sizeof(int32_t)) != cudaSuccess) {
+    if (cudaMallocHost((void **)&ctx->hostStage, (ctx->hostStageInts + 1024) * sizeof(int32_t)) != cudaSuccess) {
         delete ctx;
         return RCD_ERR_CUDA;
     }
@@ -701,11 +701,11 @@ rcd_status rcd_partition(rcd_ctx *ctx, const void *features_dev, rcd_feat_dtype 
     if (rs != RCD_OK) return rs;
 
     bool valuesWritten = false;
-    if (P.sz.graphCut) {
+    rs = launch_greedy_cluster(ctx, P.sz, P.ws, P.desc, assignment_dev, order_dev_or_null, part_values_dev_or_null, st, &valuesWritten);
+    if (rs != RCD_OK) return rs;
+    if (valuesWritten) {
+    } else if (P.sz.graphCut) {
         rs = launch_cut(ctx, P.sz, P.ws, assignment_dev, order_dev_or_null, st);
-    } else if (P.sz.maxM > 0 && cluster_form_takes(ctx, P.sz, P.desc)) {
-        valuesWritten = true;
-        rs = launch_greedy_cluster(ctx, P.sz, P.ws, P.desc, assignment_dev, order_dev_or_null, part_values_dev_or_null, st);
     } else {
         rs = launch_greedy(ctx, P.sz.floatArith ? RCD_FEAT_BF16 : RCD_FEAT_I8, P.sz, P.ws, P.desc, assignment_dev, order_dev_or_null, st);
     }

@@ -82,6 +82,7 @@ struct SimClasses {
 struct Workspace {
     // grouping
     int32_t *counter;       // [4] zero when the call starts (classes drawn by the cluster form)
+    unsigned long long *topGain;   // [L] zero when the call starts (cluster form)
     int32_t *counts;        // [L]
     int32_t *chunkHist;     // [nChunks][L]
     int32_t *perm;          // [N] class-sorted position -> dataset index
@@ -240,9 +241,8 @@ rcd_status launch_greedy(rcd_ctx *ctx, rcd_feat_dtype dtype, const Sizes &sz, co
                          cudaStream_t st);
 
 // greedy loop, one thread-block cluster per class
-bool cluster_form_takes(const rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost);
 rcd_status launch_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, const std::vector<ClassDesc> &descHost,
-                                 int32_t *assignment, int32_t *order, void *partValues, cudaStream_t st);
+                                 int32_t *assignment, int32_t *order, void *partValues, cudaStream_t st, bool *taken);
 
 rcd_status launch_bounded_wait_selftest(rcd_ctx *ctx, unsigned *counter, int32_t *status, cudaStream_t st);
 
