@@ -821,15 +821,15 @@ rcd_status rcd_objective(rcd_ctx *ctx, const void *features_dev, rcd_feat_dtype 
     rs = prepare(ctx, features_dev, dtype, N, d, labels_dev, L, W, nullptr, workspace_dev, workspace_bytes, st, &P);
     ctx->cfg.profile = savedProfile;
     if (rs != RCD_OK) return rs;
-    size_t scratchB = objective_scratch_bytes(L, P.sz.maxM, W);
-    if (P.ws.bytes + scratchB > workspace_bytes)
-        return fail(ctx, RCD_ERR_WORKSPACE_TOO_SMALL, "workspace has %zu bytes, objective needs %zu", workspace_bytes, P.ws.bytes + scratchB);
-    void *scratch = (unsigned char *)workspace_dev + P.ws.bytes;
-    if (P.sz.graphCut)
-        rs = launch_cut_objective(ctx, P.sz, P.ws.desc, P.ws.S, P.ws.perm, assignment_dev, part_values_dev, total_dev, scratch, st);
-    else
-        rs = launch_objective(ctx, P.sz.floatArith ? RCD_FEAT_BF16 : RCD_FEAT_I8, P.sz, P.ws.desc, P.desc, P.ws.S, P.ws.perm, assignment_dev,
-                              part_values_dev, total_dev, scratch, st);
+    if (P.sz.graphCut) {
+        const size_t scratchB = objective_scratch_bytes(L, P.sz.maxM, W);
+        if (P.ws.bytes + scratchB > workspace_bytes)
+            return fail(ctx, RCD_ERR_WORKSPACE_TOO_SMALL, "workspace has %zu bytes, objective needs %zu", workspace_bytes, P.ws.bytes + scratchB);
+        rs = launch_cut_objective(ctx, P.sz, P.ws.desc, P.ws.S, P.ws.perm, assignment_dev, part_values_dev, total_dev,
+                                  (unsigned char *)workspace_dev + P.ws.bytes, st);
+    } else {
+        rs = launch_objective(ctx, P.sz.floatArith ? RCD_FEAT_BF16 : RCD_FEAT_I8, P.sz, P.ws, assignment_dev, part_values_dev, total_dev, st);
+    }
     return rs;
 }
 

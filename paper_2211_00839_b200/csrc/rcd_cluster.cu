@@ -32,14 +32,27 @@ constexpr int kRaisedPerWarp = 64;        // raised columns a team lists at a ti
 constexpr int kClusterBlocks = 128;       // blocks a cluster can lead (their notes sit in one CTA's shared memory)
 constexpr int kEntries = 16;              // candidates per note
 constexpr uint32_t kScanCmd = 0u;         // a command's low word: look again;
-constexpr uint32_t kStopCmd = ~0u;        //   the class is done;  anything else: sample + 1 joins the block
-constexpr unsigned kPollLimit = 1u << 25;
+constexpr uint32_t kStopCmd = 0xfffffu;   //   the class is done;  anything else: sample + 1 joins the block
+constexpr int kRefreshers = 3;            // warps per CTA that refresh notes (17 warps would occupy the registers of 20 anyway)
+constexpr unsigned kPollLimit = 1u << 28;
 constexpr unsigned long long kZeroValue = 1ull << 55;   // (tracked values of the graph cut can be negative)
 
-// What a team tells the leader about a block: the key of its best candidate (0: none), and for the case that other
-// blocks took that one: [1, 17) keys of leading candidates, [17, 17 + T) per team warp a key that no other exceeds.
-struct Note {
-    unsigned long long word[1 + kEntries + kMaxWarps];
+// What the leader is told about a block (a note, words of 64 bits):
+//   [0]            the key of its best candidate (0: none)
+//   [1, 17)        for the case that other blocks took that one: keys of leading candidates
+//   [17, 17 + T)   per team warp a key that no candidate left out exceeds
+// and, where blocks sit in shared memory, two words that a refreshing warp rewrites whenever the best candidate has been
+// taken (with many blocks that happens often before the block's turn comes):
+//   [17 + T, 19 + T)     gain << 16 | tag and update number << 32 | (65535 - sample) << 16 | tag, where tag is the update
+//                        number's last byte << 8 | a running number from 1
+// A candidate that was a block's best and is still unassigned is still its best: gains move only when the block itself
+// receives a sample.
+struct NoteLayout {
+    int T;
+    __host__ __device__ int bounds() const { return 1 + kEntries; }
+    __host__ __device__ int now() const { return 1 + kEntries + T; }
+    __host__ __device__ int words() const { return 3 + kEntries + T; }
+    __host__ __device__ uint32_t tracked() const { return (uint32_t)(1 + kEntries + T) * 8; }   // bytes a new note brings
 };
 
 struct __align__(16) Raised {
@@ -79,8 +92,10 @@ struct ClusterParams {
     int32_t rowPieces;         // 16-byte pieces of a team's row buffer
     unsigned long long *topGain;   // [L] zero at the start: largest gain for an empty block (graph cut: row sum of |S|)
     uint32_t one;              // the value 1, opaque to the compiler
+    int32_t logC, logTeams;
     // byte offsets into dynamic shared memory
-    int32_t offTeams, offLists, offRows, offCmd, offBits, offNotes, offBars, offCover, offGains;
+    int32_t offTeams, offLists, offRows, offCmd, offBits, offNotes, offBars, offQueue, offFresh, offCover, offGains;
+    int32_t ring;              // command words per team (a power of two)
 };
 
 namespace {
@@ -136,6 +151,12 @@ __device__ __forceinline__ void team_barrier(int team, int T)
     else asm volatile("bar.sync %0, %1;" :: "r"(1 + team), "r"(T * 32) : "memory");
 }
 
+__device__ __forceinline__ int4 ld_row_shared(const int4 *p)       // (other teams of the CTA read the same rows: L1 may serve them)
+{
+    int4 v;
+    asm volatile("ld.global.nc.v4.s32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
 __device__ __forceinline__ int4 ld_row_once(const int4 *p)
 {
     int4 v;
@@ -157,6 +178,13 @@ __device__ __forceinline__ unsigned long long take_off(unsigned long long g, int
     unsigned long long r;
     asm("mad.wide.s32 %0, %1, -1, %2;" : "=l"(r) : "r"(l), "l"(g));
     return r;
+}
+
+// g - l for an unsigned l (minusOne: the value -1 as an unsigned 32-bit number times l, low 64 bits, plus l << 32)
+__device__ __forceinline__ unsigned long long take_off_wide(unsigned long long g, uint32_t l, uint32_t one)
+{
+    (void)one;
+    return g - l;
 }
 
 // Sum of a value below 2^43 per lane over the warp.
@@ -318,96 +346,184 @@ __device__ __forceinline__ int list_raised(const TeamView &t, int32_t *count, in
     return up;
 }
 
-// The n listed columns (an odd list is completed by an entry without effect) taken off the stored gains of a thread's
-// pieces.  The rows of S travel through a ring of asynchronous copies in shared memory, each thread reading back only what
-// it copied itself, two rows of one piece per step and kRing / 2 steps under way, across the ends of the list too: 80 KB
-// in flight per SM cover the latency of L2 and HBM without holding registers.
-constexpr int kRing = 10;
-struct RowStream {
-    int4 *ring;
-    const int4 *S4;
-    const Raised *list;
-    int n, step, ld4;
-    int fq, fe, fs, at;                                    // what is fetched next, and to which stage; the stage read next
-    __device__ __forceinline__ void fetch()
-    {
-        if (fq < ld4) {
-            copy16(ring + fs, S4 + (list[fe].row + fq));
-            copy16(ring + fs + step, S4 + (list[fe + 1].row + fq));
-            fe += 2;
-            if (fe >= n) { fe = 0; fq += step; }
+// Four listed columns taken off the stored gains of one piece.  Their losses (each below 2^30) add up in 32 bits, so that
+// widening and subtracting is paid once for four: 156 cycles of arithmetic per row of 20 KB and SM, 248 with two at a time.
+__device__ __forceinline__ uint32_t apply_four(const int4 &x, const int4 &y, const int4 &z, const int4 &w, const Raised &a, const Raised &b,
+                                               const Raised &c, const Raised &d, uint32_t one, unsigned long long (&g)[4])
+{
+    const uint32_t l0 = (uint32_t)loss(x.x, a) + loss(y.x, b) + loss(z.x, c) + loss(w.x, d);
+    const uint32_t l1 = (uint32_t)loss(x.y, a) + loss(y.y, b) + loss(z.y, c) + loss(w.y, d);
+    const uint32_t l2 = (uint32_t)loss(x.z, a) + loss(y.z, b) + loss(z.z, c) + loss(w.z, d);
+    const uint32_t l3 = (uint32_t)loss(x.w, a) + loss(y.w, b) + loss(z.w, c) + loss(w.w, d);
+    g[0] = take_off_wide(g[0], l0, one);
+    g[1] = take_off_wide(g[1], l1, one);
+    g[2] = take_off_wide(g[2], l2, one);
+    g[3] = take_off_wide(g[3], l3, one);
+    return l0 | l1 | l2 | l3;
+}
+// (entry e of n, or one without effect)
+__device__ __forceinline__ Raised entry_or_none(const Raised *list, int e, int n)
+{
+    Raised r = list[min(e, n - 1)];
+    if (e >= n) r.minusOld = r.by = 0;
+    return r;
+}
+
+// The n listed columns taken off one piece, rows straight to registers, up to eight in flight.
+__device__ __forceinline__ bool correct_piece(const int4 *S4q, const Raised *list, int n, uint32_t one, unsigned long long (&g)[4])
+{
+    uint32_t changed = 0;
+    int e = 0;
+#pragma unroll 1
+    for (; e + 8 <= n; e += 8) {
+        int4 x[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) x[u] = ld_row_shared(S4q + list[e + u].row);
+        changed |= apply_four(x[0], x[1], x[2], x[3], list[e], list[e + 1], list[e + 2], list[e + 3], one, g);
+        changed |= apply_four(x[4], x[5], x[6], x[7], list[e + 4], list[e + 5], list[e + 6], list[e + 7], one, g);
+    }
+#pragma unroll 1
+    for (; e < n; e += 4) {
+        Raised r[4];
+        int4 x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            r[u] = entry_or_none(list, e + u, n);
+            x[u] = ld_row_shared(S4q + r[u].row);
         }
-        copies_commit();
-        fs += 2 * step;
-        if (fs == kRing * step) fs = 0;
+        changed |= apply_four(x[0], x[1], x[2], x[3], r[0], r[1], r[2], r[3], one, g);
     }
-    __device__ __forceinline__ RowStream(const TeamView &t, int count)
-    {
-        const int first = t.warpIn * 32 + t.lane;
-        step = t.T * 32;
-        ring = t.rowBuf + first;
-        S4 = t.S4; list = t.list; n = count; ld4 = t.ld4;
-        fq = first; fe = 0; fs = 0; at = 0;
+    return changed != 0;
+}
+
+// The same for a team that keeps its P pieces per thread in registers.  The rows travel through asynchronous copies in
+// shared memory, each thread reading back only what it copied itself, so that loads in flight hold no registers.
+// Up to three pieces: row by row over all pieces (a list entry and a row's address serve them all), eight rows of room,
+// four under way while four are applied: 403 cycles per row of 20 KB and SM with 80 SMs at it, of which L2 and HBM take 350
+// (538 with two rows at a time).  More pieces, or less room: piece by piece through a ring of twelve 16-byte slots per
+// thread (480 - 500 cycles).
+template <int P> struct RowRing { static constexpr bool byRow = P <= 3; };
+constexpr int kRowStages = 8, kPieceStages = 12;
+template <int P, int kT>
+__device__ __forceinline__ void apply_list(const TeamView &t, int n, uint32_t one, unsigned long long (&g)[P][4])
+{
+    const int first = t.warpIn * 32 + t.lane, step = (kT ? kT : t.T) * 32;
+    int4 *const ring = t.rowBuf + first;
+    const Raised *list = t.list;
+    if constexpr (RowRing<P>::byRow) {
+        const int stride = t.ld4;
+        int fe = 0, fs = 0, at = 0;
+        auto fetch = [&] {                                 // four rows
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (fe + u < n) {
+                    const int4 *src = t.S4 + (list[fe + u].row + first);
+#pragma unroll
+                    for (int p = 0; p < P; ++p)
+                        if (p * step + first < t.ld4) copy16(ring + fs + u * stride + p * step, src + p * step);
+                }
+            }
+            copies_commit();
+            fe += 4;
+            fs = fs == 0 ? 4 * stride : 0;
+        };
+        fetch();
 #pragma unroll 1
-        for (int k = 0; k < kRing / 2 - 1; ++k) fetch();
-    }
-    // all n columns for the piece whose turn it is
-    __device__ __forceinline__ int piece(unsigned long long (&g)[4])
-    {
-        int changed = 0;
-#pragma unroll 1
-        for (int e = 0; e < n; e += 2) {
-            copies_wait<kRing / 2 - 2>();
-            const int4 x = ring[at], y = ring[at + step];
-            const Raised a = list[e], b = list[e + 1];
-            at += 2 * step;
-            if (at == kRing * step) at = 0;
+        for (int e = 0; e < n; e += 4) {
             fetch();
-            const int l0 = loss(x.x, a) + loss(y.x, b), l1 = loss(x.y, a) + loss(y.y, b);
-            const int l2 = loss(x.z, a) + loss(y.z, b), l3 = loss(x.w, a) + loss(y.w, b);
-            changed |= l0 | l1 | l2 | l3;
-            g[0] = take_off(g[0], l0);
-            g[1] = take_off(g[1], l1);
-            g[2] = take_off(g[2], l2);
-            g[3] = take_off(g[3], l3);
+            copies_wait<1>();
+            const int4 *x = ring + at;
+            at = at == 0 ? 4 * stride : 0;
+            Raised r[4];
+            if (e + 4 <= n) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) r[u] = list[e + u];
+            } else {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) r[u] = entry_or_none(list, e + u, n);
+            }
+#pragma unroll
+            for (int p = 0; p < P; ++p)
+                if (p * step + first < t.ld4)
+                    apply_four(x[p * step], x[p * step + stride], x[p * step + 2 * stride], x[p * step + 3 * stride], r[0], r[1], r[2], r[3], one, g[p]);
         }
-        return changed;
+    } else {
+        int fq = first, fe = 0, fs = 0, at = 0;
+        auto fetch = [&] {                                 // one piece of four rows
+            if (fq < t.ld4) {
+                const int4 *src = t.S4 + fq;
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (fe + u < n) copy16(ring + (fs + u) * step, src + list[fe + u].row);
+                fe += 4;
+                if (fe >= n) { fe = 0; fq += step; }
+            }
+            copies_commit();
+            fs += 4;
+            if (fs == kPieceStages) fs = 0;
+        };
+        fetch();
+        fetch();
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            if (p * step + first < t.ld4) {
+#pragma unroll 1
+                for (int e = 0; e < n; e += 4) {
+                    copies_wait<1>();
+                    const int4 *x = ring + at * step;
+                    at += 4;
+                    if (at == kPieceStages) at = 0;
+                    const int4 x0 = x[0], x1 = x[step], x2 = x[2 * step], x3 = x[3 * step];
+                    fetch();
+                    if (e + 4 <= n) {
+                        apply_four(x0, x1, x2, x3, list[e], list[e + 1], list[e + 2], list[e + 3], one, g[p]);
+                    } else {
+                        Raised r[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) r[u] = entry_or_none(list, e + u, n);
+                        apply_four(x0, x1, x2, x3, r[0], r[1], r[2], r[3], one, g[p]);
+                    }
+                }
+            }
+        }
     }
-};
+    copies_wait<0>();
+}
 
 // Folds a sample's row into the coverage, list by list; `apply(n)` corrects the stored gains for the n listed columns.
+// `par`: which of two list lengths is in use (the other one is zero).
 template <typename Apply>
-__device__ __forceinline__ void take_in_lists(const TeamView &t, int v, int4 *cov, unsigned &rows, Apply apply)
+__device__ __forceinline__ void take_in_lists(const TeamView &t, int v, int4 *cov, int32_t *counts, int &par, unsigned &rows, Apply apply)
 {
     const int tid = t.warpIn * 32 + t.lane, step = t.T * 32;
     const int room = t.T * kRaisedPerWarp;
-    int32_t *count = &t.tm->count[2];
     const int4 *row = t.S4 + (int64_t)v * t.ld4;
     for (;;) {
         team_barrier(t.team, t.T);                         // (the list's last readers are done)
-        if (tid == 0) *count = 0;
-        team_barrier(t.team, t.T);
+        int32_t *count = counts + par;
         for (int q = tid; q < t.ld4; q += step) {
             const int4 r = __ldg(row + q), m = cov[q];
             if (list_raised(t, count, q, r, m)) cov[q] = make_int4(max(r.x, m.x), max(r.y, m.y), max(r.z, m.z), max(r.w, m.w));
         }
         team_barrier(t.team, t.T);
         const int all = *(volatile int32_t *)count;
+        par ^= 1;
+        if (tid == 0) counts[par] = 0;
         const int n = min(all, room);
         rows += n;
-        if (tid == 0 && (n & 1)) t.list[n] = Raised{0, 0, 0, 0};
-        team_barrier(t.team, t.T);
         if (n > 0) apply(n);
         if (all <= room) break;
     }
 }
 
 // A team with one block, its stored gains in registers: P pieces of four columns per thread.  Coverage in shared memory.
-template <int P, bool kCut>
+// kT: warps per team (0: known at run time).  Registers are what this function is short of (17 warps share the file as 20
+// would: 96 per thread), hence the constants.
+template <int P, int kT, bool kCut>
 __device__ __forceinline__ void team_of_one(const ClusterParams &prm, const ClassDesc &c, const TeamView &t, int4 *cov, int shift, unsigned long long bias,
                                             uint32_t cmdAddr, uint32_t noteAddr, uint32_t barAddr, unsigned &corrected, unsigned &rows)
 {
-    const int T = t.T, tid = t.warpIn * 32 + t.lane, step = T * 32, lane = t.lane;
+    const int T = kT ? kT : t.T, tid = t.warpIn * 32 + t.lane, step = T * 32, lane = t.lane;
     const int room = T * kRaisedPerWarp;
     unsigned long long g[P][4];
 #pragma unroll
@@ -417,7 +533,8 @@ __device__ __forceinline__ void team_of_one(const ClusterParams &prm, const Clas
 #pragma unroll
         for (int u = 0; u < 4; ++u) g[p][u] = 4 * q + u < c.M ? (unsigned long long)__ldcg(prm.g0 + c.row0 + 4 * q + u) + bias : 0ull;
     }
-    if (tid == 0) t.tm->count[0] = t.tm->count[1] = 0;
+    if (tid == 0) t.tm->count[0] = t.tm->count[1] = t.tm->count[2] = t.tm->count[3] = 0;
+    int other = 0;
     Lead best;
     lead_init(best);
     Summary sum{0, 0, 0};
@@ -484,10 +601,6 @@ __device__ __forceinline__ void team_of_one(const ClusterParams &prm, const Clas
                 }
                 team_barrier(t.team, T);
                 all = *(volatile int32_t *)count;
-                if (all & 1) {                             // (an entry without effect completes the last pair)
-                    if (tid == 0 && all < room) t.list[all] = Raised{0, 0, 0, 0};
-                    team_barrier(t.team, T);
-                }
             }
         }
         if (tid == 0) t.tm->count[par ^ 1] = 0;
@@ -527,17 +640,15 @@ __device__ __forceinline__ void team_of_one(const ClusterParams &prm, const Clas
             continue;
         }
         auto apply = [&](int n) {
-            RowStream rs(t, n);
-            int changed = 0;
-#pragma unroll
-            for (int p = 0; p < P; ++p)
-                if (tid + p * step < t.ld4) changed |= rs.piece(g[p]);
-            copies_wait<0>();
-            dirty = dirty || changed != 0;
+            // (nothing about candidates is kept meanwhile)
+            lead_init(best);
+            sum = Summary{0, 0, 0};
+            dirty = true;
+            apply_list<P, kT>(t, n, prm.one, g);
         };
         if ((int)what - 1 != v || all > room) {
             // another sample than foreseen, or more raised columns than one list holds
-            take_in_lists(t, (int)what - 1, cov, rows, apply);
+            take_in_lists(t, (int)what - 1, cov, t.tm->count + 2, other, rows, apply);
             continue;
         }
         rows += all;
@@ -567,106 +678,189 @@ __device__ __forceinline__ void team_of_one(const ClusterParams &prm, const Clas
     copies_wait<0>();
 }
 
-// A one-warp team with several blocks (coverage and gains in memory): it serves whichever has a command.
-template <typename Where>
-__device__ __forceinline__ void team_of_many(const ClusterParams &prm, int l, const ClassDesc &c, const TeamView &t, int mine, int shift, uint32_t cmd0,
-                                             int cmdStride, Where where, unsigned &corrected, unsigned &rows)
+// The leading candidates among a thread's pieces of a block's stored gains.
+__device__ __forceinline__ Lead scan_gains(const uint32_t *bits, const unsigned long long *gains, int ld4, int first, int step, int shift)
 {
-    const int lane = t.lane;
+    Lead best;
+    lead_init(best);
+    for (int q = first; q < ld4; q += step) {
+        const uint32_t nib = bits[q >> 3] >> ((q & 7) * 4);
+        const ulonglong2 a0 = reinterpret_cast<const ulonglong2 *>(gains)[2 * q], a1 = reinterpret_cast<const ulonglong2 *>(gains)[2 * q + 1];
+        const unsigned long long g[4] = {a0.x, a0.y, a1.x, a1.y};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const uint32_t k = (nib >> u & 1) ? 0u : lead_part(g[u], shift);
+            best.o = max(best.o, min(best.e, k));
+            if (k >= best.e && k) {
+                const uint32_t low = low_part(g[u], shift, 4 * q + u);
+                best.low = k > best.e ? low : max(best.low, low);
+                best.e = k;
+            }
+        }
+    }
+    return best;
+}
+
+// What a team tells the refreshing warps about a block, the update number last: from then on the stored gains are those
+// after that many updates, until the leader has given the block another sample -- and then it takes no candidate of the
+// earlier update any more, so a scan that ran into the next update does no harm.
+struct Fresh {
+    int32_t sample;            // the block's best candidate
+    uint32_t update;           // number of updates (kNotYet: none told)
+};
+constexpr uint32_t kNotYet = 0xffffffffu;
+
+// A refreshing warp: lane i watches the best candidate of the CTA's block first + i step, and when that one has been
+// taken by another block, the warp looks for the best of those left and tells the leader.
+template <typename Slot>
+__device__ void refresh_notes(const ClusterParams &prm, const uint32_t *bits, int ld4, int shift, volatile Fresh *fresh, int first, int step, int slots,
+                              const volatile uint32_t *stop, uint32_t turn, Slot where)
+{
+    const int lane = threadIdx.x & 31;
+    const NoteLayout note{prm.teamWarps};
+    const int slot = first + lane * step;
+    const bool watch = slot < slots;
+    uint32_t update = kNotYet, tag = 0;
+    int sample = -1;
+    for (unsigned spin = 0; spin < kPollLimit; ++spin) {
+        if (*stop == turn) break;
+        bool taken = false;
+        if (watch) {
+            const uint32_t u = fresh[slot].update;
+            const int s = fresh[slot].sample;
+            if (u != update) {
+                update = u;
+                sample = s;
+                tag = (u & 0xffu) << 8;
+            }
+            if (update != kNotYet && sample >= 0) taken = *(volatile const uint32_t *)&bits[sample >> 5] >> (sample & 31) & 1;
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, taken);
+        if (!m) continue;
+        const int i = __ffs(m) - 1;
+        const unsigned long long *gains;
+        const uint32_t noteAddr = where(first + i * step, gains);
+        const Lead best = scan_gains(bits, gains, ld4, lane, 32, shift);
+        const uint32_t e = __reduce_max_sync(0xffffffffu, best.e);
+        const unsigned long long k = key_of(e, __reduce_max_sync(0xffffffffu, best.e == e ? best.low : 0u), shift);
+        if (lane == i) {
+            sample = k ? key_sample(k) : -1;
+            tag = (tag & 0xff00u) | ((tag & 0xffu) == 255u ? 1u : (tag & 0xffu) + 1u);
+            st_remote(noteAddr + (uint32_t)note.now() * 8, (k & ~0xffffull) | tag);
+            st_remote(noteAddr + (uint32_t)(note.now() + 1) * 8, (unsigned long long)update << 32 | (k & 0xffffull) << 16 | tag);
+        }
+        __syncwarp();
+    }
+}
+
+// A team with several blocks, coverage and stored gains in memory (shared memory where they fit).  Its commands come
+// through a ring, in the order given.
+template <bool kCut, typename Where>
+__device__ __forceinline__ void team_of_many(const ClusterParams &prm, int l, const ClassDesc &c, const TeamView &t, int mine, int shift,
+                                             unsigned long long bias, uint32_t cmds, Where where, unsigned &corrected, unsigned &rows)
+{
+    const int lane = t.lane, T = t.T, tid = t.warpIn * 32 + lane, step = T * 32;
     int4 *cov;
     unsigned long long *gains;
     uint32_t noteAddr, barAddr;
-    auto tell = [&] {
-        Lead best;
-        lead_init(best);
-        unsigned long long at = 0;
-        for (int q = lane; q < t.ld4; q += 32) {
-            const uint32_t nib = t.bits[q >> 3] >> ((q & 7) * 4);
-            const ulonglong2 a0 = reinterpret_cast<const ulonglong2 *>(gains)[2 * q], a1 = reinterpret_cast<const ulonglong2 *>(gains)[2 * q + 1];
-            const unsigned long long g[4] = {a0.x, a0.y, a1.x, a1.y};
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const uint32_t k = (nib >> u & 1) ? 0u : lead_part(g[u], shift);
-                best.o = max(best.o, min(best.e, k));
-                if (k >= best.e && k) {
-                    const uint32_t low = low_part(g[u], shift, 4 * q + u);
-                    best.low = k > best.e ? low : max(best.low, low);
-                    best.e = k;
-                }
-            }
+    volatile Fresh *fresh;
+    uint32_t updates = 0;                                  // lane i: of block i
+    auto tell = [&](int i) {
+        const Summary sum = summarize(scan_gains(t.bits, gains, t.ld4, tid, step, shift), shift, T, lane);
+        unsigned long long top = sum.top;
+        if (T > 1) {
+            if (lane == 0) t.tm->best[t.warpIn] = top;
+            team_barrier(t.team, T);
+            if (t.warpIn == 0) top = warp_max_u64(lane < T ? t.tm->best[lane] : 0ull);
         }
-        (void)at;
-        const Summary sum = summarize(best, shift, 1, lane);
+        if (tid == 0) st_async(noteAddr, top, barAddr);
         post(t, sum, noteAddr, barAddr);
-        if (lane == 0) st_async(noteAddr, sum.top, barAddr);
-    };
-    for (int i = 0; i < mine; ++i) {
-        const int j = where(i, cov, gains, noteAddr, barAddr);
-        for (int q = lane; q < t.ld4; q += 32) {
-            cov[q] = make_int4(0, 0, 0, 0);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) gains[4 * q + u] = 4 * q + u < c.M ? (unsigned long long)__ldcg(prm.g0 + c.row0 + 4 * q + u) : 0ull;
+        if (t.warpIn == 0 && lane == i) {
+            fresh->sample = top ? key_sample(top) : -1;
+            __threadfence_block();
+            fresh->update = updates;
         }
-        if (prm.quota[(int64_t)l * prm.W + j] > 0) tell();
+    };
+    if (tid == 0) t.tm->count[0] = t.tm->count[1] = 0;
+    int par = 0;
+    for (int i = 0; i < mine; ++i) {
+        const int j = where(i, cov, gains, noteAddr, barAddr, fresh);
+        for (int q = tid; q < t.ld4; q += step) {
+            if (!kCut) cov[q] = make_int4(0, 0, 0, 0);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) gains[4 * q + u] = 4 * q + u < c.M ? (unsigned long long)__ldcg(prm.g0 + c.row0 + 4 * q + u) + bias : 0ull;
+        }
+        if (prm.quota[(int64_t)l * prm.W + j] > 0) tell(i);
     }
-    // lane i watches the command of the team's i-th block
-    const uint32_t at = cmd0 + (uint32_t)(min(lane, mine - 1) * cmdStride);
-    uint32_t had = 0;
-    for (;;) {
+    team_barrier(t.team, T);
+    for (uint32_t n = 1;; ++n) {
+        const uint32_t at = cmds + ((n - 1) & (uint32_t)(prm.ring - 1)) * 8;
         unsigned long long cmd = 0;
-        unsigned pending = 0, spin = 0;
-        do {
+        unsigned spin = 0;
+        for (;;) {
             cmd = ld_relaxed(at);
-            pending = __ballot_sync(0xffffffffu, lane < mine && (uint32_t)(cmd >> 32) != had);
-        } while (pending == 0 && ++spin < kPollLimit);
-        if (pending == 0) {
+            if ((uint32_t)(cmd >> 32) == n) break;
+            if (++spin >= kPollLimit) break;
+        }
+        if (spin >= kPollLimit) {
             if (lane == 0) atomicOr(prm.status, kDevTimeout);
             break;
         }
-        const int who = __ffs(pending) - 1;
-        const uint32_t what = __shfl_sync(0xffffffffu, (uint32_t)cmd, who);
-        if (lane == who) had = (uint32_t)(cmd >> 32);
+        __syncwarp();
+        const uint32_t what = (uint32_t)cmd & 0xfffffu;
+        const int i = (int)((uint32_t)cmd >> 20);
         if (what == kStopCmd) break;
-        where(who, cov, gains, noteAddr, barAddr);
-        if (what == kScanCmd) {
-            cluster_fence();
+        where(i, cov, gains, noteAddr, barAddr, fresh);
+        ++corrected;
+        if (kCut) {
+            // gain = column sum - twice the tie to the block: the sample's row is the tie's growth
+            const int4 *row = t.S4 + (int64_t)((int)what - 1) * t.ld4;
+            for (int q = tid; q < t.ld4; q += step) {
+                const int4 r = __ldg(row + q);
+                ulonglong2 *p = reinterpret_cast<ulonglong2 *>(gains) + 2 * q;
+                const ulonglong2 k0 = p[0], k1 = p[1];
+                p[0] = make_ulonglong2(take_off(k0.x, 2 * r.x), take_off(k0.y, 2 * r.y));
+                p[1] = make_ulonglong2(take_off(k1.x, 2 * r.z), take_off(k1.y, 2 * r.w));
+            }
         } else {
-            ++corrected;
-            take_in_lists(t, (int)what - 1, cov, rows, [&](int n) {
-                RowStream rs(t, n);
+            take_in_lists(t, (int)what - 1, cov, t.tm->count, par, rows, [&](int m) {
 #pragma unroll 1
-                for (int q = lane; q < t.ld4; q += 32) {
+                for (int q = tid; q < t.ld4; q += step) {
                     ulonglong2 *p = reinterpret_cast<ulonglong2 *>(gains) + 2 * q;
                     const ulonglong2 k0 = p[0], k1 = p[1];
                     unsigned long long k[4] = {k0.x, k0.y, k1.x, k1.y};
-                    if (rs.piece(k)) {
+                    if (correct_piece(t.S4 + q, t.list, m, prm.one, k)) {
                         p[0] = make_ulonglong2(k[0], k[1]);
                         p[1] = make_ulonglong2(k[2], k[3]);
                     }
                 }
-                copies_wait<0>();
             });
         }
+        if (lane == i) ++updates;
         __syncwarp();
-        tell();
+        tell(i);
     }
 }
 
 // The leader's loop over the picks of class c.  One warp; lane p % 32 keeps the value and the room of block p, and the
 // parity of the mbarrier on which the block's notes arrive (they go on from class to class).
-template <int KW>
-__device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsigned char *shared, uint32_t C, unsigned long long bias, uint32_t &parities)
+template <int KW, bool kMany>
+__device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsigned char *shared, uint32_t C, unsigned long long bias, uint32_t turn, uint32_t &parities)
 {
     const int lane = threadIdx.x & 31, W = prm.W, T = prm.teamWarps;
-    const uint32_t noteBytes = (1 + kEntries + T) * 8;
+    const NoteLayout layout{T};
+    const uint32_t noteBytes = layout.tracked();
+    const int nTeams = prm.warps / T;
+    volatile uint32_t *queue = reinterpret_cast<uint32_t *>(shared + prm.offQueue);      // commands given to each team
     const uint32_t base = smem32(shared);
     volatile uint32_t *bits = reinterpret_cast<uint32_t *>(shared + prm.offBits);
     const uint32_t myBits = remote(base + prm.offBits, (uint32_t)lane < C ? lane : 0);
-    volatile const Note *notes = reinterpret_cast<const Note *>(shared + prm.offNotes);
+    volatile const unsigned long long *notes = reinterpret_cast<const unsigned long long *>(shared + prm.offNotes);
     const uint32_t bars = base + prm.offBars;
     unsigned long long f[KW];              // (value + kZeroValue) << 7 | block
     int room[KW];
     uint32_t seq[KW], cmdAddr[KW];
+    uint32_t qWord[KW];                    // kMany: block's number in its team << 20 | its team's entry of queue
     uint32_t awaited = 0;                  // bit k: block lane + 32 k owes a note
 #pragma unroll
     for (int k = 0; k < KW; ++k) {
@@ -674,12 +868,28 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
         f[k] = (kZeroValue << 7) | (unsigned long long)p;
         seq[k] = 0;
         room[k] = p < W ? prm.quota[(int64_t)l * W + p] : 0;
-        cmdAddr[k] = remote(base + prm.offCmd + (uint32_t)((p < W ? p : 0) / C) * 8, (uint32_t)(p < W ? p : 0) % C);
+        const uint32_t owner = (uint32_t)(p < W ? p : 0) & (C - 1), slot = (uint32_t)(p < W ? p : 0) >> prm.logC;
+        cmdAddr[k] = remote(base + prm.offCmd + (slot & (nTeams - 1)) * prm.ring * 8, owner);
+        qWord[k] = slot >> prm.logTeams << 20 | (owner * nTeams + (slot & (nTeams - 1)));
         if (room[k] > 0) {
             bar_expect(bars + p * 8, noteBytes);
             awaited |= 1u << k;
         }
     }
+    // (run by the lane that keeps block p, k = p / 32)
+    auto command = [&](int k, uint32_t what) {
+#pragma unroll
+        for (int i = 0; i < KW; ++i)
+            if (i == k) {
+                uint32_t n = ++seq[i];
+                if (kMany) {
+                    n = queue[qWord[i] & 0xfffffu] + 1;
+                    queue[qWord[i] & 0xfffffu] = n;
+                    what |= qWord[i] & 0xfff00000u;
+                }
+                st_remote(cmdAddr[i] + ((n - 1) & (uint32_t)(prm.ring - 1)) * 8, ((unsigned long long)n << 32) | what);
+            }
+    };
     __syncwarp();
     unsigned rescans = 0;
     bool ok = true;
@@ -704,6 +914,13 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
         for (int k = 0; k < KW; ++k) others = room[k] > 0 && lane + 32 * k != j ? umin(others, f[k]) : others;
         others = ~warp_max_u64(~others);
         unsigned long long best = 0;
+        uint32_t updates = 0;
+        if (kMany) {
+#pragma unroll
+            for (int k = 0; k < KW; ++k) if (k == jk) updates = seq[k];
+            updates = __shfl_sync(0xffffffffu, updates, jl);
+        }
+        unsigned polls = 0;
         for (;;) {
             if (waits) {
                 unsigned spin = 0;
@@ -716,17 +933,38 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
                 parity ^= 1;
                 if (lane == jl) { awaited &= ~(1u << jk); parities ^= 1u << jk; }
             }
-            best = notes[j].word[0];
+            volatile const unsigned long long *note = notes + j * layout.words();
+            best = note[0];
+            if (kMany) {
+                const unsigned long long x = note[layout.now()], y = note[layout.now() + 1];
+                const uint32_t tag = (uint32_t)x & 0xffffu;
+                if (tag == ((uint32_t)y & 0xffffu) && (tag & 0xffu) != 0 && (uint32_t)(y >> 32) == updates) best = (x & ~0xffffull) | (y >> 16 & 0xffffull);
+            }
             {
                 const int s = key_sample(best);
-                if (best != 0 && !(bits[s >> 5] >> (s & 31) & 1)) break;
+                if (kMany ? __all_sync(0xffffffffu, best != 0 && best == __shfl_sync(0xffffffffu, best, 0) && !(bits[s >> 5] >> (s & 31) & 1))
+                          : best != 0 && !(bits[s >> 5] >> (s & 31) & 1))
+                    break;
             }
-            // the best one has been taken: the best of those left, if none that the note leaves out can lead
-            const unsigned long long k = lane < kEntries + T ? notes[j].word[1 + lane] : 0ull;
-            const int s = key_sample(k);
-            const bool free = lane < kEntries && k != 0 && !(bits[s >> 5] >> (s & 31) & 1);
-            best = warp_max_u64(free ? k : 0ull);
-            if (best != 0 && __ballot_sync(0xffffffffu, lane >= kEntries && k >= best) == 0) break;
+            if (!kMany || polls == 0) {
+                // the best one has been taken: the best of those left, if none that the note leaves out can lead
+                const unsigned long long k = lane < kEntries + T ? note[1 + lane] : 0ull;
+                const int s = key_sample(k);
+                const bool free = lane < kEntries && k != 0 && !(bits[s >> 5] >> (s & 31) & 1);
+                best = warp_max_u64(free ? k : 0ull);
+                if (best != 0 && __ballot_sync(0xffffffffu, lane >= kEntries && k >= best) == 0) break;
+            }
+            if (kMany) {
+                // a refreshing warp is looking for others already
+                waits = 0;
+                if (polls == 0) ++rescans;
+                if (++polls >= kPollLimit) {
+                    if (lane == 0) atomicOr(prm.status, kDevTimeout);
+                    ok = false;
+                    break;
+                }
+                continue;
+            }
             // every candidate that is sure to lead has been taken by other blocks: look again
             ++rescans;
             waits = 1;
@@ -734,8 +972,7 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
             if (lane == jl) {
                 bar_expect(bars + j * 8, noteBytes);
                 awaited |= 1u << jk;
-#pragma unroll
-                for (int q = 0; q < KW; ++q) if (q == jk) st_remote(cmdAddr[q], ((unsigned long long)++seq[q] << 32) | kScanCmd);
+                command(jk, kScanCmd);
             }
         }
         if (!ok) break;
@@ -751,7 +988,7 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
                     if (left > 0) {                   // (a full block needs no gains any more)
                         bar_expect(bars + j * 8, noteBytes);
                         awaited |= 1u << k;
-                        st_remote(cmdAddr[k], ((unsigned long long)++seq[k] << 32) | (unsigned long long)(v + 1));
+                        command(k, (uint32_t)(v + 1));
                     }
                 }
         }
@@ -777,29 +1014,32 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
             parities ^= 1u << k;
         }
         if (p < W) {
-            st_remote(cmdAddr[k], ((unsigned long long)++seq[k] << 32) | kStopCmd);
+            if (!kMany || p >> prm.logC < nTeams) command(k, kStopCmd);
             const long long value = (long long)(f[k] >> 7) - (long long)kZeroValue;
             prm.fval[(int64_t)l * W + p] = prm.fixedExp ? __double_as_longlong(ldexp((double)value, -prm.fixedExp[l])) : value;
         }
     }
+    if (kMany && lane < (int)C) st_remote32(remote(base + prm.offFresh, lane), turn);
     if (lane == 0 && rescans) atomicAdd(prm.stats + 9, (unsigned long long)rescans);
 }
 
-// P: pieces per thread of teams with one block; 0: teams of one warp with several blocks (kSmemState: which all fit the
+// P: pieces per thread of teams with one block; 0: teams with several blocks (kSmemState: which all fit the
 // CTAs' shared memory).  kCut: graph-cut objective.
-template <int KW, int P, bool kSmemState, bool kCut>
-__global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) greedy_cluster_kernel(const __grid_constant__ ClusterParams prm)
+template <int KW, int P, int kT, bool kSmemState, bool kCut>
+__global__ void __launch_bounds__((kMaxWarps + 1 + (P == 0 ? kRefreshers : 0)) * 32, 1) greedy_cluster_kernel(const __grid_constant__ ClusterParams prm)
 {
     extern __shared__ __align__(128) unsigned char shared[];
     __shared__ int shClass[2];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t rank = cluster_rank(), C = cluster_size();
-    const int NW = prm.warps, T = prm.teamWarps, nTeams = NW / T;
+    const int NW = kMaxWarps, T = kT ? kT : prm.teamWarps, nTeams = NW / T;
     const uint32_t base = smem32(shared);
     uint32_t *bits = reinterpret_cast<uint32_t *>(shared + prm.offBits);
     volatile unsigned long long *cmds = reinterpret_cast<volatile unsigned long long *>(shared + prm.offCmd);
     const int W = prm.W;
     uint32_t parities = 0;
+    const NoteLayout layout{T};
+    uint32_t classes = 0;                                  // this cluster has begun
 
     if (rank == 0)
         for (int p = threadIdx.x; p < W; p += blockDim.x) bar_init(base + prm.offBars + p * 8, 1);
@@ -814,6 +1054,7 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) greedy_cluster_kernel
         cluster_barrier();
         const int l = *(volatile int *)&shClass[turn];
         if (l < 0) break;
+        ++classes;
         const ClassDesc c = prm.desc[l];
         if (c.M == 0) {
             if (rank == 0) for (int p = threadIdx.x; p < W; p += blockDim.x) prm.fval[(int64_t)l * W + p] = 0;
@@ -835,7 +1076,17 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) greedy_cluster_kernel
         }
         for (int i = threadIdx.x; i < (c.ld + 31) / 32; i += blockDim.x)
             bits[i] = 32 * i + 32 <= c.M ? 0u : (32 * i >= c.M ? ~0u : ~0u << (c.M - 32 * i));
-        for (int i = threadIdx.x; i < prm.slots; i += blockDim.x) cmds[i] = 0;
+        for (int i = threadIdx.x; i < nTeams * prm.ring; i += blockDim.x) cmds[i] = 0;
+        // (shared memory for the refreshing warps: the number of the class that has ended last, then what teams tell them)
+        volatile uint32_t *ended = reinterpret_cast<uint32_t *>(shared + prm.offFresh);
+        volatile Fresh *fresh0 = reinterpret_cast<Fresh *>(shared + prm.offFresh + 16);
+        if (P == 0)
+            for (int i = threadIdx.x; i < prm.slots; i += blockDim.x) { fresh0[i].sample = -1; fresh0[i].update = kNotYet; }
+        if (P == 0 && threadIdx.x == 0 && classes == 1) *ended = 0;
+        if (P == 0 && rank == 0) {
+            for (int i = threadIdx.x; i < (int)C * nTeams; i += blockDim.x) reinterpret_cast<uint32_t *>(shared + prm.offQueue)[i] = 0;
+            for (int i = threadIdx.x; i < W * layout.words(); i += blockDim.x) reinterpret_cast<unsigned long long *>(shared + prm.offNotes)[i] = 0;
+        }
         cluster_barrier();
         // graph cut: gains lie within three times the largest sum of |S| over a row, either way
         const unsigned long long top = __ldcg(prm.topGain + l);
@@ -843,7 +1094,15 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) greedy_cluster_kernel
         const int shift = shift_for(bias + (kCut ? 3 : 1) * top);
 
         if (warp == NW) {
-            if (rank == 0) lead<KW>(prm, l, c, shared, C, bias, parities);
+            if (rank == 0) lead<KW, P == 0>(prm, l, c, shared, C, bias, classes, parities);
+        } else if (warp > NW) {
+            // refreshing warps (kSmemState: gains elsewhere may still be on their way)
+            refresh_notes(prm, bits, ld4, shift, fresh0, warp - NW - 1, kRefreshers, prm.slots, ended, classes, [&](int slot, const unsigned long long *&gains) {
+                const int j = slot * (int)C + (int)rank;
+                if (kSmemState) gains = reinterpret_cast<const unsigned long long *>(shared + prm.offGains) + (size_t)slot * prm.maxLd;
+                else gains = reinterpret_cast<const unsigned long long *>(prm.gains + c.vOff) + (size_t)j * c.ld;
+                return remote(base + prm.offNotes, 0) + (uint32_t)(j * layout.words()) * 8;
+            });
         } else {
             const int team = warp / T;
             TeamView t;
@@ -858,11 +1117,11 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) greedy_cluster_kernel
             if (P > 0) {
                 const int j = team * (int)C + (int)rank;
                 if (team < prm.slots && j < W && prm.quota[(int64_t)l * W + j] > 0)
-                    team_of_one<(P > 0 ? P : 1), kCut>(prm, c, t, reinterpret_cast<int4 *>(shared + prm.offCover) + (size_t)team * (prm.maxLd >> 2), shift, bias,
-                                                       base + prm.offCmd + team * 8, notes0 + j * (uint32_t)sizeof(Note), bars0 + j * 8, corrected, rows);
+                    team_of_one<(P > 0 ? P : 1), kT, kCut>(prm, c, t, reinterpret_cast<int4 *>(shared + prm.offCover) + (size_t)team * (prm.maxLd >> 2), shift, bias,
+                                                       base + prm.offCmd + team * prm.ring * 8, notes0 + j * (uint32_t)layout.words() * 8, bars0 + j * 8, corrected, rows);
             } else {
                 // the i-th block of the team
-                auto where = [&](int i, int4 *&cov, unsigned long long *&gains, uint32_t &noteAddr, uint32_t &barAddr) -> int {
+                auto where = [&](int i, int4 *&cov, unsigned long long *&gains, uint32_t &noteAddr, uint32_t &barAddr, volatile Fresh *&fresh) -> int {
                     const int slot = team + i * nTeams, j = slot * (int)C + (int)rank;
                     if (kSmemState) {
                         cov = reinterpret_cast<int4 *>(shared + prm.offCover) + (size_t)slot * (prm.maxLd >> 2);
@@ -871,13 +1130,14 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) greedy_cluster_kernel
                         cov = reinterpret_cast<int4 *>(prm.cover + c.vOff) + (size_t)j * ld4;
                         gains = reinterpret_cast<unsigned long long *>(prm.gains + c.vOff) + (size_t)j * c.ld;
                     }
-                    noteAddr = notes0 + j * (uint32_t)sizeof(Note);
+                    noteAddr = notes0 + j * (uint32_t)layout.words() * 8;
+                    fresh = fresh0 + slot;
                     barAddr = bars0 + j * 8;
                     return j;
                 };
                 int mine = 0;
                 while (team + mine * nTeams < prm.slots && (team + mine * nTeams) * (int)C + (int)rank < W) ++mine;
-                if (mine > 0) team_of_many(prm, l, c, t, mine, shift, base + prm.offCmd + team * 8, nTeams * 8, where, corrected, rows);
+                if (mine > 0) team_of_many<kCut>(prm, l, c, t, mine, shift, bias, base + prm.offCmd + team * prm.ring * 8, where, corrected, rows);
             }
             if (lane == 0 && t.warpIn == 0 && corrected) {
                 atomicAdd(prm.stats + 15, (unsigned long long)corrected);
@@ -940,24 +1200,36 @@ static int pow2_at_least(int x)
 
 typedef void (*ClusterKernel)(ClusterParams);
 
-template <int KW, bool kCut>
-static ClusterKernel pick_kernel(int P, bool smemState)
+template <int KW, int kT, bool kCut>
+static ClusterKernel pick_one(int P)
 {
-    if (P == 1) return greedy_cluster_kernel<KW, 1, true, kCut>;
-    if (P == 2) return greedy_cluster_kernel<KW, 2, true, kCut>;
-    if (P == 3) return greedy_cluster_kernel<KW, 3, true, kCut>;
-    if (P > 0 && P <= 4) return greedy_cluster_kernel<KW, 4, true, kCut>;
-    if (P > 0) return greedy_cluster_kernel<KW, kMaxPieces, true, kCut>;
-    return smemState ? greedy_cluster_kernel<KW, 0, true, false> : greedy_cluster_kernel<KW, 0, false, false>;
+    switch (P) {
+    case 1: return greedy_cluster_kernel<KW, 1, kT, true, kCut>;
+    case 2: return greedy_cluster_kernel<KW, 2, kT, true, kCut>;
+    case 3: return greedy_cluster_kernel<KW, 3, kT, true, kCut>;
+    case 4: return greedy_cluster_kernel<KW, 4, kT, true, kCut>;
+    default: return greedy_cluster_kernel<KW, kMaxPieces, kT, true, kCut>;
+    }
+}
+// (P = 0: teams with several blocks)
+template <int KW, bool kCut>
+static ClusterKernel pick_kernel(int P, int T, bool smemState)
+{
+    if (P == 0) return smemState ? greedy_cluster_kernel<KW, 0, 0, true, kCut> : greedy_cluster_kernel<KW, 0, 0, false, kCut>;
+    if constexpr (KW == 1 && !kCut) {
+        if (T == 16) return pick_one<KW, 16, kCut>(P);
+        if (T == 8) return pick_one<KW, 8, kCut>(P);
+    }
+    return pick_one<KW, 0, kCut>(P);
 }
 
-static rcd_status launch_cluster(rcd_ctx *ctx, ClusterKernel kernel, const ClusterParams &prm, int C, int clusters, size_t smem, cudaStream_t st, int *active)
+static rcd_status launch_cluster(rcd_ctx *ctx, ClusterKernel kernel, const ClusterParams &prm, int threads, int C, int clusters, size_t smem, cudaStream_t st, int *active)
 {
     RCD_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     RCD_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(clusters * C));
-    cfg.blockDim = dim3((unsigned)((prm.warps + 1) * 32));
+    cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -982,30 +1254,76 @@ struct ClusterPlan {
     size_t smem;
     ClusterParams prm;         // teamWarps, slots, maxLd, rowPieces and the offsets are set
 };
-static size_t cluster_layout(const Sizes &sz, int maxLd, int C, bool state, ClusterPlan &plan)
+static size_t cluster_layout(const Sizes &sz, int maxLd, int C, bool state, size_t cap, ClusterPlan &plan)
 {
     ClusterParams &prm = plan.prm;
     prm.warps = kMaxWarps;
     prm.maxLd = maxLd;
     prm.slots = (sz.W + C - 1) / C;
-    // a team per block, of as many warps as a row has work for
+    prm.logC = 0;
+    while ((1 << prm.logC) < C) ++prm.logC;
+    const int ld4 = maxLd / 4;
+    // A team per block, of as many warps as there are, or teams of several blocks: then a team has as many warps as a row
+    // keeps busy (at least three quarters of their threads).
     const int most = kMaxWarps / std::min(kMaxWarps, pow2_at_least(prm.slots));
-    prm.teamWarps = std::min(most, pow2_at_least((maxLd / 4 + 31) / 32));
-    const int step = prm.teamWarps * 32, teams = kMaxWarps / prm.teamWarps;
-    plan.P = prm.slots > kMaxWarps ? 0 : (maxLd / 4 + step - 1) / step;
-    size_t off = 0;
-    auto take = [&](size_t bytes) { const size_t at = off; off = (off + bytes + 15) / 16 * 16; return (int32_t)at; };
-    prm.offTeams = take(sizeof(Team) * (size_t)teams);
-    prm.offCmd = take(8 * (size_t)prm.slots);
-    prm.offBits = take((size_t)(maxLd + 31) / 32 * 4);
-    prm.offLists = take(sizeof(Raised) * (size_t)(kMaxWarps * kRaisedPerWarp + teams));
-    prm.offNotes = take(sizeof(Note) * (size_t)sz.W);
-    prm.offBars = take(8 * (size_t)sz.W);
-    prm.rowPieces = std::max(kRing, plan.P) * step;
-    prm.offRows = take((size_t)std::min(teams, prm.slots) * prm.rowPieces * 16);
-    prm.offCover = take(plan.P > 0 || state ? (size_t)prm.slots * maxLd * 4 : 0);
-    prm.offGains = take(plan.P == 0 && state ? (size_t)prm.slots * maxLd * 8 : 0);
-    return off;
+    const int one = std::min(most, pow2_at_least((ld4 + 31) / 32));
+    int busy = 1;
+    for (int T = 2; T <= kMaxWarps; T *= 2)
+        if (4 * ld4 >= 3 * ((ld4 + 32 * T - 1) / (32 * T)) * 32 * T) busy = T;
+    const int onePieces = (ld4 + 32 * one - 1) / (32 * one);
+    int pieces = onePieces;
+    auto place = [&](bool many, bool state) -> size_t {
+        prm.teamWarps = many ? busy : one;
+        plan.P = many ? 0 : pieces;
+        const int step = prm.teamWarps * 32, teams = kMaxWarps / prm.teamWarps;
+        const int perTeam = (prm.slots + teams - 1) / teams;
+        prm.ring = many ? pow2_at_least(perTeam + 1) : 1;
+        const NoteLayout note{prm.teamWarps};
+        size_t off = 0;
+        auto take = [&](size_t bytes) { const size_t at = off; off = (off + bytes + 15) / 16 * 16; return (int32_t)at; };
+        prm.offTeams = take(sizeof(Team) * (size_t)teams);
+        prm.offCmd = take(8 * (size_t)teams * prm.ring);
+        prm.offBits = take((size_t)(maxLd + 31) / 32 * 4);
+        prm.offLists = take(sizeof(Raised) * (size_t)(kMaxWarps * kRaisedPerWarp + teams));
+        prm.offNotes = take((size_t)note.words() * 8 * (size_t)sz.W);
+        prm.offBars = take(8 * (size_t)sz.W);
+        prm.offQueue = take(many ? 4 * (size_t)C * teams : 0);
+        prm.offFresh = take(many ? 16 + sizeof(Fresh) * (size_t)prm.slots : 0);
+        prm.logTeams = 0;
+        while ((1 << prm.logTeams) < teams) ++prm.logTeams;
+        // (a team's row buffer: the row of the sample foreseen, and the rows on their way through apply_list)
+        prm.rowPieces = many ? 0 : (std::max(plan.P * step, plan.P <= 3 ? kRowStages * ld4 : kPieceStages * step) + 7) / 8 * 8;
+        // (asynchronous 16-byte copies whose destination sits differently in its 32-byte sector than the source fetch two
+        // sectors each: rows of S start on sectors, so the buffers do)
+        off = (off + 127) / 128 * 128;
+        prm.offRows = take((size_t)std::min(teams, prm.slots) * prm.rowPieces * 16);
+        prm.offCover = take(!many || state ? (size_t)prm.slots * maxLd * 4 : 0);
+        prm.offGains = take(many && state ? (size_t)prm.slots * maxLd * 8 : 0);
+        plan.smemState = state;
+        return off;
+    };
+    const bool oneFits = prm.slots <= kMaxWarps && onePieces <= kMaxPieces;
+    const bool manyFits = (prm.slots + kMaxWarps / busy - 1) / (kMaxWarps / busy) <= 31;
+    // (graph cut: the blocks' best candidates are mostly the same samples, so notes have to be kept fresh)
+    if (oneFits && !(sz.graphCut && manyFits && prm.slots > 1) && (prm.slots == 1 || 2 * one >= busy || !manyFits)) {
+        const size_t need = place(false, true);
+        if (need <= cap) return need;
+    }
+    if (manyFits) {
+        const size_t need = place(true, true);
+        if (need <= cap) return need;
+    }
+    if (oneFits) {
+        size_t need = place(false, true);
+        if (need <= cap) return need;
+        if (plan.P == 3) {                                 // (less room: the four-piece kernel's ring)
+            pieces = 4;
+            need = place(false, true);
+            if (need <= cap) return need;
+        }
+    }
+    if (!state && manyFits) return place(true, false);     // (coverage and gains in global memory)
+    return cap + 1;
 }
 
 // Whether the cluster form takes a problem, and how: chosen by the library (no pass-based form or option asked for),
@@ -1029,7 +1347,7 @@ static bool cluster_plan(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassD
     for (int i = 0; i < 5; ++i)
         if (ctx->maxClusters[i] == 0) {
             plan.prm.warps = kMaxWarps;
-            if (launch_cluster(ctx, pick_kernel<1, false>(3, true), plan.prm, 1 << i, 1, cap, nullptr, &ctx->maxClusters[i]) != RCD_OK) return false;
+            if (launch_cluster(ctx, pick_kernel<1, false>(3, 16, true), plan.prm, (kMaxWarps + 1) * 32, 1 << i, 1, cap, nullptr, &ctx->maxClusters[i]) != RCD_OK) return false;
         }
     // Cluster size: the one whose clusters, drawing classes largest first, finish soonest by the estimate that a class of
     // M samples takes M (M / C + 300) (corrections, shared by the CTAs, and the chain of picks); blocks have to stay on
@@ -1043,8 +1361,7 @@ static bool cluster_plan(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassD
     for (int i = 0; (1 << i) <= most; ++i) {
         const int C = 1 << i, n = ctx->maxClusters[i];
         if (n < 1) continue;
-        const size_t smem = cluster_layout(sz, maxLd, C, true, plan);
-        if (smem > cap || plan.P > kMaxPieces || (sz.graphCut && plan.P == 0)) continue;
+        if (cluster_layout(sz, maxLd, C, true, cap, plan) > cap) continue;
         double time = 0;
         std::vector<double> busy((size_t)std::min<size_t>((size_t)n, sizes.size()), 0.0);      // (a heap of the clusters' finishing times)
         for (int M : sizes) {
@@ -1056,16 +1373,12 @@ static bool cluster_plan(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassD
         if (plan.C == 0 || time < bestTime) { plan.C = C; bestTime = time; }
     }
     if (plan.C > 0) {
-        plan.smem = cluster_layout(sz, maxLd, plan.C, true, plan);
-        plan.smemState = true;
+        plan.smem = cluster_layout(sz, maxLd, plan.C, true, cap, plan);
     } else {
-        // several blocks per warp, in global memory
-        plan.C = 1;
-        plan.smem = cluster_layout(sz, maxLd, plan.C, false, plan);
-        plan.smemState = false;
-        if (plan.P > 0 || plan.smem > cap) return false;
+        plan.C = std::min(8, most);
+        plan.smem = cluster_layout(sz, maxLd, plan.C, false, cap, plan);
+        if (plan.smem > cap) return false;
     }
-    if (sz.graphCut && plan.P == 0) return false;
     int idx = 0;
     while ((1 << idx) < plan.C) ++idx;
     if (ctx->maxClusters[idx] < 1) return false;
@@ -1109,9 +1422,10 @@ rcd_status launch_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const Workspace 
         ctx->kernelLaunches += 2;
         RCD_CUDA(ctx, cudaGetLastError());
     }
-    ClusterKernel kernel = sz.graphCut ? (sz.W <= 32 ? pick_kernel<1, true>(plan.P, plan.smemState) : pick_kernel<4, true>(plan.P, plan.smemState))
-                                       : (sz.W <= 32 ? pick_kernel<1, false>(plan.P, plan.smemState) : pick_kernel<4, false>(plan.P, plan.smemState));
-    const rcd_status rs = launch_cluster(ctx, kernel, prm, plan.C, plan.clusters, plan.smem, st, nullptr);
+    ClusterKernel kernel = sz.graphCut ? (sz.W <= 32 ? pick_kernel<1, true>(plan.P, prm.teamWarps, plan.smemState) : pick_kernel<4, true>(plan.P, prm.teamWarps, plan.smemState))
+                                       : (sz.W <= 32 ? pick_kernel<1, false>(plan.P, prm.teamWarps, plan.smemState)
+                                          : sz.W <= 64 ? pick_kernel<2, false>(plan.P, prm.teamWarps, plan.smemState) : pick_kernel<4, false>(plan.P, prm.teamWarps, plan.smemState));
+    const rcd_status rs = launch_cluster(ctx, kernel, prm, (kMaxWarps + 1 + (plan.P == 0 ? kRefreshers : 0)) * 32, plan.C, plan.clusters, plan.smem, st, nullptr);
     if (rs != RCD_OK) return rs;
     ctx->steps = sz.maxM;
     ctx->phaseNsDev = ws.phaseNs;

@@ -252,10 +252,8 @@ rcd_status launch_cut_objective(rcd_ctx *ctx, const Sizes &sz, const ClassDesc *
                                 const int32_t *assignment, void *partValues, void *total, void *scratch, cudaStream_t st);
 
 // objective from an assignment
-rcd_status launch_objective(rcd_ctx *ctx, rcd_feat_dtype dtype, const Sizes &sz, const ClassDesc *descDev,
-                            const std::vector<ClassDesc> &descHost, const void *S, const int32_t *perm,
-                            const int32_t *assignment, void *partValues, void *total, void *scratch,
-                            cudaStream_t st);
+rcd_status launch_objective(rcd_ctx *ctx, rcd_feat_dtype dtype, const Sizes &sz, const Workspace &ws, const int32_t *assignment,
+                            void *partValues, void *total, cudaStream_t st);
 
 
 #ifdef __CUDACC__

@@ -1,86 +1,145 @@
 // f(A_j^l) = sum_{i in V_l} max(0, max_{v' in A_j^l} S[i][v'])  for every class l and block j,
 // straight from the definition (Section 4, item 2), given an assignment vector.  Independent of
-// the greedy state: one pass over S; per row i a per-block running maximum, then fixed-order sums
-// so that the fp64 result is reproducible.
+// the greedy state: one pass over S, then sums in a fixed order so that the fp64 result is reproducible.
+//
+// S is symmetric, so the maximum over a block's members may be taken down the members' rows: a thread owns four columns
+// and keeps their running maximum, nothing is shared and every load is coalesced.  The rows are walked in block order (a
+// counting sort of each class's samples); where the block changes, or at the end of a unit of work, the maxima join the
+// block's coverage vector by atomic maxima.  Bound by reading S once (1 GB for ten classes of 5000: 1.25 ms with a
+// shared-memory atomic maximum per element, @@ now, of which 0.15 ms is the copy bandwidth's share).
 #include "rcd_internal.h"
 
 #include <type_traits>
 
 namespace rcd {
 
-constexpr int kObjWarps = 8;
-constexpr int kObjRowsPerCta = 64;
+constexpr int kObjThreads = 128;          // x 4 columns
+constexpr int kObjRows = 128;             // rows of S per unit of work
 
-template <typename SV, typename FV>
-__global__ void __launch_bounds__(kObjWarps * 32, 4) objective_rows_kernel(const ClassDesc *__restrict__ desc,
-                                                                       const SV *__restrict__ S,
-                                                                       const int32_t *__restrict__ perm,
-                                                                       const int32_t *__restrict__ assignment,
-                                                                       int32_t W, int32_t maxBlocks,
-                                                                       FV *__restrict__ partial)
+// Class-sorted positions of a class's samples, sorted by block (samples in no block left out); counts[l][W] members.
+__global__ void __launch_bounds__(512) objective_members_kernel(const ClassDesc *__restrict__ desc, const int32_t *__restrict__ perm,
+                                                               const int32_t *__restrict__ assignment, int32_t W,
+                                                               int32_t *__restrict__ members, int32_t *__restrict__ counts)
 {
-    extern __shared__ unsigned char shraw[];
-    // per warp: running maxima of the current row [W] (int bits) and accumulated sums [W]
-    FV *shAcc = reinterpret_cast<FV *>(shraw);                        // [kObjWarps][W]
-    int32_t *shMax = reinterpret_cast<int32_t *>(shAcc + (size_t)kObjWarps * W);   // [kObjWarps][W]
-    const int l = blockIdx.y;
-    const ClassDesc c = desc[l];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int row0 = blockIdx.x * kObjRowsPerCta;
-    if (row0 >= c.M) return;
-    FV *acc = shAcc + (size_t)warp * W;
-    int32_t *mx = shMax + (size_t)warp * W;
-    for (int p = lane; p < W; p += 32) acc[p] = (FV)0;
-    const SV *Sl = S + c.sOff;
+    extern __shared__ int32_t shCount[];
+    const ClassDesc c = desc[blockIdx.x];
     const int32_t *pl = perm + c.row0;
-    for (int r = warp; r < kObjRowsPerCta; r += kObjWarps) {
-        const int i = row0 + r;
-        if (i >= c.M) break;
-        for (int p = lane; p < W; p += 32) mx[p] = 0;
-        __syncwarp();
-        const SV *row = Sl + (int64_t)i * c.ld;
-        for (int v = lane; v < c.M; v += 32) {
-            const int a = assignment[pl[v]];
-            if (a < 0 || a >= W) continue;
-            const SV s = row[v];
-            if (s > (SV)0) {
-                // positive int32 and positive fp32 both order like their bit patterns
-                int32_t bits;
-                if constexpr (sizeof(SV) == 4 && !std::is_integral<SV>::value) bits = __float_as_int((float)s);
-                else bits = (int32_t)s;
-                atomicMax(&mx[a], bits);
-            }
-        }
-        __syncwarp();
-        for (int p = lane; p < W; p += 32) {
-            int32_t bits = mx[p];
-            FV val;
-            if constexpr (!std::is_integral<SV>::value) val = (FV)__int_as_float(bits);
-            else val = (FV)bits;
-            acc[p] += val;
-        }
-        __syncwarp();
+    for (int p = threadIdx.x; p < W; p += 512) shCount[p] = 0;
+    __syncthreads();
+    for (int v = threadIdx.x; v < c.M; v += 512) {
+        const int a = assignment[pl[v]];
+        if (a >= 0 && a < W) atomicAdd(&shCount[a], 1);
     }
     __syncthreads();
-    FV *out = partial + ((int64_t)l * maxBlocks + blockIdx.x) * W;
-    for (int p = threadIdx.x; p < W; p += blockDim.x) {
-        FV s = (FV)0;
-        for (int w = 0; w < kObjWarps; ++w) s += shAcc[(size_t)w * W + p];
-        out[p] = s;
+    if (threadIdx.x < 32) {
+        int run = 0;
+        for (int p0 = 0; p0 < W; p0 += 32) {
+            const int p = p0 + threadIdx.x;
+            const int n = p < W ? shCount[p] : 0;
+            int sum = n;
+            for (int off = 1; off < 32; off <<= 1) {
+                const int up = __shfl_up_sync(0xffffffffu, sum, off);
+                if ((int)threadIdx.x >= off) sum += up;
+            }
+            if (p < W) {
+                counts[(int64_t)blockIdx.x * W + p] = n;
+                shCount[p] = run + sum - n;
+            }
+            run += __shfl_sync(0xffffffffu, sum, 31);
+        }
+    }
+    __syncthreads();
+    // (the order inside a block does not matter: a maximum is taken over it)
+    for (int v = threadIdx.x; v < c.M; v += 512) {
+        const int a = assignment[pl[v]];
+        if (a >= 0 && a < W) members[c.row0 + atomicAdd(&shCount[a], 1)] = v;
     }
 }
 
-template <typename FV>
-__global__ void objective_reduce_kernel(const ClassDesc *__restrict__ desc, const FV *__restrict__ partial,
-                                        int32_t L, int32_t W, int32_t maxBlocks, FV *__restrict__ partValues)
+template <typename SV>
+__device__ __forceinline__ int32_t above_zero(SV s)
 {
-    int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    // positive int32 and positive fp32 both order like their bit patterns
+    if constexpr (std::is_integral<SV>::value) return max((int32_t)s, 0);
+    else return s > 0.f ? __float_as_int(s) : 0;
+}
+
+template <typename SV>
+__global__ void __launch_bounds__(kObjThreads, 8) objective_cover_kernel(const ClassDesc *__restrict__ desc, const SV *__restrict__ S,
+                                                                        const int32_t *__restrict__ members, const int32_t *__restrict__ counts,
+                                                                        int32_t W, int32_t *__restrict__ cover)
+{
+    __shared__ int32_t shMember[kObjRows];
+    __shared__ int32_t shBlock[kObjRows];
+    const int l = blockIdx.z;
+    const ClassDesc c = desc[l];
+    const int first = blockIdx.y * kObjRows;
+    if (first >= c.M || (int)blockIdx.x * kObjThreads * 4 >= c.ld) return;
+    // the block of every row of this unit
+    {
+        const int32_t *cnt = counts + (int64_t)l * W;
+        const int k = first + threadIdx.x;
+        int run = 0, p = 0;
+        for (; p < W; ++p) {
+            const int n = cnt[p];
+            if (k < run + n) break;
+            run += n;
+        }
+        shBlock[threadIdx.x] = p < W ? p : -1;
+        shMember[threadIdx.x] = p < W ? members[c.row0 + k] : 0;
+    }
+    __syncthreads();
+    const int q = blockIdx.x * kObjThreads + threadIdx.x;
+    if (4 * q >= c.ld) return;
+    typedef typename std::conditional<std::is_integral<SV>::value, int4, float4>::type V4;
+    const V4 *col = reinterpret_cast<const V4 *>(S + c.sOff) + q;
+    const int ld4 = c.ld >> 2;
+    int4 m = make_int4(0, 0, 0, 0);
+    int block = shBlock[0];
+    auto flush = [&] {
+        int32_t *to = cover + c.vOff + (int64_t)block * c.ld + 4 * q;
+        if (m.x) atomicMax(to, m.x);
+        if (m.y) atomicMax(to + 1, m.y);
+        if (m.z) atomicMax(to + 2, m.z);
+        if (m.w) atomicMax(to + 3, m.w);
+        m = make_int4(0, 0, 0, 0);
+    };
+    for (int k0 = 0; k0 < kObjRows && shBlock[k0] >= 0; k0 += 8) {
+        V4 x[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) x[u] = __ldcs(col + (int64_t)shMember[k0 + u] * ld4);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int b = shBlock[k0 + u];
+            if (b < 0) break;
+            if (b != block) { flush(); block = b; }
+            m.x = max(m.x, above_zero<SV>(x[u].x));
+            m.y = max(m.y, above_zero<SV>(x[u].y));
+            m.z = max(m.z, above_zero<SV>(x[u].z));
+            m.w = max(m.w, above_zero<SV>(x[u].w));
+        }
+    }
+    if (block >= 0) flush();
+}
+
+// f of one (class, block): the sum of its coverage vector, by one warp.
+template <typename SV, typename FV>
+__global__ void __launch_bounds__(256) objective_sum_kernel(const ClassDesc *__restrict__ desc, const int32_t *__restrict__ cover, int32_t L, int32_t W,
+                                                           FV *__restrict__ partValues)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t idx = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (idx >= (int64_t)L * W) return;
-    int l = (int)(idx / W), p = (int)(idx % W);
-    int nb = (desc[l].M + kObjRowsPerCta - 1) / kObjRowsPerCta;
+    const ClassDesc c = desc[idx / W];
+    const int4 *v = reinterpret_cast<const int4 *>(cover + c.vOff + (idx % W) * c.ld);
     FV s = (FV)0;
-    for (int b = 0; b < nb; ++b) s += partial[((int64_t)l * maxBlocks + b) * W + p];
-    partValues[idx] = s;
+    for (int q = lane; q < c.ld / 4; q += 32) {
+        const int4 x = v[q];
+        if constexpr (std::is_integral<SV>::value) s += (FV)x.x + (FV)x.y + (FV)x.z + (FV)x.w;
+        else s += (FV)__int_as_float(x.x) + (FV)__int_as_float(x.y) + (FV)__int_as_float(x.z) + (FV)__int_as_float(x.w);
+    }
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (lane == 0) partValues[idx] = s;
 }
 
 // one CTA, fixed strided partials then a fixed tree: reproducible
@@ -101,40 +160,32 @@ __global__ void __launch_bounds__(256, 1) objective_total_kernel(const FV *__res
 }
 
 template <typename SV, typename FV>
-static rcd_status run_objective(rcd_ctx *ctx, const Sizes &sz, const ClassDesc *descDev,
-                                const std::vector<ClassDesc> &descHost, const void *S, const int32_t *perm,
-                                const int32_t *assignment, void *partValues, void *total, void *scratch,
+static rcd_status run_objective(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, const int32_t *assignment, void *partValues, void *total,
                                 cudaStream_t st)
 {
-    const int maxBlocks = (int)((sz.maxM + kObjRowsPerCta - 1) / kObjRowsPerCta);
-    const size_t smem = (size_t)kObjWarps * sz.W * (sizeof(FV) + sizeof(int32_t));
-    if ((int64_t)smem > ctx->maxSmemOptin - 1024)
-        return fail(ctx, RCD_ERR_UNSUPPORTED, "W=%d needs %zu bytes of shared memory in the objective kernel", sz.W, smem);
-    if (sz.L > 65535) return fail(ctx, RCD_ERR_UNSUPPORTED, "objective: more than 65535 classes");
-    RCD_CUDA(ctx, cudaFuncSetAttribute(objective_rows_kernel<SV, FV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if (maxBlocks > 0) {
-        dim3 grid(maxBlocks, sz.L);
-        objective_rows_kernel<SV, FV><<<grid, kObjWarps * 32, smem, st>>>(descDev, (const SV *)S, perm, assignment, sz.W,
-                                                                         maxBlocks, (FV *)scratch);
-        ctx->kernelLaunches++;
+    const int64_t rowBlocks = (sz.maxM + kObjRows - 1) / kObjRows;
+    if (sz.L > 65535 || rowBlocks > 65535) return fail(ctx, RCD_ERR_UNSUPPORTED, "objective: more than 65535 classes or row blocks");
+    int32_t *members = ws.cand, *counts = ws.cnt, *cover = (int32_t *)ws.cover;
+    if (sz.maxM > 0) {
+        RCD_CUDA(ctx, cudaMemsetAsync(cover, 0, (size_t)sz.vElems * sizeof(int32_t), st));
+        objective_members_kernel<<<sz.L, 512, (size_t)sz.W * 4, st>>>(ws.desc, ws.perm, assignment, sz.W, members, counts);
+        const dim3 grid((unsigned)((pad_row(sz.maxM) + 4 * kObjThreads - 1) / (4 * kObjThreads)), (unsigned)rowBlocks, (unsigned)sz.L);
+        objective_cover_kernel<SV><<<grid, kObjThreads, 0, st>>>(ws.desc, (const SV *)ws.S, members, counts, sz.W, cover);
+        ctx->kernelLaunches += 2;
     }
-    int64_t n = (int64_t)sz.L * sz.W;
-    objective_reduce_kernel<FV><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(descDev, (const FV *)scratch, sz.L, sz.W,
-                                                                           maxBlocks, (FV *)partValues);
+    const int64_t n = (int64_t)sz.L * sz.W;
+    objective_sum_kernel<SV, FV><<<(unsigned)((n + 7) / 8), 256, 0, st>>>(ws.desc, cover, sz.L, sz.W, (FV *)partValues);
     objective_total_kernel<FV><<<1, 256, 0, st>>>((const FV *)partValues, n, (FV *)total);
     ctx->kernelLaunches += 2;
     RCD_CUDA(ctx, cudaGetLastError());
     return RCD_OK;
 }
 
-rcd_status launch_objective(rcd_ctx *ctx, rcd_feat_dtype dtype, const Sizes &sz, const ClassDesc *descDev,
-                            const std::vector<ClassDesc> &descHost, const void *S, const int32_t *perm,
-                            const int32_t *assignment, void *partValues, void *total, void *scratch,
-                            cudaStream_t st)
+rcd_status launch_objective(rcd_ctx *ctx, rcd_feat_dtype dtype, const Sizes &sz, const Workspace &ws, const int32_t *assignment,
+                            void *partValues, void *total, cudaStream_t st)
 {
-    if (dtype == RCD_FEAT_I8)
-        return run_objective<int32_t, long long>(ctx, sz, descDev, descHost, S, perm, assignment, partValues, total, scratch, st);
-    return run_objective<float, double>(ctx, sz, descDev, descHost, S, perm, assignment, partValues, total, scratch, st);
+    if (dtype == RCD_FEAT_I8) return run_objective<int32_t, long long>(ctx, sz, ws, assignment, partValues, total, st);
+    return run_objective<float, double>(ctx, sz, ws, assignment, partValues, total, st);
 }
 
 }  // namespace rcd
