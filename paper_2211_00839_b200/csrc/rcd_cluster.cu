@@ -26,33 +26,39 @@ namespace rcd {
 
 namespace {
 
-constexpr int kMaxWarps = 16;             // team warps per CTA (one more warp leads in the cluster's first CTA)
-constexpr int kMaxPieces = 5;             // pieces per thread of a team that keeps its block's gains in registers
+constexpr int kMaxWarps = 16;             // team warps per CTA; one more warp leads in the cluster's first CTA
+// One block per CTA and long rows: a team of 15 warps, so that with the leader there are 16 and a thread may hold 128
+// registers (17 warps get the share of 20: 96).
+__host__ __device__ constexpr int team_warps(int T) { return T == 15 ? 15 : kMaxWarps; }
+constexpr int kMaxPieces = 7;             // pieces per thread of a team that keeps its block's gains in registers
 constexpr int kRaisedPerWarp = 64;        // raised columns a team lists at a time, per warp
 constexpr int kClusterBlocks = 128;       // blocks a cluster can lead (their notes sit in one CTA's shared memory)
-constexpr int kEntries = 16;              // candidates per note
 constexpr uint32_t kScanCmd = 0u;         // a command's low word: look again;
 constexpr uint32_t kStopCmd = 0xfffffu;   //   the class is done;  anything else: sample + 1 joins the block
 constexpr int kRefreshers = 3;            // warps per CTA that refresh notes (17 warps would occupy the registers of 20 anyway)
 constexpr unsigned kPollLimit = 1u << 28;
 constexpr unsigned long long kZeroValue = 1ull << 55;   // (tracked values of the graph cut can be negative)
 
-// What the leader is told about a block (a note, words of 64 bits):
+// Candidates a warp of a team of T contributes to a note: a power of two, at most 16 in all.
+__host__ __device__ constexpr int entries_per_warp(int T) { return T <= 1 ? 16 : T <= 2 ? 8 : T <= 4 ? 4 : T <= 8 ? 2 : 1; }
+
+// What the leader is told about a block (a note, words of 64 bits; E = candidates per warp):
 //   [0]            the key of its best candidate (0: none)
-//   [1, 17)        for the case that other blocks took that one: keys of leading candidates
-//   [17, 17 + T)   per team warp a key that no candidate left out exceeds
+//   [1, 1 + TE)    for the case that other blocks took that one: keys of leading candidates
+//   then T words   per team warp a key that no candidate left out exceeds
 // and, where blocks sit in shared memory, two words that a refreshing warp rewrites whenever the best candidate has been
 // taken (with many blocks that happens often before the block's turn comes):
-//   [17 + T, 19 + T)     gain << 16 | tag and update number << 32 | (65535 - sample) << 16 | tag, where tag is the update
-//                        number's last byte << 8 | a running number from 1
+//   gain << 16 | tag  and  update number << 32 | (65535 - sample) << 16 | tag,  where tag is the update number's last byte
+//   << 8 | a running number from 1
 // A candidate that was a block's best and is still unassigned is still its best: gains move only when the block itself
 // receives a sample.
 struct NoteLayout {
     int T;
-    __host__ __device__ int bounds() const { return 1 + kEntries; }
-    __host__ __device__ int now() const { return 1 + kEntries + T; }
-    __host__ __device__ int words() const { return 3 + kEntries + T; }
-    __host__ __device__ uint32_t tracked() const { return (uint32_t)(1 + kEntries + T) * 8; }   // bytes a new note brings
+    __host__ __device__ int entries() const { return T * entries_per_warp(T); }
+    __host__ __device__ int bounds() const { return 1 + entries(); }
+    __host__ __device__ int now() const { return 1 + entries() + T; }
+    __host__ __device__ int words() const { return 3 + entries() + T; }
+    __host__ __device__ uint32_t tracked() const { return (uint32_t)(1 + entries() + T) * 8; }   // bytes a new note brings
 };
 
 struct __align__(16) Raised {
@@ -85,14 +91,13 @@ struct ClusterParams {
     int32_t *status;
     unsigned long long *stats; // phase words
     int32_t L, W;
-    int32_t warps;             // team warps per CTA
     int32_t teamWarps;         // T
     int32_t slots;             // blocks per CTA at most
     int32_t maxLd;
     int32_t rowPieces;         // 16-byte pieces of a team's row buffer
     unsigned long long *topGain;   // [L] zero at the start: largest gain for an empty block (graph cut: row sum of |S|)
     uint32_t one;              // the value 1, opaque to the compiler
-    int32_t logC, logTeams;
+    int32_t logC;
     // byte offsets into dynamic shared memory
     int32_t offTeams, offLists, offRows, offCmd, offBits, offNotes, offBars, offQueue, offFresh, offCover, offGains;
     int32_t ring;              // command words per team (a power of two)
@@ -277,7 +282,7 @@ __device__ __forceinline__ uint32_t low_part(unsigned long long g, int shift, in
 // (shift for gains up to g: gain >> shift stays below 2^31)
 __device__ __forceinline__ int shift_for(unsigned long long g) { return max(0, 33 - __clzll((long long)g)); }
 
-// A warp's part of a note: entries (one per tile of 2 T lanes, at the tile's first lane), a bound on every gain that is
+// A warp's part of a note: entries (one per tile of 32 / E lanes, at the tile's first lane), a bound on every gain that is
 // no entry, and the best of all, as keys.
 struct Summary {
     unsigned long long entry, bound, top;
@@ -290,8 +295,9 @@ __device__ __forceinline__ unsigned long long key_of(uint32_t e, uint32_t low, i
 __device__ __forceinline__ Summary summarize(Lead b, int shift, int T, int lane)
 {
     Summary s;
-    if (T <= 2) {
-        for (int off = 1; off < 2 * T; off <<= 1) {
+    const int tile = 32 / entries_per_warp(T);
+    if (tile <= 4) {
+        for (int off = 1; off < tile; off <<= 1) {
             const uint32_t e2 = __shfl_xor_sync(0xffffffffu, b.e, off), o2 = __shfl_xor_sync(0xffffffffu, b.o, off), l2 = __shfl_xor_sync(0xffffffffu, b.low, off);
             b.o = max(max(b.o, o2), min(b.e, e2));
             b.low = b.e > e2 ? b.low : (b.e < e2 ? l2 : max(b.low, l2));
@@ -303,7 +309,6 @@ __device__ __forceinline__ Summary summarize(Lead b, int shift, int T, int lane)
         const uint32_t m = __reduce_max_sync(0xffffffffu, b.e);
         s.top = key_of(m, __reduce_max_sync(0xffffffffu, b.e == m ? b.low : 0u), shift);
     } else {
-        const int tile = 2 * T;
         const uint32_t mask = tile == 32 ? 0xffffffffu : ((1u << tile) - 1u) << (lane & ~(tile - 1));
         const uint32_t m = __reduce_max_sync(mask, b.e);
         const uint32_t low = __reduce_max_sync(mask, b.e == m ? b.low : 0u);
@@ -318,11 +323,11 @@ __device__ __forceinline__ Summary summarize(Lead b, int shift, int T, int lane)
     }
     return s;
 }
-__device__ __forceinline__ void post(const TeamView &t, const Summary &s, uint32_t noteAddr, uint32_t barAddr)
+__device__ __forceinline__ void post(const TeamView &t, int T, const Summary &s, uint32_t noteAddr, uint32_t barAddr)
 {
-    const int tile = 2 * t.T;
-    if ((t.lane & (tile - 1)) == 0) st_async(noteAddr + (uint32_t)(1 + (t.warpIn * 32 + t.lane) / tile) * 8, s.entry, barAddr);
-    if (t.lane == 1) st_async(noteAddr + (uint32_t)(1 + kEntries + t.warpIn) * 8, s.bound, barAddr);
+    const int E = entries_per_warp(T), tile = 32 / E;
+    if ((t.lane & (tile - 1)) == 0) st_async(noteAddr + (uint32_t)(1 + t.warpIn * E + t.lane / tile) * 8, s.entry, barAddr);
+    if (t.lane == 1) st_async(noteAddr + (uint32_t)(1 + T * E + t.warpIn) * 8, s.bound, barAddr);
 }
 
 // Columns of one piece that rose join the list, as far as it has room.  Returns which did.
@@ -400,10 +405,10 @@ __device__ __forceinline__ bool correct_piece(const int4 *S4q, const Raised *lis
 // shared memory, each thread reading back only what it copied itself, so that loads in flight hold no registers.
 // Up to three pieces: row by row over all pieces (a list entry and a row's address serve them all), eight rows of room,
 // four under way while four are applied: 403 cycles per row of 20 KB and SM with 80 SMs at it, of which L2 and HBM take 350
-// (538 with two rows at a time).  More pieces, or less room: piece by piece through a ring of twelve 16-byte slots per
-// thread (480 - 500 cycles).
+// (538 with two rows at a time).  More pieces, or less room: piece by piece through a ring of sixteen 16-byte slots per
+// thread, twelve under way (530 cycles; 620 with eight).
 template <int P> struct RowRing { static constexpr bool byRow = P <= 3; };
-constexpr int kRowStages = 8, kPieceStages = 12;
+constexpr int kRowStages = 8, kPieceStages = 16;
 template <int P, int kT>
 __device__ __forceinline__ void apply_list(const TeamView &t, int n, uint32_t one, unsigned long long (&g)[P][4])
 {
@@ -464,12 +469,13 @@ __device__ __forceinline__ void apply_list(const TeamView &t, int n, uint32_t on
         };
         fetch();
         fetch();
+        fetch();
 #pragma unroll
         for (int p = 0; p < P; ++p) {
             if (p * step + first < t.ld4) {
 #pragma unroll 1
                 for (int e = 0; e < n; e += 4) {
-                    copies_wait<1>();
+                    copies_wait<2>();
                     const int4 *x = ring + at * step;
                     at += 4;
                     if (at == kPieceStages) at = 0;
@@ -517,8 +523,7 @@ __device__ __forceinline__ void take_in_lists(const TeamView &t, int v, int4 *co
 }
 
 // A team with one block, its stored gains in registers: P pieces of four columns per thread.  Coverage in shared memory.
-// kT: warps per team (0: known at run time).  Registers are what this function is short of (17 warps share the file as 20
-// would: 96 per thread), hence the constants.
+// kT: warps per team (0: known at run time; a constant saves registers and address arithmetic).
 template <int P, int kT, bool kCut>
 __device__ __forceinline__ void team_of_one(const ClusterParams &prm, const ClassDesc &c, const TeamView &t, int4 *cov, int shift, unsigned long long bias,
                                             uint32_t cmdAddr, uint32_t noteAddr, uint32_t barAddr, unsigned &corrected, unsigned &rows)
@@ -578,7 +583,7 @@ __device__ __forceinline__ void team_of_one(const ClusterParams &prm, const Clas
             top = warp_max_u64(lane < T ? t.tm->best[lane] : 0ull);
         }
         if (tid == 0) st_async(noteAddr, top, barAddr);
-        post(t, sum, noteAddr, barAddr);
+        post(t, T, sum, noteAddr, barAddr);
         // (the warp's best may be the block's best some picks from now: its row comes to L2 meanwhile)
         if (T > 1 && newTop && sum.top) {
             newTop = false;
@@ -774,7 +779,7 @@ __device__ __forceinline__ void team_of_many(const ClusterParams &prm, int l, co
             if (t.warpIn == 0) top = warp_max_u64(lane < T ? t.tm->best[lane] : 0ull);
         }
         if (tid == 0) st_async(noteAddr, top, barAddr);
-        post(t, sum, noteAddr, barAddr);
+        post(t, T, sum, noteAddr, barAddr);
         if (t.warpIn == 0 && lane == i) {
             fresh->sample = top ? key_sample(top) : -1;
             __threadfence_block();
@@ -850,7 +855,7 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
     const int lane = threadIdx.x & 31, W = prm.W, T = prm.teamWarps;
     const NoteLayout layout{T};
     const uint32_t noteBytes = layout.tracked();
-    const int nTeams = prm.warps / T;
+    const int nTeams = team_warps(T) / T;
     volatile uint32_t *queue = reinterpret_cast<uint32_t *>(shared + prm.offQueue);      // commands given to each team
     const uint32_t base = smem32(shared);
     volatile uint32_t *bits = reinterpret_cast<uint32_t *>(shared + prm.offBits);
@@ -869,8 +874,8 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
         seq[k] = 0;
         room[k] = p < W ? prm.quota[(int64_t)l * W + p] : 0;
         const uint32_t owner = (uint32_t)(p < W ? p : 0) & (C - 1), slot = (uint32_t)(p < W ? p : 0) >> prm.logC;
-        cmdAddr[k] = remote(base + prm.offCmd + (slot & (nTeams - 1)) * prm.ring * 8, owner);
-        qWord[k] = slot >> prm.logTeams << 20 | (owner * nTeams + (slot & (nTeams - 1)));
+        cmdAddr[k] = remote(base + prm.offCmd + slot % nTeams * prm.ring * 8, owner);
+        qWord[k] = slot / nTeams << 20 | (owner * nTeams + slot % nTeams);
         if (room[k] > 0) {
             bar_expect(bars + p * 8, noteBytes);
             awaited |= 1u << k;
@@ -948,11 +953,11 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
             }
             if (!kMany || polls == 0) {
                 // the best one has been taken: the best of those left, if none that the note leaves out can lead
-                const unsigned long long k = lane < kEntries + T ? note[1 + lane] : 0ull;
+                const unsigned long long k = lane < layout.entries() + T ? note[1 + lane] : 0ull;
                 const int s = key_sample(k);
-                const bool free = lane < kEntries && k != 0 && !(bits[s >> 5] >> (s & 31) & 1);
+                const bool free = lane < layout.entries() && k != 0 && !(bits[s >> 5] >> (s & 31) & 1);
                 best = warp_max_u64(free ? k : 0ull);
-                if (best != 0 && __ballot_sync(0xffffffffu, lane >= kEntries && k >= best) == 0) break;
+                if (best != 0 && __ballot_sync(0xffffffffu, lane >= layout.entries() && k >= best) == 0) break;
             }
             if (kMany) {
                 // a refreshing warp is looking for others already
@@ -1026,13 +1031,14 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
 // P: pieces per thread of teams with one block; 0: teams with several blocks (kSmemState: which all fit the
 // CTAs' shared memory).  kCut: graph-cut objective.
 template <int KW, int P, int kT, bool kSmemState, bool kCut>
-__global__ void __launch_bounds__((kMaxWarps + 1 + (P == 0 ? kRefreshers : 0)) * 32, 1) greedy_cluster_kernel(const __grid_constant__ ClusterParams prm)
+__global__ void __launch_bounds__((P == 0 ? kMaxWarps + 1 + kRefreshers : team_warps(kT) + 1) * 32, 1) greedy_cluster_kernel(const __grid_constant__ ClusterParams prm)
 {
     extern __shared__ __align__(128) unsigned char shared[];
     __shared__ int shClass[2];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t rank = cluster_rank(), C = cluster_size();
-    const int NW = kMaxWarps, T = kT ? kT : prm.teamWarps, nTeams = NW / T;
+    constexpr int NW = team_warps(kT);
+    const int T = kT ? kT : prm.teamWarps, nTeams = NW / T;
     const uint32_t base = smem32(shared);
     uint32_t *bits = reinterpret_cast<uint32_t *>(shared + prm.offBits);
     volatile unsigned long long *cmds = reinterpret_cast<volatile unsigned long long *>(shared + prm.offCmd);
@@ -1116,7 +1122,7 @@ __global__ void __launch_bounds__((kMaxWarps + 1 + (P == 0 ? kRefreshers : 0)) *
             const uint32_t notes0 = remote(base + prm.offNotes, 0), bars0 = remote(base + prm.offBars, 0);
             if (P > 0) {
                 const int j = team * (int)C + (int)rank;
-                if (team < prm.slots && j < W && prm.quota[(int64_t)l * W + j] > 0)
+                if (team < prm.slots && team < nTeams && j < W && prm.quota[(int64_t)l * W + j] > 0)
                     team_of_one<(P > 0 ? P : 1), kT, kCut>(prm, c, t, reinterpret_cast<int4 *>(shared + prm.offCover) + (size_t)team * (prm.maxLd >> 2), shift, bias,
                                                        base + prm.offCmd + team * prm.ring * 8, notes0 + j * (uint32_t)layout.words() * 8, bars0 + j * 8, corrected, rows);
             } else {
@@ -1208,6 +1214,7 @@ static ClusterKernel pick_one(int P)
     case 2: return greedy_cluster_kernel<KW, 2, kT, true, kCut>;
     case 3: return greedy_cluster_kernel<KW, 3, kT, true, kCut>;
     case 4: return greedy_cluster_kernel<KW, 4, kT, true, kCut>;
+    case 5: return greedy_cluster_kernel<KW, 5, kT, true, kCut>;
     default: return greedy_cluster_kernel<KW, kMaxPieces, kT, true, kCut>;
     }
 }
@@ -1216,9 +1223,10 @@ template <int KW, bool kCut>
 static ClusterKernel pick_kernel(int P, int T, bool smemState)
 {
     if (P == 0) return smemState ? greedy_cluster_kernel<KW, 0, 0, true, kCut> : greedy_cluster_kernel<KW, 0, 0, false, kCut>;
-    if constexpr (KW == 1 && !kCut) {
-        if (T == 16) return pick_one<KW, 16, kCut>(P);
-        if (T == 8) return pick_one<KW, 8, kCut>(P);
+    if constexpr (KW == 1) {
+        if (T == 15) return pick_one<KW, 15, kCut>(P);         // (one block per CTA: 16 at most)
+        if constexpr (!kCut)
+            if (T == 8) return pick_one<KW, 8, kCut>(P);
     }
     return pick_one<KW, 0, kCut>(P);
 }
@@ -1257,7 +1265,6 @@ struct ClusterPlan {
 static size_t cluster_layout(const Sizes &sz, int maxLd, int C, bool state, size_t cap, ClusterPlan &plan)
 {
     ClusterParams &prm = plan.prm;
-    prm.warps = kMaxWarps;
     prm.maxLd = maxLd;
     prm.slots = (sz.W + C - 1) / C;
     prm.logC = 0;
@@ -1265,8 +1272,9 @@ static size_t cluster_layout(const Sizes &sz, int maxLd, int C, bool state, size
     const int ld4 = maxLd / 4;
     // A team per block, of as many warps as there are, or teams of several blocks: then a team has as many warps as a row
     // keeps busy (at least three quarters of their threads).
-    const int most = kMaxWarps / std::min(kMaxWarps, pow2_at_least(prm.slots));
-    const int one = std::min(most, pow2_at_least((ld4 + 31) / 32));
+    const int rowWarps = (ld4 + 31) / 32;
+    int one = std::min(kMaxWarps / std::min(kMaxWarps, pow2_at_least(prm.slots)), pow2_at_least(rowWarps));
+    if (prm.slots == 1 && rowWarps > 8) one = 15;
     int busy = 1;
     for (int T = 2; T <= kMaxWarps; T *= 2)
         if (4 * ld4 >= 3 * ((ld4 + 32 * T - 1) / (32 * T)) * 32 * T) busy = T;
@@ -1275,7 +1283,8 @@ static size_t cluster_layout(const Sizes &sz, int maxLd, int C, bool state, size
     auto place = [&](bool many, bool state) -> size_t {
         prm.teamWarps = many ? busy : one;
         plan.P = many ? 0 : pieces;
-        const int step = prm.teamWarps * 32, teams = kMaxWarps / prm.teamWarps;
+        const int warps = many ? kMaxWarps : team_warps(prm.teamWarps);
+        const int step = prm.teamWarps * 32, teams = warps / prm.teamWarps;
         const int perTeam = (prm.slots + teams - 1) / teams;
         prm.ring = many ? pow2_at_least(perTeam + 1) : 1;
         const NoteLayout note{prm.teamWarps};
@@ -1284,13 +1293,11 @@ static size_t cluster_layout(const Sizes &sz, int maxLd, int C, bool state, size
         prm.offTeams = take(sizeof(Team) * (size_t)teams);
         prm.offCmd = take(8 * (size_t)teams * prm.ring);
         prm.offBits = take((size_t)(maxLd + 31) / 32 * 4);
-        prm.offLists = take(sizeof(Raised) * (size_t)(kMaxWarps * kRaisedPerWarp + teams));
+        prm.offLists = take(sizeof(Raised) * (size_t)(warps * kRaisedPerWarp + teams));
         prm.offNotes = take((size_t)note.words() * 8 * (size_t)sz.W);
         prm.offBars = take(8 * (size_t)sz.W);
         prm.offQueue = take(many ? 4 * (size_t)C * teams : 0);
         prm.offFresh = take(many ? 16 + sizeof(Fresh) * (size_t)prm.slots : 0);
-        prm.logTeams = 0;
-        while ((1 << prm.logTeams) < teams) ++prm.logTeams;
         // (a team's row buffer: the row of the sample foreseen, and the rows on their way through apply_list)
         prm.rowPieces = many ? 0 : (std::max(plan.P * step, plan.P <= 3 ? kRowStages * ld4 : kPieceStages * step) + 7) / 8 * 8;
         // (asynchronous 16-byte copies whose destination sits differently in its 32-byte sector than the source fetch two
@@ -1305,7 +1312,7 @@ static size_t cluster_layout(const Sizes &sz, int maxLd, int C, bool state, size
     const bool oneFits = prm.slots <= kMaxWarps && onePieces <= kMaxPieces;
     const bool manyFits = (prm.slots + kMaxWarps / busy - 1) / (kMaxWarps / busy) <= 31;
     // (graph cut: the blocks' best candidates are mostly the same samples, so notes have to be kept fresh)
-    if (oneFits && !(sz.graphCut && manyFits && prm.slots > 1) && (prm.slots == 1 || 2 * one >= busy || !manyFits)) {
+    if (oneFits && !(sz.graphCut && manyFits && prm.slots > 1) && (prm.slots == 1 || 2 * one + 2 >= busy || !manyFits)) {
         const size_t need = place(false, true);
         if (need <= cap) return need;
     }
@@ -1346,8 +1353,7 @@ static bool cluster_plan(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassD
     plan.prm = ClusterParams{};
     for (int i = 0; i < 5; ++i)
         if (ctx->maxClusters[i] == 0) {
-            plan.prm.warps = kMaxWarps;
-            if (launch_cluster(ctx, pick_kernel<1, false>(3, 16, true), plan.prm, (kMaxWarps + 1) * 32, 1 << i, 1, cap, nullptr, &ctx->maxClusters[i]) != RCD_OK) return false;
+            if (launch_cluster(ctx, pick_kernel<1, false>(3, 15, true), plan.prm, 16 * 32, 1 << i, 1, cap, nullptr, &ctx->maxClusters[i]) != RCD_OK) return false;
         }
     // Cluster size: the one whose clusters, drawing classes largest first, finish soonest by the estimate that a class of
     // M samples takes M (M / C + 300) (corrections, shared by the CTAs, and the chain of picks); blocks have to stay on
@@ -1425,7 +1431,7 @@ rcd_status launch_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const Workspace 
     ClusterKernel kernel = sz.graphCut ? (sz.W <= 32 ? pick_kernel<1, true>(plan.P, prm.teamWarps, plan.smemState) : pick_kernel<4, true>(plan.P, prm.teamWarps, plan.smemState))
                                        : (sz.W <= 32 ? pick_kernel<1, false>(plan.P, prm.teamWarps, plan.smemState)
                                           : sz.W <= 64 ? pick_kernel<2, false>(plan.P, prm.teamWarps, plan.smemState) : pick_kernel<4, false>(plan.P, prm.teamWarps, plan.smemState));
-    const rcd_status rs = launch_cluster(ctx, kernel, prm, (kMaxWarps + 1 + (plan.P == 0 ? kRefreshers : 0)) * 32, plan.C, plan.clusters, plan.smem, st, nullptr);
+    const rcd_status rs = launch_cluster(ctx, kernel, prm, (plan.P == 0 ? kMaxWarps + 1 + kRefreshers : team_warps(prm.teamWarps) + 1) * 32, plan.C, plan.clusters, plan.smem, st, nullptr);
     if (rs != RCD_OK) return rs;
     ctx->steps = sz.maxM;
     ctx->phaseNsDev = ws.phaseNs;
