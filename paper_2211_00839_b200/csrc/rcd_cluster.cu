@@ -99,7 +99,7 @@ struct ClusterParams {
     uint32_t one;              // the value 1, opaque to the compiler
     int32_t logC;
     // byte offsets into dynamic shared memory
-    int32_t offTeams, offLists, offRows, offCmd, offBits, offNotes, offBars, offQueue, offFresh, offCover, offGains;
+    int32_t offTeams, offLists, offRows, offCmd, offBits, offNotes, offBars, offQueue, offFresh, offFirsts, offCover, offGains;
     int32_t ring;              // command words per team (a power of two)
 };
 
@@ -795,7 +795,7 @@ __device__ __forceinline__ void team_of_many(const ClusterParams &prm, int l, co
 #pragma unroll
             for (int u = 0; u < 4; ++u) gains[4 * q + u] = 4 * q + u < c.M ? (unsigned long long)__ldcg(prm.g0 + c.row0 + 4 * q + u) + bias : 0ull;
         }
-        if (prm.quota[(int64_t)l * prm.W + j] > 0) tell(i);
+        (void)j;
     }
     team_barrier(t.team, T);
     for (uint32_t n = 1;; ++n) {
@@ -816,6 +816,11 @@ __device__ __forceinline__ void team_of_many(const ClusterParams &prm, int l, co
         const int i = (int)((uint32_t)cmd >> 20);
         if (what == kStopCmd) break;
         where(i, cov, gains, noteAddr, barAddr, fresh);
+        if (what == kScanCmd) {
+            cluster_fence();
+            tell(i);
+            continue;
+        }
         ++corrected;
         if (kCut) {
             // gain = column sum - twice the tie to the block: the sample's row is the tie's growth
@@ -848,11 +853,16 @@ __device__ __forceinline__ void team_of_many(const ClusterParams &prm, int l, co
 }
 
 // The leader's loop over the picks of class c.  One warp; lane p % 32 keeps the value and the room of block p, and the
-// parity of the mbarrier on which the block's notes arrive (they go on from class to class).
+// parity of the mbarrier on which the block's notes arrive (they go on from class to class).  A pick is a chain of dependent
+// latencies (shuffle, mbarrier, two shared-memory loads, the command); what does not depend on the pick
+// (the least of the other blocks) is computed under them, and a block's state travels in one shuffle.
+// kMany: every block's first sample comes from `firsts`, the greatest gains for an empty block in order (they are the same
+// for all blocks, so notes would be overtaken by one another).
 template <int KW, bool kMany>
-__device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsigned char *shared, uint32_t C, unsigned long long bias, uint32_t turn, uint32_t &parities)
+__device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsigned char *shared, uint32_t C, int T, unsigned long long bias, uint32_t turn,
+                     uint32_t &parities)
 {
-    const int lane = threadIdx.x & 31, W = prm.W, T = prm.teamWarps;
+    const int lane = threadIdx.x & 31, W = prm.W;
     const NoteLayout layout{T};
     const uint32_t noteBytes = layout.tracked();
     const int nTeams = team_warps(T) / T;
@@ -861,47 +871,59 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
     volatile uint32_t *bits = reinterpret_cast<uint32_t *>(shared + prm.offBits);
     const uint32_t myBits = remote(base + prm.offBits, (uint32_t)lane < C ? lane : 0);
     volatile const unsigned long long *notes = reinterpret_cast<const unsigned long long *>(shared + prm.offNotes);
+    volatile const unsigned long long *firsts = reinterpret_cast<const unsigned long long *>(shared + prm.offFirsts);
     const uint32_t bars = base + prm.offBars;
     unsigned long long f[KW];              // (value + kZeroValue) << 7 | block
     int room[KW];
-    uint32_t seq[KW], cmdAddr[KW];
+    uint32_t given[KW];                    // samples (one team per block: commands) given to the block
+    uint32_t cmdAddr[KW];
     uint32_t qWord[KW];                    // kMany: block's number in its team << 20 | its team's entry of queue
-    uint32_t awaited = 0;                  // bit k: block lane + 32 k owes a note
+    // four bits for each k: the block owes a note; parity of its mbarrier; its next sample is its last; it is empty
+    constexpr uint32_t kOwes = 1, kParity = 2, kLast = 4, kEmpty = 8;
+    uint32_t state = 0;
 #pragma unroll
     for (int k = 0; k < KW; ++k) {
         const int p = lane + 32 * k;
         f[k] = (kZeroValue << 7) | (unsigned long long)p;
-        seq[k] = 0;
+        given[k] = 0;
         room[k] = p < W ? prm.quota[(int64_t)l * W + p] : 0;
         const uint32_t owner = (uint32_t)(p < W ? p : 0) & (C - 1), slot = (uint32_t)(p < W ? p : 0) >> prm.logC;
         cmdAddr[k] = remote(base + prm.offCmd + slot % nTeams * prm.ring * 8, owner);
         qWord[k] = slot / nTeams << 20 | (owner * nTeams + slot % nTeams);
-        if (room[k] > 0) {
+        uint32_t st = (parities >> k & 1 ? kParity : 0u) | (room[k] == 1 ? kLast : 0u);
+        if (kMany) {
+            st |= kEmpty;
+        } else if (room[k] > 0) {
             bar_expect(bars + p * 8, noteBytes);
-            awaited |= 1u << k;
+            st |= kOwes;
         }
+        state |= st << (4 * k);
     }
-    // (run by the lane that keeps block p, k = p / 32)
+    // (run by the lane that keeps block lane + 32 k)
     auto command = [&](int k, uint32_t what) {
 #pragma unroll
         for (int i = 0; i < KW; ++i)
             if (i == k) {
-                uint32_t n = ++seq[i];
+                uint32_t n;
                 if (kMany) {
                     n = queue[qWord[i] & 0xfffffu] + 1;
                     queue[qWord[i] & 0xfffffu] = n;
                     what |= qWord[i] & 0xfff00000u;
+                } else {
+                    n = ++given[i];
                 }
                 st_remote(cmdAddr[i] + ((n - 1) & (uint32_t)(prm.ring - 1)) * 8, ((unsigned long long)n << 32) | what);
             }
     };
     __syncwarp();
     unsigned rescans = 0;
+    int nextFirst = 0;
     bool ok = true;
     unsigned long long others = ~0ull, last = ~0ull;       // least of the blocks but the one picked last, and that one's
 #pragma unroll
     for (int k = 0; k < KW; ++k) others = room[k] > 0 ? umin(others, f[k]) : others;
     others = ~warp_max_u64(~others);
+    uint32_t *picks = prm.picks + c.row0;
     for (int t = 0; t < c.M; ++t) {
         const unsigned long long least = umin(others, last);
         if (least == ~0ull) {
@@ -911,113 +933,126 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
         }
         const int j = (int)(least & 127);
         const int jk = KW == 1 ? 0 : j >> 5, jl = j & 31;
-        const uint32_t state = __shfl_sync(0xffffffffu, awaited | parities << 16, jl) >> jk;
-        uint32_t waits = state & 1, parity = state >> 16 & 1;
-        // the least of the other blocks: known before this pick is made
+        const uint32_t st = __shfl_sync(0xffffffffu, state, jl) >> (4 * jk);
+        uint32_t parity = st & kParity;
+        volatile const unsigned long long *note = notes + j * layout.words();
+        auto await = [&]() -> bool {
+            unsigned spin = 0;
+            while (!bar_done(bars + j * 8, parity ? 1u : 0u) && ++spin < kPollLimit) { }
+            parity ^= kParity;
+            if (spin < kPollLimit) return true;
+            if (lane == 0) atomicOr(prm.status, kDevTimeout);
+            return false;
+        };
+        if (st & kOwes) ok = await();
+        if (!ok) break;
+        unsigned long long best = kMany && (st & kEmpty) ? 0ull : note[0];
+        // the least of the other blocks: does not depend on this pick
         others = ~0ull;
 #pragma unroll
         for (int k = 0; k < KW; ++k) others = room[k] > 0 && lane + 32 * k != j ? umin(others, f[k]) : others;
         others = ~warp_max_u64(~others);
-        unsigned long long best = 0;
-        uint32_t updates = 0;
-        if (kMany) {
+        int v = key_sample(best);
+        uint32_t word = bits[v >> 5];
+        if (best == 0 || (word >> (v & 31) & 1)) {
+            // the block's best candidate has been taken by another block, or the block is empty
+            best = 0;
+            if (kMany && (st & kEmpty)) {
+                for (; nextFirst < W; ++nextFirst) {
+                    const unsigned long long k = firsts[nextFirst];
+                    const int s = key_sample(k);
+                    if (k == 0) { nextFirst = W; break; }
+                    if (!(bits[s >> 5] >> (s & 31) & 1)) { best = k; break; }
+                }
+            }
+            uint32_t updates = 0;
+            if (kMany) {
 #pragma unroll
-            for (int k = 0; k < KW; ++k) if (k == jk) updates = seq[k];
-            updates = __shfl_sync(0xffffffffu, updates, jl);
-        }
-        unsigned polls = 0;
-        for (;;) {
-            if (waits) {
-                unsigned spin = 0;
-                while (!bar_done(bars + j * 8, parity) && ++spin < kPollLimit) { }
-                if (spin >= kPollLimit) {
-                    if (lane == 0) atomicOr(prm.status, kDevTimeout);
-                    ok = false;
-                    break;
+                for (int k = 0; k < KW; ++k) if (k == jk) updates = given[k];
+                updates = __shfl_sync(0xffffffffu, updates, jl);
+            }
+            bool noted = !kMany || !(st & kEmpty);         // the note stands for the block's present gains
+            for (unsigned polls = 0; best == 0; ++polls) {
+                if (noted && (!kMany || polls == 0)) {
+                    // the best of the candidates left, if none that the note leaves out can lead
+                    const unsigned long long k = lane < layout.entries() + T ? note[1 + lane] : 0ull;
+                    const int s = key_sample(k);
+                    const bool free = lane < layout.entries() && k != 0 && !(bits[s >> 5] >> (s & 31) & 1);
+                    best = warp_max_u64(free ? k : 0ull);
+                    if (__any_sync(0xffffffffu, lane >= layout.entries() && k >= best)) best = 0;
+                    if (best) break;
                 }
-                parity ^= 1;
-                if (lane == jl) { awaited &= ~(1u << jk); parities ^= 1u << jk; }
-            }
-            volatile const unsigned long long *note = notes + j * layout.words();
-            best = note[0];
-            if (kMany) {
-                const unsigned long long x = note[layout.now()], y = note[layout.now() + 1];
-                const uint32_t tag = (uint32_t)x & 0xffffu;
-                if (tag == ((uint32_t)y & 0xffffu) && (tag & 0xffu) != 0 && (uint32_t)(y >> 32) == updates) best = (x & ~0xffffull) | (y >> 16 & 0xffffull);
-            }
-            {
-                const int s = key_sample(best);
-                if (kMany ? __all_sync(0xffffffffu, best != 0 && best == __shfl_sync(0xffffffffu, best, 0) && !(bits[s >> 5] >> (s & 31) & 1))
-                          : best != 0 && !(bits[s >> 5] >> (s & 31) & 1))
-                    break;
-            }
-            if (!kMany || polls == 0) {
-                // the best one has been taken: the best of those left, if none that the note leaves out can lead
-                const unsigned long long k = lane < layout.entries() + T ? note[1 + lane] : 0ull;
+                ++rescans;
+                if (kMany && noted) {
+                    // a refreshing warp is looking for others already (every lane polls; lane 0's reading counts)
+                    const unsigned long long x = note[layout.now()], y = note[layout.now() + 1];
+                    const uint32_t tag = (uint32_t)x & 0xffffu;
+                    unsigned long long k = 0;
+                    if (tag == ((uint32_t)y & 0xffffu) && (tag & 0xffu) != 0 && (uint32_t)(y >> 32) == updates) k = (x & ~0xffffull) | (y >> 16 & 0xffffull);
+                    k = __shfl_sync(0xffffffffu, k, 0);
+                    const int s = key_sample(k);
+                    if (k != 0 && !(bits[s >> 5] >> (s & 31) & 1)) best = k;
+                    if (polls >= kPollLimit) {
+                        if (lane == 0) atomicOr(prm.status, kDevTimeout);
+                        ok = false;
+                        break;
+                    }
+                    continue;
+                }
+                // every candidate that is sure to lead has been taken by other blocks: the team looks again
+                cluster_fence();                           // (it must see which samples are taken)
+                if (lane == jl) {
+                    bar_expect(bars + j * 8, noteBytes);
+                    command(jk, kScanCmd);
+                }
+                ok = await();
+                if (!ok) break;
+                noted = true;
+                const unsigned long long k = note[0];
                 const int s = key_sample(k);
-                const bool free = lane < layout.entries() && k != 0 && !(bits[s >> 5] >> (s & 31) & 1);
-                best = warp_max_u64(free ? k : 0ull);
-                if (best != 0 && __ballot_sync(0xffffffffu, lane >= layout.entries() && k >= best) == 0) break;
+                if (k != 0 && !(bits[s >> 5] >> (s & 31) & 1)) best = k;
             }
-            if (kMany) {
-                // a refreshing warp is looking for others already
-                waits = 0;
-                if (polls == 0) ++rescans;
-                if (++polls >= kPollLimit) {
-                    if (lane == 0) atomicOr(prm.status, kDevTimeout);
-                    ok = false;
-                    break;
-                }
-                continue;
-            }
-            // every candidate that is sure to lead has been taken by other blocks: look again
-            ++rescans;
-            waits = 1;
-            cluster_fence();                               // (the team must see which samples are taken)
-            if (lane == jl) {
-                bar_expect(bars + j * 8, noteBytes);
-                awaited |= 1u << jk;
-                command(jk, kScanCmd);
-            }
+            if (!ok) break;
+            v = key_sample(best);
+            word = bits[v >> 5];
         }
-        if (!ok) break;
-        const int v = key_sample(best);
-        last = least + (((best >> 16) - bias) << 7);
-        int left = 0;
+        const unsigned long long inc = ((best >> 16) - bias) << 7;
+        last = (st & kLast) ? ~0ull : least + inc;         // (a full block is out)
+        word |= 1u << (v & 31);
         if (lane == jl) {
+            if (!(st & kLast)) {                           // (and needs no gains any more)
+                bar_expect(bars + j * 8, noteBytes);
+                command(jk, (uint32_t)(v + 1));
+            }
 #pragma unroll
             for (int k = 0; k < KW; ++k)
                 if (k == jk) {
-                    f[k] += ((best >> 16) - bias) << 7;
-                    left = --room[k];
-                    if (left > 0) {                   // (a full block needs no gains any more)
-                        bar_expect(bars + j * 8, noteBytes);
-                        awaited |= 1u << k;
-                        command(k, (uint32_t)(v + 1));
-                    }
+                    f[k] += inc;
+                    --room[k];
+                    if (kMany) ++given[k];
+                    const uint32_t now = parity | (st & kLast ? 0u : kOwes) | (room[k] == 1 ? kLast : 0u);
+                    state = (state & ~(15u << (4 * k))) | now << (4 * k);
                 }
         }
-        if (__shfl_sync(0xffffffffu, left, jl) == 0) last = ~0ull;
-        const uint32_t word = bits[v >> 5] | (1u << (v & 31));
-        __syncwarp();
         if (lane == 0) {
             bits[v >> 5] = word;
-            prm.picks[c.row0 + t] = (uint32_t)v | ((uint32_t)j << 16);
-        } else if (lane < (int)C) {
-            st_remote32(myBits + (uint32_t)(v >> 5) * 4, word);
+            picks[t] = (uint32_t)v | ((uint32_t)j << 16);
         }
+        if (lane > 0 && lane < (int)C) st_remote32(myBits + (uint32_t)(v >> 5) * 4, word);
         __syncwarp();
     }
     // notes still under way land before the class ends; then every team is sent home
 #pragma unroll
     for (int k = 0; k < KW; ++k) {
         const int p = lane + 32 * k;
-        if (ok && (awaited >> k & 1)) {
+        uint32_t st = state >> (4 * k) & 15u;
+        if (ok && (st & kOwes)) {
             unsigned spin = 0;
-            while (!bar_done(bars + p * 8, parities >> k & 1) && ++spin < kPollLimit) { }
+            while (!bar_done(bars + p * 8, st & kParity ? 1u : 0u) && ++spin < kPollLimit) { }
             if (spin >= kPollLimit) atomicOr(prm.status, kDevTimeout);
-            parities ^= 1u << k;
+            st ^= kParity;
         }
+        parities = (parities & ~(1u << k)) | (st & kParity ? 1u << k : 0u);
         if (p < W) {
             if (!kMany || p >> prm.logC < nTeams) command(k, kStopCmd);
             const long long value = (long long)(f[k] >> 7) - (long long)kZeroValue;
@@ -1094,13 +1129,36 @@ __global__ void __launch_bounds__((P == 0 ? kMaxWarps + 1 + kRefreshers : team_w
             for (int i = threadIdx.x; i < W * layout.words(); i += blockDim.x) reinterpret_cast<unsigned long long *>(shared + prm.offNotes)[i] = 0;
         }
         cluster_barrier();
+        if constexpr (P == 0) {
+            // The greatest gains for an empty block in order: every sample's rank by counting, a share of the samples per CTA.
+            if (rank == 0) for (int i = threadIdx.x; i < W; i += blockDim.x) reinterpret_cast<unsigned long long *>(shared + prm.offFirsts)[i] = 0;
+            cluster_barrier();
+            const uint32_t firsts0 = remote(base + prm.offFirsts, 0);
+            const unsigned long long bias0 = kCut ? 3 * __ldcg(prm.topGain + l) + 1 : 0ull;
+            auto key0 = [&](int v) { return make_key((unsigned long long)__ldcg(prm.g0 + c.row0 + v) + bias0, v); };
+            for (int v = rank * (NW + 1 + kRefreshers) + warp; v < c.M; v += C * (NW + 1 + kRefreshers)) {
+                const unsigned long long mine = key0(v);
+                int above = 0;
+                for (int u0 = 0; u0 < c.M && above < W; u0 += 256) {
+                    int n = 0;
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const int w = u0 + u * 32 + lane;
+                        n += w < c.M && key0(w) > mine ? 1 : 0;
+                    }
+                    above += __reduce_add_sync(0xffffffffu, n);
+                }
+                if (above < W && lane == 0) st_remote(firsts0 + above * 8, mine);
+            }
+            cluster_barrier();
+        }
         // graph cut: gains lie within three times the largest sum of |S| over a row, either way
         const unsigned long long top = __ldcg(prm.topGain + l);
         const unsigned long long bias = kCut ? 3 * top + 1 : 0ull;
         const int shift = shift_for(bias + (kCut ? 3 : 1) * top);
 
         if (warp == NW) {
-            if (rank == 0) lead<KW, P == 0>(prm, l, c, shared, C, bias, classes, parities);
+            if (rank == 0) lead<KW, P == 0>(prm, l, c, shared, C, T, bias, classes, parities);
         } else if (warp > NW) {
             // refreshing warps (kSmemState: gains elsewhere may still be on their way)
             refresh_notes(prm, bits, ld4, shift, fresh0, warp - NW - 1, kRefreshers, prm.slots, ended, classes, [&](int slot, const unsigned long long *&gains) {
@@ -1297,6 +1355,7 @@ static size_t cluster_layout(const Sizes &sz, int maxLd, int C, bool state, size
         prm.offNotes = take((size_t)note.words() * 8 * (size_t)sz.W);
         prm.offBars = take(8 * (size_t)sz.W);
         prm.offQueue = take(many ? 4 * (size_t)C * teams : 0);
+        prm.offFirsts = take(many ? 8 * (size_t)sz.W : 0);
         prm.offFresh = take(many ? 16 + sizeof(Fresh) * (size_t)prm.slots : 0);
         // (a team's row buffer: the row of the sample foreseen, and the rows on their way through apply_list)
         prm.rowPieces = many ? 0 : (std::max(plan.P * step, plan.P <= 3 ? kRowStages * ld4 : kPieceStages * step) + 7) / 8 * 8;
@@ -1312,7 +1371,7 @@ static size_t cluster_layout(const Sizes &sz, int maxLd, int C, bool state, size
     const bool oneFits = prm.slots <= kMaxWarps && onePieces <= kMaxPieces;
     const bool manyFits = (prm.slots + kMaxWarps / busy - 1) / (kMaxWarps / busy) <= 31;
     // (graph cut: the blocks' best candidates are mostly the same samples, so notes have to be kept fresh)
-    if (oneFits && !(sz.graphCut && manyFits && prm.slots > 1) && (prm.slots == 1 || 2 * one + 2 >= busy || !manyFits)) {
+    if (oneFits && !(sz.graphCut && manyFits && prm.slots > 1) && (prm.slots == 1 || one >= 8 || (onePieces <= 3 && 2 * one >= busy) || !manyFits)) {
         const size_t need = place(false, true);
         if (need <= cap) return need;
     }
