@@ -35,29 +35,30 @@ constexpr int kRaisedPerWarp = 64;        // raised columns a team lists at a ti
 constexpr int kClusterBlocks = 128;       // blocks a cluster can lead (their notes sit in one CTA's shared memory)
 constexpr uint32_t kScanCmd = 0u;         // a command's low word: look again;
 constexpr uint32_t kStopCmd = 0xfffffu;   //   the class is done;  anything else: sample + 1 joins the block
-constexpr int kRefreshers = 3;            // warps per CTA that refresh notes (17 warps would occupy the registers of 20 anyway)
+constexpr int kListers = 3;               // listing warps per CTA (17 warps would occupy the registers of 20 anyway)
 constexpr unsigned kPollLimit = 1u << 28;
 constexpr unsigned long long kZeroValue = 1ull << 55;   // (tracked values of the graph cut can be negative)
 
 // Candidates a warp of a team of T contributes to a note: a power of two, at most 16 in all.
 __host__ __device__ constexpr int entries_per_warp(int T) { return T <= 1 ? 16 : T <= 2 ? 8 : T <= 4 ? 4 : T <= 8 ? 2 : 1; }
 
-// What the leader is told about a block (a note, words of 64 bits; E = candidates per warp):
+// What the leader is told about a block (a note, words of 64 bits):
 //   [0]            the key of its best candidate (0: none)
-//   [1, 1 + TE)    for the case that other blocks took that one: keys of leading candidates
+// and for the case that other blocks took that one (E = candidates per warp):
+//   [1, 1 + TE)    keys of leading candidates
 //   then T words   per team warp a key that no candidate left out exceeds
-// and, where blocks sit in shared memory, two words that a refreshing warp rewrites whenever the best candidate has been
-// taken (with many blocks that happens often before the block's turn comes):
-//   gain << 16 | tag  and  update number << 32 | (65535 - sample) << 16 | tag,  where tag is the update number's last byte
-//   << 8 | a running number from 1
-// A candidate that was a block's best and is still unassigned is still its best: gains move only when the block itself
-// receives a sample.
+// and, where teams have several blocks, from a listing warp, some thousand cycles later (with many blocks the best candidates
+// are often taken before the block's turn comes):
+//   64 words       keys of leading candidates
+//   1 word         a key that no candidate left out exceeds
+//   1 word         number of the command that the list answers << 16 | number of the list, 0 while the list is being written
 struct NoteLayout {
     int T;
+    bool many;
+    static constexpr int kList = 64;
     __host__ __device__ int entries() const { return T * entries_per_warp(T); }
-    __host__ __device__ int bounds() const { return 1 + entries(); }
-    __host__ __device__ int now() const { return 1 + entries() + T; }
-    __host__ __device__ int words() const { return 3 + entries() + T; }
+    __host__ __device__ int list() const { return 1 + entries() + T; }
+    __host__ __device__ int words() const { return list() + (many ? kList + 2 : 0); }
     __host__ __device__ uint32_t tracked() const { return (uint32_t)(1 + entries() + T) * 8; }   // bytes a new note brings
 };
 
@@ -99,7 +100,7 @@ struct ClusterParams {
     uint32_t one;              // the value 1, opaque to the compiler
     int32_t logC;
     // byte offsets into dynamic shared memory
-    int32_t offTeams, offLists, offRows, offCmd, offBits, offNotes, offBars, offQueue, offFresh, offFirsts, offCover, offGains;
+    int32_t offTeams, offLists, offRows, offCmd, offBits, offNotes, offBars, offQueue, offTold, offListed, offFirsts, offCover, offGains;
     int32_t ring;              // command words per team (a power of two)
 };
 
@@ -374,11 +375,20 @@ __device__ __forceinline__ Raised entry_or_none(const Raised *list, int e, int n
     return r;
 }
 
-// The n listed columns taken off one piece, rows straight to registers, up to eight in flight.
+// The n listed columns taken off one piece, rows straight to registers, up to sixteen in flight
+// (a warp waits about 1100 cycles for a batch: 137 -> @@ cycles per row of 5 KB with eleven warps at it).
 __device__ __forceinline__ bool correct_piece(const int4 *S4q, const Raised *list, int n, uint32_t one, unsigned long long (&g)[4])
 {
     uint32_t changed = 0;
     int e = 0;
+#pragma unroll 1
+    for (; e + 16 <= n; e += 16) {
+        int4 x[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) x[u] = ld_row_shared(S4q + list[e + u].row);
+#pragma unroll
+        for (int u = 0; u < 16; u += 4) changed |= apply_four(x[u], x[u + 1], x[u + 2], x[u + 3], list[e + u], list[e + u + 1], list[e + u + 2], list[e + u + 3], one, g);
+    }
 #pragma unroll 1
     for (; e + 8 <= n; e += 8) {
         int4 x[8];
@@ -706,55 +716,95 @@ __device__ __forceinline__ Lead scan_gains(const uint32_t *bits, const unsigned 
     return best;
 }
 
-// What a team tells the refreshing warps about a block, the update number last: from then on the stored gains are those
-// after that many updates, until the leader has given the block another sample -- and then it takes no candidate of the
-// earlier update any more, so a scan that ran into the next update does no harm.
-struct Fresh {
-    int32_t sample;            // the block's best candidate
-    uint32_t update;           // number of updates (kNotYet: none told)
+// What a listing warp remembers of a block's list: per lane the two gains >> shift (+ 1) it listed, and whose they are.
+struct Listed {
+    uint32_t lead[NoteLayout::kList];
+    uint16_t sample[NoteLayout::kList];
+    uint32_t bound;
+    uint32_t pad_;
 };
-constexpr uint32_t kNotYet = 0xffffffffu;
 
-// A refreshing warp: lane i watches the best candidate of the CTA's block first + i step, and when that one has been
-// taken by another block, the warp looks for the best of those left and tells the leader.
+// A listing warp serves the CTA's blocks first, first + step, ...  When a team has told the leader a block's best candidate
+// (serial: number of the command that this answers), the warp lists the leading candidates, the two best of every lane;
+// when other blocks have taken all but a few of those, it lists anew.
+// From the moment a team writes its serial the stored gains are those of that command, until the leader has given the block
+// another one -- and then it does not use lists of the earlier one any more, so a scan that ran into the next update
+// does no harm.
 template <typename Slot>
-__device__ void refresh_notes(const ClusterParams &prm, const uint32_t *bits, int ld4, int shift, volatile Fresh *fresh, int first, int step, int slots,
-                              const volatile uint32_t *stop, uint32_t turn, Slot where)
+__device__ void list_candidates(const ClusterParams &prm, const uint32_t *bits, int ld4, int shift, const volatile uint32_t *serials, Listed *listed, int first,
+                                int step, int slots, const volatile uint32_t *ended, uint32_t turn, Slot where)
 {
     const int lane = threadIdx.x & 31;
-    const NoteLayout note{prm.teamWarps};
-    const int slot = first + lane * step;
-    const bool watch = slot < slots;
-    uint32_t update = kNotYet, tag = 0;
-    int sample = -1;
+    const NoteLayout layout{prm.teamWarps, true};
+    uint32_t had = 0, lists = 0;                           // lane i: of block first + i step: command listed last, and how often
+    int turnOf = 0;
+    const int mine = first < slots ? (slots - first + step - 1) / step : 0;
     for (unsigned spin = 0; spin < kPollLimit; ++spin) {
-        if (*stop == turn) break;
-        bool taken = false;
-        if (watch) {
-            const uint32_t u = fresh[slot].update;
-            const int s = fresh[slot].sample;
-            if (u != update) {
-                update = u;
-                sample = s;
-                tag = (u & 0xffu) << 8;
+        if (*ended == turn) break;
+        // a block told anew comes first; else a look at one block's list
+        const uint32_t now = lane < mine ? serials[first + lane * step] : 0u;
+        const unsigned m = __ballot_sync(0xffffffffu, now != had && now != 0);
+        const bool fresh = m != 0;
+        if (!fresh) turnOf = turnOf + 1 < mine ? turnOf + 1 : 0;
+        const int i = fresh ? __ffs(m) - 1 : turnOf;
+        const int slot = first + i * step;
+        const uint32_t serial = __shfl_sync(0xffffffffu, now, i);
+        if (mine == 0 || serial == 0) { __nanosleep(200); continue; }
+        Listed &li = listed[slot];
+        {
+            if (!fresh) {
+                // how many of the listed are left that are sure to lead?
+                const uint32_t bound = li.bound;
+                const int s0 = li.sample[lane], s1 = li.sample[32 + lane];
+                const bool taken0 = *(volatile const uint32_t *)&bits[s0 >> 5] >> (s0 & 31) & 1, taken1 = *(volatile const uint32_t *)&bits[s1 >> 5] >> (s1 & 31) & 1;
+                const unsigned sure = __popc(__ballot_sync(0xffffffffu, li.lead[lane] > bound && !taken0)) + __popc(__ballot_sync(0xffffffffu, li.lead[32 + lane] > bound && !taken1));
+                const bool any = __any_sync(0xffffffffu, (li.lead[lane] && taken0) || (li.lead[32 + lane] && taken1));
+                if (bound == 0 || sure > 2 || !any) {
+                    __nanosleep(50);                       // (the teams need the issue slots)
+                    continue;
+                }
             }
-            if (update != kNotYet && sample >= 0) taken = *(volatile const uint32_t *)&bits[sample >> 5] >> (sample & 31) & 1;
+            const unsigned long long *gains;
+            const uint32_t listAddr = where(slot, gains) + (uint32_t)layout.list() * 8;
+            if (lane == i) {
+                st_remote(listAddr + (uint32_t)(NoteLayout::kList + 1) * 8, 0ull);
+                lists = fresh ? 1 : lists + 1;
+                had = serial;
+            }
+            uint32_t e = 0, f = 0, o = 0;                  // greatest, second and third gain >> shift (+ 1), and whose they are
+            int ev = 0, fv = 0;
+            for (int q = lane; q < ld4; q += 32) {
+                const uint32_t nib = *(volatile const uint32_t *)&bits[q >> 3] >> ((q & 7) * 4);
+                const ulonglong2 a0 = reinterpret_cast<const ulonglong2 *>(gains)[2 * q], a1 = reinterpret_cast<const ulonglong2 *>(gains)[2 * q + 1];
+                const unsigned long long g[4] = {a0.x, a0.y, a1.x, a1.y};
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const uint32_t k = (nib >> u & 1) ? 0u : lead_part(g[u], shift);
+                    if (k > f) {
+                        o = f;
+                        if (k > e) { f = e; fv = ev; e = k; ev = 4 * q + u; }
+                        else { f = k; fv = 4 * q + u; }
+                    } else {
+                        o = max(o, k);
+                    }
+                }
+            }
+            o = __reduce_max_sync(0xffffffffu, o);
+            li.lead[lane] = e;
+            li.lead[32 + lane] = f;
+            li.sample[lane] = (uint16_t)ev;
+            li.sample[32 + lane] = (uint16_t)fv;
+            if (lane == 0) li.bound = o;
+            cluster_fence();                               // (the list that was there is withdrawn)
+            __syncwarp();
+            st_remote(listAddr + (uint32_t)lane * 8, e ? key_of(e, low_part(gains[ev], shift, ev), shift) : 0ull);
+            st_remote(listAddr + (uint32_t)(32 + lane) * 8, f ? key_of(f, low_part(gains[fv], shift, fv), shift) : 0ull);
+            if (lane == 0) st_remote(listAddr + (uint32_t)NoteLayout::kList * 8, o ? key_of(o, ((1u << shift) - 1u) << 16 | 0xffffu, shift) : 0ull);
+            cluster_fence();
+            __syncwarp();
+            if (lane == i) st_remote(listAddr + (uint32_t)(NoteLayout::kList + 1) * 8, (unsigned long long)serial << 16 | (lists & 0xffffu));
+            __syncwarp();
         }
-        const unsigned m = __ballot_sync(0xffffffffu, taken);
-        if (!m) continue;
-        const int i = __ffs(m) - 1;
-        const unsigned long long *gains;
-        const uint32_t noteAddr = where(first + i * step, gains);
-        const Lead best = scan_gains(bits, gains, ld4, lane, 32, shift);
-        const uint32_t e = __reduce_max_sync(0xffffffffu, best.e);
-        const unsigned long long k = key_of(e, __reduce_max_sync(0xffffffffu, best.e == e ? best.low : 0u), shift);
-        if (lane == i) {
-            sample = k ? key_sample(k) : -1;
-            tag = (tag & 0xff00u) | ((tag & 0xffu) == 255u ? 1u : (tag & 0xffu) + 1u);
-            st_remote(noteAddr + (uint32_t)note.now() * 8, (k & ~0xffffull) | tag);
-            st_remote(noteAddr + (uint32_t)(note.now() + 1) * 8, (unsigned long long)update << 32 | (k & 0xffffull) << 16 | tag);
-        }
-        __syncwarp();
     }
 }
 
@@ -768,28 +818,29 @@ __device__ __forceinline__ void team_of_many(const ClusterParams &prm, int l, co
     int4 *cov;
     unsigned long long *gains;
     uint32_t noteAddr, barAddr;
-    volatile Fresh *fresh;
-    uint32_t updates = 0;                                  // lane i: of block i
+    volatile uint32_t *told;
+    uint32_t serial = 0;                                   // lane i: commands for block i so far
+    // the block's best candidate goes to the leader, and the command it answers to the listing warps
     auto tell = [&](int i) {
         const Summary sum = summarize(scan_gains(t.bits, gains, t.ld4, tid, step, shift), shift, T, lane);
         unsigned long long top = sum.top;
+        post(t, T, sum, noteAddr, barAddr);
         if (T > 1) {
             if (lane == 0) t.tm->best[t.warpIn] = top;
             team_barrier(t.team, T);
             if (t.warpIn == 0) top = warp_max_u64(lane < T ? t.tm->best[lane] : 0ull);
         }
-        if (tid == 0) st_async(noteAddr, top, barAddr);
-        post(t, T, sum, noteAddr, barAddr);
+        if (lane == i) ++serial;
         if (t.warpIn == 0 && lane == i) {
-            fresh->sample = top ? key_sample(top) : -1;
+            st_async(noteAddr, top, barAddr);
             __threadfence_block();
-            fresh->update = updates;
+            *told = serial;
         }
     };
     if (tid == 0) t.tm->count[0] = t.tm->count[1] = 0;
     int par = 0;
     for (int i = 0; i < mine; ++i) {
-        const int j = where(i, cov, gains, noteAddr, barAddr, fresh);
+        const int j = where(i, cov, gains, noteAddr, barAddr, told);
         for (int q = tid; q < t.ld4; q += step) {
             if (!kCut) cov[q] = make_int4(0, 0, 0, 0);
 #pragma unroll
@@ -815,7 +866,7 @@ __device__ __forceinline__ void team_of_many(const ClusterParams &prm, int l, co
         const uint32_t what = (uint32_t)cmd & 0xfffffu;
         const int i = (int)((uint32_t)cmd >> 20);
         if (what == kStopCmd) break;
-        where(i, cov, gains, noteAddr, barAddr, fresh);
+        where(i, cov, gains, noteAddr, barAddr, told);
         if (what == kScanCmd) {
             cluster_fence();
             tell(i);
@@ -846,7 +897,6 @@ __device__ __forceinline__ void team_of_many(const ClusterParams &prm, int l, co
                 }
             });
         }
-        if (lane == i) ++updates;
         __syncwarp();
         tell(i);
     }
@@ -863,7 +913,7 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
                      uint32_t &parities)
 {
     const int lane = threadIdx.x & 31, W = prm.W;
-    const NoteLayout layout{T};
+    const NoteLayout layout{T, kMany};
     const uint32_t noteBytes = layout.tracked();
     const int nTeams = team_warps(T) / T;
     volatile uint32_t *queue = reinterpret_cast<uint32_t *>(shared + prm.offQueue);      // commands given to each team
@@ -875,7 +925,7 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
     const uint32_t bars = base + prm.offBars;
     unsigned long long f[KW];              // (value + kZeroValue) << 7 | block
     int room[KW];
-    uint32_t given[KW];                    // samples (one team per block: commands) given to the block
+    uint32_t given[KW];                    // commands given to the block
     uint32_t cmdAddr[KW];
     uint32_t qWord[KW];                    // kMany: block's number in its team << 20 | its team's entry of queue
     // four bits for each k: the block owes a note; parity of its mbarrier; its next sample is its last; it is empty
@@ -904,13 +954,11 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
 #pragma unroll
         for (int i = 0; i < KW; ++i)
             if (i == k) {
-                uint32_t n;
+                uint32_t n = ++given[i];
                 if (kMany) {
                     n = queue[qWord[i] & 0xfffffu] + 1;
                     queue[qWord[i] & 0xfffffu] = n;
                     what |= qWord[i] & 0xfff00000u;
-                } else {
-                    n = ++given[i];
                 }
                 st_remote(cmdAddr[i] + ((n - 1) & (uint32_t)(prm.ring - 1)) * 8, ((unsigned long long)n << 32) | what);
             }
@@ -965,49 +1013,55 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
                     if (!(bits[s >> 5] >> (s & 31) & 1)) { best = k; break; }
                 }
             }
-            uint32_t updates = 0;
+            uint32_t serial = 0;
             if (kMany) {
 #pragma unroll
-                for (int k = 0; k < KW; ++k) if (k == jk) updates = given[k];
-                updates = __shfl_sync(0xffffffffu, updates, jl);
+                for (int k = 0; k < KW; ++k) if (k == jk) serial = given[k];
+                serial = __shfl_sync(0xffffffffu, serial, jl);
             }
-            bool noted = !kMany || !(st & kEmpty);         // the note stands for the block's present gains
-            for (unsigned polls = 0; best == 0; ++polls) {
-                if (noted && (!kMany || polls == 0)) {
+            while (best == 0) {
+                if (!kMany || serial > 0) {
                     // the best of the candidates left, if none that the note leaves out can lead
                     const unsigned long long k = lane < layout.entries() + T ? note[1 + lane] : 0ull;
                     const int s = key_sample(k);
                     const bool free = lane < layout.entries() && k != 0 && !(bits[s >> 5] >> (s & 31) & 1);
                     best = warp_max_u64(free ? k : 0ull);
                     if (__any_sync(0xffffffffu, lane >= layout.entries() && k >= best)) best = 0;
-                    if (best) break;
                 }
-                ++rescans;
-                if (kMany && noted) {
-                    // a refreshing warp is looking for others already (every lane polls; lane 0's reading counts)
-                    const unsigned long long x = note[layout.now()], y = note[layout.now() + 1];
-                    const uint32_t tag = (uint32_t)x & 0xffffu;
-                    unsigned long long k = 0;
-                    if (tag == ((uint32_t)y & 0xffffu) && (tag & 0xffu) != 0 && (uint32_t)(y >> 32) == updates) k = (x & ~0xffffull) | (y >> 16 & 0xffffull);
-                    k = __shfl_sync(0xffffffffu, k, 0);
-                    const int s = key_sample(k);
-                    if (k != 0 && !(bits[s >> 5] >> (s & 31) & 1)) best = k;
-                    if (polls >= kPollLimit) {
+                if (kMany && serial > 0 && best == 0) {
+                    // the list, and its next edition when all that are sure to lead in this one have been taken
+                    volatile const unsigned long long *list = note + layout.list();
+                    unsigned spin = 0, spent = 0;
+                    while (best == 0 && ++spin < kPollLimit) {
+                        const unsigned long long tag = list[NoteLayout::kList + 1];
+                        const unsigned long long k = list[lane], k2 = list[32 + lane], bound = list[NoteLayout::kList];
+                        const unsigned long long again = list[NoteLayout::kList + 1];
+                        if (!__all_sync(0xffffffffu, tag == again && (uint32_t)(tag >> 16) == serial && (tag & 0xffffu) == (__shfl_sync(0xffffffffu, (uint32_t)tag, 0) & 0xffffu))) continue;
+                        const int s = key_sample(k), s2 = key_sample(k2);
+                        const bool free = k != 0 && !(bits[s >> 5] >> (s & 31) & 1), free2 = k2 != 0 && !(bits[s2 >> 5] >> (s2 & 31) & 1);
+                        best = warp_max_u64(umax(free ? k : 0ull, free2 ? k2 : 0ull));
+                        if (bound >= best) {
+                            best = 0;
+                            if (++spent > 200) break;      // (equal gains: the team decides)
+                        }
+                    }
+                    if (spin >= kPollLimit) {
                         if (lane == 0) atomicOr(prm.status, kDevTimeout);
                         ok = false;
                         break;
                     }
-                    continue;
                 }
+                if (best) break;
                 // every candidate that is sure to lead has been taken by other blocks: the team looks again
+                ++rescans;
                 cluster_fence();                           // (it must see which samples are taken)
                 if (lane == jl) {
                     bar_expect(bars + j * 8, noteBytes);
                     command(jk, kScanCmd);
                 }
+                ++serial;
                 ok = await();
                 if (!ok) break;
-                noted = true;
                 const unsigned long long k = note[0];
                 const int s = key_sample(k);
                 if (k != 0 && !(bits[s >> 5] >> (s & 31) & 1)) best = k;
@@ -1029,7 +1083,6 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
                 if (k == jk) {
                     f[k] += inc;
                     --room[k];
-                    if (kMany) ++given[k];
                     const uint32_t now = parity | (st & kLast ? 0u : kOwes) | (room[k] == 1 ? kLast : 0u);
                     state = (state & ~(15u << (4 * k))) | now << (4 * k);
                 }
@@ -1059,14 +1112,14 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
             prm.fval[(int64_t)l * W + p] = prm.fixedExp ? __double_as_longlong(ldexp((double)value, -prm.fixedExp[l])) : value;
         }
     }
-    if (kMany && lane < (int)C) st_remote32(remote(base + prm.offFresh, lane), turn);
+    if (kMany && lane < (int)C) st_remote32(remote(base + prm.offTold, lane), turn);
     if (lane == 0 && rescans) atomicAdd(prm.stats + 9, (unsigned long long)rescans);
 }
 
 // P: pieces per thread of teams with one block; 0: teams with several blocks (kSmemState: which all fit the
 // CTAs' shared memory).  kCut: graph-cut objective.
 template <int KW, int P, int kT, bool kSmemState, bool kCut>
-__global__ void __launch_bounds__((P == 0 ? kMaxWarps + 1 + kRefreshers : team_warps(kT) + 1) * 32, 1) greedy_cluster_kernel(const __grid_constant__ ClusterParams prm)
+__global__ void __launch_bounds__((P == 0 ? kMaxWarps + 1 + kListers : team_warps(kT) + 1) * 32, 1) greedy_cluster_kernel(const __grid_constant__ ClusterParams prm)
 {
     extern __shared__ __align__(128) unsigned char shared[];
     __shared__ int shClass[2];
@@ -1079,7 +1132,7 @@ __global__ void __launch_bounds__((P == 0 ? kMaxWarps + 1 + kRefreshers : team_w
     volatile unsigned long long *cmds = reinterpret_cast<volatile unsigned long long *>(shared + prm.offCmd);
     const int W = prm.W;
     uint32_t parities = 0;
-    const NoteLayout layout{T};
+    const NoteLayout layout{T, P == 0};
     uint32_t classes = 0;                                  // this cluster has begun
 
     if (rank == 0)
@@ -1118,11 +1171,11 @@ __global__ void __launch_bounds__((P == 0 ? kMaxWarps + 1 + kRefreshers : team_w
         for (int i = threadIdx.x; i < (c.ld + 31) / 32; i += blockDim.x)
             bits[i] = 32 * i + 32 <= c.M ? 0u : (32 * i >= c.M ? ~0u : ~0u << (c.M - 32 * i));
         for (int i = threadIdx.x; i < nTeams * prm.ring; i += blockDim.x) cmds[i] = 0;
-        // (shared memory for the refreshing warps: the number of the class that has ended last, then what teams tell them)
-        volatile uint32_t *ended = reinterpret_cast<uint32_t *>(shared + prm.offFresh);
-        volatile Fresh *fresh0 = reinterpret_cast<Fresh *>(shared + prm.offFresh + 16);
+        // (for the listing warps: the number of the class that has ended last, then per block the command told last)
+        volatile uint32_t *ended = reinterpret_cast<uint32_t *>(shared + prm.offTold);
+        volatile uint32_t *told0 = ended + 4;
         if (P == 0)
-            for (int i = threadIdx.x; i < prm.slots; i += blockDim.x) { fresh0[i].sample = -1; fresh0[i].update = kNotYet; }
+            for (int i = threadIdx.x; i < prm.slots; i += blockDim.x) told0[i] = 0;
         if (P == 0 && threadIdx.x == 0 && classes == 1) *ended = 0;
         if (P == 0 && rank == 0) {
             for (int i = threadIdx.x; i < (int)C * nTeams; i += blockDim.x) reinterpret_cast<uint32_t *>(shared + prm.offQueue)[i] = 0;
@@ -1136,7 +1189,7 @@ __global__ void __launch_bounds__((P == 0 ? kMaxWarps + 1 + kRefreshers : team_w
             const uint32_t firsts0 = remote(base + prm.offFirsts, 0);
             const unsigned long long bias0 = kCut ? 3 * __ldcg(prm.topGain + l) + 1 : 0ull;
             auto key0 = [&](int v) { return make_key((unsigned long long)__ldcg(prm.g0 + c.row0 + v) + bias0, v); };
-            for (int v = rank * (NW + 1 + kRefreshers) + warp; v < c.M; v += C * (NW + 1 + kRefreshers)) {
+            for (int v = rank * (NW + 1 + kListers) + warp; v < c.M; v += C * (NW + 1 + kListers)) {
                 const unsigned long long mine = key0(v);
                 int above = 0;
                 for (int u0 = 0; u0 < c.M && above < W; u0 += 256) {
@@ -1160,8 +1213,7 @@ __global__ void __launch_bounds__((P == 0 ? kMaxWarps + 1 + kRefreshers : team_w
         if (warp == NW) {
             if (rank == 0) lead<KW, P == 0>(prm, l, c, shared, C, T, bias, classes, parities);
         } else if (warp > NW) {
-            // refreshing warps (kSmemState: gains elsewhere may still be on their way)
-            refresh_notes(prm, bits, ld4, shift, fresh0, warp - NW - 1, kRefreshers, prm.slots, ended, classes, [&](int slot, const unsigned long long *&gains) {
+            list_candidates(prm, bits, ld4, shift, told0, reinterpret_cast<Listed *>(shared + prm.offListed), warp - NW - 1, kListers, prm.slots, ended, classes, [&](int slot, const unsigned long long *&gains) {
                 const int j = slot * (int)C + (int)rank;
                 if (kSmemState) gains = reinterpret_cast<const unsigned long long *>(shared + prm.offGains) + (size_t)slot * prm.maxLd;
                 else gains = reinterpret_cast<const unsigned long long *>(prm.gains + c.vOff) + (size_t)j * c.ld;
@@ -1185,7 +1237,7 @@ __global__ void __launch_bounds__((P == 0 ? kMaxWarps + 1 + kRefreshers : team_w
                                                        base + prm.offCmd + team * prm.ring * 8, notes0 + j * (uint32_t)layout.words() * 8, bars0 + j * 8, corrected, rows);
             } else {
                 // the i-th block of the team
-                auto where = [&](int i, int4 *&cov, unsigned long long *&gains, uint32_t &noteAddr, uint32_t &barAddr, volatile Fresh *&fresh) -> int {
+                auto where = [&](int i, int4 *&cov, unsigned long long *&gains, uint32_t &noteAddr, uint32_t &barAddr, volatile uint32_t *&told) -> int {
                     const int slot = team + i * nTeams, j = slot * (int)C + (int)rank;
                     if (kSmemState) {
                         cov = reinterpret_cast<int4 *>(shared + prm.offCover) + (size_t)slot * (prm.maxLd >> 2);
@@ -1195,7 +1247,7 @@ __global__ void __launch_bounds__((P == 0 ? kMaxWarps + 1 + kRefreshers : team_w
                         gains = reinterpret_cast<unsigned long long *>(prm.gains + c.vOff) + (size_t)j * c.ld;
                     }
                     noteAddr = notes0 + j * (uint32_t)layout.words() * 8;
-                    fresh = fresh0 + slot;
+                    told = told0 + slot;
                     barAddr = bars0 + j * 8;
                     return j;
                 };
@@ -1329,13 +1381,15 @@ static size_t cluster_layout(const Sizes &sz, int maxLd, int C, bool state, size
     while ((1 << prm.logC) < C) ++prm.logC;
     const int ld4 = maxLd / 4;
     // A team per block, of as many warps as there are, or teams of several blocks: then a team has as many warps as a row
-    // keeps busy (at least three quarters of their threads).
+    // keeps busy (at least three fifths of their threads; measured on 300 to 1300 samples), half of that with more than 16
+    // blocks to serve.
     const int rowWarps = (ld4 + 31) / 32;
     int one = std::min(kMaxWarps / std::min(kMaxWarps, pow2_at_least(prm.slots)), pow2_at_least(rowWarps));
     if (prm.slots == 1 && rowWarps > 8) one = 15;
     int busy = 1;
     for (int T = 2; T <= kMaxWarps; T *= 2)
-        if (4 * ld4 >= 3 * ((ld4 + 32 * T - 1) / (32 * T)) * 32 * T) busy = T;
+        if (5 * ld4 >= 3 * 32 * T) busy = T;
+    if (prm.slots > kMaxWarps && busy > 1) busy /= 2;
     const int onePieces = (ld4 + 32 * one - 1) / (32 * one);
     int pieces = onePieces;
     auto place = [&](bool many, bool state) -> size_t {
@@ -1345,7 +1399,7 @@ static size_t cluster_layout(const Sizes &sz, int maxLd, int C, bool state, size
         const int step = prm.teamWarps * 32, teams = warps / prm.teamWarps;
         const int perTeam = (prm.slots + teams - 1) / teams;
         prm.ring = many ? pow2_at_least(perTeam + 1) : 1;
-        const NoteLayout note{prm.teamWarps};
+        const NoteLayout note{prm.teamWarps, many};
         size_t off = 0;
         auto take = [&](size_t bytes) { const size_t at = off; off = (off + bytes + 15) / 16 * 16; return (int32_t)at; };
         prm.offTeams = take(sizeof(Team) * (size_t)teams);
@@ -1356,7 +1410,8 @@ static size_t cluster_layout(const Sizes &sz, int maxLd, int C, bool state, size
         prm.offBars = take(8 * (size_t)sz.W);
         prm.offQueue = take(many ? 4 * (size_t)C * teams : 0);
         prm.offFirsts = take(many ? 8 * (size_t)sz.W : 0);
-        prm.offFresh = take(many ? 16 + sizeof(Fresh) * (size_t)prm.slots : 0);
+        prm.offListed = take(many ? sizeof(Listed) * (size_t)prm.slots : 0);
+        prm.offTold = take(many ? 16 + 4 * (size_t)prm.slots : 0);
         // (a team's row buffer: the row of the sample foreseen, and the rows on their way through apply_list)
         prm.rowPieces = many ? 0 : (std::max(plan.P * step, plan.P <= 3 ? kRowStages * ld4 : kPieceStages * step) + 7) / 8 * 8;
         // (asynchronous 16-byte copies whose destination sits differently in its 32-byte sector than the source fetch two
@@ -1490,7 +1545,7 @@ rcd_status launch_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const Workspace 
     ClusterKernel kernel = sz.graphCut ? (sz.W <= 32 ? pick_kernel<1, true>(plan.P, prm.teamWarps, plan.smemState) : pick_kernel<4, true>(plan.P, prm.teamWarps, plan.smemState))
                                        : (sz.W <= 32 ? pick_kernel<1, false>(plan.P, prm.teamWarps, plan.smemState)
                                           : sz.W <= 64 ? pick_kernel<2, false>(plan.P, prm.teamWarps, plan.smemState) : pick_kernel<4, false>(plan.P, prm.teamWarps, plan.smemState));
-    const rcd_status rs = launch_cluster(ctx, kernel, prm, (plan.P == 0 ? kMaxWarps + 1 + kRefreshers : team_warps(prm.teamWarps) + 1) * 32, plan.C, plan.clusters, plan.smem, st, nullptr);
+    const rcd_status rs = launch_cluster(ctx, kernel, prm, (plan.P == 0 ? kMaxWarps + 1 + kListers : team_warps(prm.teamWarps) + 1) * 32, plan.C, plan.clusters, plan.smem, st, nullptr);
     if (rs != RCD_OK) return rs;
     ctx->steps = sz.maxM;
     ctx->phaseNsDev = ws.phaseNs;
