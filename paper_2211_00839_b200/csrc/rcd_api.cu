@@ -38,12 +38,17 @@ static cudaError_t status_begin(rcd_ctx *ctx, cudaStream_t st)
     return cudaMemsetAsync(ctx->statusOwn, 0, sizeof(int32_t), st);
 }
 
-// Pinned memory for what a call's host side hands to the device.  Grows to the largest call; the wait is for the last
-// copy out of it (done long ago unless the context changed streams).
-static rcd_status blob_begin(rcd_ctx *ctx, size_t bytes)
+// Pinned memory for what a call's host side hands to the device: the second half of the staging buffer, or, for calls that
+// need more, a buffer that grows to the largest of them.  The wait is for the last copy out of it (done long ago unless the
+// context changed streams).
+static rcd_status blob_begin(rcd_ctx *ctx, size_t bytes, size_t stageIntsUsed, unsigned char **out)
 {
     if (ctx->evBlob) RCD_CUDA(ctx, cudaEventSynchronize(ctx->evBlob));
     else RCD_CUDA(ctx, cudaEventCreateWithFlags(&ctx->evBlob, cudaEventDisableTiming));
+    if (stageIntsUsed <= ctx->hostStageInts / 2 && bytes <= ctx->hostStageInts / 2 * sizeof(int32_t)) {
+        *out = (unsigned char *)(ctx->hostStage + ctx->hostStageInts / 2);
+        return RCD_OK;
+    }
     if (bytes > ctx->hostBlobBytes) {
         if (ctx->hostBlob) cudaFreeHost(ctx->hostBlob);
         ctx->hostBlob = nullptr;
@@ -52,6 +57,7 @@ static rcd_status blob_begin(rcd_ctx *ctx, size_t bytes)
         RCD_CUDA(ctx, cudaMallocHost((void **)&ctx->hostBlob, want));
         ctx->hostBlobBytes = want;
     }
+    *out = ctx->hostBlob;
     return RCD_OK;
 }
 
@@ -256,7 +262,8 @@ static rcd_status prepare(rcd_ctx *ctx, const void *features, rcd_feat_dtype dty
     if (!ctx->evCounts) RCD_CUDA(ctx, cudaEventCreateWithFlags(&ctx->evCounts, cudaEventDisableTiming));
     RCD_CUDA(ctx, cudaEventRecord(ctx->evCounts, st));
     const size_t blobBytes = (size_t)((unsigned char *)(hw.quota + (size_t)L * W) - (unsigned char *)hw.desc);
-    rs = blob_begin(ctx, blobBytes);
+    unsigned char *blob = nullptr;
+    rs = blob_begin(ctx, blobBytes, statusInts + (size_t)L, &blob);
     if (rs != RCD_OK) return rs;
     RCD_CUDA(ctx, cudaEventSynchronize(ctx->evCounts));
     if (ctx->hostStage[0] & kDevBadLabel) return fail(ctx, RCD_ERR_INVALID_ARG, "a label lies outside [0, %d)", L);
@@ -287,7 +294,7 @@ static rcd_status prepare(rcd_ctx *ctx, const void *features, rcd_feat_dtype dty
     P.sz = sz;
 
     // descriptors, tile prefixes, classes by size and quotas: one copy from pinned memory
-    auto at = [&](void *dev) { return ctx->hostBlob + ((unsigned char *)dev - (unsigned char *)hw.desc); };
+    auto at = [&](void *dev) { return blob + ((unsigned char *)dev - (unsigned char *)hw.desc); };
     memcpy(at(hw.desc), P.desc.data(), (size_t)L * sizeof(ClassDesc));
     int32_t *prefix = (int32_t *)at(hw.tilePrefix), *order = (int32_t *)at(hw.classOrder), *sorted = (int32_t *)at(hw.sizesSorted);
     SimClasses cls{};
@@ -318,7 +325,7 @@ static rcd_status prepare(rcd_ctx *ctx, const void *features, rcd_feat_dtype dty
     const bool early = capacities && L <= 64;               // (few quotas: not worth a copy of their own behind the similarity kernel)
     if (early) quotas();
     const size_t firstBytes = early ? blobBytes : (size_t)((unsigned char *)hw.quota - (unsigned char *)hw.desc);
-    RCD_CUDA(ctx, cudaMemcpyAsync(P.ws.desc, ctx->hostBlob, firstBytes, cudaMemcpyHostToDevice, st));
+    RCD_CUDA(ctx, cudaMemcpyAsync(P.ws.desc, blob, firstBytes, cudaMemcpyHostToDevice, st));
     rs = launch_stable_split(ctx, labels, N, L, P.ws.chunkHist, P.ws.desc, nullptr, nullptr, nullptr, P.ws.perm,
                              features, d * (int64_t)feat_bytes(dtype), sz.pitch, P.ws.Xs, st);
     if (rs != RCD_OK) return rs;
