@@ -1149,6 +1149,7 @@ __global__ void __launch_bounds__((P == 0 ? kMaxWarps + 1 + kListers : team_warp
         const int l = *(volatile int *)&shClass[turn];
         if (l < 0) break;
         ++classes;
+        if (prm.fixedExp && prm.fixedExp[l] == kNotFixed) continue;
         const ClassDesc c = prm.desc[l];
         if (c.M == 0) {
             if (rank == 0) for (int p = threadIdx.x; p < W; p += blockDim.x) prm.fval[(int64_t)l * W + p] = 0;
@@ -1276,25 +1277,39 @@ __global__ void __launch_bounds__((P == 0 ? kMaxWarps + 1 + kListers : team_warp
 // Floating-point similarities as fixed-point integers, so that sums of them are exact.  The largest similarity of a class
 // is the largest squared norm (Cauchy-Schwarz), i.e. on the diagonal; it lands in [2^29, 2^30), which leaves every entry
 // an absolute precision of 2^-30 of it: finer than the fp32 dot products themselves (2^-24 of the products they add up).
+// That holds for rows of about one norm (normalised features, and the Gaussian kernel, whose diagonal is 1).  A class whose
+// squared norms differ by more than a factor of 16, or are not finite, is left in floating point (kNotFixed) for
+// launch_greedy_not_fixed.
 __global__ void __launch_bounds__(256, 8) fixed_exponent_kernel(const ClassDesc *__restrict__ desc, const float *__restrict__ S, int32_t *__restrict__ fixedExp)
 {
-    __shared__ float shMax[8];
+    __shared__ float shMax[8], shMin[8];
     const ClassDesc c = desc[blockIdx.x];
-    float m = 0.f;
-    for (int v = threadIdx.x; v < c.M; v += 256) m = fmaxf(m, S[c.sOff + (int64_t)v * c.ld + v]);
-    for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-    if ((threadIdx.x & 31) == 0) shMax[threadIdx.x >> 5] = m;
-    __syncthreads();
+    float m = 0.f, least = INFINITY;                       // (zero rows have similarity 0 with everything: exact at any scale)
+    bool odd = false;
+    for (int v = threadIdx.x; v < c.M; v += 256) {
+        const float x = S[c.sOff + (int64_t)v * c.ld + v];
+        odd = odd || !(x >= 0.f && x <= 1e30f);
+        m = fmaxf(m, x);
+        if (x > 0.f) least = fminf(least, x);
+    }
+    for (int off = 16; off > 0; off >>= 1) {
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+        least = fminf(least, __shfl_xor_sync(0xffffffffu, least, off));
+    }
+    if ((threadIdx.x & 31) == 0) { shMax[threadIdx.x >> 5] = m; shMin[threadIdx.x >> 5] = least; }
+    odd = __syncthreads_or(odd);
     if (threadIdx.x == 0) {
-        for (int w = 1; w < 8; ++w) m = fmaxf(m, shMax[w]);
+        for (int w = 1; w < 8; ++w) { m = fmaxf(m, shMax[w]); least = fminf(least, shMin[w]); }
         int e = 0;
-        if (m > 0.f && m <= 3.4e38f) frexpf(m, &e);         // m = x 2^e, x in [0.5, 1)
-        fixedExp[blockIdx.x] = 30 - e;
+        if (m > 0.f && !odd) frexpf(m, &e);                // m = x 2^e, x in [0.5, 1)
+        odd = odd || (m > 0.f && (m > 16.f * least || m < 1e-30f));
+        fixedExp[blockIdx.x] = odd ? kNotFixed : 30 - e;
     }
 }
 __global__ void __launch_bounds__(256, 8) fixed_point_kernel(const ClassDesc *__restrict__ desc, const int32_t *__restrict__ fixedExp, float *__restrict__ S)
 {
     const ClassDesc c = desc[blockIdx.y];
+    if (fixedExp[blockIdx.y] == kNotFixed) return;
     const float scale = ldexpf(1.f, fixedExp[blockIdx.y]);
     float4 *p = reinterpret_cast<float4 *>(S + c.sOff);
     const int64_t n = (int64_t)c.M * (c.ld >> 2);
@@ -1549,6 +1564,7 @@ rcd_status launch_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const Workspace 
     if (rs != RCD_OK) return rs;
     ctx->steps = sz.maxM;
     ctx->phaseNsDev = ws.phaseNs;
+    if (sz.floatArith) return launch_greedy_not_fixed(ctx, sz, ws, descHost, assignment, order, partValues, st);
     return RCD_OK;
 }
 

@@ -105,6 +105,8 @@ struct GreedyParams {
     int32_t denseRing;          // 8-block dense passes stream through shared-memory rings when the coverage vectors leave room
     const int32_t *classOrder;  // [L] classes by descending size (the order in which the one-CTA-per-class loop draws them)
     const int32_t *sizesSorted; // [L] class sizes in ascending order
+    const int32_t *only;        // one CTA per class: run (and set up) only the classes marked kNotFixed; null: every class
+    int32_t *drawn;             // one CTA per class: classes drawn so far
     int32_t minM;               // smallest non-empty class
     int32_t nonEmpty;           // classes that hold at least one sample
 };
@@ -471,11 +473,9 @@ __device__ void plan_decide(const GreedyParams<SV> &prm, int l, const ClassDesc 
 
 // ---------------------------------------------------------------------------------------------
 template <typename SV>
-__global__ void __launch_bounds__(kSelectThreads, 4) init_kernel(GreedyParams<SV> prm)
+__device__ __forceinline__ void init_class(const GreedyParams<SV> &prm, int l, PlanShared<typename Arith<SV>::FV> &shPlan)
 {
     using FV = typename Arith<SV>::FV;
-    __shared__ PlanShared<FV> shPlan;
-    const int l = blockIdx.x;
     const ClassDesc c = prm.desc[l];
     const int W = prm.W;
     SV *cover = prm.cover + c.vOff;
@@ -512,6 +512,13 @@ __global__ void __launch_bounds__(kSelectThreads, 4) init_kernel(GreedyParams<SV
     plan_load(prm, l, shPlan);
     __syncthreads();
     if (threadIdx.x < 32) plan_decide(prm, l, c, c.M, 0, shPlan);
+}
+
+template <typename SV>
+__global__ void __launch_bounds__(kSelectThreads, 4) init_kernel(GreedyParams<SV> prm)
+{
+    __shared__ PlanShared<typename Arith<SV>::FV> shPlan;
+    init_class(prm, blockIdx.x, shPlan);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -2318,17 +2325,23 @@ __global__ void __launch_bounds__(kSweepThreads, 1) greedy_owner_kernel(const __
     __shared__ SweepShared<SV> shSweep;
     __shared__ int shClass;
     __shared__ int shKeep[2];
+    __shared__ PlanShared<typename Arith<SV>::FV> shInit;
     unsigned long long tSweep = 0, tPick = 0, tThreshold = 0;
     for (;;) {
         __syncthreads();
         if (threadIdx.x == 0) {
-            const int k = atomicAdd(&prm.nSweep[0], 1);
+            const int k = atomicAdd(prm.drawn, 1);
             shClass = k < prm.L ? prm.classOrder[k] : -1;
         }
         __syncthreads();
         const int l = shClass;
         if (l < 0) break;
         if (prm.desc[l].M == 0) continue;
+        if (prm.only) {
+            if (prm.only[l] != kNotFixed) continue;
+            init_class(prm, l, shInit);
+            __syncthreads();
+        }
         for (int round = 0; round <= prm.desc[l].M; ++round) {
             if (*(volatile int32_t *)prm.status != 0) break;
             unsigned long long t0 = 0;
@@ -2373,7 +2386,7 @@ static cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 template <typename SV>
 static rcd_status run_greedy(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws,
                              const std::vector<ClassDesc> &descHost, int32_t *assignment, int32_t *order,
-                             cudaStream_t st)
+                             cudaStream_t st, const int32_t *only = nullptr, void *partValues = nullptr)
 {
     using GV = typename Arith<SV>::GV;
     using FV = typename Arith<SV>::FV;
@@ -2382,7 +2395,9 @@ static rcd_status run_greedy(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws,
     prm.S = (const SV *)ws.S;
     prm.cover = (SV *)ws.cover;
     prm.gains = (GV *)ws.gains;
-    prm.fval = (FV *)ws.fval;
+    prm.fval = (FV *)(partValues ? partValues : ws.fval);
+    prm.only = only;
+    prm.drawn = only ? ws.counter + 1 : ws.nSweep;
     prm.cnt = ws.cnt;
     prm.quota = ws.quota;
     prm.valid = ws.valid;
@@ -2479,6 +2494,7 @@ static rcd_status run_greedy(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws,
     const bool perSweep = ctx->cfg.profile >= 2;
     int path = ctx->cfg.greedy_path;
     if (perSweep || !ctx->cooperative) path = 1;
+    if (only) path = 4;
     if (path == 0) path = (sz.L * 4 <= ctx->smCount) ? 3 : 4;
     if (path == 3 && ctx->smCount < 2) path = 2;
     if (path == 4) {
@@ -2515,6 +2531,13 @@ static rcd_status run_greedy(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws,
         prm.asyncGroup = ctx->cfg.async_group > 0 ? ctx->cfg.async_group : std::max<int>(sz.L, 1);
     }
 
+    if (only) {
+        // (classes are set up as they are drawn; the counter and the statistics were cleared when the call began)
+        greedy_owner_kernel<SV><<<std::min<int>(ctx->smCount, sz.L), kSweepThreads, (size_t)smem, st>>>(prm);
+        ctx->kernelLaunches += 1;
+        RCD_CUDA(ctx, cudaGetLastError());
+        return RCD_OK;
+    }
     if (path == 3) RCD_CUDA(ctx, cudaMemsetAsync(ws.tickets, 0, (size_t)(sz.N + sz.L) * sizeof(int32_t), st));
     RCD_CUDA(ctx, cudaMemsetAsync(ws.nSweep, 0, 4 * sizeof(int32_t), st));
     RCD_CUDA(ctx, cudaMemsetAsync(ws.phaseNs, 0, kPhaseWords * sizeof(unsigned long long), st));
@@ -2591,6 +2614,12 @@ rcd_status launch_greedy(rcd_ctx *ctx, rcd_feat_dtype dtype, const Sizes &sz, co
     if (sz.L == 0 || sz.maxM == 0) return RCD_OK;
     if (dtype == RCD_FEAT_I8) return run_greedy<int32_t>(ctx, sz, ws, descHost, assignment, order, st);
     return run_greedy<float>(ctx, sz, ws, descHost, assignment, order, st);
+}
+
+rcd_status launch_greedy_not_fixed(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, const std::vector<ClassDesc> &descHost,
+                                   int32_t *assignment, int32_t *order, void *partValues, cudaStream_t st)
+{
+    return run_greedy<float>(ctx, sz, ws, descHost, assignment, order, st, ws.fixedExp, partValues);
 }
 
 }  // namespace rcd

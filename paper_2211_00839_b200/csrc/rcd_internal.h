@@ -130,10 +130,13 @@ struct Workspace {
     unsigned long long *stepOps;     // [steps+1] element x block pairs of that sweep
     unsigned long long *phaseNs;     // [6] sweep-/pick-phase ns of the persistent kernel, barrier counter, threshold-pass hits / elements / max blocks
     long long *g0;          // [N] cluster form: gain of every sample for an empty block
-    int32_t *fixedExp;      // [L] cluster form, floating-point similarities: S holds round(sim * 2^fixedExp)
+    int32_t *fixedExp;      // [L] cluster form, floating-point similarities: S holds round(sim * 2^fixedExp), or kNotFixed
     int32_t *status;        // [1]
     size_t bytes;           // total bytes laid out
 };
+
+// A class whose samples' norms lie too far apart for one fixed-point scale (see fixed_exponent_kernel).
+constexpr int32_t kNotFixed = INT32_MIN;
 
 struct Sizes {
     int64_t N, d;
@@ -239,6 +242,10 @@ size_t gaussian_scratch_bytes(int64_t N, int32_t L, int64_t maxM);
 rcd_status launch_greedy(rcd_ctx *ctx, rcd_feat_dtype dtype, const Sizes &sz, const Workspace &ws,
                          const std::vector<ClassDesc> &descHost, int32_t *assignment, int32_t *order,
                          cudaStream_t st);
+
+// the floating-point classes that the cluster form left (ws.fixedExp[l] == kNotFixed)
+rcd_status launch_greedy_not_fixed(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, const std::vector<ClassDesc> &descHost,
+                                   int32_t *assignment, int32_t *order, void *partValues, cudaStream_t st);
 
 // greedy loop, one thread-block cluster per class
 rcd_status launch_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, const std::vector<ClassDesc> &descHost,
