@@ -335,7 +335,7 @@ static rcd_status prepare(rcd_ctx *ctx, const void *features, rcd_feat_dtype dty
     if (rs != RCD_OK) return rs;
     if (ctx->cfg.similarity_kind == RCD_SIM_GAUSSIAN) {
         rs = launch_gaussian(ctx, P.ws.Xs, dtype, N, dPitch, cls, P.ws.S, P.ws.gaussNorms, P.ws.gaussPartial, P.ws.gaussSigma,
-                             P.ws.gaussScale, st);
+                             P.ws.gaussScale, capacities && greedy_cluster_takes(ctx, sz, P.desc) ? P.ws.fixedExp : nullptr, st);
         if (rs != RCD_OK) return rs;
     }
     if (capacities && !early) {
@@ -661,7 +661,7 @@ rcd_status rcd_similarity_gaussian(rcd_ctx *ctx, const void *X_dev, rcd_feat_dty
     cls.src.uniLd = (int32_t)ldS;
     cls.L = (int32_t)batch;
     cls.maxM = M;
-    rs = launch_gaussian(ctx, X_dev, dtype, M * batch, d, cls, S_dev, norms, partial, sigma, scale, st);
+    rs = launch_gaussian(ctx, X_dev, dtype, M * batch, d, cls, S_dev, norms, partial, sigma, scale, nullptr, st);
     if (rs != RCD_OK) return rs;
     if (sigma_dev_or_null)
         RCD_CUDA(ctx, cudaMemcpyAsync(sigma_dev_or_null, sigma, (size_t)batch * sizeof(float), cudaMemcpyDeviceToDevice, st));

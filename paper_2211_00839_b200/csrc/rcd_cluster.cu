@@ -1277,7 +1277,7 @@ __global__ void __launch_bounds__((P == 0 ? kMaxWarps + 1 + kListers : team_warp
 // Floating-point similarities as fixed-point integers, so that sums of them are exact.  The largest similarity of a class
 // is the largest squared norm (Cauchy-Schwarz), i.e. on the diagonal; it lands in [2^29, 2^30), which leaves every entry
 // an absolute precision of 2^-30 of it: finer than the fp32 dot products themselves (2^-24 of the products they add up).
-// That holds for rows of about one norm (normalised features, and the Gaussian kernel, whose diagonal is 1).  A class whose
+// That holds for rows of about one norm (normalised features).  A class whose
 // squared norms differ by more than a factor of 16, or are not finite, is left in floating point (kNotFixed) for
 // launch_greedy_not_fixed.
 __global__ void __launch_bounds__(256, 8) fixed_exponent_kernel(const ClassDesc *__restrict__ desc, const float *__restrict__ S, int32_t *__restrict__ fixedExp)
@@ -1521,6 +1521,12 @@ static bool cluster_plan(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassD
     return true;
 }
 
+bool greedy_cluster_takes(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost)
+{
+    ClusterPlan plan;
+    return cluster_plan(ctx, sz, descHost, plan);
+}
+
 // Runs the greedy loop if the cluster form takes the problem (*taken).  partValues (may be null) receives the tracked values.
 rcd_status launch_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, const std::vector<ClassDesc> &descHost,
                                  int32_t *assignment, int32_t *order, void *partValues, cudaStream_t st, bool *taken)
@@ -1549,7 +1555,8 @@ rcd_status launch_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const Workspace 
     prm.L = sz.L;
     prm.W = sz.W;
     prm.one = 1u;
-    if (sz.floatArith) {
+    const bool toFix = sz.floatArith && ctx->cfg.similarity_kind != RCD_SIM_GAUSSIAN;     // (the Gaussian kernel writes fixed point itself)
+    if (toFix) {
         fixed_exponent_kernel<<<sz.L, 256, 0, st>>>(ws.desc, (const float *)ws.S, ws.fixedExp);
         const int64_t pieces = sz.maxM * (int64_t)(prm.maxLd / 4);
         const dim3 grid((unsigned)std::min<int64_t>((pieces + 1023) / 1024, std::max(1, 16 * ctx->smCount / sz.L)), (unsigned)sz.L);
@@ -1564,7 +1571,7 @@ rcd_status launch_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const Workspace 
     if (rs != RCD_OK) return rs;
     ctx->steps = sz.maxM;
     ctx->phaseNsDev = ws.phaseNs;
-    if (sz.floatArith) return launch_greedy_not_fixed(ctx, sz, ws, descHost, assignment, order, partValues, st);
+    if (toFix) return launch_greedy_not_fixed(ctx, sz, ws, descHost, assignment, order, partValues, st);
     return RCD_OK;
 }
 

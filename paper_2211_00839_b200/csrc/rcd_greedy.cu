@@ -2325,7 +2325,6 @@ __global__ void __launch_bounds__(kSweepThreads, 1) greedy_owner_kernel(const __
     __shared__ SweepShared<SV> shSweep;
     __shared__ int shClass;
     __shared__ int shKeep[2];
-    __shared__ PlanShared<typename Arith<SV>::FV> shInit;
     unsigned long long tSweep = 0, tPick = 0, tThreshold = 0;
     for (;;) {
         __syncthreads();
@@ -2339,7 +2338,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1) greedy_owner_kernel(const __
         if (prm.desc[l].M == 0) continue;
         if (prm.only) {
             if (prm.only[l] != kNotFixed) continue;
-            init_class(prm, l, shInit);
+            init_class(prm, l, *reinterpret_cast<PlanShared<typename Arith<SV>::FV> *>(shCover));
             __syncthreads();
         }
         for (int round = 0; round <= prm.desc[l].M; ++round) {
@@ -2470,6 +2469,7 @@ static rcd_status run_greedy(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws,
         const int64_t withRing = (int64_t)thr_bytes_aligned(8 * maxLd * (int)sizeof(SV)) + dense_ring_bytes(4);
         if (withRing <= smemCap) { smem = std::max<int64_t>(smem, withRing); prm.denseRing = 1; }
     }
+    if (only) smem = std::max<int64_t>(smem, (int64_t)sizeof(PlanShared<FV>));       // (the owner kernel sets its classes up there)
     if (smem > smemCap) smem = smemCap;
     if ((int64_t)maxLd * (int64_t)sizeof(SV) > smem)
         return fail(ctx, RCD_ERR_UNSUPPORTED,

@@ -233,9 +233,10 @@ rcd_status launch_stable_split(rcd_ctx *ctx, const int32_t *labels, int64_t N, i
 rcd_status launch_similarity(rcd_ctx *ctx, const void *Xs, rcd_feat_dtype dtype, int64_t Ntot, int64_t d,
                              const SimClasses &cls, void *S, cudaStream_t st);
 
-// Gaussian-kernel similarity: transforms the dot products in S in place
+// Gaussian-kernel similarity: transforms the dot products in S in place, to fp32 or (fixedExp not null) to the fixed-point
+// integers of the cluster form, whose scale it writes to fixedExp[l]
 rcd_status launch_gaussian(rcd_ctx *ctx, const void *Xs, rcd_feat_dtype dtype, int64_t N, int64_t d, const SimClasses &cls,
-                           void *S, void *norms, double *partial, float *sigma, float *scale, cudaStream_t st);
+                           void *S, void *norms, double *partial, float *sigma, float *scale, int32_t *fixedExp, cudaStream_t st);
 size_t gaussian_scratch_bytes(int64_t N, int32_t L, int64_t maxM);
 
 // greedy loop
@@ -247,7 +248,8 @@ rcd_status launch_greedy(rcd_ctx *ctx, rcd_feat_dtype dtype, const Sizes &sz, co
 rcd_status launch_greedy_not_fixed(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, const std::vector<ClassDesc> &descHost,
                                    int32_t *assignment, int32_t *order, void *partValues, cudaStream_t st);
 
-// greedy loop, one thread-block cluster per class
+// greedy loop, one thread-block cluster per class: whether it takes a problem, and the loop
+bool greedy_cluster_takes(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost);
 rcd_status launch_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, const std::vector<ClassDesc> &descHost,
                                  int32_t *assignment, int32_t *order, void *partValues, cudaStream_t st, bool *taken);
 

@@ -1,0 +1,133 @@
+"""The cluster form of the greedy loop (the library's own choice) against the oracle, at the sizes where its layout changes:
+one or several blocks per team, one to seven 16-byte pieces per thread, lists of raised columns longer than their room, blocks
+in shared or in global memory; and the class split, the objective and the fixed-point scale at their own edges."""
+import numpy as np
+import pytest
+
+from test_gpu_parity import check_exact, check_float, rcd, orc, run_partition  # noqa: F401  (fixtures)
+
+pytestmark = pytest.mark.gpu
+
+
+def workload(sizes, d, W, seed, dtype="int8", scale=None, copies=0):
+    from paper_2211_00839_b200.workloads import Workload, make_mixture, fp32_to_bf16_bits
+    rng = np.random.default_rng(seed)
+    feats, labels = [], []
+    for l, M in enumerate(sizes):
+        x = make_mixture(rng, M, d, 4, "dirichlet", "gauss", 4.0) if M else np.zeros((0, d), np.float32)
+        if copies and M > copies:
+            x[rng.choice(M, copies, replace=False)] = x[0]                   # equal gains: the lowest index wins
+        if dtype == "int8":
+            x = np.clip(np.rint(x), -127, 127).astype(np.int8)
+        else:
+            x = x / np.maximum(np.sqrt((x ** 2).sum(1, keepdims=True)), 1e-30)
+            x = fp32_to_bf16_bits(x if scale is None else x * scale(rng, M)[:, None])
+        feats.append(x)
+        labels.append(np.full(M, l, np.int32))
+    feats, labels = np.concatenate(feats), np.concatenate(labels)
+    perm = rng.permutation(len(labels))
+    caps = np.exp(rng.uniform(0, np.log(8.0), size=W))
+    return Workload("edges", dtype, np.ascontiguousarray(feats[perm]), np.ascontiguousarray(labels[perm]), caps, len(sizes), W)
+
+
+@pytest.mark.parametrize("sizes,d,W", [
+    ([1, 2, 3, 0, 33], 17, 1),            # one block; classes of a few samples
+    ([127, 128, 129], 64, 2),             # edges of a warp's columns
+    ([500], 32, 3),                       # one class over a whole cluster
+    ([1921, 60], 96, 5),                  # more columns than one piece per thread of 15 warps; a tiny class beside
+    ([700, 300, 5], 64, 16),              # one block per CTA of the largest cluster
+    ([900] * 9, 48, 20),                  # several blocks per CTA
+    ([130] * 160, 24, 33),                # more classes than SMs: all blocks of a class in one CTA
+    ([40] * 20, 16, 128),                 # the most blocks the form takes; more blocks than samples
+    ([40] * 3, 16, 129),                  # one more: the pass-based forms
+])
+def test_int8_exact(rcd, orc, sizes, d, W):
+    check_exact(rcd, orc, workload(sizes, d, W, 7 + len(sizes) + W))
+
+
+@pytest.mark.parametrize("sizes,d,W", [
+    ([3841], 40, 2),                      # three pieces per thread
+    ([13441, 14500], 32, 5),              # the most pieces the registers take, and one class beyond: gains in shared memory
+    ([2300] * 20, 64, 40),                # teams of 16 warps with several blocks
+    ([5000] * 10, 48, 100),               # two blocks of one team each per CTA
+])
+def test_int8_like_the_passes(rcd, sizes, d, W):
+    """Sizes that would hold the oracle up: the pass-based form, itself checked against it, is the reference."""
+    wl = workload(sizes, d, W, W)
+    for got, want in zip(run_partition(rcd, wl), run_partition(rcd, wl, greedy_path=3)):
+        assert np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("W", [3, 24])
+def test_int8_ties_exact(rcd, orc, W):
+    check_exact(rcd, orc, workload([600, 90], 32, W, W, copies=80))
+
+
+@pytest.mark.parametrize("sizes,W", [([257, 31], 4), ([800] * 3, 24)])
+def test_float(rcd, orc, sizes, W):
+    check_float(rcd, orc, workload(sizes, 96, W, W, dtype="bf16"))
+
+
+def test_float_norms_far_apart(rcd, orc):
+    """Classes whose norms span three orders of magnitude stay in floating point, beside classes that do not."""
+    wl = workload([300, 220, 64], 64, 6, 3, dtype="bf16", scale=lambda rng, M: 10.0 ** rng.uniform(-1.5 if M != 220 else 0.0, 1.5 if M != 220 else 0.1, M))
+    check_float(rcd, orc, wl)
+
+
+@pytest.mark.parametrize("sizes,W", [([400, 3], 5), ([600] * 4, 24), ([90] * 150, 20)])
+def test_graph_cut_int8_exact(rcd, orc, sizes, W):
+    wl = workload(sizes, 48, W, W)
+    a, o, v = run_partition(rcd, wl, objective=rcd.RCD_OBJ_GRAPH_CUT)
+    ref = orc.partition(wl.features, wl.labels, wl.capacities, wl.L, variant="incremental", objective="cut")
+    assert np.array_equal(a, ref.assignment) and np.array_equal(o, ref.order) and np.array_equal(v, ref.part_values)
+
+
+@pytest.mark.parametrize("L", [255, 6000, 6001])
+def test_class_split_many_labels(rcd, orc, L):
+    """Chunk counters in shared memory up to 6000 labels, in global memory beyond."""
+    rng = np.random.default_rng(L)
+    wl = workload([3, 2], 32, 2, L)
+    wl.labels = np.sort(rng.integers(0, L, 3000).astype(np.int32))[rng.permutation(3000)]
+    wl.features = rng.integers(-9, 10, size=(3000, 32)).astype(np.int8)
+    wl.L = L
+    check_exact(rcd, orc, wl)
+
+
+@pytest.mark.parametrize("dtype", ["int8", "bf16"])
+def test_objective_samples_in_no_block(rcd, orc, dtype):
+    """Rows in units of 128, columns in units of 512; entries below zero belong to no block, one block is empty."""
+    import torch
+    wl = workload([129, 513, 1], 96, 4, 11, dtype=dtype)
+    rng = np.random.default_rng(5)
+    a = rng.integers(-1, 3, size=len(wl.labels)).astype(np.int32)
+    with rcd.Context(0) as ctx:
+        X = rcd.features_to_torch(wl.features, device="cuda")
+        vals, total = ctx.rcd_objective(X, torch.from_numpy(wl.labels).cuda(), torch.from_numpy(a).cuda(), wl.W, wl.L)
+        ctx.sync_status()
+        vals, total = vals.cpu().numpy(), total.cpu().numpy()
+    want = np.zeros((wl.L, wl.W))
+    for l, ids in enumerate(orc.split_by_label(wl.labels, wl.L)):
+        S = np.asarray(orc.similarity(wl.features[ids]), dtype=np.float64)
+        for p in range(wl.W):
+            m = a[ids] == p
+            if m.any():
+                want[l, p] = np.maximum(S[:, m].max(1), 0).sum()
+    if dtype == "int8":
+        assert np.array_equal(vals, want.astype(np.int64)) and total[0] == vals.sum()
+    else:
+        assert np.allclose(vals, want, rtol=1e-5, atol=1e-5) and np.isclose(total[0], want.sum(), rtol=1e-5)
+
+
+@pytest.mark.parametrize("M", [1, 2, 64, 65, 127, 130, 1027])
+def test_gaussian_edges(rcd, orc, M):
+    """Row groups of 64, column groups of 128 and, from 1025 on, a warp's second group."""
+    wl = workload([M, M], 40, 1, M, dtype="bf16")
+    x = np.concatenate([wl.features[wl.labels == l] for l in (0, 1)])
+    with rcd.Context(0) as ctx:
+        S, sigma = ctx.rcd_similarity_gaussian(rcd.features_to_torch(x, device="cuda").view(2, M, 40))
+        ctx.sync_status()
+        S, sigma = S.cpu().numpy(), sigma.cpu().numpy()
+    for b in range(2):
+        want, sg = orc.similarity_gaussian(x[b * M:(b + 1) * M])
+        assert sigma[b] == pytest.approx(sg, rel=2e-6)
+        assert np.allclose(S[b, :, :M], want, rtol=2e-5, atol=1e-7) and np.all(S[b, :, M:] == 0)
