@@ -401,7 +401,8 @@ rcd_status rcd_create(rcd_ctx **out, int cuda_device, const rcd_config *cfg)
         delete ctx;
         return RCD_ERR_CUDA;
     }
-    if (cudaMalloc((void **)&ctx->statusOwn, 256) != cudaSuccess || cudaMemset(ctx->statusOwn, 0, 256) != cudaSuccess) {
+    if (cudaMalloc((void **)&ctx->statusOwn, kStatusWords * sizeof(int32_t)) != cudaSuccess ||
+        cudaMemset(ctx->statusOwn, 0, kStatusWords * sizeof(int32_t)) != cudaSuccess) {
         rcd_destroy(ctx);
         return RCD_ERR_CUDA;
     }

@@ -135,6 +135,10 @@ struct Workspace {
     size_t bytes;           // total bytes laid out
 };
 
+// Words of rcd_ctx::statusOwn, and where the similarity kernel's tile tickets (zero between launches) begin.
+constexpr int kStatusWords = 1024;
+constexpr int kFirstTicket = 64;
+
 // A class whose samples' norms lie too far apart for one fixed-point scale (see fixed_exponent_kernel).
 constexpr int32_t kNotFixed = INT32_MIN;
 
@@ -188,7 +192,8 @@ struct rcd_ctx {
     rcd_config cfg{};
     std::string err;
     int32_t *hostStage = nullptr;       // pinned, counts / status read-back
-    int32_t *statusOwn = nullptr;       // device status word for calls that take no workspace
+    int32_t *statusOwn = nullptr;       // device status word for calls that take no workspace; from kFirstTicket on, tile tickets
+    unsigned simTurn = 0;               // similarity launches so far: each takes the next ticket
     size_t hostStageInts = 0;
     unsigned char *hostBlob = nullptr;  // pinned, what a call's host side hands to its kernels
     size_t hostBlobBytes = 0;

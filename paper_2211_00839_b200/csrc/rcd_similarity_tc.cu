@@ -1,7 +1,7 @@
 // Tensor-core similarity kernel for sm_100a:  S_l = X_l X_l^T  per class (Section 3.1: similarities
 // from the feature vectors; int8 -> int32 exact, bf16 -> fp32).
 //
-// Persistent CTAs (one per SM) walk tiles of 128 rows x 256 columns of every class, those that reach the
+// Persistent CTAs (one per SM) take tiles of 128 rows x 256 columns of every class, those that reach the
 // diagonal or lie above it; S is symmetric, so each 128 x 128 block above the diagonal is computed once
 // and written twice (itself and its mirror image), which halves the tensor work and the operand traffic
 // (a tile whose left half lies below the diagonal computes its right half only).  The tile is twice as wide
@@ -34,6 +34,7 @@ constexpr int kSlabBytes = 128;                         // k-slab per stage and 
 constexpr int kStages = 4;
 constexpr int kOperandBytes = kTileM * kSlabBytes;      // 16 KB: 128 rows of one k-slab
 constexpr int kStageBytes = 3 * kOperandBytes;          // A (128 rows) + B (256 rows)
+constexpr int kTileSlots = 2;                           // tiles between the producer, which draws them, and the other roles
 constexpr int kEpiWarps = 8;                            // two per quarter of the TMEM lanes
 constexpr int kTcThreads = 64 + 32 * kEpiWarps;
 constexpr int kTmemCols = 512;                           // two accumulator buffers of 256 columns
@@ -44,6 +45,9 @@ struct __align__(8) TcShared {
     uint64_t empty[kStages];
     uint64_t accFull[2];
     uint64_t accEmpty[2];
+    uint64_t tileFull[kTileSlots];
+    uint64_t tileEmpty[kTileSlots];
+    int32_t tile[kTileSlots];                           // tiles this CTA has drawn (-1: no more)
     uint32_t tmemBase;
     int32_t abort;
 };
@@ -140,10 +144,10 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_addr(bar)) : "memory");
 }
 
-// Tile idx of the launch -> (class, row block tm of 128 rows, column block sn of 256 columns).  A class lists, row
-// block after row block, the tiles with sn >= tm / 2: those that contain a 128 x 128 block on or above the diagonal.
-// skip = 128 when the left half of the tile lies below the diagonal (tm odd, sn = tm / 2): that half is the mirror
-// image of a block another tile computes, so only the right half is computed.
+// Tile idx of the launch -> (class, row block tm of 128 rows, column block sn of 256 columns).  The tiles of a class are
+// those with sn >= tm / 2, which contain a 128 x 128 block on or above the diagonal.  skip = 128 when the left half of the
+// tile lies below the diagonal (tm odd, sn = tm / 2): that half is the mirror image of a block another tile computes, so
+// only the right half is computed.
 struct TileCoord { int l, tm, sn, skip, n; };         // n: columns computed, from column sn * 256 + skip on
 __device__ __forceinline__ TileCoord decode_tile(const DescSource &src, const int32_t *__restrict__ prefix, int L, int uniTiles, int idx)
 {
@@ -181,7 +185,7 @@ __device__ __forceinline__ TileCoord decode_tile(const DescSource &src, const in
 template <bool kInt8>
 __global__ void __launch_bounds__(kTcThreads, 1) sim_tc_kernel(const __grid_constant__ CUtensorMap map, DescSource src, int32_t L,
                                                               const int32_t *__restrict__ tilePrefix, int32_t uniTiles,
-                                                              int32_t totalTiles, int32_t numSlabs, uint32_t *__restrict__ S,
+                                                              int32_t *ticket, int32_t totalTiles, int32_t numSlabs, uint32_t *__restrict__ S,
                                                               int32_t *status)
 {
     extern __shared__ unsigned char smemRaw[];
@@ -195,6 +199,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) sim_tc_kernel(const __grid_cons
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(&sh.accFull[b], 1); mbar_init(&sh.accEmpty[b], kEpiWarps); }
+        for (int k = 0; k < kTileSlots; ++k) { mbar_init(&sh.tileFull[k], 1); mbar_init(&sh.tileEmpty[k], 1 + kEpiWarps); }
         sh.abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -212,21 +217,39 @@ __global__ void __launch_bounds__(kTcThreads, 1) sim_tc_kernel(const __grid_cons
         if (lane == 0) {
             uint32_t it = 0;                             // k-slabs issued so far, over all tiles
             bool ok = true;
-            for (int idx = blockIdx.x; idx < totalTiles && ok; idx += gridDim.x) {
+            int idx = blockIdx.x;
+            // the next tile: every gridDim.x-th, or drawn from the launch's ticket, which whoever draws last puts back to zero
+            auto draw = [&]() { return ticket ? atomicAdd(ticket, 1) : idx; };
+            auto tile_of = [&](int k) {
+                if (ticket && k == totalTiles - 1) atomicExch(ticket, 0);
+                return k + (int)gridDim.x < totalTiles ? k + (int)gridDim.x : -1;
+            };
+            for (uint32_t nt = 0; ok; ++nt) {
+                const int slot = nt % kTileSlots;
+                if (!mbar_wait(&sh.tileEmpty[slot], ((nt / kTileSlots) & 1) ^ 1, &sh)) break;
+                *(volatile int32_t *)&sh.tile[slot] = idx;
+                mbar_arrive(&sh.tileFull[slot]);
+                if (idx < 0) break;
+                int next = -1;
                 const TileCoord t = decode_tile(src, tilePrefix, L, uniTiles, idx);
                 const ClassDesc c = src.get(t.l);
                 const int rowA = c.row0 + t.tm * kTileM, rowB = c.row0 + t.sn * kTileN + t.skip;
                 const int halves = (t.n + kTileM - 1) / kTileM;         // 128-row pieces of B to bring in: 2, or 1
+                const bool shared = t.sn == t.tm / 2;                   // on the diagonal the first of them is A
                 for (int kb = 0; kb < numSlabs; ++kb, ++it) {
+                    if (kb == max(numSlabs - kStages, 0)) next = draw();       // (looked at behind the last slab)
                     const int s = it % kStages;
                     if (!mbar_wait(&sh.empty[s], ((it / kStages) & 1) ^ 1, &sh)) { ok = false; break; }
                     unsigned char *a = tiles + (size_t)s * kStageBytes;
-                    mbar_expect_tx(&sh.full[s], (1 + halves) * kOperandBytes);
+                    mbar_expect_tx(&sh.full[s], ((shared ? 0 : 1) + halves) * kOperandBytes);
                     const int k0 = kb * (kInt8 ? kSlabBytes : kSlabBytes / 2);         // element coordinate
-                    tma_load_2d(a, &map, k0, rowA, &sh.full[s]);
+                    if (!shared) tma_load_2d(a, &map, k0, rowA, &sh.full[s]);
                     for (int h = 0; h < halves; ++h) tma_load_2d(a + (1 + h) * kOperandBytes, &map, k0, rowB + h * kTileM, &sh.full[s]);
                 }
+                if (next < 0) next = draw();
+                idx = tile_of(next);
             }
+            while (idx >= 0) idx = tile_of(draw());       // (given up: the tickets still have to run out)
             // after an abort: let the copies already issued land before the CTA leaves
             if (*(volatile int32_t *)&sh.abort) {
                 for (uint32_t k = (it > (uint32_t)kStages ? it - kStages : 0); k < it; ++k) {
@@ -244,7 +267,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) sim_tc_kernel(const __grid_cons
                                        | ((uint32_t)(kTileM >> 4) << 24);
             uint32_t it = 0, nt = 0;
             bool ok = true;
-            for (int idx = blockIdx.x; idx < totalTiles && ok; idx += gridDim.x, ++nt) {
+            for (; ok; ++nt) {
+                const int slot = nt % kTileSlots;
+                if (!mbar_wait(&sh.tileFull[slot], (nt / kTileSlots) & 1, &sh)) break;
+                const int idx = *(volatile int32_t *)&sh.tile[slot];
+                mbar_arrive(&sh.tileEmpty[slot]);
+                if (idx < 0) break;
                 const TileCoord t = decode_tile(src, tilePrefix, L, uniTiles, idx);
                 const uint32_t idesc = idescBase | ((uint32_t)(t.n >> 3) << 17);   // N = 256, less for a half tile or at the class's edge
                 const uint32_t buf = nt & 1;
@@ -257,7 +285,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) sim_tc_kernel(const __grid_cons
                     if (!mbar_wait(&sh.full[s], (it / kStages) & 1, &sh)) { ok = false; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint32_t aAddr = smem_addr(tiles + (size_t)s * kStageBytes);
-                    const uint64_t descA = make_smem_desc(aAddr);
+                    const uint64_t descA = make_smem_desc(t.sn == t.tm / 2 ? aAddr + kOperandBytes : aAddr);
                     const uint64_t descB = make_smem_desc(aAddr + kOperandBytes);
 #pragma unroll
                     for (int k = 0; k < kSlabBytes / 32; ++k)          // one MMA consumes 32 bytes of k per row
@@ -273,7 +301,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) sim_tc_kernel(const __grid_cons
         const int ew = warp - 2;
         const int half = ew >> 2;                                      // which column blocks of the tile: even or odd
         uint32_t nt = 0;
-        for (int idx = blockIdx.x; idx < totalTiles; idx += gridDim.x, ++nt) {
+        for (;; ++nt) {
+            const int slot = nt % kTileSlots;
+            if (!mbar_wait(&sh.tileFull[slot], (nt / kTileSlots) & 1, &sh)) break;
+            const int idx = *(volatile int32_t *)&sh.tile[slot];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sh.tileEmpty[slot]);
+            if (idx < 0) break;
             const TileCoord t = decode_tile(src, tilePrefix, L, uniTiles, idx);
             const ClassDesc c = src.get(t.l);
             const int rowA = t.tm * kTileM, colB = t.sn * kTileN + t.skip;   // class-local: first row, first column computed
@@ -395,13 +429,19 @@ rcd_status launch_similarity_tc(rcd_ctx *ctx, const void *Xs, rcd_feat_dtype dty
     const int totalTiles = (int)cls.upperTiles;
     const int grid = totalTiles < ctx->smCount ? totalTiles : ctx->smCount;
     int32_t *status = const_cast<int32_t *>(ctx->statusDev);
+    // Tiles are drawn, since they are not equally long and an uneven share leaves most SMs idle at the end: 10 classes of
+    // 5000 x 256 int8 217 -> 177 us, 50 of 1300 x 192 bf16 112 -> 99, 100 of 500 x 512 bf16 47 -> 44.  Not so for short rows
+    // in classes of at most 8 tiles (500 samples: 6): every gridDim.x-th is as even then, and a CTA has to draw such tiles
+    // up to three ahead of their turn (200 of 257 x 256 int8: 29 -> 34 us).  A ticket of its own for every launch that can
+    // be under way at once: calls may overlap on several streams.
+    int32_t *ticket = totalTiles <= 8LL * cls.L && numSlabs < 8 ? nullptr : ctx->statusOwn + kFirstTicket + ctx->simTurn++ % (kStatusWords - kFirstTicket);
     if (dtype == RCD_FEAT_I8) {
         RCD_CUDA(ctx, cudaFuncSetAttribute(sim_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        sim_tc_kernel<true><<<grid, kTcThreads, smem, st>>>(map, cls.src, cls.L, cls.tilePrefixDev, cls.uniTiles, totalTiles,
+        sim_tc_kernel<true><<<grid, kTcThreads, smem, st>>>(map, cls.src, cls.L, cls.tilePrefixDev, cls.uniTiles, ticket, totalTiles,
                                                            numSlabs, (uint32_t *)S, status);
     } else {
         RCD_CUDA(ctx, cudaFuncSetAttribute(sim_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        sim_tc_kernel<false><<<grid, kTcThreads, smem, st>>>(map, cls.src, cls.L, cls.tilePrefixDev, cls.uniTiles, totalTiles,
+        sim_tc_kernel<false><<<grid, kTcThreads, smem, st>>>(map, cls.src, cls.L, cls.tilePrefixDev, cls.uniTiles, ticket, totalTiles,
                                                             numSlabs, (uint32_t *)S, status);
     }
     ctx->kernelLaunches++;
