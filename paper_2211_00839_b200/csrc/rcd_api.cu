@@ -304,7 +304,7 @@ static rcd_status prepare(rcd_ctx *ctx, const void *features, rcd_feat_dtype dty
     cls.tilePrefixDev = P.ws.tilePrefix;
     for (int32_t l = 0; l < L; ++l) {
         prefix[l] = (int32_t)cls.upperTiles;
-        cls.upperTiles += sim_tiles(P.desc[(size_t)l].M);
+        cls.upperTiles += sim_tiles(P.desc[(size_t)l].M, sim_pairs(sz.pitch, maxM));
         if (cls.upperTiles > 0x7fffffffLL) return fail(ctx, RCD_ERR_UNSUPPORTED, "too many similarity tiles");
         order[l] = l;
         sorted[l] = P.desc[(size_t)l].M;
@@ -617,7 +617,7 @@ rcd_status rcd_similarity(rcd_ctx *ctx, const void *X_dev, rcd_feat_dtype dtype,
     cls.L = (int32_t)batch;
     cls.maxM = M;
     cls.tilePrefixDev = nullptr;
-    cls.uniTiles = (int32_t)sim_tiles(M);
+    cls.uniTiles = (int32_t)sim_tiles(M, sim_pairs(d * (int64_t)feat_bytes(dtype), M));
     cls.upperTiles = batch * (int64_t)cls.uniTiles;
     ctx->kernelLaunches = 0;
     ctx->tcLaunches = 0;

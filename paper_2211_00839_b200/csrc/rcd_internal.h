@@ -169,10 +169,15 @@ inline int32_t pad4(int64_t m) { return (int32_t)((m + 3) / 4 * 4); }
 // the sweeps copy then pair up into whole sectors.
 inline int32_t pad_row(int64_t m) { return (int32_t)((m + 7) / 8 * 8); }
 
-// Tiles the tensor-core similarity kernel computes for a class of M samples: 128 rows x 256 columns each, those that
-// reach the diagonal or lie above it (row block tm pairs with the column blocks from tm / 2 on).
-inline int64_t sim_tiles(int64_t M)
+// Classes of 129 to 1024 samples with rows of at least 1 KB: 256 x 256 tiles, a pair of SMs each.  Shorter rows are bound by
+// writing S, one block of rows leaves half a pair idle, and in larger classes drawn tiles of half the size share the work out
+// better (20 classes of 1300 x 1024 int8: 55 us, pairs 61; 50 of 1300 x 768 bf16: 130 either way).
+inline bool sim_pairs(int64_t rowBytes, int64_t maxM) { return rowBytes >= 1024 && maxM > 128 && maxM <= 1024; }
+// Tiles the tensor-core similarity kernels compute for a class of M samples: those that reach the diagonal or lie above it, of
+// 256 x 256, or of 128 rows x 256 columns (row block tm with the column blocks from tm / 2 on).
+inline int64_t sim_tiles(int64_t M, bool pairs)
 {
+    if (pairs) { const int64_t blocks = (M + 255) / 256; return blocks * (blocks + 1) / 2; }
     const int64_t rowBlocks = (M + 127) / 128, colBlocks = (M + 255) / 256;
     int64_t n = 0;
     for (int64_t tm = 0; tm < rowBlocks; ++tm) n += colBlocks - tm / 2;

@@ -24,6 +24,8 @@
 
 #include <cuda.h>
 
+#include <algorithm>
+
 namespace rcd {
 
 namespace {
@@ -182,6 +184,60 @@ __device__ __forceinline__ TileCoord decode_tile(const DescSource &src, const in
     return t;
 }
 
+// An epilogue warp's column blocks (every other one of a tile's, from `half` on) -> S: the 32 rows from row0 on in 32 x 32
+// blocks, transposed through shared memory, and the mirror image of those that are mirrored.  v: the first block, on its way.
+template <typename Mirrored>
+__device__ __forceinline__ void write_columns(uint32_t (*stage)[33], uint32_t *Sl, const ClassDesc &c, int row0, int colB, uint32_t tmemRow,
+                                              int half, int nCb, uint32_t (&v)[32], Mirrored mirrored)
+{
+    const int lane = threadIdx.x & 31;
+    const int cg = (lane & 7) * 4;                             // this lane's 4 columns of a 32-wide block
+#pragma unroll 1
+    for (int cb = half; cb < nCb; cb += kEpiWarps / 4) {
+        tmem_load_wait();
+#pragma unroll
+        for (int j = 0; j < 32; ++j) stage[lane][j] = v[j];         // lane = row inside the quarter
+        __syncwarp();
+        // the next block of this warp travels from tensor memory while this one is written out
+        if (cb + kEpiWarps / 4 < nCb) tmem_load_32cols(tmemRow + (uint32_t)((cb + kEpiWarps / 4) * 32), v);
+        // block rows -> S[rowA + ..][colB + ..]: 8 lanes cover 32 columns with 128-bit stores, 4 rows per pass
+        {
+            const int col = colB + cb * 32 + cg;
+#pragma unroll
+            for (int pass = 0; pass < 8; ++pass) {
+                const int r = pass * 4 + (lane >> 3);
+                const int row = row0 + r;
+                if (row < c.M && col < c.ld) {
+                    uint4 o;
+                    o.x = col + 0 < c.M ? stage[r][cg + 0] : 0u;
+                    o.y = col + 1 < c.M ? stage[r][cg + 1] : 0u;
+                    o.z = col + 2 < c.M ? stage[r][cg + 2] : 0u;
+                    o.w = col + 3 < c.M ? stage[r][cg + 3] : 0u;
+                    *reinterpret_cast<uint4 *>(Sl + (int64_t)row * c.ld + col) = o;
+                }
+            }
+        }
+        // the mirrored block -> S[colB + ..][rowA + ..] (blocks below the diagonal are never computed)
+        if (mirrored(cb)) {
+            const int col = row0 + cg;
+#pragma unroll
+            for (int pass = 0; pass < 8; ++pass) {
+                const int jj = pass * 4 + (lane >> 3);
+                const int row = colB + cb * 32 + jj;
+                if (row < c.M && col < c.ld) {
+                    uint4 o;
+                    o.x = col + 0 < c.M ? stage[cg + 0][jj] : 0u;
+                    o.y = col + 1 < c.M ? stage[cg + 1][jj] : 0u;
+                    o.z = col + 2 < c.M ? stage[cg + 2][jj] : 0u;
+                    o.w = col + 3 < c.M ? stage[cg + 3][jj] : 0u;
+                    *reinterpret_cast<uint4 *>(Sl + (int64_t)row * c.ld + col) = o;
+                }
+            }
+        }
+        __syncwarp();
+    }
+}
+
 template <bool kInt8>
 __global__ void __launch_bounds__(kTcThreads, 1) sim_tc_kernel(const __grid_constant__ CUtensorMap map, DescSource src, int32_t L,
                                                               const int32_t *__restrict__ tilePrefix, int32_t uniTiles,
@@ -316,58 +372,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) sim_tc_kernel(const __grid_cons
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             if (*(volatile int32_t *)&sh.abort) break;
             uint32_t *Sl = S + c.sOff;
-            const int cg = (lane & 7) * 4;                             // this lane's 4 columns of a 32-wide block
             const int nCb = t.n / 32;
             const uint32_t tmemRow = tmemBase + buf * kTileN + ((uint32_t)(q * 32) << 16);
             uint32_t v[32];
             if (half < nCb) tmem_load_32cols(tmemRow + (uint32_t)(half * 32), v);
-#pragma unroll 1
-            for (int cb = half; cb < nCb; cb += kEpiWarps / 4) {
-                // the 128 x 128 block this column block belongs to lies on the diagonal (stored once) or above it
-                // (stored twice: itself and its mirror image)
-                const bool diag = (colB + cb * 32) / kTileM == t.tm;
-                tmem_load_wait();
-#pragma unroll
-                for (int j = 0; j < 32; ++j) stage32[ew][lane][j] = v[j];         // lane = row inside the quarter
-                __syncwarp();
-                // the next block of this warp travels from tensor memory while this one is written out
-                if (cb + kEpiWarps / 4 < nCb) tmem_load_32cols(tmemRow + (uint32_t)((cb + kEpiWarps / 4) * 32), v);
-                // block rows -> S[rowA + ..][colB + ..]: 8 lanes cover 32 columns with 128-bit stores, 4 rows per pass
-                {
-                    const int col = colB + cb * 32 + cg;
-#pragma unroll
-                    for (int pass = 0; pass < 8; ++pass) {
-                        const int r = pass * 4 + (lane >> 3);
-                        const int row = rowA + q * 32 + r;
-                        if (row < c.M && col < c.ld) {
-                            uint4 o;
-                            o.x = col + 0 < c.M ? stage32[ew][r][cg + 0] : 0u;
-                            o.y = col + 1 < c.M ? stage32[ew][r][cg + 1] : 0u;
-                            o.z = col + 2 < c.M ? stage32[ew][r][cg + 2] : 0u;
-                            o.w = col + 3 < c.M ? stage32[ew][r][cg + 3] : 0u;
-                            *reinterpret_cast<uint4 *>(Sl + (int64_t)row * c.ld + col) = o;
-                        }
-                    }
-                }
-                // the mirrored block -> S[colB + ..][rowA + ..] (blocks below the diagonal are never computed)
-                if (!diag) {
-                    const int col = rowA + q * 32 + cg;
-#pragma unroll
-                    for (int pass = 0; pass < 8; ++pass) {
-                        const int jj = pass * 4 + (lane >> 3);
-                        const int row = colB + cb * 32 + jj;
-                        if (row < c.M && col < c.ld) {
-                            uint4 o;
-                            o.x = col + 0 < c.M ? stage32[ew][cg + 0][jj] : 0u;
-                            o.y = col + 1 < c.M ? stage32[ew][cg + 1][jj] : 0u;
-                            o.z = col + 2 < c.M ? stage32[ew][cg + 2][jj] : 0u;
-                            o.w = col + 3 < c.M ? stage32[ew][cg + 3][jj] : 0u;
-                            *reinterpret_cast<uint4 *>(Sl + (int64_t)row * c.ld + col) = o;
-                        }
-                    }
-                }
-                __syncwarp();
-            }
+            // a 128 x 128 block lies on the diagonal (stored once) or above it (stored twice: itself and its mirror image)
+            write_columns(stage32[ew], Sl, c, rowA + q * 32, colB, tmemRow, half, nCb, v, [&](int cb) { return (colB + cb * 32) / kTileM != t.tm; });
             // hand the accumulator buffer back to the MMA warp
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
@@ -379,6 +389,238 @@ __global__ void __launch_bounds__(kTcThreads, 1) sim_tc_kernel(const __grid_cons
     if (warp == 1) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmemBase), "r"(kTmemCols) : "memory");
+    }
+    if (threadIdx.x == 0 && sh.abort && status) atomicOr(status, kDevTimeout);
+}
+
+// ---------------------------------------------------------------------------------------------
+// Long rows: a pair of SMs per 256 x 256 tile (cta_group::2).  Each CTA holds 128 of the tile's rows (A and the accumulator)
+// and half of its columns (B), so every operand row comes in once: 32 KB per SM and k-slab, 16 on the diagonal, where both
+// operands are the same rows, against 48 and 32 above.  CTA 0 issues the MMAs of both.  Tiles on the diagonal are computed
+// whole and stored as they are, the others stored twice.  Bound by the tensor cores: a slab takes 0.43 us where its MMAs
+// alone take 0.37 at the rate of a large cuBLAS product.  100 classes of 500 x 2048 bf16: 92 -> 82 us (67 GFLOP, at least
+// 40 us; writing S and reading X, 47), 300 of 200 x 1024: 55 -> 48.
+constexpr int kPairStages = 6;
+constexpr int kPairStageBytes = 2 * kOperandBytes;
+constexpr int kPairTile = 256;
+
+struct __align__(8) PairShared {
+    uint64_t full[kPairStages];                         // CTA 0's: both CTAs' copies of a slab have landed
+    uint64_t empty[kPairStages];
+    uint64_t accFull[2];
+    uint64_t accEmpty[2];                               // CTA 0's: the epilogue warps of both CTAs have read the accumulator
+    uint32_t tmemBase;
+    int32_t abort;
+};
+
+__device__ __forceinline__ uint32_t leader_addr(const void *p)
+{
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(a) : "r"(smem_addr(p)));
+    return a;
+}
+__device__ __forceinline__ bool pair_wait(uint64_t *bar, uint32_t parity, PairShared *sh)
+{
+    for (uint32_t spin = 0; spin < kSpinLimit; ++spin) {
+        uint32_t ok;
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(ok) : "r"(smem_addr(bar)), "r"(parity) : "memory");
+        if (ok) return true;
+        if (spin > 64) {
+            if (*(volatile int32_t *)&sh->abort) return false;
+            __nanosleep(64);
+        }
+    }
+    atomicExch(&sh->abort, 1);
+    return false;
+}
+__device__ __forceinline__ void pair_load_2d(void *dst, const CUtensorMap *map, int c0, int c1, uint32_t leaderBar)
+{
+    asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                 :: "r"(smem_addr(dst)), "l"(map), "r"(c0), "r"(c1), "r"(leaderBar) : "memory");
+}
+template <bool kInt8>
+__device__ __forceinline__ void pair_mma(uint32_t tmemD, uint64_t descA, uint64_t descB, uint32_t idesc, uint32_t accumulate)
+{
+    if constexpr (kInt8) {
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                     "tcgen05.mma.cta_group::2.kind::i8 [%0], %1, %2, %3, p;\n\t}"
+                     :: "r"(tmemD), "l"(descA), "l"(descB), "r"(idesc), "r"(accumulate) : "memory");
+    } else {
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                     "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+                     :: "r"(tmemD), "l"(descA), "l"(descB), "r"(idesc), "r"(accumulate) : "memory");
+    }
+}
+// arrives at the barrier of this offset in both CTAs
+__device__ __forceinline__ void pair_commit(uint64_t *bar)
+{
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+                 :: "r"(smem_addr(bar)), "h"((uint16_t)3) : "memory");
+}
+__device__ __forceinline__ void cluster_barrier()
+{
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// Unit -> class, row block of 256, first column and columns computed.  The units are the tiles (column blocks from the row
+// block on), as long as they fill rounds of one per pair; those left over are cut into 2, 4 or 8 strips of columns, which
+// share the last round out to more pairs (100 classes of 500 x 2048: 300 tiles on 74 pairs leave 4; 85 -> 82 us).
+struct PairUnits { int whole, strips, count; };
+__host__ __device__ inline PairUnits pair_units(int tiles, int pairs)
+{
+    PairUnits u;
+    u.whole = tiles / pairs * pairs;
+    u.strips = 1;
+    while (u.strips < 8 && (tiles - u.whole) * u.strips * 2 <= pairs) u.strips *= 2;
+    u.count = u.whole + (tiles - u.whole) * u.strips;
+    return u;
+}
+struct PairTile { int l, tb, col, n; bool diag, shared; };      // diag: stored once; shared: A's rows are B's
+__device__ __forceinline__ PairTile decode_pair_tile(const DescSource &src, const int32_t *__restrict__ prefix, int L, int uniTiles,
+                                                     const PairUnits &units, int unit)
+{
+    PairTile t;
+    int local, idx = unit, strip = 0;
+    const bool cut = unit >= units.whole && units.strips > 1;
+    if (cut) {
+        idx = units.whole + (unit - units.whole) / units.strips;
+        strip = (unit - units.whole) % units.strips;
+    }
+    if (prefix) {
+        int lo = 0, hi = L;                              // prefix[lo] <= idx < prefix[hi]
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (prefix[mid] <= idx) lo = mid; else hi = mid;
+        }
+        t.l = lo;
+        local = idx - prefix[lo];
+    } else {
+        t.l = idx / uniTiles;
+        local = idx - t.l * uniTiles;
+    }
+    const ClassDesc c = src.get(t.l);
+    const int blocks = (c.M + kPairTile - 1) / kPairTile;
+    for (t.tb = 0; local >= blocks - t.tb; ++t.tb) local -= blocks - t.tb;
+    const int width = cut ? kPairTile / units.strips : kPairTile;
+    t.diag = local == 0;
+    t.shared = t.diag && !cut;                           // (each CTA's 128 rows are its half of the columns too)
+    t.col = (t.tb + local) * kPairTile + strip * width;
+    t.n = t.shared ? kPairTile : max(32, min(width, (c.ld - t.col + 31) & ~31));
+    return t;
+}
+
+template <bool kInt8>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) sim_pair_kernel(
+    const __grid_constant__ CUtensorMap map, DescSource src, int32_t L, const int32_t *__restrict__ tilePrefix, int32_t uniTiles,
+    int32_t totalTiles, int32_t kernelPairs, int32_t numSlabs, uint32_t *__restrict__ S, int32_t *status)
+{
+    extern __shared__ unsigned char smemRaw[];
+    unsigned char *tiles = reinterpret_cast<unsigned char *>(((uintptr_t)smemRaw + 1023) & ~(uintptr_t)1023);
+    __shared__ PairShared sh;
+    __shared__ uint32_t stage32[kEpiWarps][32][33];
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = blockIdx.x & 1;                     // (clusters are consecutive pairs of blocks)
+    const int firstUnit = blockIdx.x >> 1, pairs = gridDim.x >> 1;
+    const PairUnits units = pair_units(totalTiles, kernelPairs);
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kPairStages; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&sh.accFull[b], 1); mbar_init(&sh.accEmpty[b], 2 * kEpiWarps); }
+        sh.abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(smem_addr(&sh.tmemBase)), "r"(kTmemCols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    cluster_barrier();                                   // the other CTA's barriers exist
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmemBase = sh.tmemBase;
+
+    if (warp == 0) {
+        // ---------------- TMA producer: this CTA's half of both operands ----------------
+        if (lane == 0) {
+            uint32_t it = 0;
+            bool ok = true;
+            for (int idx = firstUnit; idx < units.count && ok; idx += pairs) {
+                const PairTile t = decode_pair_tile(src, tilePrefix, L, uniTiles, units, idx);
+                const ClassDesc c = src.get(t.l);
+                const int rowA = c.row0 + t.tb * kPairTile + rank * kTileM, rowB = c.row0 + t.col + rank * (t.n / 2);
+                for (int kb = 0; kb < numSlabs; ++kb, ++it) {
+                    const int s = it % kPairStages;
+                    if (!pair_wait(&sh.empty[s], ((it / kPairStages) & 1) ^ 1, &sh)) { ok = false; break; }
+                    unsigned char *a = tiles + (size_t)s * kPairStageBytes;
+                    if (rank == 0) mbar_expect_tx(&sh.full[s], 2 * (t.shared ? 1 : 2) * kOperandBytes);
+                    const uint32_t bar = leader_addr(&sh.full[s]);
+                    const int k0 = kb * (kInt8 ? kSlabBytes : kSlabBytes / 2);
+                    pair_load_2d(a, &map, k0, rowA, bar);
+                    if (!t.shared) pair_load_2d(a + kOperandBytes, &map, k0, rowB, bar);
+                }
+            }
+            // after an abort: let the copies already issued land (they report to CTA 0, so by time: some 2 ms)
+            if (*(volatile int32_t *)&sh.abort)
+                for (uint32_t spin = 0; spin < (1u << 15); ++spin) __nanosleep(64);
+        }
+    } else if (warp == 1) {
+        // ---------------- MMA issuer: CTA 0, for both ----------------
+        if (lane == 0 && rank == 0) {
+            const uint32_t idescBase = (kInt8 ? (2u << 4) | (1u << 7) | (1u << 10) : (1u << 4) | (1u << 7) | (1u << 10)) | ((uint32_t)(kPairTile >> 4) << 24);
+            uint32_t it = 0, nt = 0;
+            bool ok = true;
+            for (int idx = firstUnit; idx < units.count && ok; idx += pairs, ++nt) {
+                const PairTile t = decode_pair_tile(src, tilePrefix, L, uniTiles, units, idx);
+                const uint32_t idesc = idescBase | ((uint32_t)(t.n >> 3) << 17);
+                const uint32_t buf = nt & 1;
+                if (!pair_wait(&sh.accEmpty[buf], ((nt >> 1) & 1) ^ 1, &sh)) { ok = false; break; }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint32_t tmemD = tmemBase + buf * kPairTile;
+                for (int kb = 0; kb < numSlabs; ++kb, ++it) {
+                    const int s = it % kPairStages;
+                    if (!pair_wait(&sh.full[s], (it / kPairStages) & 1, &sh)) { ok = false; break; }
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const uint32_t aAddr = smem_addr(tiles + (size_t)s * kPairStageBytes);
+                    const uint64_t descA = make_smem_desc(aAddr);
+                    const uint64_t descB = make_smem_desc(t.shared ? aAddr : aAddr + kOperandBytes);
+#pragma unroll
+                    for (int k = 0; k < kSlabBytes / 32; ++k)
+                        pair_mma<kInt8>(tmemD, descA + (uint64_t)(2 * k), descB + (uint64_t)(2 * k), idesc, (kb > 0 || k > 0) ? 1u : 0u);
+                    pair_commit(&sh.empty[s]);
+                }
+                pair_commit(&sh.accFull[buf]);
+            }
+        }
+    } else {
+        // ---------------- epilogue: this CTA's 128 rows ----------------
+        const int q = warp & 3, ew = warp - 2, half = ew >> 2;
+        uint32_t nt = 0;
+        for (int idx = firstUnit; idx < units.count; idx += pairs, ++nt) {
+            const PairTile t = decode_pair_tile(src, tilePrefix, L, uniTiles, units, idx);
+            const ClassDesc c = src.get(t.l);
+            const uint32_t buf = nt & 1;
+            if (!pair_wait(&sh.accFull[buf], (nt >> 1) & 1, &sh)) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            if (*(volatile int32_t *)&sh.abort) break;
+            const int row0 = t.tb * kPairTile + rank * kTileM + q * 32;
+            const int nCb = row0 < c.M ? t.n / 32 : 0;
+            const uint32_t tmemRow = tmemBase + buf * kPairTile + ((uint32_t)(q * 32) << 16);
+            uint32_t v[32];
+            if (half < nCb) tmem_load_32cols(tmemRow + (uint32_t)(half * 32), v);
+            write_columns(stage32[ew], S + c.sOff, c, row0, t.col, tmemRow, half, nCb, v, [&](int) { return !t.diag; });
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" :: "r"(leader_addr(&sh.accEmpty[buf])) : "memory");
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    cluster_barrier();                                   // nothing of the other CTA is on its way here any more
+    if (warp == 1) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" :: "r"(tmemBase), "r"(kTmemCols) : "memory");
     }
     if (threadIdx.x == 0 && sh.abort && status) atomicOr(status, kDevTimeout);
 }
@@ -429,6 +671,20 @@ rcd_status launch_similarity_tc(rcd_ctx *ctx, const void *Xs, rcd_feat_dtype dty
     const int totalTiles = (int)cls.upperTiles;
     const int grid = totalTiles < ctx->smCount ? totalTiles : ctx->smCount;
     int32_t *status = const_cast<int32_t *>(ctx->statusDev);
+    if (sim_pairs(rowBytes, cls.maxM)) {
+        const size_t pairSmem = (size_t)kPairStages * kPairStageBytes + 1024;
+        const int pairs = std::max(1, ctx->smCount / 2);
+        const int pairGrid = 2 * std::min(pairs, pair_units(totalTiles, pairs).count);
+        auto *kernel = dtype == RCD_FEAT_I8 ? sim_pair_kernel<true> : sim_pair_kernel<false>;
+        RCD_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pairSmem));
+        kernel<<<pairGrid, kTcThreads, pairSmem, st>>>(map, cls.src, cls.L, cls.tilePrefixDev, cls.uniTiles, totalTiles, pairs,
+                                                        numSlabs, (uint32_t *)S, status);
+        ctx->kernelLaunches++;
+        ctx->tcLaunches++;
+        RCD_CUDA(ctx, cudaGetLastError());
+        *handled = true;
+        return RCD_OK;
+    }
     // Tiles are drawn, since they are not equally long and an uneven share leaves most SMs idle at the end: 10 classes of
     // 5000 x 256 int8 217 -> 177 us, 50 of 1300 x 192 bf16 112 -> 99, 100 of 500 x 512 bf16 47 -> 44.  Not so for short rows
     // in classes of at most 8 tiles (500 samples: 6): every gridDim.x-th is as even then, and a CTA has to draw such tiles

@@ -131,3 +131,28 @@ def test_gaussian_edges(rcd, orc, M):
         want, sg = orc.similarity_gaussian(x[b * M:(b + 1) * M])
         assert sigma[b] == pytest.approx(sg, rel=2e-6)
         assert np.allclose(S[b, :, :M], want, rtol=2e-5, atol=1e-7) and np.all(S[b, :, M:] == 0)
+
+
+@pytest.mark.parametrize("M,batch,d,dtype", [(129, 1, 1024, "int8"), (256, 3, 1040, "int8"), (257, 2, 512, "bf16"), (500, 80, 520, "bf16"),
+                                             (1000, 9, 1024, "int8"), (1024, 1, 1024, "int8")])
+def test_similarity_long_rows(rcd, orc, M, batch, d, dtype):
+    """Pairs of SMs: one and several row blocks, whole rounds of tiles and rounds cut into strips; two calls overlap on two streams."""
+    import torch
+    g = torch.Generator().manual_seed(M)
+    X = torch.randint(-128, 128, (batch, M, d), generator=g).to(torch.int8) if dtype == "int8" else torch.randn(batch, M, d, generator=g).to(torch.bfloat16)
+    X = X.cuda()
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    torch.cuda.synchronize()
+    with rcd.Context(0) as ctx:
+        got = []
+        for st in streams:
+            with torch.cuda.stream(st):
+                got.append(ctx.rcd_similarity(X))
+        torch.cuda.synchronize()
+        ctx.sync_status()
+    w = X.double()
+    want = torch.matmul(w, w.transpose(1, 2))
+    for S in got:
+        assert bool((S[:, :, M:] == 0).all()) and torch.equal(S[:, :, :M], S[:, :, :M].transpose(1, 2))
+        err = (S[:, :, :M].double() - want).abs().max().item()
+        assert err == 0 if dtype == "int8" else err <= 2e-5 * want.abs().max().item()
