@@ -14,6 +14,7 @@ from __future__ import annotations
 import ctypes as C
 import os
 import subprocess
+import threading
 from concurrent.futures import ThreadPoolExecutor
 from typing import List, Optional, Sequence, Tuple
 
@@ -29,7 +30,7 @@ def build(force: bool = False) -> str:
     """Compile the oracle with gcc (no fast-math, no FP contraction)."""
     newest = max(os.path.getmtime(p) for p in _SRC)
     if force or not os.path.exists(_SO) or os.path.getmtime(_SO) < newest:
-        tmp = _SO + ".tmp.%d" % os.getpid()
+        tmp = _SO + ".tmp.%d.%d" % (os.getpid(), threading.get_ident())    # (several threads may find it missing)
         subprocess.check_call(["gcc", "-O2", "-std=c99", "-fPIC", "-shared", "-fno-fast-math",
                                "-ffp-contract=off", "-o", tmp, _SRC[0], "-lm"])
         os.replace(tmp, _SO)

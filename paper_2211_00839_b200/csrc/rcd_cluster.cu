@@ -376,7 +376,8 @@ __device__ __forceinline__ Raised entry_or_none(const Raised *list, int e, int n
 }
 
 // The n listed columns taken off one piece, rows straight to registers, up to sixteen in flight
-// (a warp waits about 1100 cycles for a batch: 137 -> @@ cycles per row of 5 KB with eleven warps at it).
+// (a warp waits about 1100 cycles for a batch; with sixteen warps at it a row of 5 KB takes an SM about 140 cycles, the share
+// of the copy bandwidth that 148 SMs get).
 __device__ __forceinline__ bool correct_piece(const int4 *S4q, const Raised *list, int n, uint32_t one, unsigned long long (&g)[4])
 {
     uint32_t changed = 0;
