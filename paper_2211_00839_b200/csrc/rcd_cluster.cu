@@ -1488,7 +1488,9 @@ static bool cluster_plan(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassD
     // Cluster size: the one whose clusters, drawing classes largest first, finish soonest by the estimate that a class of
     // M samples takes M (M / C + 300) (corrections, shared by the CTAs, and the chain of picks); blocks have to stay on
     // the chip.
-    const int most = std::min(16, pow2_at_least(sz.W));
+    // (graph cut, small classes: an update is one row, so the time goes into stale notes, and several blocks per CTA with lists
+    // of candidates do better than one: 2 classes of 400 into 8 blocks 791 us with 8 CTAs, 517 with 4, pass-free chain 583)
+    const int most = std::min(sz.graphCut && sz.maxM <= 1536 ? 4 : 16, pow2_at_least(sz.W));
     std::vector<int> sizes;
     for (const ClassDesc &d : descHost) if (d.M > 0) sizes.push_back(d.M);
     std::sort(sizes.begin(), sizes.end(), std::greater<int>());
@@ -1515,6 +1517,10 @@ static bool cluster_plan(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassD
         plan.smem = cluster_layout(sz, maxLd, plan.C, false, cap, plan);
         if (plan.smem > cap) return false;
     }
+    // Graph cut with many blocks per CTA: every pick makes most of the other blocks' notes stale, and the listing warps fall
+    // behind the chain of one CTA per class (2 classes of 1000, 16 blocks per CTA: 2625 us against 1981; 2 of 3000 into 100
+    // blocks 12.6 ms against 11.7; but 30 of 600, 15 blocks per CTA, 1124 against 1255).
+    if (sz.graphCut && (sz.W > 64 || (sz.W + plan.C - 1) / plan.C > 15)) return false;
     int idx = 0;
     while ((1 << idx) < plan.C) ++idx;
     if (ctx->maxClusters[idx] < 1) return false;
