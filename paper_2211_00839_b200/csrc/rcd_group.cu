@@ -116,6 +116,25 @@ __device__ __forceinline__ void copy_row(const uint8_t *__restrict__ src, uint8_
             d[i] = a; d[i + 32] = b; d[i + 64] = c; d[i + 96] = e;
         }
         for (; i < np; i += 32) d[i] = i < n ? __ldg(s + i) : make_int4(0, 0, 0, 0);
+    } else if (pitch % 16 == 0 && ((uintptr_t)dst) % 16 == 0) {
+        // rows that start anywhere: 16 bytes of the copy from the five aligned words that hold them (only words with a byte of
+        // the row in them are read).  Byte by byte a row of 2.7 KB took a warp 30 us.
+        const uint32_t *s = reinterpret_cast<const uint32_t *>((uintptr_t)src & ~(uintptr_t)3);
+        const int off = (int)((uintptr_t)src & 3), words = (int)((off + bytes + 3) >> 2), np = (int)(pitch >> 4);
+        int4 *d = reinterpret_cast<int4 *>(dst);
+#pragma unroll 2
+        for (int i = lane; i < np; i += 32) {
+            uint32_t w[5], o[4];
+#pragma unroll
+            for (int e = 0; e < 5; ++e) w[e] = 4 * i + e < words ? __ldg(s + 4 * i + e) : 0u;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int64_t left = bytes - 16 * (int64_t)i - 4 * e;            // bytes of the row from this word on
+                const uint32_t x = __funnelshift_r(w[e], w[e + 1], 8 * off);
+                o[e] = left >= 4 ? x : left <= 0 ? 0u : x & ((1u << (8 * (int)left)) - 1u);
+            }
+            d[i] = make_int4((int)o[0], (int)o[1], (int)o[2], (int)o[3]);
+        }
     } else {
         for (int64_t i = lane; i < pitch; i += 32) dst[i] = i < bytes ? src[i] : (uint8_t)0;
     }
@@ -159,14 +178,14 @@ __global__ void __launch_bounds__(kGroupThreads) label_place_kernel(const int32_
         if (in && rank == 0) mine[lab] = pos + __popc(same);
         __syncwarp();
         if (in) {
-            perm[pos] = (int32_t)(base + i + lane);
+            if (blockIdx.y == 0) perm[pos] = (int32_t)(base + i + lane);
             if (Xs) shPos[i + lane] = pos;
         }
     }
     if (!Xs) return;
     __syncthreads();
     const bool vec = rowBytes % 16 == 0 && pitch % 16 == 0 && ((uintptr_t)X) % 16 == 0 && ((uintptr_t)Xs) % 16 == 0;
-    for (int i = warp; i < n; i += kGroupWarps)
+    for (int i = warp + blockIdx.y * kGroupWarps; i < n; i += kGroupWarps * gridDim.y)
         copy_row(X + (base + i) * rowBytes, Xs + (int64_t)shPos[i] * pitch, rowBytes, pitch, vec, lane);
 }
 
@@ -275,7 +294,9 @@ rcd_status launch_stable_split(rcd_ctx *ctx, const int32_t *labels, int64_t N, i
     if (shared_labels(L)) {
         const size_t smem = ((size_t)kGroupWarps * L + (Xs ? chunk : 0)) * 4;
         if (smem > 48 * 1024) RCD_CUDA(ctx, cudaFuncSetAttribute(label_place_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        label_place_kernel<<<nChunks, kGroupThreads, smem, st>>>(labels, N, L, chunk, chunkHist, perm, (const uint8_t *)X, rowBytes, pitch,
+        // (few samples: several CTAs rank the same chunk and share its rows out, so that wide rows occupy more than a few SMs)
+        const dim3 grid(nChunks, Xs ? std::max(1, std::min(16, 2 * ctx->smCount / nChunks)) : 1);
+        label_place_kernel<<<grid, kGroupThreads, smem, st>>>(labels, N, L, chunk, chunkHist, perm, (const uint8_t *)X, rowBytes, pitch,
                                                                 (uint8_t *)Xs, status);
         ctx->kernelLaunches++;
     } else {
