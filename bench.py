@@ -309,10 +309,9 @@ def run_ours(args):
     h2d = Xh.numel() * Xh.element_size() + yh.numel() * 4
     d2h = sum(t.numel() * t.element_size() for t in host_out)
 
-    # Roofline of the dominant kernel.  The whole greedy loop is ONE launch (greedy_async_kernel when
-    # classes are few: pick CTAs and sweep CTAs hand classes back and forth; greedy_persistent_kernel
-    # otherwise: sweep phases and pick phases separated by grid barriers); it is HBM-bound through its
-    # sweeps.  Algorithmic bytes = for every sweep of a class, the rows of S of its unassigned samples
+    # Roofline of the dominant kernel.  The whole greedy loop is ONE launch (greedy_cluster_kernel, or, where a form with
+    # passes over S is asked for or needed: greedy_async_kernel when classes are few, greedy_owner_kernel when they are
+    # many).  For the forms with passes: algorithmic bytes = for every sweep of a class, the rows of S of its unassigned samples
     # plus the coverage vectors of the blocks refreshed (4*ld*(n_R + n) bytes), summed on the device.
     # Duration = CUDA events around the greedy loop on the launching stream (last timed step).
     peaks = load_peaks()
@@ -323,10 +322,15 @@ def run_ours(args):
         yard = box[0]
     default_setup = args.classes == 0 and args.sweep_batch in (0, 8) and args.async_group == 0 and args.async_help_min == 0 and args.similarity == "dot"
     loop_s = prof["greedy_ms"] * 1e-3
-    achieved = prof["sweep_bytes"] / loop_s / 1e9 if loop_s > 0 else 0.0
+    # The cluster form makes no sweeps: it reads the row of S of every pick and one per column that the pick raised.
+    clustered = prof["sweep_bytes"] == 0 and prof["incremental_rows"] > 0
+    loop_bytes = 4 * ((M + 7) // 8 * 8) * (prof["incremental_rows"] + prof["incremental_updates"]) if clustered else prof["sweep_bytes"]
+    achieved = loop_bytes / loop_s / 1e9 if loop_s > 0 else 0.0
     sms = torch.cuda.get_device_properties(local).multi_processor_count
     path = args.greedy_path if args.greedy_path else (3 if wl.L * 4 <= sms else 4)
-    if args.objective != "facility":
+    if clustered:
+        kernel_name = "greedy_cluster_kernel"
+    elif args.objective != "facility":
         kernel_name = "cut_chain_kernel"
     else:
         kernel_name = {1: "sweep_kernel", 2: "greedy_persistent_kernel", 3: "greedy_async_kernel", 4: "greedy_owner_kernel"}[path]
@@ -341,7 +345,7 @@ def run_ours(args):
                 # dram__bytes_read.sum + dram__bytes_write.sum of one launch of that kernel on this workload, from the
                 # ncu capture summarised under profiles/ (None: no capture of the kernel as it stands)
                 "traffic": MEASURED_TRAFFIC.get((args.config, kernel_name)) if default_setup else None,
-                "launch_ms": prof["greedy_ms"], "bytes_per_launch": prof["sweep_bytes"],
+                "launch_ms": prof["greedy_ms"], "bytes_per_launch": loop_bytes,
                 "rounds_with_sweeps": int(prof["sweep_launches"])}
     # the same bytes against the time the kernel spends sweeping (its own clock: the sweep phases of the
     # round-based kernel, the busy time of the first sweep CTA of the asynchronous one)
@@ -362,8 +366,8 @@ def run_ours(args):
         a3 = p3["sweep_bytes"] / (p3["greedy_ms"] * 1e-3) / 1e9
         roofline["note"] = ("default run: %d of %d picks correct their block's stored gains in place, so the launch reads %.1fx fewer bytes "
                             "than the passes-only form and is bound by the latency of each class's chain of picks, not by bandwidth; "
-                            "the bandwidth-bound form of the same kernel on the same dataset is under passes_only"
-                            % (int(prof["incremental_updates"]), wl.N, p3["sweep_bytes"] / max(1.0, prof["sweep_bytes"])))
+                            "the bandwidth-bound form of the loop on the same dataset is under passes_only"
+                            % (int(prof["incremental_updates"]), wl.N, p3["sweep_bytes"] / max(1.0, loop_bytes)))
         roofline["passes_only"] = {"what": "same dataset, in-place correction of stored gains off: every out-of-date block waits for a pass over S",
                                    "ms_per_step": p3["total_ms"], "launch_ms": p3["greedy_ms"], "bytes_per_launch": p3["sweep_bytes"],
                                    "achieved": a3, "frac": a3 / sweep_peak}
