@@ -32,11 +32,6 @@ rcd_status cuda_fail(rcd_ctx *ctx, cudaError_t e, const char *what)
 
 // Device-side errors of a call are collected in a status word of the context (the kernels' target, ctx->statusDev), so
 // rcd_sync_status never touches a workspace the caller may have freed.
-static cudaError_t status_begin(rcd_ctx *ctx, cudaStream_t st)
-{
-    ctx->statusDev = ctx->statusOwn;
-    return cudaMemsetAsync(ctx->statusOwn, 0, sizeof(int32_t), st);
-}
 
 // Pinned memory for what a call's host side hands to the device: the second half of the staging buffer, or, for calls that
 // need more, a buffer that grows to the largest of them.  The wait is for the last copy out of it (done long ago unless the
@@ -302,9 +297,15 @@ static rcd_status prepare(rcd_ctx *ctx, const void *features, rcd_feat_dtype dty
     cls.L = L;
     cls.maxM = maxM;
     cls.tilePrefixDev = P.ws.tilePrefix;
+    int64_t tiles = 0, pairTiles = 0;
+    for (int32_t l = 0; l < L; ++l) {
+        tiles += sim_tiles(P.desc[(size_t)l].M, false);
+        pairTiles += sim_tiles(P.desc[(size_t)l].M, true);
+    }
+    cls.pairs = sim_pairs(sz.pitch, maxM, tiles, pairTiles, ctx->smCount);
     for (int32_t l = 0; l < L; ++l) {
         prefix[l] = (int32_t)cls.upperTiles;
-        cls.upperTiles += sim_tiles(P.desc[(size_t)l].M, sim_pairs(sz.pitch, maxM));
+        cls.upperTiles += sim_tiles(P.desc[(size_t)l].M, cls.pairs);
         if (cls.upperTiles > 0x7fffffffLL) return fail(ctx, RCD_ERR_UNSUPPORTED, "too many similarity tiles");
         order[l] = l;
         sorted[l] = P.desc[(size_t)l].M;
@@ -617,11 +618,13 @@ rcd_status rcd_similarity(rcd_ctx *ctx, const void *X_dev, rcd_feat_dtype dtype,
     cls.L = (int32_t)batch;
     cls.maxM = M;
     cls.tilePrefixDev = nullptr;
-    cls.uniTiles = (int32_t)sim_tiles(M, sim_pairs(d * (int64_t)feat_bytes(dtype), M));
+    cls.pairs = sim_pairs(d * (int64_t)feat_bytes(dtype), M, batch * sim_tiles(M, false), batch * sim_tiles(M, true), ctx->smCount);
+    cls.uniTiles = (int32_t)sim_tiles(M, cls.pairs);
     cls.upperTiles = batch * (int64_t)cls.uniTiles;
     ctx->kernelLaunches = 0;
     ctx->tcLaunches = 0;
-    RCD_CUDA(ctx, status_begin(ctx, st));
+    ctx->statusDev = ctx->statusOwn;
+    cls.clearStatus = true;
     return launch_similarity(ctx, X_dev, dtype, M * batch, d, cls, S_dev, st);
 }
 

@@ -72,10 +72,13 @@ struct SimClasses {
     DescSource src;
     int32_t L;
     int64_t maxM;
-    // tensor-core kernel: 128 x 256 tiles that reach the diagonal or lie above it, listed class after class
+    // tensor-core kernels: tiles that reach the diagonal or lie above it, listed class after class
     const int32_t *tilePrefixDev;   // [L+1] first tile index of every class (null: equal classes)
     int32_t uniTiles;               // tiles per class when the classes are equal
     int64_t upperTiles;             // tiles in all
+    bool pairs;                     // tiles of 256 x 256 on pairs of SMs (see sim_pairs)
+    bool clearStatus;               // the launch is a call of its own: its first CTA clears the status word (a memset in front of a
+                                    // small call takes 2 us of 14)
 };
 
 // Pointers into the caller's workspace for one rcd_partition call.
@@ -169,19 +172,40 @@ inline int32_t pad4(int64_t m) { return (int32_t)((m + 3) / 4 * 4); }
 // the sweeps copy then pair up into whole sectors.
 inline int32_t pad_row(int64_t m) { return (int32_t)((m + 7) / 8 * 8); }
 
-// Classes of 129 to 1024 samples with rows of at least 1 KB: 256 x 256 tiles, a pair of SMs each.  Shorter rows are bound by
-// writing S, one block of rows leaves half a pair idle, and in larger classes drawn tiles of half the size share the work out
-// better (20 classes of 1300 x 1024 int8: 55 us, pairs 61; 50 of 1300 x 768 bf16: 130 either way).
-inline bool sim_pairs(int64_t rowBytes, int64_t maxM) { return rowBytes >= 1024 && maxM > 128 && maxM <= 1024; }
 // Tiles the tensor-core similarity kernels compute for a class of M samples: those that reach the diagonal or lie above it, of
-// 256 x 256, or of 128 rows x 256 columns (row block tm with the column blocks from tm / 2 on).
+// 256 x 256 (pairs), or of 128 rows x 256 columns (row block tm with the column blocks from tm / 2 on).
 inline int64_t sim_tiles(int64_t M, bool pairs)
 {
-    if (pairs) { const int64_t blocks = (M + 255) / 256; return blocks * (blocks + 1) / 2; }
     const int64_t rowBlocks = (M + 127) / 128, colBlocks = (M + 255) / 256;
+    if (pairs) return colBlocks * (colBlocks + 1) / 2;
     int64_t n = 0;
     for (int64_t tm = 0; tm < rowBlocks; ++tm) n += colBlocks - tm / 2;
     return n;
+}
+// Units of work on pairs of SMs: tiles, as long as they fill rounds of one per pair; those left over are cut into 2, 4 or 8
+// strips of columns, which share the last round out to more pairs (100 classes of 500 x 2048: 300 tiles on 74 pairs leave 4;
+// 85 -> 82 us).
+struct PairUnits { int whole, strips, count; };
+__host__ __device__ inline PairUnits pair_units(int tiles, int pairs)
+{
+    PairUnits u;
+    u.whole = tiles / pairs * pairs;
+    u.strips = 1;
+    while (u.strips < 8 && (tiles - u.whole) * u.strips * 2 <= pairs) u.strips *= 2;
+    u.count = u.whole + (tiles - u.whole) * u.strips;
+    return u;
+}
+// Whether pairs of SMs take a similarity launch: rows of at least 2 KB (40 classes of 1300 x 2048 bf16: 188 -> 170 us), or of
+// 1 KB in classes of up to 1024 samples; in larger classes of such rows drawn tiles of half the size share the work out better
+// (20 of 1300 x 1024 int8: 55 us, pairs 61), and below that writing S is the bound.  And where pairs need no more rounds, which
+// take the same time: a tile a round, 0.7 of one for tiles in two strips, 0.5 for more (10 of 1025 x 2048: 2 rounds, 43 us;
+// pairs 2.5 and 48).
+inline bool sim_pairs(int64_t rowBytes, int64_t maxM, int64_t tiles, int64_t pairTiles, int sms)
+{
+    if (sms < 2 || maxM <= 128 || pairTiles > 0x7fffffffLL || (rowBytes < 2048 && (rowBytes < 1024 || maxM > 1024))) return false;
+    const PairUnits u = pair_units((int)pairTiles, sms / 2);
+    const double last = u.count == u.whole ? 0.0 : u.strips == 1 ? 1.0 : u.strips == 2 ? 0.7 : 0.5;
+    return (double)(u.whole / (sms / 2)) + last <= (double)((tiles + sms - 1) / sms);
 }
 
 // Lays the workspace out at `base` (may be null to measure).  Returns total bytes.
@@ -198,6 +222,7 @@ struct rcd_ctx {
     std::string err;
     int32_t *hostStage = nullptr;       // pinned, counts / status read-back
     int32_t *statusOwn = nullptr;       // device status word for calls that take no workspace; from kFirstTicket on, tile tickets
+    unsigned simReady = 0;              // tensor-core similarity kernels whose shared memory has been asked for, a bit each
     unsigned simTurn = 0;               // similarity launches so far: each takes the next ticket
     size_t hostStageInts = 0;
     unsigned char *hostBlob = nullptr;  // pinned, what a call's host side hands to its kernels

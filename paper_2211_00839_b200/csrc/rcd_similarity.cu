@@ -162,6 +162,7 @@ rcd_status launch_similarity(rcd_ctx *ctx, const void *Xs, rcd_feat_dtype dtype,
         if (rs != RCD_OK) return rs;
         if (handled) return RCD_OK;
     }
+    if (cls.clearStatus) RCD_CUDA(ctx, cudaMemsetAsync(const_cast<int32_t *>(ctx->statusDev), 0, sizeof(int32_t), st));
     return launch_similarity_generic(ctx, Xs, dtype, d, cls, S, st);
 }
 

@@ -242,7 +242,7 @@ template <bool kInt8>
 __global__ void __launch_bounds__(kTcThreads, 1) sim_tc_kernel(const __grid_constant__ CUtensorMap map, DescSource src, int32_t L,
                                                               const int32_t *__restrict__ tilePrefix, int32_t uniTiles,
                                                               int32_t *ticket, int32_t totalTiles, int32_t numSlabs, uint32_t *__restrict__ S,
-                                                              int32_t *status)
+                                                              int32_t *status, bool clearStatus)
 {
     extern __shared__ unsigned char smemRaw[];
     // operand stages need 1024-byte alignment for the 128-byte swizzle pattern
@@ -251,6 +251,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) sim_tc_kernel(const __grid_cons
     __shared__ uint32_t stage32[kEpiWarps][32][33];             // per epilogue warp: one 32 x 32 block, padded
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (clearStatus && blockIdx.x == 0 && threadIdx.x == 0) *(volatile int32_t *)status = 0;    // (no wait runs out for a quarter of a second)
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], 1); }
@@ -463,19 +464,7 @@ __device__ __forceinline__ void cluster_barrier()
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
-// Unit -> class, row block of 256, first column and columns computed.  The units are the tiles (column blocks from the row
-// block on), as long as they fill rounds of one per pair; those left over are cut into 2, 4 or 8 strips of columns, which
-// share the last round out to more pairs (100 classes of 500 x 2048: 300 tiles on 74 pairs leave 4; 85 -> 82 us).
-struct PairUnits { int whole, strips, count; };
-__host__ __device__ inline PairUnits pair_units(int tiles, int pairs)
-{
-    PairUnits u;
-    u.whole = tiles / pairs * pairs;
-    u.strips = 1;
-    while (u.strips < 8 && (tiles - u.whole) * u.strips * 2 <= pairs) u.strips *= 2;
-    u.count = u.whole + (tiles - u.whole) * u.strips;
-    return u;
-}
+// Unit -> class, row block of 256, first column and columns computed; column blocks run from the row block on.
 struct PairTile { int l, tb, col, n; bool diag, shared; };      // diag: stored once; shared: A's rows are B's
 __device__ __forceinline__ PairTile decode_pair_tile(const DescSource &src, const int32_t *__restrict__ prefix, int L, int uniTiles,
                                                      const PairUnits &units, int unit)
@@ -513,7 +502,7 @@ __device__ __forceinline__ PairTile decode_pair_tile(const DescSource &src, cons
 template <bool kInt8>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) sim_pair_kernel(
     const __grid_constant__ CUtensorMap map, DescSource src, int32_t L, const int32_t *__restrict__ tilePrefix, int32_t uniTiles,
-    int32_t totalTiles, int32_t kernelPairs, int32_t numSlabs, uint32_t *__restrict__ S, int32_t *status)
+    int32_t totalTiles, int32_t kernelPairs, int32_t numSlabs, uint32_t *__restrict__ S, int32_t *status, bool clearStatus)
 {
     extern __shared__ unsigned char smemRaw[];
     unsigned char *tiles = reinterpret_cast<unsigned char *>(((uintptr_t)smemRaw + 1023) & ~(uintptr_t)1023);
@@ -521,6 +510,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) sim_p
     __shared__ uint32_t stage32[kEpiWarps][32][33];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (clearStatus && blockIdx.x == 0 && threadIdx.x == 0) *(volatile int32_t *)status = 0;    // (no wait runs out for a quarter of a second)
     const int rank = blockIdx.x & 1;                     // (clusters are consecutive pairs of blocks)
     const int firstUnit = blockIdx.x >> 1, pairs = gridDim.x >> 1;
     const PairUnits units = pair_units(totalTiles, kernelPairs);
@@ -671,34 +661,32 @@ rcd_status launch_similarity_tc(rcd_ctx *ctx, const void *Xs, rcd_feat_dtype dty
     const int totalTiles = (int)cls.upperTiles;
     const int grid = totalTiles < ctx->smCount ? totalTiles : ctx->smCount;
     int32_t *status = const_cast<int32_t *>(ctx->statusDev);
-    if (sim_pairs(rowBytes, cls.maxM)) {
+    const bool isInt8 = dtype == RCD_FEAT_I8;
+    // (shared memory beyond 48 KB is asked for once per context and kernel, not on every call)
+    auto allow = [&](auto *kernel, int bit, size_t bytes) {
+        if (ctx->simReady >> bit & 1) return cudaSuccess;
+        ctx->simReady |= 1 << bit;
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
+    if (cls.pairs) {
         const size_t pairSmem = (size_t)kPairStages * kPairStageBytes + 1024;
         const int pairs = std::max(1, ctx->smCount / 2);
         const int pairGrid = 2 * std::min(pairs, pair_units(totalTiles, pairs).count);
-        auto *kernel = dtype == RCD_FEAT_I8 ? sim_pair_kernel<true> : sim_pair_kernel<false>;
-        RCD_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pairSmem));
+        auto *kernel = isInt8 ? sim_pair_kernel<true> : sim_pair_kernel<false>;
+        RCD_CUDA(ctx, allow(kernel, isInt8 ? 3 : 2, pairSmem));
         kernel<<<pairGrid, kTcThreads, pairSmem, st>>>(map, cls.src, cls.L, cls.tilePrefixDev, cls.uniTiles, totalTiles, pairs,
-                                                        numSlabs, (uint32_t *)S, status);
-        ctx->kernelLaunches++;
-        ctx->tcLaunches++;
-        RCD_CUDA(ctx, cudaGetLastError());
-        *handled = true;
-        return RCD_OK;
-    }
-    // Tiles are drawn, since they are not equally long and an uneven share leaves most SMs idle at the end: 10 classes of
-    // 5000 x 256 int8 217 -> 177 us, 50 of 1300 x 192 bf16 112 -> 99, 100 of 500 x 512 bf16 47 -> 44.  Not so for short rows
-    // in classes of at most 8 tiles (500 samples: 6): every gridDim.x-th is as even then, and a CTA has to draw such tiles
-    // up to three ahead of their turn (200 of 257 x 256 int8: 29 -> 34 us).  A ticket of its own for every launch that can
-    // be under way at once: calls may overlap on several streams.
-    int32_t *ticket = totalTiles <= 8LL * cls.L && numSlabs < 8 ? nullptr : ctx->statusOwn + kFirstTicket + ctx->simTurn++ % (kStatusWords - kFirstTicket);
-    if (dtype == RCD_FEAT_I8) {
-        RCD_CUDA(ctx, cudaFuncSetAttribute(sim_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        sim_tc_kernel<true><<<grid, kTcThreads, smem, st>>>(map, cls.src, cls.L, cls.tilePrefixDev, cls.uniTiles, ticket, totalTiles,
-                                                           numSlabs, (uint32_t *)S, status);
+                                                       numSlabs, (uint32_t *)S, status, cls.clearStatus);
     } else {
-        RCD_CUDA(ctx, cudaFuncSetAttribute(sim_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        sim_tc_kernel<false><<<grid, kTcThreads, smem, st>>>(map, cls.src, cls.L, cls.tilePrefixDev, cls.uniTiles, ticket, totalTiles,
-                                                            numSlabs, (uint32_t *)S, status);
+        // Tiles are drawn, since they are not equally long and an uneven share leaves most SMs idle at the end: 10 classes of
+        // 5000 x 256 int8 217 -> 177 us, 50 of 1300 x 192 bf16 112 -> 99, 100 of 500 x 512 bf16 47 -> 44.  Not so for short
+        // rows in classes of at most 8 tiles (500 samples: 6): every gridDim.x-th is as even then, and a CTA has to draw such
+        // tiles up to three ahead of their turn (200 of 257 x 256 int8: 29 -> 34 us).  A ticket of its own for every launch
+        // that can be under way at once: calls may overlap on several streams.
+        int32_t *ticket = totalTiles <= 8LL * cls.L && numSlabs < 8 ? nullptr : ctx->statusOwn + kFirstTicket + ctx->simTurn++ % (kStatusWords - kFirstTicket);
+        auto *kernel = isInt8 ? sim_tc_kernel<true> : sim_tc_kernel<false>;
+        RCD_CUDA(ctx, allow(kernel, isInt8 ? 1 : 0, smem));
+        kernel<<<grid, kTcThreads, smem, st>>>(map, cls.src, cls.L, cls.tilePrefixDev, cls.uniTiles, ticket, totalTiles,
+                                               numSlabs, (uint32_t *)S, status, cls.clearStatus);
     }
     ctx->kernelLaunches++;
     ctx->tcLaunches++;
