@@ -77,7 +77,8 @@ typedef struct {
     int32_t sweep_batch_max;   /* blocks whose gains one pass over S may refresh: 1,2,4 or 8; 0 = default (8) */
     int32_t similarity_path;   /* 0 = tensor-core kernel when the shape allows, 2 = always the generic kernel */
     int32_t profile;           /* 0 off; 1 time the phases of rcd_partition; 2 also time every sweep launch */
-    int32_t greedy_path;       /* form of the greedy loop.  0 = choose: asynchronous classes (3) when there are at most a quarter
+    int32_t greedy_path;       /* form of the greedy loop.  0 = choose: one thread-block cluster per class (at most 128 blocks,
+                                  none of the options below set), else asynchronous classes (3) when there are at most a quarter
                                   as many classes as SMs, else one CTA per class (4);  1 = two launches per round (always
                                   used with profile 2);  2 = one cooperative launch, rounds of a sweep phase and a pick phase
                                   separated by grid barriers;  3 = one cooperative launch, every class cycles between sweep and
