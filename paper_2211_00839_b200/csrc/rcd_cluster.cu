@@ -1134,8 +1134,12 @@ __global__ void __launch_bounds__((P == 0 ? kMaxWarps + 1 + kListers : team_warp
     const int W = prm.W;
     uint32_t parities = 0;
     const NoteLayout layout{T, P == 0};
-    uint32_t classes = 0;                                  // this cluster has begun
+    uint32_t classes = 0;                                  // this cluster has drawn (classes left in floating point and empty ones too)
 
+    // (for the listing warps: the number of the class that has ended last, 0 at first, then per block the command told last)
+    volatile uint32_t *const ended = reinterpret_cast<uint32_t *>(shared + prm.offTold);
+    volatile uint32_t *const told0 = ended + 4;
+    if (P == 0 && threadIdx.x == 0) *ended = 0;
     if (rank == 0)
         for (int p = threadIdx.x; p < W; p += blockDim.x) bar_init(base + prm.offBars + p * 8, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1173,12 +1177,8 @@ __global__ void __launch_bounds__((P == 0 ? kMaxWarps + 1 + kListers : team_warp
         for (int i = threadIdx.x; i < (c.ld + 31) / 32; i += blockDim.x)
             bits[i] = 32 * i + 32 <= c.M ? 0u : (32 * i >= c.M ? ~0u : ~0u << (c.M - 32 * i));
         for (int i = threadIdx.x; i < nTeams * prm.ring; i += blockDim.x) cmds[i] = 0;
-        // (for the listing warps: the number of the class that has ended last, then per block the command told last)
-        volatile uint32_t *ended = reinterpret_cast<uint32_t *>(shared + prm.offTold);
-        volatile uint32_t *told0 = ended + 4;
         if (P == 0)
             for (int i = threadIdx.x; i < prm.slots; i += blockDim.x) told0[i] = 0;
-        if (P == 0 && threadIdx.x == 0 && classes == 1) *ended = 0;
         if (P == 0 && rank == 0) {
             for (int i = threadIdx.x; i < (int)C * nTeams; i += blockDim.x) reinterpret_cast<uint32_t *>(shared + prm.offQueue)[i] = 0;
             for (int i = threadIdx.x; i < W * layout.words(); i += blockDim.x) reinterpret_cast<unsigned long long *>(shared + prm.offNotes)[i] = 0;

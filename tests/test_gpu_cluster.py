@@ -74,6 +74,22 @@ def test_float_norms_far_apart(rcd, orc):
     check_float(rcd, orc, wl)
 
 
+@pytest.mark.parametrize("sizes,W,apart", [([800, 500, 300], 100, 1), ([140] * 12 + [130] * 148, 33, 12)])
+def test_float_norms_far_apart_with_lists(rcd, orc, sizes, W, apart):
+    """The largest classes, which clusters draw first, stay in floating point; the next ones use lists of candidates (several
+    blocks per team).  Twice on one context: shared memory then holds what the first call left."""
+    import torch
+    M0 = sizes[apart - 1]
+    wl = workload(sizes, 32, W, W, dtype="bf16", scale=lambda rng, M: 10.0 ** rng.uniform(-1.5 if M == M0 else 0.0, 1.5 if M == M0 else 0.1, M))
+    X, y = rcd.features_to_torch(wl.features, device="cuda"), torch.from_numpy(wl.labels).cuda()
+    with rcd.Context(0) as ctx:
+        first = [t.clone() for t in ctx.rcd_partition(X, y, wl.capacities, wl.L)]
+        again = ctx.rcd_partition(X, y, wl.capacities, wl.L)
+        ctx.sync_status()
+    assert all(torch.equal(a, b) for a, b in zip(first, again))
+    check_float(rcd, orc, wl)
+
+
 @pytest.mark.parametrize("sizes,W", [([400, 3], 5), ([600] * 4, 24), ([90] * 150, 20)])
 def test_graph_cut_int8_exact(rcd, orc, sizes, W):
     wl = workload(sizes, 48, W, W)
