@@ -131,16 +131,30 @@ __device__ __forceinline__ unsigned long long ld_relaxed(uint32_t addr)      // 
     asm volatile("ld.volatile.shared::cta.u64 %0, [%1];" : "=l"(v) : "r"(addr) : "memory");
     return v;
 }
-__device__ __forceinline__ void cluster_fence() { asm volatile("fence.acq_rel.cluster;" ::: "memory"); }
+// What the thread reads from the cluster's shared memory after this is not read before it.  Only that: a fence of both
+// directions waits for the thread's own stores to other CTAs, and an acquire at cluster scope without the restriction drops the
+// SM's L1 lines, which hold rows that several teams read (1000 classes of 1300 into 64 blocks: lists of candidates read with
+// ld.acquire 166.8 ms, with this fence 165.0; 10 of 5000 with the graph cut, whose teams are told to look again often: their
+// fence of both directions 9.58 ms, this one 8.84).
+__device__ __forceinline__ void shared_acquire_fence() { asm volatile("fence.acquire.sync_restrict::shared::cluster.cluster;" ::: "memory"); }
+__device__ __forceinline__ uint32_t ld_acquire_block(uint32_t addr)          // (own shared memory, written by this CTA)
+{
+    uint32_t v;
+    asm volatile("ld.acquire.cta.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+}
+// What the thread has written, or seen written, comes before what it writes after this.
+__device__ __forceinline__ void release_fence() { asm volatile("fence.release.cluster;" ::: "memory"); }
 __device__ __forceinline__ void bar_init(uint32_t bar, uint32_t count) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(bar), "r"(count) : "memory"); }
 __device__ __forceinline__ void bar_expect(uint32_t bar, uint32_t bytes)
 {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(bar), "r"(bytes) : "memory");
 }
+// (orders nothing by itself)
 __device__ __forceinline__ bool bar_done(uint32_t bar, uint32_t parity)
 {
     uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
                  : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
@@ -631,7 +645,7 @@ __device__ __forceinline__ void team_of_one(const ClusterParams &prm, const Clas
         const uint32_t what = (uint32_t)cmd;
         if (what == kStopCmd) break;
         if (what == kScanCmd) {
-            cluster_fence();
+            shared_acquire_fence();
             dirty = true;
             continue;
         }
@@ -732,7 +746,7 @@ struct Listed {
 // another one -- and then it does not use lists of the earlier one any more, so a scan that ran into the next update
 // does no harm.
 template <typename Slot>
-__device__ void list_candidates(const ClusterParams &prm, const uint32_t *bits, int ld4, int shift, const volatile uint32_t *serials, Listed *listed, int first,
+__device__ void list_candidates(const ClusterParams &prm, const uint32_t *bits, int ld4, int shift, uint32_t serials, Listed *listed, int first,
                                 int step, int slots, const volatile uint32_t *ended, uint32_t turn, Slot where)
 {
     const int lane = threadIdx.x & 31;
@@ -743,7 +757,7 @@ __device__ void list_candidates(const ClusterParams &prm, const uint32_t *bits, 
     for (unsigned spin = 0; spin < kPollLimit; ++spin) {
         if (*ended == turn) break;
         // a block told anew comes first; else a look at one block's list
-        const uint32_t now = lane < mine ? serials[first + lane * step] : 0u;
+        const uint32_t now = lane < mine ? ld_acquire_block(serials + (first + lane * step) * 4) : 0u;
         const unsigned m = __ballot_sync(0xffffffffu, now != had && now != 0);
         const bool fresh = m != 0;
         if (!fresh) turnOf = turnOf + 1 < mine ? turnOf + 1 : 0;
@@ -751,6 +765,7 @@ __device__ void list_candidates(const ClusterParams &prm, const uint32_t *bits, 
         const int slot = first + i * step;
         const uint32_t serial = __shfl_sync(0xffffffffu, now, i);
         if (mine == 0 || serial == 0) { __nanosleep(200); continue; }
+        __syncwarp();                                      // (what the lane that read the serial sees, the warp sees)
         Listed &li = listed[slot];
         {
             if (!fresh) {
@@ -796,13 +811,15 @@ __device__ void list_candidates(const ClusterParams &prm, const uint32_t *bits, 
             li.sample[lane] = (uint16_t)ev;
             li.sample[32 + lane] = (uint16_t)fv;
             if (lane == 0) li.bound = o;
-            cluster_fence();                               // (the list that was there is withdrawn)
+            // the list that was there is withdrawn before any word of the new one is written, and the new one complete
+            // before its tag: the barrier hands every lane what the others stored, the fence after it orders that
             __syncwarp();
+            release_fence();
             st_remote(listAddr + (uint32_t)lane * 8, e ? key_of(e, low_part(gains[ev], shift, ev), shift) : 0ull);
             st_remote(listAddr + (uint32_t)(32 + lane) * 8, f ? key_of(f, low_part(gains[fv], shift, fv), shift) : 0ull);
             if (lane == 0) st_remote(listAddr + (uint32_t)NoteLayout::kList * 8, o ? key_of(o, ((1u << shift) - 1u) << 16 | 0xffffu, shift) : 0ull);
-            cluster_fence();
             __syncwarp();
+            release_fence();
             if (lane == i) st_remote(listAddr + (uint32_t)(NoteLayout::kList + 1) * 8, (unsigned long long)serial << 16 | (lists & 0xffffu));
             __syncwarp();
         }
@@ -832,6 +849,7 @@ __device__ __forceinline__ void team_of_many(const ClusterParams &prm, int l, co
             if (t.warpIn == 0) top = warp_max_u64(lane < T ? t.tm->best[lane] : 0ull);
         }
         if (lane == i) ++serial;
+        // (the whole team's gains are written: a barrier lies between them and here, in front of this call or above)
         if (t.warpIn == 0 && lane == i) {
             st_async(noteAddr, top, barAddr);
             __threadfence_block();
@@ -869,7 +887,7 @@ __device__ __forceinline__ void team_of_many(const ClusterParams &prm, int l, co
         if (what == kStopCmd) break;
         where(i, cov, gains, noteAddr, barAddr, told);
         if (what == kScanCmd) {
-            cluster_fence();
+            shared_acquire_fence();
             tell(i);
             continue;
         }
@@ -923,7 +941,7 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
     const uint32_t myBits = remote(base + prm.offBits, (uint32_t)lane < C ? lane : 0);
     volatile const unsigned long long *notes = reinterpret_cast<const unsigned long long *>(shared + prm.offNotes);
     volatile const unsigned long long *firsts = reinterpret_cast<const unsigned long long *>(shared + prm.offFirsts);
-    const uint32_t bars = base + prm.offBars;
+    const uint32_t bars = base + prm.offBars, notesAt = base + prm.offNotes;
     unsigned long long f[KW];              // (value + kZeroValue) << 7 | block
     int room[KW];
     uint32_t given[KW];                    // commands given to the block
@@ -989,7 +1007,10 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
             unsigned spin = 0;
             while (!bar_done(bars + j * 8, parity ? 1u : 0u) && ++spin < kPollLimit) { }
             parity ^= kParity;
-            if (spin < kPollLimit) return true;
+            if (spin < kPollLimit) {
+                shared_acquire_fence();                    // (the note)
+                return true;
+            }
             if (lane == 0) atomicOr(prm.status, kDevTimeout);
             return false;
         };
@@ -1031,12 +1052,17 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
                 }
                 if (kMany && serial > 0 && best == 0) {
                     // the list, and its next edition when all that are sure to lead in this one have been taken
-                    volatile const unsigned long long *list = note + layout.list();
+                    // (Tag, words, tag: the first fence keeps the words behind the tag, and with the second a word of the next
+                    // edition comes with the withdrawal of this one.)
+                    const uint32_t list = notesAt + (uint32_t)(j * layout.words() + layout.list()) * 8;
                     unsigned spin = 0, spent = 0;
                     while (best == 0 && ++spin < kPollLimit) {
-                        const unsigned long long tag = list[NoteLayout::kList + 1];
-                        const unsigned long long k = list[lane], k2 = list[32 + lane], bound = list[NoteLayout::kList];
-                        const unsigned long long again = list[NoteLayout::kList + 1];
+                        const unsigned long long tag = ld_relaxed(list + (NoteLayout::kList + 1) * 8);
+                        shared_acquire_fence();
+                        const unsigned long long k = ld_relaxed(list + (uint32_t)lane * 8), k2 = ld_relaxed(list + (uint32_t)(32 + lane) * 8);
+                        const unsigned long long bound = ld_relaxed(list + NoteLayout::kList * 8);
+                        shared_acquire_fence();
+                        const unsigned long long again = ld_relaxed(list + (NoteLayout::kList + 1) * 8);
                         if (!__all_sync(0xffffffffu, tag == again && (uint32_t)(tag >> 16) == serial && (tag & 0xffffu) == (__shfl_sync(0xffffffffu, (uint32_t)tag, 0) & 0xffffu))) continue;
                         const int s = key_sample(k), s2 = key_sample(k2);
                         const bool free = k != 0 && !(bits[s >> 5] >> (s & 31) & 1), free2 = k2 != 0 && !(bits[s2 >> 5] >> (s2 & 31) & 1);
@@ -1055,7 +1081,7 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
                 if (best) break;
                 // every candidate that is sure to lead has been taken by other blocks: the team looks again
                 ++rescans;
-                cluster_fence();                           // (it must see which samples are taken)
+                release_fence();                           // (it must see which samples are taken)
                 if (lane == jl) {
                     bar_expect(bars + j * 8, noteBytes);
                     command(jk, kScanCmd);
@@ -1215,7 +1241,7 @@ __global__ void __launch_bounds__((P == 0 ? kMaxWarps + 1 + kListers : team_warp
         if (warp == NW) {
             if (rank == 0) lead<KW, P == 0>(prm, l, c, shared, C, T, bias, classes, parities);
         } else if (warp > NW) {
-            list_candidates(prm, bits, ld4, shift, told0, reinterpret_cast<Listed *>(shared + prm.offListed), warp - NW - 1, kListers, prm.slots, ended, classes, [&](int slot, const unsigned long long *&gains) {
+            list_candidates(prm, bits, ld4, shift, smem32((const void *)told0), reinterpret_cast<Listed *>(shared + prm.offListed), warp - NW - 1, kListers, prm.slots, ended, classes, [&](int slot, const unsigned long long *&gains) {
                 const int j = slot * (int)C + (int)rank;
                 if (kSmemState) gains = reinterpret_cast<const unsigned long long *>(shared + prm.offGains) + (size_t)slot * prm.maxLd;
                 else gains = reinterpret_cast<const unsigned long long *>(prm.gains + c.vOff) + (size_t)j * c.ld;

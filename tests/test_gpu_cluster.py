@@ -63,6 +63,23 @@ def test_int8_ties_exact(rcd, orc, W):
     check_exact(rcd, orc, workload([600, 90], 32, W, W, copies=80))
 
 
+@pytest.mark.parametrize("sizes,W", [([130] * 160, 33), ([900] * 9, 100), ([300] * 40, 128)])
+def test_lists_under_contention(rcd, sizes, W):
+    """Many blocks that compete for the same samples: teams of one, two and eight warps hand stored gains to the listing warps,
+    and those hand lists to the leader, thousands of times over.  Results do not depend on the timing of any of it: twenty calls
+    give the first one's, which is the pass-based form's."""
+    import torch
+    wl = workload(sizes, 24, W, W, copies=16)
+    X, y = rcd.features_to_torch(wl.features, device="cuda"), torch.from_numpy(wl.labels).cuda()
+    with rcd.Context(0) as ctx:
+        first = [t.clone() for t in ctx.rcd_partition(X, y, wl.capacities, wl.L)]
+        for _ in range(20):
+            assert all(torch.equal(a, b) for a, b in zip(first, ctx.rcd_partition(X, y, wl.capacities, wl.L)))
+        ctx.sync_status()
+    for got, want in zip(first, run_partition(rcd, wl, greedy_path=4)):
+        assert np.array_equal(got.cpu().numpy(), want)
+
+
 @pytest.mark.parametrize("sizes,W", [([257, 31], 4), ([800] * 3, 24)])
 def test_float(rcd, orc, sizes, W):
     check_float(rcd, orc, workload(sizes, 96, W, W, dtype="bf16"))
