@@ -120,14 +120,14 @@ size_t layout_workspace(void *base, rcd_feat_dtype dtype, const Sizes &sz, Works
     w.rowCtr = c.take<int32_t>(L);
     w.sweepList = c.take<int32_t>(3 * L);
     w.sync = c.take<ClassSync>(L);
-    w.tickets = c.take<int32_t>(N + L);
+    w.tickets = c.take<int32_t>(2 * N + L);
     w.sweepF = c.take<long long>(L * 8);
     w.floorv = c.take<unsigned char>(L * kLazyBlocks * 8);
     w.theta = c.take<unsigned char>(L * kLazyBlocks * 8);
     w.sweepTheta = c.take<unsigned char>(L * kLazyBlocks * 8);
     w.lazyStat = c.take<int32_t>(L * 4);
-    w.stepBytes = c.take<unsigned long long>((size_t)sz.maxM + 1);
-    w.stepOps = c.take<unsigned long long>((size_t)sz.maxM + 1);
+    w.stepBytes = c.take<unsigned long long>(2 * (size_t)sz.maxM + 1);
+    w.stepOps = c.take<unsigned long long>(2 * (size_t)sz.maxM + 1);
     w.g0 = c.take<long long>(N);
     w.fixedExp = c.take<int32_t>(L);
     w.bytes = align_up(c.off);
@@ -487,11 +487,11 @@ rcd_status rcd_get_profile(rcd_ctx *ctx, rcd_profile *out)
         out->async_visits = (int64_t)(ns[7] & 0xffffffffull);
         out->async_attempts = (int64_t)(ns[7] >> 32);
     }
-    if (ctx->stepBytesDev && ctx->steps > 0) {
-        std::vector<unsigned long long> bytes((size_t)ctx->steps + 1), ops((size_t)ctx->steps + 1);
+    if (ctx->stepBytesDev && ctx->passes > 0) {
+        std::vector<unsigned long long> bytes((size_t)ctx->passes + 1), ops((size_t)ctx->passes + 1);
         RCD_CUDA(ctx, cudaMemcpy(bytes.data(), ctx->stepBytesDev, bytes.size() * sizeof(unsigned long long), cudaMemcpyDeviceToHost));
         RCD_CUDA(ctx, cudaMemcpy(ops.data(), ctx->stepOpsDev, ops.size() * sizeof(unsigned long long), cudaMemcpyDeviceToHost));
-        for (int64_t t = 0; t < ctx->steps; ++t) {
+        for (int64_t t = 0; t < ctx->passes; ++t) {
             if (bytes[(size_t)t] == 0) continue;
             out->sweep_bytes += (int64_t)bytes[(size_t)t];
             out->sweep_elem_ops += (int64_t)ops[(size_t)t];
@@ -699,6 +699,7 @@ rcd_status rcd_partition(rcd_ctx *ctx, const void *features_dev, rcd_feat_dtype 
     ctx->kernelLaunches = 0;
     ctx->tcLaunches = 0;
     ctx->steps = 0;
+    ctx->passes = 0;
     ctx->phaseValid = false;
     ctx->stepBytesDev = nullptr;
     ctx->stepOpsDev = nullptr;

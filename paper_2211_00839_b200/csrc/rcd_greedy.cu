@@ -88,7 +88,7 @@ struct GreedyParams {
     int32_t sparseMinMembers;   // threshold passes start once every out-of-date block has this many members (<0: never)
     // asynchronous kernel (greedy_async_kernel); asyncMode = 0 everywhere else
     ClassSync *sync;            // [L] hand-off words
-    int32_t *tickets;           // [N + L] ticket counter of sweep k of class l at tickets[row0_l + l + k]
+    int32_t *tickets;           // [2N + L] ticket counter of sweep k of class l: see ticket_of
     long long *sweepF;          // [L][kMaxSweepBatch] int8 features: f of the blocks a dense pass refreshes
     int32_t asyncMode;
     int32_t nPick;              // CTAs [0, nPick) make picks, the others sweep
@@ -110,6 +110,15 @@ struct GreedyParams {
     int32_t minM;               // smallest non-empty class
     int32_t nonEmpty;           // classes that hold at least one sample
 };
+
+// A class of M samples makes M picks, each after at most two passes of its own: one, and where that one skipped rows and the
+// pick found a gain below its floor (a miss), one over every row.  Passes are numbered from 0, so the last has a number below 2M.
+__host__ __device__ inline int64_t passes_of(int64_t M) { return 2 * M; }
+template <typename SV>
+__device__ __forceinline__ int32_t *ticket_of(const GreedyParams<SV> &prm, const ClassDesc &c, int l, int k)
+{
+    return prm.tickets + passes_of(c.row0) + l + k;
+}
 
 __host__ __device__ inline int rows_per_group(int P) { return P == 8 ? 4 : 8; }
 
@@ -2176,7 +2185,7 @@ __device__ __forceinline__ void async_sweep_cta(const GreedyParams<SV> &prm, int
         for (int l = threadIdx.x; l < prm.L; l += blockDim.x) {
             const int4 a = ld_volatile16(&prm.sync[l]);             // epoch, nGroups, done, seq
             const int4 b = ld_volatile16(&prm.sync[l].pad_[0]);     // -, -, nR, cfg
-            const int drawn = (a.x & 1) ? 0 : ld_volatile32(prm.tickets + prm.desc[l].row0 + l + (a.x >> 1));
+            const int drawn = (a.x & 1) ? 0 : ld_volatile32(ticket_of(prm, prm.desc[l], l, a.x >> 1));
             if (!(a.x & 1) && drawn < a.y) {
                 int dist = l - home;
                 if (dist < 0) dist += prm.L;
@@ -2247,7 +2256,7 @@ __device__ __forceinline__ void async_sweep_cta(const GreedyParams<SV> &prm, int
         if (threadIdx.x == 0) {
             const int e1 = shInfo[9];
             const int teams = (kSweepThreads / 32) / (mode ? 1 : CS);
-            const int first = atomicAdd(prm.tickets + c.row0 + l + (e1 >> 1), teams);
+            const int first = atomicAdd(ticket_of(prm, c, l, e1 >> 1), teams);
             const int e2 = ld_acquire32(&prm.sync[l].epoch);
             shInfo[0] = (e1 == e2 && !(e1 & 1) && first < shInfo[6]) ? 1 : 0;
             if (clocked) shClk[2] += 1ull << 32;                   // attempts (high half), visits (low half)
@@ -2276,7 +2285,7 @@ __device__ __forceinline__ void async_sweep_cta(const GreedyParams<SV> &prm, int
             shClk[2] += 1;
         }
         const int nR = shInfo[2], first = shInfo[1];
-        int32_t *ticket = prm.tickets + c.row0 + l + shInfo[8];      // the counter of this sweep alone
+        int32_t *ticket = ticket_of(prm, c, l, shInfo[8]);      // the counter of this sweep alone
         int32_t *done = &prm.sync[l].done;
         if (mode) {
             P = shInfo[3];
@@ -2341,7 +2350,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1) greedy_owner_kernel(const __
             init_class(prm, l, *reinterpret_cast<PlanShared<typename Arith<SV>::FV> *>(shCover));
             __syncthreads();
         }
-        for (int round = 0; round <= prm.desc[l].M; ++round) {
+        for (int round = 0; round < passes_of(prm.desc[l].M); ++round) {
             if (*(volatile int32_t *)prm.status != 0) break;
             unsigned long long t0 = 0;
             if (blockIdx.x == 0 && threadIdx.x == 0) t0 = global_ns();
@@ -2538,12 +2547,12 @@ static rcd_status run_greedy(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws,
         RCD_CUDA(ctx, cudaGetLastError());
         return RCD_OK;
     }
-    if (path == 3) RCD_CUDA(ctx, cudaMemsetAsync(ws.tickets, 0, (size_t)(sz.N + sz.L) * sizeof(int32_t), st));
+    if (path == 3) RCD_CUDA(ctx, cudaMemsetAsync(ws.tickets, 0, (size_t)(passes_of(sz.N) + sz.L) * sizeof(int32_t), st));
     RCD_CUDA(ctx, cudaMemsetAsync(ws.nSweep, 0, 4 * sizeof(int32_t), st));
     RCD_CUDA(ctx, cudaMemsetAsync(ws.phaseNs, 0, kPhaseWords * sizeof(unsigned long long), st));
     ctx->phaseNsDev = ws.phaseNs;
-    RCD_CUDA(ctx, cudaMemsetAsync(ws.stepBytes, 0, (size_t)(sz.maxM + 1) * sizeof(unsigned long long), st));
-    RCD_CUDA(ctx, cudaMemsetAsync(ws.stepOps, 0, (size_t)(sz.maxM + 1) * sizeof(unsigned long long), st));
+    RCD_CUDA(ctx, cudaMemsetAsync(ws.stepBytes, 0, (size_t)(passes_of(sz.maxM) + 1) * sizeof(unsigned long long), st));
+    RCD_CUDA(ctx, cudaMemsetAsync(ws.stepOps, 0, (size_t)(passes_of(sz.maxM) + 1) * sizeof(unsigned long long), st));
     init_kernel<SV><<<sz.L, kSelectThreads, 0, st>>>(prm);
     ctx->kernelLaunches++;
     RCD_CUDA(ctx, cudaGetLastError());
@@ -2552,6 +2561,7 @@ static rcd_status run_greedy(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws,
     // One cooperative launch for the whole loop when the device can hold one sweep CTA per SM at once;
     // per-sweep event timing (profile 2) needs the sweeps as separate launches.
     const bool persistent = path != 1;
+    const int64_t rounds = prm.lazyFrom >= 0 ? passes_of(sz.maxM) : sz.maxM;
     if (path == 4) {
         // (an ordinary launch: the CTAs never wait for one another)
         greedy_owner_kernel<SV><<<std::min<int>(ctx->smCount, sz.L), kSweepThreads, (size_t)smem, st>>>(prm);
@@ -2562,20 +2572,20 @@ static rcd_status run_greedy(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws,
                                                   args, (size_t)smem, st));
         ctx->kernelLaunches += 1;
     } else if (persistent) {
-        int steps = (int)sz.maxM;
+        int steps = (int)passes_of(sz.maxM);                     // (the loop leaves as soon as every class is finished)
         void *args[] = {(void *)&prm, (void *)&steps};
         RCD_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)greedy_persistent_kernel<SV>, dim3(ctx->smCount), dim3(kSweepThreads),
                                                   args, (size_t)smem, st));
         ctx->kernelLaunches += 1;
     } else {
         if (perSweep) {
-            while ((int64_t)ctx->evSweep.size() < 2 * sz.maxM) {
+            while ((int64_t)ctx->evSweep.size() < 2 * rounds) {
                 cudaEvent_t e;
                 RCD_CUDA(ctx, cudaEventCreate(&e));
                 ctx->evSweep.push_back(e);
             }
         }
-        for (int64_t t = 0; t < sz.maxM; ++t) {
+        for (int64_t t = 0; t < rounds; ++t) {
             if (perSweep) RCD_CUDA(ctx, cudaEventRecord(ctx->evSweep[2 * t], st));
             RCD_CUDA(ctx, launch_pdl(sweep_kernel<SV>, dim3(ctx->smCount), dim3(kSweepThreads), (size_t)smem, st, prm, (int)t));
             if (perSweep) RCD_CUDA(ctx, cudaEventRecord(ctx->evSweep[2 * t + 1], st));
@@ -2583,9 +2593,10 @@ static rcd_status run_greedy(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws,
             ctx->kernelLaunches += 2;
         }
     }
-    if (perSweep) ctx->sweepEventsUsed = 2 * sz.maxM;
+    if (perSweep) ctx->sweepEventsUsed = 2 * rounds;
     RCD_CUDA(ctx, cudaGetLastError());
     ctx->steps = sz.maxM;
+    ctx->passes = rounds;
     ctx->stepBytesDev = ws.stepBytes;
     ctx->stepOpsDev = ws.stepOps;
     return RCD_OK;

@@ -119,7 +119,7 @@ struct Workspace {
     int32_t *sweepCS;       // [L] warps per row group in the next sweep
     int32_t *rowCtr;        // [L] ticket counter over row groups of the running sweep
     ClassSync *sync;        // [L] asynchronous kernel: hand-off words
-    int32_t *tickets;       // [N + L] asynchronous kernel: one ticket counter per (class, sweep number), never reused
+    int32_t *tickets;       // [2N + L] asynchronous kernel: one ticket counter per (class, sweep number), never reused
     int32_t *sizesSorted;   // [L] class sizes, ascending
     int32_t *classOrder;    // [L] classes by descending size
     void *floorv;           // [L][kLazyBlocks] per block: every stored gain at or above it is exact (int64 / double)
@@ -129,8 +129,8 @@ struct Workspace {
     long long *sweepF;      // [L][8] asynchronous kernel, int8 features: f of the first blocks in the sweep's list
     int32_t *sweepList;     // [3][L] classes that sweep in a step (three lists in rotation)
     int32_t *nSweep;        // [3] (+1 pad)
-    unsigned long long *stepBytes;   // [steps+1] bytes the sweep of step t has to read
-    unsigned long long *stepOps;     // [steps+1] element x block pairs of that sweep
+    unsigned long long *stepBytes;   // [2 maxM + 1] bytes the sweep of step t has to read
+    unsigned long long *stepOps;     // [2 maxM + 1] element x block pairs of that sweep
     unsigned long long *phaseNs;     // [6] sweep-/pick-phase ns of the persistent kernel, barrier counter, threshold-pass hits / elements / max blocks
     long long *g0;          // [N] cluster form: gain of every sample for an empty block
     int32_t *fixedExp;      // [L] cluster form, floating-point similarities: S holds round(sim * 2^fixedExp), or kNotFixed
@@ -237,6 +237,7 @@ struct rcd_ctx {
     int64_t kernelLaunches = 0;
     int64_t tcLaunches = 0;
     int64_t steps = 0;
+    int64_t passes = 0;                 // entries of stepBytes / stepOps that count
     const unsigned long long *stepBytesDev = nullptr;
     const unsigned long long *stepOpsDev = nullptr;
     const unsigned long long *phaseNsDev = nullptr;

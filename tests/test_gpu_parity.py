@@ -460,6 +460,18 @@ def test_lazy_evaluation_many_blocks_and_ragged_classes_exact(rcd, orc, lazy_fro
         check_exact(rcd, orc, wl, greedy_path=path, lazy_mode=1, lazy_from=lazy_from, incremental=2)
 
 
+@pytest.mark.parametrize("path", [1, 2, 3, 4])
+def test_lazy_evaluation_more_passes_than_picks_exact(rcd, orc, path):
+    """With one block every pick needs a pass, and a miss one more: the passes of a class outnumber its picks."""
+    from paper_2211_00839_b200.workloads import make_workload
+    wl = make_workload("C2", L=2, M=2000, d=64)
+    wl.capacities, wl.W = wl.capacities[:1], 1
+    ref = orc.partition(wl.features, wl.labels, wl.capacities, wl.L, variant="incremental")
+    a, o, v, prof = run_with_profile(rcd, wl, greedy_path=path, lazy_mode=1, lazy_from=1, incremental=2)
+    assert prof["lazy_misses"] > 0 and prof["sweep_launches"] > 2000
+    assert np.array_equal(a, ref.assignment) and np.array_equal(o, ref.order) and np.array_equal(v, ref.part_values)
+
+
 def test_lazy_evaluation_float(rcd, orc):
     from paper_2211_00839_b200.workloads import make_workload
     wl = make_workload("C3", L=2, M=900, d=512)
