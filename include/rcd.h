@@ -220,7 +220,9 @@ RCD_API rcd_status rcd_partition_workspace_bytes(rcd_ctx *ctx, rcd_feat_dtype dt
  *   part_values_dev_or_null [L][W] tracked f(A_j^l): int64 (I8 with RCD_SIM_DOT), else double
  * workspace_dev: 256-byte aligned, at least rcd_partition_workspace_bytes.
  * The call blocks once, briefly, on `cuda_stream` to read the L class sizes back (they fix the
- * launch shapes); everything after that is only enqueued.  Per class and per pick it runs:
+ * launch shapes).  With RCD_FEAT_BF16, RCD_SIM_DOT and facility location it blocks a second time, until the
+ * similarities are written (classes whose norms lie far apart take a launch of their own).  Everything
+ * else is only enqueued.  Per class and per pick it runs:
  * choose the non-full block of least f; (re)compute the marginal gains
  * sum_i max(0, S[v][i] - cover_p[i]) of every unassigned v for that block, and in the same
  * pass over S for other non-full blocks whose stored gains are out of date (a block's gains

@@ -82,8 +82,8 @@ size_t layout_workspace(void *base, rcd_feat_dtype dtype, const Sizes &sz, Works
     w.status = c.take<int32_t>(4);
     w.counter = c.take<int32_t>(4);
     w.phaseNs = c.take<unsigned long long>(kPhaseWords);   // phase clocks, the grid-barrier counter, threshold-pass and row-skipping counters
-    w.counts = c.take<int32_t>(L);
     w.nSweep = c.take<int32_t>(4);
+    w.counts = c.take<int32_t>(L);
     // what the host computes from the class sizes, copied in one piece
     w.desc = c.take<ClassDesc>(L);
     w.tilePrefix = c.take<int32_t>(L + 1);
@@ -130,6 +130,7 @@ size_t layout_workspace(void *base, rcd_feat_dtype dtype, const Sizes &sz, Works
     w.stepOps = c.take<unsigned long long>(2 * (size_t)sz.maxM + 1);
     w.g0 = c.take<long long>(N);
     w.fixedExp = c.take<int32_t>(L);
+    w.sizesLeft = c.take<int32_t>(L);
     w.bytes = align_up(c.off);
     if (ws) *ws = w;
     return w.bytes;
@@ -398,7 +399,7 @@ rcd_status rcd_create(rcd_ctx **out, int cuda_device, const rcd_config *cfg)
     ctx->cooperative = prop.cooperativeLaunch != 0;
     if (cfg) ctx->cfg = *cfg;
     ctx->hostStageInts = 1 << 20;
-    if (cudaMallocHost((void **)&ctx->hostStage, (ctx->hostStageInts + 1024) * sizeof(int32_t)) != cudaSuccess) {
+    if (cudaMallocHost((void **)&ctx->hostStage, (ctx->hostStageInts + kStageSpare) * sizeof(int32_t)) != cudaSuccess) {
         delete ctx;
         return RCD_ERR_CUDA;
     }

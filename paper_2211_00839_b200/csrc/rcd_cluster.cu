@@ -1307,7 +1307,8 @@ __global__ void __launch_bounds__((P == 0 ? kMaxWarps + 1 + kListers : team_warp
 // That holds for rows of about one norm (normalised features).  A class whose
 // squared norms differ by more than a factor of 16, or are not finite, is left in floating point (kNotFixed) for
 // launch_greedy_not_fixed.
-__global__ void __launch_bounds__(256, 8) fixed_exponent_kernel(const ClassDesc *__restrict__ desc, const float *__restrict__ S, int32_t *__restrict__ fixedExp)
+__global__ void __launch_bounds__(256, 8) fixed_exponent_kernel(const ClassDesc *__restrict__ desc, const float *__restrict__ S, int32_t *__restrict__ fixedExp,
+                                                               int32_t *__restrict__ sizesLeft, volatile int32_t *left)
 {
     __shared__ float shMax[8], shMin[8];
     const ClassDesc c = desc[blockIdx.x];
@@ -1331,6 +1332,8 @@ __global__ void __launch_bounds__(256, 8) fixed_exponent_kernel(const ClassDesc 
         if (m > 0.f && !odd) frexpf(m, &e);                // m = x 2^e, x in [0.5, 1)
         odd = odd || (m > 0.f && (m > 16.f * least || m < 1e-30f));
         fixedExp[blockIdx.x] = odd ? kNotFixed : 30 - e;
+        sizesLeft[blockIdx.x] = odd ? c.M : 0;
+        if (odd) *left = 1;                                // (the host's memory: read once the kernel is done)
     }
 }
 __global__ void __launch_bounds__(256, 8) fixed_point_kernel(const ClassDesc *__restrict__ desc, const int32_t *__restrict__ fixedExp, float *__restrict__ S)
@@ -1588,9 +1591,15 @@ rcd_status launch_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const Workspace 
     prm.L = sz.L;
     prm.W = sz.W;
     prm.one = 1u;
+    // Whether a class was left in floating point is known once the similarities are: the host waits for that under the loop's
+    // kernel.  (A launch in every call that finds out by itself would have to bring as many CTAs as such classes need, all
+    // resident at once, and so wait for whatever other streams run.)
+    volatile int32_t *const left = ctx->hostStage + ctx->hostStageInts + kStageLeft;
     const bool toFix = sz.floatArith && ctx->cfg.similarity_kind != RCD_SIM_GAUSSIAN;     // (the Gaussian kernel writes fixed point itself)
     if (toFix) {
-        fixed_exponent_kernel<<<sz.L, 256, 0, st>>>(ws.desc, (const float *)ws.S, ws.fixedExp);
+        *left = 0;
+        fixed_exponent_kernel<<<sz.L, 256, 0, st>>>(ws.desc, (const float *)ws.S, ws.fixedExp, ws.sizesLeft, left);
+        RCD_CUDA(ctx, cudaEventRecord(ctx->evCounts, st));
         const int64_t pieces = sz.maxM * (int64_t)(prm.maxLd / 4);
         const dim3 grid((unsigned)std::min<int64_t>((pieces + 1023) / 1024, std::max(1, 16 * ctx->smCount / sz.L)), (unsigned)sz.L);
         fixed_point_kernel<<<grid, 256, 0, st>>>(ws.desc, ws.fixedExp, (float *)ws.S);
@@ -1604,7 +1613,8 @@ rcd_status launch_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const Workspace 
     if (rs != RCD_OK) return rs;
     ctx->steps = sz.maxM;
     ctx->phaseNsDev = ws.phaseNs;
-    if (toFix) return launch_greedy_not_fixed(ctx, sz, ws, descHost, assignment, order, partValues, st);
+    if (toFix) RCD_CUDA(ctx, cudaEventSynchronize(ctx->evCounts));
+    if (toFix && *left) return launch_greedy_not_fixed(ctx, sz, ws, descHost, assignment, order, partValues, st);
     return RCD_OK;
 }
 

@@ -104,10 +104,10 @@ struct GreedyParams {
     int32_t deltaMax;           //     ... when the pick raised the block's coverage in at most this many columns (<= kDeltaMax)
     int32_t denseRing;          // 8-block dense passes stream through shared-memory rings when the coverage vectors leave room
     const int32_t *classOrder;  // [L] classes by descending size (the order in which the one-CTA-per-class loop draws them)
-    const int32_t *sizesSorted; // [L] class sizes in ascending order
-    const int32_t *only;        // one CTA per class: run (and set up) only the classes marked kNotFixed; null: every class
+    const int32_t *sizes;       // [L] sizes of the classes that run, in any order (0: one that does not)
+    const int32_t *only;        // run (and set up) only the classes marked kNotFixed; null: every class
     int32_t *drawn;             // one CTA per class: classes drawn so far
-    int32_t minM;               // smallest non-empty class
+    int32_t minM;               // smallest non-empty class (0: not known)
     int32_t nonEmpty;           // classes that hold at least one sample
 };
 
@@ -243,7 +243,7 @@ __device__ __forceinline__ int classes_alongside(const GreedyParams<SV> &prm, in
     if (made < prm.minM) return prm.nonEmpty;
     const int lane = threadIdx.x & 31;
     int n = 0;
-    for (int i = lane; i < prm.L; i += 32) n += __ldg(prm.sizesSorted + i) > made ? 1 : 0;
+    for (int i = lane; i < prm.L; i += 32) n += __ldg(prm.sizes + i) > made ? 1 : 0;
     for (int off = 16; off > 0; off >>= 1) n += __shfl_xor_sync(0xffffffffu, n, off);
     return n;
 }
@@ -1405,8 +1405,11 @@ __device__ __forceinline__ int key_index(unsigned long long key) { return 8191 -
 __device__ __forceinline__ void key_gain(unsigned long long key, long long &g) { g = (long long)(key >> 13); }
 __device__ __forceinline__ void key_gain(unsigned long long key, float &g) { g = from_ordered_u32((unsigned)(key >> 32)); }
 
-// kDelta: compiled with the incremental update of stored gains.
-template <typename SV, bool kDelta = false>
+// kDelta: compiled with the incremental update of stored gains.  kFloors: a block whose gains are corrected in place gets a
+// floor, a 128th of the best gain that its last pass found: below it the rounding of the corrections (a few hundred of 2^-25 of
+// that gain) would show, so the block asks for a pass first.  Norms far apart need that: once a sample covers all that is left,
+// every gain is zero and the lowest index wins, but corrected gains are what rounding left of zero.
+template <typename SV, bool kDelta = false, bool kFloors = false>
 __device__ __forceinline__ void pick_chain(const GreedyParams<SV> &prm, int l, int round, int4 *scratch, int scratchBytes,
                                            int own = 0, int *keep = nullptr)
 {
@@ -1510,6 +1513,7 @@ __device__ __forceinline__ void pick_chain(const GreedyParams<SV> &prm, int l, i
                 const unsigned long long key = warp_max_u64(lane < kWarps ? noteK[j * kWarps + lane] : 0ull);
                 if (key) { key_gain(key, bestG); bestV = key_index(key); }
                 fast = bestV != INT_MAX && (res ? shPos[bestV] : pos[bestV]) >= 0;
+                if constexpr (kFloors) fast = fast && !(j < kLazyBlocks && (FV)bestG < shPlan.floorv[j]);
                 if (!fast) { bestG = 0; bestV = INT_MAX; }
             }
         }
@@ -1676,7 +1680,7 @@ __device__ __forceinline__ void pick_chain(const GreedyParams<SV> &prm, int l, i
             prm.cnt[at] = shPlan.quota[j] - shPlan.room[j];
             book_sample();
         }
-        if (kDelta && deltaAllowed && nR > 1 && roomAfter > 0) {
+        if (kDelta && deltaAllowed && nR > 1 && roomAfter > 0 && (!kFloors || j < kLazyBlocks)) {
             // Incremental update: fold row v* into the coverage vector now, find the columns it raised, and if they are
             // few correct the stored gains of block j by one row of S per column; the block then stays up to date.
             for (int i = threadIdx.x; i < ld4; i += kSelectThreads) {
@@ -1848,6 +1852,8 @@ __device__ __forceinline__ void pick_chain(const GreedyParams<SV> &prm, int l, i
                     // block j is up to date again
                     shPlan.open[j] = (uint8_t)1;
                     prm.valid[(int64_t)l * prm.W + j] = 1;
+                    if constexpr (kFloors)
+                        if (total > 0 && !(shPlan.floorv[j] > lowest_value<FV>())) shPlan.floorv[j] = (FV)bestG / 128;
                     shStat[0] += 1ull;
                     shStat[1] += (unsigned long long)total;
                     shStat[2] += (unsigned long long)(total + 2) * (unsigned long long)c.ld * sizeof(SV) + 2ull * c.ld * sizeof(GV);
@@ -2084,13 +2090,13 @@ __device__ __forceinline__ int32_t ld_acquire32(const int32_t *p)
 }
 
 
-template <typename SV>
+template <typename SV, bool kOnly>
 __device__ __forceinline__ void async_pick_cta(const GreedyParams<SV> &prm, int4 *scratch)
 {
     __shared__ int shEpoch, shFinished;
     const int me = blockIdx.x;
     int mine = 0;                                                   // my classes that are not finished
-    for (int l = me; l < prm.L; l += prm.nPick) mine += prm.desc[l].M > 0 ? 1 : 0;
+    for (int l = me; l < prm.L; l += prm.nPick) mine += prm.desc[l].M > 0 && (!kOnly || prm.only[l] == kNotFixed) ? 1 : 0;
     unsigned idle = 0;
     unsigned long long busy = 0;
     __shared__ int shKeep[2];
@@ -2118,7 +2124,7 @@ __device__ __forceinline__ void async_pick_cta(const GreedyParams<SV> &prm, int4
             progressed = true;
             unsigned long long t0 = 0;
             if (me == 0 && threadIdx.x == 0) t0 = global_ns();
-            pick_chain<SV, true>(prm, l, e >> 1, scratch, prm.smemBytes, owner ? (kept ? 2 : 1) : 0, shKeep);
+            pick_chain<SV, true, kOnly>(prm, l, e >> 1, scratch, prm.smemBytes, owner ? (kept ? 2 : 1) : 0, shKeep);
             kept = true;
             __syncthreads();                                            // all writes of the chain are issued
             if (threadIdx.x == 0) {
@@ -2312,11 +2318,33 @@ __device__ __forceinline__ void async_sweep_cta(const GreedyParams<SV> &prm, int
     if (clocked && threadIdx.x == 0) { prm.phaseNs[0] = shClk[0]; prm.phaseNs[6] = shClk[1]; prm.phaseNs[7] = shClk[2]; }
 }
 
+// Set-up inside the kernel, for the classes marked in prm.only: the pick CTAs set their classes up (the others count as
+// finished), and nobody goes on before all have.  False: the wait ran out.
 template <typename SV>
+__device__ __forceinline__ bool async_set_up(const GreedyParams<SV> &prm, int4 *scratch)
+{
+    if ((int)blockIdx.x < prm.nPick) {
+        for (int l = blockIdx.x; l < prm.L; l += prm.nPick) {
+            if (prm.only[l] != kNotFixed) {
+                if (threadIdx.x == 0) prm.sync[l].epoch = 1;
+                continue;
+            }
+            const ClassDesc c = prm.desc[l];
+            for (int64_t i = threadIdx.x; i <= passes_of(c.M); i += blockDim.x) ticket_of(prm, c, l, 0)[i] = 0;
+            init_class(prm, l, *reinterpret_cast<PlanShared<typename Arith<SV>::FV> *>(scratch));
+            __syncthreads();
+        }
+    }
+    return grid_barrier(prm.barrier, gridDim.x, prm.status);
+}
+
+template <typename SV, bool kOnly>
 __global__ void __launch_bounds__(kSweepThreads, 1) greedy_async_kernel(const __grid_constant__ GreedyParams<SV> prm)
 {
     extern __shared__ __align__(128) int4 shCover[];
-    if ((int)blockIdx.x < prm.nPick) async_pick_cta(prm, shCover);
+    if constexpr (kOnly)
+        if (!async_set_up(prm, shCover)) return;
+    if ((int)blockIdx.x < prm.nPick) async_pick_cta<SV, kOnly>(prm, shCover);
     else async_sweep_cta(prm, shCover);
 }
 
@@ -2327,7 +2355,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1) greedy_async_kernel(const __
 // draws the next.  Nothing is shared between CTAs but that counter: no grid barrier, no hand-off, and while one
 // SM makes picks (latency-bound) the others stream, so the memory system stays busy without any phase structure.
 // Classes are drawn largest first (classOrder), which keeps the last CTAs from finishing long after the rest.
-template <typename SV>
+template <typename SV, bool kOnly>
 __global__ void __launch_bounds__(kSweepThreads, 1) greedy_owner_kernel(const __grid_constant__ GreedyParams<SV> prm)
 {
     extern __shared__ __align__(128) int4 shCover[];
@@ -2345,7 +2373,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1) greedy_owner_kernel(const __
         const int l = shClass;
         if (l < 0) break;
         if (prm.desc[l].M == 0) continue;
-        if (prm.only) {
+        if constexpr (kOnly) {
             if (prm.only[l] != kNotFixed) continue;
             init_class(prm, l, *reinterpret_cast<PlanShared<typename Arith<SV>::FV> *>(shCover));
             __syncthreads();
@@ -2363,7 +2391,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1) greedy_owner_kernel(const __
                 if (thresholdPass) tThreshold += t1 - t0;
                 t0 = t1;
             }
-            pick_chain<SV, true>(prm, l, round, shCover, prm.smemBytes, 0, shKeep);
+            pick_chain<SV, true, kOnly>(prm, l, round, shCover, prm.smemBytes, 0, shKeep);
             __syncthreads();
             if (blockIdx.x == 0 && threadIdx.x == 0) tPick += global_ns() - t0;
             if (shKeep[0] == 0 || shKeep[1] < 0) break;
@@ -2456,7 +2484,7 @@ static rcd_status run_greedy(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws,
     prm.asyncGroup = 1;
     prm.helpMin = 1;
     {
-        prm.sizesSorted = ws.sizesSorted;
+        prm.sizes = only ? ws.sizesLeft : ws.sizesSorted;
         prm.classOrder = ws.classOrder;
         prm.nonEmpty = 0;
         prm.minM = 0;
@@ -2465,6 +2493,7 @@ static rcd_status run_greedy(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws,
             prm.minM = prm.nonEmpty == 0 ? c.M : std::min<int32_t>(prm.minM, c.M);
             ++prm.nonEmpty;
         }
+        if (only) prm.minM = 0;                                      // (the host does not know which classes are marked)
     }
     int maxLd = 0;
     for (const auto &c : descHost) if (c.ld > maxLd) maxLd = c.ld;
@@ -2500,30 +2529,38 @@ static rcd_status run_greedy(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws,
     // barriers, 3 = one launch, asynchronous classes, 0 = choose.  With few classes the pick phases of
     // the round-based kernel leave most SMs idle, and giving every class a pick CTA of its own costs
     // few SMs: the asynchronous kernel is chosen when there are at most a quarter as many classes as SMs.
+    // The classes that the cluster form left in floating point (`only`) run in the same two forms.  Norms spread over a factor of
+    // ten, every class left, asynchronous against one CTA per class without corrections in place: 10 of 5000 into 16 blocks
+    // 24.8 ms, 79.1; 4 of 1000 into 8 blocks 2.9, 24.4; 4 of 300 1.15, 2.6; 37 of 1000 3.6, 35.7.
     const bool perSweep = ctx->cfg.profile >= 2;
     int path = ctx->cfg.greedy_path;
-    if (perSweep || !ctx->cooperative) path = 1;
-    if (only) path = 4;
-    if (path == 0) path = (sz.L * 4 <= ctx->smCount) ? 3 : 4;
-    if (path == 3 && ctx->smCount < 2) path = 2;
+    if (only) path = 0;
+    else if (perSweep || !ctx->cooperative) path = 1;
+    if (path == 0) path = (sz.L * 4 <= ctx->smCount && ctx->cooperative) ? 3 : 4;
+    if (path == 3 && ctx->smCount < 2) path = only ? 4 : 2;
+    auto *const ownerKernel = only ? greedy_owner_kernel<SV, !Arith<SV>::kInt> : greedy_owner_kernel<SV, false>;
+    auto *const asyncKernel = only ? greedy_async_kernel<SV, !Arith<SV>::kInt> : greedy_async_kernel<SV, false>;
+    if (path == 2 || path == 3) {
+        // one cooperative launch needs one CTA per SM resident at once
+        int perSm = 0;
+        if (path == 3) {
+            RCD_CUDA(ctx, cudaFuncSetAttribute(asyncKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            RCD_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&perSm, asyncKernel, kSweepThreads, (size_t)smem));
+        } else {
+            RCD_CUDA(ctx, cudaFuncSetAttribute(greedy_persistent_kernel<SV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            RCD_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&perSm, greedy_persistent_kernel<SV>, kSweepThreads, (size_t)smem));
+        }
+        if (perSm < 1) path = only ? 4 : 1;
+    }
     if (path == 4) {
-        RCD_CUDA(ctx, cudaFuncSetAttribute(greedy_owner_kernel<SV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        RCD_CUDA(ctx, cudaFuncSetAttribute(ownerKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         // (in-place correction of stored gains: a class's passes are made by one SM here, so their cost grows with the
         // square of the class size while a correction reads a few dozen rows; measured: it wins on 1300-sample classes
         // with 64 blocks (208 -> 183 ms) and loses on 500-sample classes with 32 (3.9 -> 5.0 ms))
-        if (ctx->cfg.incremental == 0) prm.incremental = sz.maxM >= 1024 ? 1 : 0;
+        if (ctx->cfg.incremental == 0) prm.incremental = sz.maxM >= 1024 || only ? 1 : 0;
         if (ctx->cfg.incremental_max <= 0) prm.deltaMax = 64;
         prm.asyncMode = 2;
         prm.sweepWarps = kSweepThreads / 32;                     // a class is swept by the warps of its own CTA
-    }
-    if (path == 2 || path == 3) {
-        // one cooperative launch needs one CTA per SM resident at once
-        RCD_CUDA(ctx, cudaFuncSetAttribute(greedy_persistent_kernel<SV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        RCD_CUDA(ctx, cudaFuncSetAttribute(greedy_async_kernel<SV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        int perSm = 0;
-        if (path == 3) RCD_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&perSm, greedy_async_kernel<SV>, kSweepThreads, (size_t)smem));
-        else RCD_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&perSm, greedy_persistent_kernel<SV>, kSweepThreads, (size_t)smem));
-        if (perSm < 1) path = 1;
     }
     if (path == 3) {
         // (a pass over a class is cheap here, the whole GPU serves it: beyond a few dozen raised columns it is the faster way)
@@ -2532,7 +2569,10 @@ static rcd_status run_greedy(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws,
         // out-of-date block at once, so its cost per pick falls with the number of blocks.  Measured on CIFAR-10-shaped
         // classes: with 8 blocks the correction wins (99 -> 35 ms), with 16 it wins a little once the picks take their v* from
         // the notes (72.6 -> 70.7 ms); with 32 blocks and small classes it loses.
-        if (ctx->cfg.incremental == 0) prm.incremental = sz.W <= 16 ? 1 : 0;
+        // (Classes left in floating point: always, and in the other form too.  A block there often receives several samples in a
+        // row, each of which would need a pass: 10 classes of 5000 into 16 blocks, norms spread over a factor of ten, 24.8 ms,
+        // with passes only 536; one CTA per class, 100 of 500 into 8 blocks 2.3 ms, 7.0 with passes only, into 32 4.2, 4.8.)
+        if (ctx->cfg.incremental == 0) prm.incremental = sz.W <= 16 || only ? 1 : 0;
         prm.asyncMode = 1;
         prm.nPick = std::min<int>(sz.L, std::max(1, ctx->smCount / 4));
         prm.sweepWarps = (ctx->smCount - prm.nPick) * (kSweepThreads / 32);
@@ -2541,8 +2581,13 @@ static rcd_status run_greedy(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws,
     }
 
     if (only) {
-        // (classes are set up as they are drawn; the counter and the statistics were cleared when the call began)
-        greedy_owner_kernel<SV><<<std::min<int>(ctx->smCount, sz.L), kSweepThreads, (size_t)smem, st>>>(prm);
+        // (the kernels set their classes up themselves; counters and statistics were cleared when the call began)
+        if (path == 3) {
+            void *args[] = {(void *)&prm};
+            RCD_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)asyncKernel, dim3(ctx->smCount), dim3(kSweepThreads), args, (size_t)smem, st));
+        } else {
+            ownerKernel<<<std::min<int>(ctx->smCount, sz.L), kSweepThreads, (size_t)smem, st>>>(prm);
+        }
         ctx->kernelLaunches += 1;
         RCD_CUDA(ctx, cudaGetLastError());
         return RCD_OK;
@@ -2564,11 +2609,11 @@ static rcd_status run_greedy(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws,
     const int64_t rounds = prm.lazyFrom >= 0 ? passes_of(sz.maxM) : sz.maxM;
     if (path == 4) {
         // (an ordinary launch: the CTAs never wait for one another)
-        greedy_owner_kernel<SV><<<std::min<int>(ctx->smCount, sz.L), kSweepThreads, (size_t)smem, st>>>(prm);
+        ownerKernel<<<std::min<int>(ctx->smCount, sz.L), kSweepThreads, (size_t)smem, st>>>(prm);
         ctx->kernelLaunches += 1;
     } else if (persistent && path == 3) {
         void *args[] = {(void *)&prm};
-        RCD_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)greedy_async_kernel<SV>, dim3(ctx->smCount), dim3(kSweepThreads),
+        RCD_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)asyncKernel, dim3(ctx->smCount), dim3(kSweepThreads),
                                                   args, (size_t)smem, st));
         ctx->kernelLaunches += 1;
     } else if (persistent) {

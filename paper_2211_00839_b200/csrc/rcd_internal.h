@@ -134,6 +134,7 @@ struct Workspace {
     unsigned long long *phaseNs;     // [6] sweep-/pick-phase ns of the persistent kernel, barrier counter, threshold-pass hits / elements / max blocks
     long long *g0;          // [N] cluster form: gain of every sample for an empty block
     int32_t *fixedExp;      // [L] cluster form, floating-point similarities: S holds round(sim * 2^fixedExp), or kNotFixed
+    int32_t *sizesLeft;     // [L] sizes of the classes marked kNotFixed, 0 for the others
     int32_t *status;        // [1]
     size_t bytes;           // total bytes laid out
 };
@@ -141,6 +142,9 @@ struct Workspace {
 // Words of rcd_ctx::statusOwn, and where the similarity kernel's tile tickets (zero between launches) begin.
 constexpr int kStatusWords = 1024;
 constexpr int kFirstTicket = 64;
+// The staging buffer holds as many class sizes as a call may have, behind them the status words that come along, and last a word
+// that the device writes: a class was left in floating point.
+constexpr int kStageSpare = 1024, kStageLeft = kStageSpare - 1;
 
 // A class whose samples' norms lie too far apart for one fixed-point scale (see fixed_exponent_kernel).
 constexpr int32_t kNotFixed = INT32_MIN;

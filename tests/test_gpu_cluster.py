@@ -91,6 +91,21 @@ def test_float_norms_far_apart(rcd, orc):
     check_float(rcd, orc, wl)
 
 
+@pytest.mark.parametrize("sizes,W,apart", [([900, 700], 6, 2), ([1200, 33, 700], 24, 3), ([600, 300, 1, 500], 100, 2)])
+def test_float_norms_far_apart_on_all_sms(rcd, orc, sizes, W, apart):
+    """Few classes left in floating point are swept by every SM, as they are when the asynchronous form is asked for; the first
+    `apart` classes are such.  Once a few long rows cover all that is left every gain is zero, so most picks are ties."""
+    import torch
+    spread = set(sizes[:apart])
+    wl = workload(sizes, 64, W, W, dtype="bf16", scale=lambda rng, M: 10.0 ** rng.uniform(-1.5 if M in spread else 0.0, 1.5 if M in spread else 0.1, M))
+    X, y = rcd.features_to_torch(wl.features, device="cuda"), torch.from_numpy(wl.labels).cuda()
+    with rcd.Context(0, profile=1) as ctx:
+        ctx.rcd_partition(X, y, wl.capacities, wl.L)
+        ctx.sync_status()
+        assert ctx.profile()["async_visits"] > 0
+    check_float(rcd, orc, wl)
+
+
 @pytest.mark.parametrize("sizes,W,apart", [([800, 500, 300], 100, 1), ([140] * 12 + [130] * 148, 33, 12)])
 def test_float_norms_far_apart_with_lists(rcd, orc, sizes, W, apart):
     """The largest classes, which clusters draw first, stay in floating point; the next ones use lists of candidates (several
