@@ -122,6 +122,36 @@ def test_float_norms_far_apart_with_lists(rcd, orc, sizes, W, apart):
     check_float(rcd, orc, wl)
 
 
+@pytest.mark.parametrize("similarity", ["gaussian", "dot"])
+@pytest.mark.parametrize("sizes,W", [([128, 1, 77], 5), ([120] * 6, 48)])
+def test_float_is_exact_in_fixed_point(rcd, orc, similarity, sizes, W):
+    """Floating-point similarities become integers once, and from there on nothing is rounded: picks and values are those of the
+    oracle's integer arithmetic on those integers, bit for bit.  And where no two candidates lie closer than the similarities'
+    own rounding, the picks are the fp64 oracle's with no tolerance (asserted on the first set of classes)."""
+    wl = workload(sizes, 64, W, 5 * W, dtype="bf16")
+    kind = rcd.RCD_SIM_GAUSSIAN if similarity == "gaussian" else rcd.RCD_SIM_DOT
+    a, o, v = run_partition(rcd, wl, similarity_kind=kind)
+    off = 0
+    for l, ids in enumerate(orc.split_by_label(wl.labels, wl.L)):
+        M = len(ids)
+        with rcd.Context(0) as ctx:
+            X = rcd.features_to_torch(wl.features[ids], device="cuda").view(1, M, -1)
+            S = ctx.rcd_similarity_gaussian(X)[0] if similarity == "gaussian" else ctx.rcd_similarity(X)
+            ctx.sync_status()
+            S = S.cpu().numpy()[0, :, :M].astype(np.float64)
+        # the largest value lands in [2^29, 2^30); the Gaussian kernel's is 1
+        e = 29 if similarity == "gaussian" else 30 - int(np.frexp(np.float32(S.diagonal().max()))[1])
+        F = np.clip(np.rint(S * 2.0 ** e), 1 - 2 ** 30, 2 ** 30 - 1).astype(np.int64)
+        q = orc.quotas(M, wl.capacities)
+        want, oj, ov, fv = orc.partition_class(F, q, "incremental")
+        assert np.array_equal(o[off:off + M], ids[ov]) and np.array_equal(a[ids], want)
+        assert np.array_equal(v[l], np.ldexp(fv.astype(np.float64), -e))
+        if len(sizes) == 3:
+            exact = orc.class_similarity(wl.features[ids], similarity)
+            assert orc.replay_class(exact, q, oj, ov, 0.0)[0] == -1
+        off += M
+
+
 @pytest.mark.parametrize("sizes,W", [([400, 3], 5), ([600] * 4, 24), ([90] * 150, 20)])
 def test_graph_cut_int8_exact(rcd, orc, sizes, W):
     wl = workload(sizes, 48, W, W)
