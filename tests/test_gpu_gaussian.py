@@ -54,6 +54,39 @@ def test_gaussian_similarity_of_coincident_points(rcd):
         assert float(sigma[0]) == 0.0 and bool((S[0, :, :40] == 1).all())
 
 
+def test_distance_roots_to_one_unit_in_the_last_place(rcd):
+    """Distances are rooted by two of Heron's steps from a 22-bit reciprocal root: 2^-65 of the root is left after them, so the
+    last rounding leaves half a unit in the last place of fp64 and next to nothing more; one unit is allowed.  Classes of two
+    samples, the second zero: the class's sum of distances, an fp64 word of the scratch buffer, is twice the first one's norm.
+    Squared norms n 2^2k, n < 2^24 a sum of squares of whole numbers: exact in fp32."""
+    import torch
+    rng = np.random.default_rng(3)
+    d, cases = 1024, []
+    for k in (-74, -70, -63, -40, -1, 0, 1, 30, 52):
+        for n in (1, 2, 3, 40):
+            cases.append((rng.integers(1, 256, size=n), k))
+    most = np.concatenate([np.full(258, 255), [27, 6]])                  # 2^24 - 1: the largest fp32 at k = 52
+    cases += [(np.zeros(1, np.int64), 0), (most, 52), (most, -74), (np.ones(1, np.int64), 64)]       # (the last: infinity)
+    x = np.zeros((len(cases), 2, d), np.float32)
+    square = np.zeros(len(cases))
+    for i, (n, k) in enumerate(cases):
+        x[i, 0, :len(n)] = n * np.float32(2.0) ** k
+        square[i] = float((n.astype(np.int64) ** 2).sum()) * 2.0 ** (2 * k)
+    square[square >= 2.0 ** 128] = np.inf
+    assert np.array_equal(square.astype(np.float32).astype(np.float64), square)
+    with rcd.Context(0) as ctx:
+        X = torch.from_numpy(x).to(torch.bfloat16).cuda()
+        assert np.array_equal(X.float().cpu().numpy(), x)
+        ctx.rcd_similarity_gaussian(X)
+        ctx.sync_status()
+        at = (2 * len(cases) * 4 + 255) // 256 * 256                     # behind the norms of the rows
+        got = ctx.workspace(at + 8 * len(cases))[at:at + 8 * len(cases)].cpu().numpy().view(np.float64)
+    want = np.sqrt(square)
+    fin = np.isfinite(want)
+    assert np.array_equal(got[~fin], want[~fin])
+    assert np.all(np.abs(got[fin] / 2 - want[fin]) <= np.spacing(want[fin]) * (want[fin] > 0))
+
+
 @pytest.mark.parametrize("name,L,M,d,path", [("C1", 2, 200, 64, 0), ("C2", 2, 700, 128, 0), ("C4", 3, 400, 256, 1)])
 def test_partition_with_gaussian_similarity(rcd, orc, name, L, M, d, path):
     import torch
