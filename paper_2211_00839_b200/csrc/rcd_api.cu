@@ -228,6 +228,7 @@ struct Prepared {
     Sizes sz{};
     Workspace ws{};
     std::vector<ClassDesc> desc;
+    std::shared_ptr<ClusterPlan> cluster;   // null: another form of the greedy loop, or none
 };
 
 // capacities null: no quotas wanted.
@@ -335,9 +336,10 @@ static rcd_status prepare(rcd_ctx *ctx, const void *features, rcd_feat_dtype dty
     const int64_t dPitch = sz.pitch / (int64_t)feat_bytes(dtype);
     rs = launch_similarity(ctx, P.ws.Xs, dtype, N, dPitch, cls, P.ws.S, st);
     if (rs != RCD_OK) return rs;
+    if (capacities) P.cluster = plan_greedy_cluster(ctx, sz, P.desc);
     if (ctx->cfg.similarity_kind == RCD_SIM_GAUSSIAN) {
         rs = launch_gaussian(ctx, P.ws.Xs, dtype, N, dPitch, cls, P.ws.S, P.ws.gaussNorms, P.ws.gaussPartial, P.ws.gaussSigma,
-                             P.ws.gaussScale, capacities && greedy_cluster_takes(ctx, sz, P.desc) ? P.ws.fixedExp : nullptr, st);
+                             P.ws.gaussScale, P.cluster ? P.ws.fixedExp : nullptr, st);
         if (rs != RCD_OK) return rs;
     }
     if (capacities && !early) {
@@ -713,10 +715,9 @@ rcd_status rcd_partition(rcd_ctx *ctx, const void *features_dev, rcd_feat_dtype 
     rs = prepare(ctx, features_dev, dtype, N, d, labels_dev, L, W, capacities_host, workspace_dev, workspace_bytes, st, &P);
     if (rs != RCD_OK) return rs;
 
-    bool valuesWritten = false;
-    rs = launch_greedy_cluster(ctx, P.sz, P.ws, P.desc, assignment_dev, order_dev_or_null, part_values_dev_or_null, st, &valuesWritten);
-    if (rs != RCD_OK) return rs;
-    if (valuesWritten) {
+    const bool valuesWritten = P.cluster != nullptr;
+    if (P.cluster) {
+        rs = launch_greedy_cluster(ctx, *P.cluster, P.sz, P.ws, P.desc, assignment_dev, order_dev_or_null, part_values_dev_or_null, st);
     } else if (P.sz.graphCut) {
         rs = launch_cut(ctx, P.sz, P.ws, assignment_dev, order_dev_or_null, st);
     } else {

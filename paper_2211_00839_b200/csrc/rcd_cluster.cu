@@ -1557,19 +1557,16 @@ static bool cluster_plan(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassD
     return true;
 }
 
-bool greedy_cluster_takes(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost)
+std::shared_ptr<ClusterPlan> plan_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost)
 {
-    ClusterPlan plan;
-    return cluster_plan(ctx, sz, descHost, plan);
+    auto plan = std::make_shared<ClusterPlan>();
+    return cluster_plan(ctx, sz, descHost, *plan) ? plan : nullptr;
 }
 
-// Runs the greedy loop if the cluster form takes the problem (*taken).  partValues (may be null) receives the tracked values.
-rcd_status launch_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, const std::vector<ClassDesc> &descHost,
-                                 int32_t *assignment, int32_t *order, void *partValues, cudaStream_t st, bool *taken)
+// Runs the greedy loop.  partValues (may be null) receives the tracked values.
+rcd_status launch_greedy_cluster(rcd_ctx *ctx, ClusterPlan &plan, const Sizes &sz, const Workspace &ws, const std::vector<ClassDesc> &descHost,
+                                 int32_t *assignment, int32_t *order, void *partValues, cudaStream_t st)
 {
-    ClusterPlan plan;
-    *taken = cluster_plan(ctx, sz, descHost, plan);
-    if (!*taken) return RCD_OK;
     ClusterParams &prm = plan.prm;
     prm.desc = ws.desc;
     prm.S = (const int32_t *)ws.S;

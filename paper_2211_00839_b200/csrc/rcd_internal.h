@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <stddef.h>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -288,10 +289,11 @@ rcd_status launch_greedy(rcd_ctx *ctx, rcd_feat_dtype dtype, const Sizes &sz, co
 rcd_status launch_greedy_not_fixed(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, const std::vector<ClassDesc> &descHost,
                                    int32_t *assignment, int32_t *order, void *partValues, cudaStream_t st);
 
-// greedy loop, one thread-block cluster per class: whether it takes a problem, and the loop
-bool greedy_cluster_takes(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost);
-rcd_status launch_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, const std::vector<ClassDesc> &descHost,
-                                 int32_t *assignment, int32_t *order, void *partValues, cudaStream_t st, bool *taken);
+// greedy loop, one thread-block cluster per class: how it takes a problem (null: it does not), and the loop
+struct ClusterPlan;
+std::shared_ptr<ClusterPlan> plan_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost);
+rcd_status launch_greedy_cluster(rcd_ctx *ctx, ClusterPlan &plan, const Sizes &sz, const Workspace &ws, const std::vector<ClassDesc> &descHost,
+                                 int32_t *assignment, int32_t *order, void *partValues, cudaStream_t st);
 
 rcd_status launch_bounded_wait_selftest(rcd_ctx *ctx, unsigned *counter, int32_t *status, cudaStream_t st);
 
