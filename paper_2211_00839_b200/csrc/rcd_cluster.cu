@@ -1511,8 +1511,10 @@ static bool cluster_plan(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassD
     const size_t cap = (size_t)ctx->maxSmemOptin - 1024;
     plan.prm = ClusterParams{};
     for (int i = 0; i < 5; ++i)
-        if (ctx->maxClusters[i] == 0) {
-            if (launch_cluster(ctx, pick_kernel<1, false>(3, 15, true), plan.prm, 16 * 32, 1 << i, 1, cap, nullptr, &ctx->maxClusters[i]) != RCD_OK) return false;
+        if (ctx->maxClusters[i] < 0) {
+            int active = 0;
+            if (launch_cluster(ctx, pick_kernel<1, false>(3, 15, true), plan.prm, 16 * 32, 1 << i, 1, cap, nullptr, &active) != RCD_OK) return false;
+            ctx->maxClusters[i] = active;
         }
     // Cluster size: the one whose clusters, drawing classes largest first, finish soonest by the estimate that a class of
     // M samples takes M (M / C + 300) (corrections, shared by the CTAs, and the chain of picks); blocks have to stay on

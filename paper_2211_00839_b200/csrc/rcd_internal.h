@@ -247,7 +247,7 @@ struct rcd_ctx {
     const unsigned long long *stepOpsDev = nullptr;
     const unsigned long long *phaseNsDev = nullptr;
     const int32_t *statusDev = nullptr;
-    int maxClusters[5]{};               // clusters of 1, 2, 4, 8, 16 CTAs of the cluster form resident at once (0: not asked yet)
+    int maxClusters[5] = {-1, -1, -1, -1, -1};   // clusters of 1, 2, 4, 8, 16 CTAs of the cluster form resident at once (-1: not asked yet)
 };
 
 namespace rcd {
