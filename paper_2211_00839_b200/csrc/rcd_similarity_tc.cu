@@ -665,8 +665,9 @@ rcd_status launch_similarity_tc(rcd_ctx *ctx, const void *Xs, rcd_feat_dtype dty
     // (shared memory beyond 48 KB is asked for once per context and kernel, not on every call)
     auto allow = [&](auto *kernel, int bit, size_t bytes) {
         if (ctx->simReady >> bit & 1) return cudaSuccess;
-        ctx->simReady |= 1 << bit;
-        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        if (e == cudaSuccess) ctx->simReady |= 1u << bit;
+        return e;
     };
     if (cls.pairs) {
         const size_t pairSmem = (size_t)kPairStages * kPairStageBytes + 1024;
