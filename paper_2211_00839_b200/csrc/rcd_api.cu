@@ -56,6 +56,13 @@ static rcd_status blob_begin(rcd_ctx *ctx, size_t bytes, size_t stageIntsUsed, u
     return RCD_OK;
 }
 
+// From the first copy out of that memory on it is in use, however the call ends: the event comes after the last copy.
+struct BlobInUse {
+    rcd_ctx *ctx;
+    cudaStream_t st;
+    ~BlobInUse() { cudaEventRecord(ctx->evBlob, st); }
+};
+
 // Bump allocator over the caller's workspace.
 struct Carver {
     unsigned char *base;
@@ -261,8 +268,8 @@ static rcd_status prepare(rcd_ctx *ctx, const void *features, rcd_feat_dtype dty
     const size_t blobBytes = (size_t)((unsigned char *)(hw.quota + (size_t)L * W) - (unsigned char *)hw.desc);
     unsigned char *blob = nullptr;
     rs = blob_begin(ctx, blobBytes, statusInts + (size_t)L, &blob);
+    RCD_CUDA(ctx, cudaEventSynchronize(ctx->evCounts));     // (also where that failed: the sizes are on their way to the staging buffer)
     if (rs != RCD_OK) return rs;
-    RCD_CUDA(ctx, cudaEventSynchronize(ctx->evCounts));
     if (ctx->hostStage[0] & kDevBadLabel) return fail(ctx, RCD_ERR_INVALID_ARG, "a label lies outside [0, %d)", L);
     const int32_t *counts = ctx->hostStage + statusInts;      // (behind the zeroed words that came along)
 
@@ -327,6 +334,7 @@ static rcd_status prepare(rcd_ctx *ctx, const void *features, rcd_feat_dtype dty
     }
     const bool early = capacities && L <= 64;               // (few quotas: not worth a copy of their own behind the similarity kernel)
     if (early) quotas();
+    const BlobInUse inUse{ctx, st};
     const size_t firstBytes = early ? blobBytes : (size_t)((unsigned char *)hw.quota - (unsigned char *)hw.desc);
     RCD_CUDA(ctx, cudaMemcpyAsync(P.ws.desc, blob, firstBytes, cudaMemcpyHostToDevice, st));
     rs = launch_stable_split(ctx, labels, N, L, P.ws.chunkHist, P.ws.desc, nullptr, nullptr, nullptr, P.ws.perm,
@@ -346,7 +354,6 @@ static rcd_status prepare(rcd_ctx *ctx, const void *features, rcd_feat_dtype dty
         quotas();
         RCD_CUDA(ctx, cudaMemcpyAsync(P.ws.quota, at(hw.quota), (size_t)L * W * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     }
-    RCD_CUDA(ctx, cudaEventRecord(ctx->evBlob, st));
     if (ctx->cfg.profile >= 1) RCD_CUDA(ctx, cudaEventRecord(ctx->evPhase[2], st));
     return RCD_OK;
 }
@@ -572,8 +579,8 @@ rcd_status rcd_worker_lists(rcd_ctx *ctx, const int32_t *assignment_dev, int64_t
     // the list boundaries are sums of the sizes, and a stable split by block number fills the lists (inside a list the
     // dataset indices ascend): enqueued behind the check of the entries, whose verdict they read themselves
     rs = launch_stable_split(ctx, assignment_dev, N, W, ws.chunkHist, nullptr, ws.counts, offsets_dev, ws.status, indices_dev, nullptr, 0, 0, nullptr, st);
-    if (rs != RCD_OK) return rs;
     RCD_CUDA(ctx, cudaEventSynchronize(ctx->evCounts));
+    if (rs != RCD_OK) return rs;
     if (ctx->hostStage[0] & kDevBadLabel) return fail(ctx, RCD_ERR_INVALID_ARG, "an assignment entry lies outside [0, %d)", W);
     return RCD_OK;
 }

@@ -54,6 +54,27 @@ def test_gaussian_similarity_of_coincident_points(rcd):
         assert float(sigma[0]) == 0.0 and bool((S[0, :, :40] == 1).all())
 
 
+def test_call_after_one_that_was_given_up_under_way(rcd):
+    """More classes than the Gaussian kernel takes are refused once the class sizes are known, with copies out of the context's
+    pinned memory under way: the next call, on another stream, must not write into that memory before they are done."""
+    import torch
+    rng = np.random.default_rng(1)
+    X = torch.from_numpy(rng.integers(-9, 10, size=(70000, 128)).astype(np.int8)).cuda()
+    many = (torch.arange(70000, device="cuda") % 66000).to(torch.int32)
+    few = (torch.arange(70000, device="cuda") % 200).to(torch.int32)
+    with rcd.Context(0, similarity_kind=rcd.RCD_SIM_GAUSSIAN) as ctx:
+        want = [t.clone() for t in ctx.rcd_partition(X, few, [1.0, 2.0], 200)]
+        torch.cuda.synchronize()
+        for _ in range(3):
+            with pytest.raises(rcd.RcdError):
+                ctx.rcd_partition(X, many, [1.0, 2.0], 66000, M_max=2)
+            still_used, ctx._ws = ctx._ws, None                          # (streams that overlap need a workspace each)
+            with torch.cuda.stream(torch.cuda.Stream()):
+                got = ctx.rcd_partition(X, few, [1.0, 2.0], 200)
+                ctx.sync_status()
+            assert all(torch.equal(a, b) for a, b in zip(want, got))
+
+
 def test_distance_roots_to_one_unit_in_the_last_place(rcd):
     """Distances are rooted by two of Heron's steps from a 22-bit reciprocal root: 2^-65 of the root is left after them, so the
     last rounding leaves half a unit in the last place of fp64 and next to nothing more; one unit is allowed.  Classes of two
