@@ -806,8 +806,8 @@ rcd_status rcd_partition_host(rcd_ctx *ctx, const void *features_host, rcd_feat_
     return rcd_sync_status(ctx, st);
 }
 
-// Objective scratch: per class and row block, W partial sums.
-static size_t objective_scratch_bytes(int32_t L, int64_t Mmax, int32_t W)
+// Graph cut: per class and row block, W partial sums.  (Facility location uses arrays of the greedy loop.)
+static size_t cut_scratch_bytes(int32_t L, int64_t Mmax, int32_t W)
 {
     size_t blocks = (size_t)((Mmax + 63) / 64);
     return align_up(std::max<size_t>(1, (size_t)L * blocks * (size_t)W * 8));
@@ -820,7 +820,7 @@ rcd_status rcd_objective_workspace_bytes(rcd_ctx *ctx, rcd_feat_dtype dtype, int
     if (rs != RCD_OK) return rs;
     if (!bytes_out || M_max < 0) return fail(ctx, RCD_ERR_INVALID_ARG, "bad M_max or null output");
     Sizes sz = bound_sizes(ctx, dtype, N, d, L, M_max, W);
-    *bytes_out = layout_workspace(nullptr, dtype, sz, nullptr) + objective_scratch_bytes(L, std::min(M_max, N), W);
+    *bytes_out = layout_workspace(nullptr, dtype, sz, nullptr) + (sz.graphCut ? cut_scratch_bytes(L, std::min(M_max, N), W) : 0);
     return RCD_OK;
 }
 
@@ -843,7 +843,7 @@ rcd_status rcd_objective(rcd_ctx *ctx, const void *features_dev, rcd_feat_dtype 
     ctx->cfg.profile = savedProfile;
     if (rs != RCD_OK) return rs;
     if (P.sz.graphCut) {
-        const size_t scratchB = objective_scratch_bytes(L, P.sz.maxM, W);
+        const size_t scratchB = cut_scratch_bytes(L, P.sz.maxM, W);
         if (P.ws.bytes + scratchB > workspace_bytes)
             return fail(ctx, RCD_ERR_WORKSPACE_TOO_SMALL, "workspace has %zu bytes, objective needs %zu", workspace_bytes, P.ws.bytes + scratchB);
         rs = launch_cut_objective(ctx, P.sz, P.ws.desc, P.ws.S, P.ws.perm, assignment_dev, part_values_dev, total_dev,

@@ -200,13 +200,6 @@ __device__ __forceinline__ unsigned long long take_off(unsigned long long g, int
     return r;
 }
 
-// g - l for an unsigned l (minusOne: the value -1 as an unsigned 32-bit number times l, low 64 bits, plus l << 32)
-__device__ __forceinline__ unsigned long long take_off_wide(unsigned long long g, uint32_t l, uint32_t one)
-{
-    (void)one;
-    return g - l;
-}
-
 // Sum of a value below 2^43 per lane over the warp.
 __device__ __forceinline__ unsigned long long warp_sum(unsigned long long x)
 {
@@ -369,16 +362,16 @@ __device__ __forceinline__ int list_raised(const TeamView &t, int32_t *count, in
 // Four listed columns taken off the stored gains of one piece.  Their losses (each below 2^30) add up in 32 bits, so that
 // widening and subtracting is paid once for four: 156 cycles of arithmetic per row of 20 KB and SM, 248 with two at a time.
 __device__ __forceinline__ uint32_t apply_four(const int4 &x, const int4 &y, const int4 &z, const int4 &w, const Raised &a, const Raised &b,
-                                               const Raised &c, const Raised &d, uint32_t one, unsigned long long (&g)[4])
+                                               const Raised &c, const Raised &d, unsigned long long (&g)[4])
 {
     const uint32_t l0 = (uint32_t)loss(x.x, a) + loss(y.x, b) + loss(z.x, c) + loss(w.x, d);
     const uint32_t l1 = (uint32_t)loss(x.y, a) + loss(y.y, b) + loss(z.y, c) + loss(w.y, d);
     const uint32_t l2 = (uint32_t)loss(x.z, a) + loss(y.z, b) + loss(z.z, c) + loss(w.z, d);
     const uint32_t l3 = (uint32_t)loss(x.w, a) + loss(y.w, b) + loss(z.w, c) + loss(w.w, d);
-    g[0] = take_off_wide(g[0], l0, one);
-    g[1] = take_off_wide(g[1], l1, one);
-    g[2] = take_off_wide(g[2], l2, one);
-    g[3] = take_off_wide(g[3], l3, one);
+    g[0] -= l0;
+    g[1] -= l1;
+    g[2] -= l2;
+    g[3] -= l3;
     return l0 | l1 | l2 | l3;
 }
 // (entry e of n, or one without effect)
@@ -392,7 +385,7 @@ __device__ __forceinline__ Raised entry_or_none(const Raised *list, int e, int n
 // The n listed columns taken off one piece, rows straight to registers, up to sixteen in flight
 // (a warp waits about 1100 cycles for a batch; with sixteen warps at it a row of 5 KB takes an SM about 140 cycles, the share
 // of the copy bandwidth that 148 SMs get).
-__device__ __forceinline__ bool correct_piece(const int4 *S4q, const Raised *list, int n, uint32_t one, unsigned long long (&g)[4])
+__device__ __forceinline__ bool correct_piece(const int4 *S4q, const Raised *list, int n, unsigned long long (&g)[4])
 {
     uint32_t changed = 0;
     int e = 0;
@@ -402,15 +395,15 @@ __device__ __forceinline__ bool correct_piece(const int4 *S4q, const Raised *lis
 #pragma unroll
         for (int u = 0; u < 16; ++u) x[u] = ld_row_shared(S4q + list[e + u].row);
 #pragma unroll
-        for (int u = 0; u < 16; u += 4) changed |= apply_four(x[u], x[u + 1], x[u + 2], x[u + 3], list[e + u], list[e + u + 1], list[e + u + 2], list[e + u + 3], one, g);
+        for (int u = 0; u < 16; u += 4) changed |= apply_four(x[u], x[u + 1], x[u + 2], x[u + 3], list[e + u], list[e + u + 1], list[e + u + 2], list[e + u + 3], g);
     }
 #pragma unroll 1
     for (; e + 8 <= n; e += 8) {
         int4 x[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) x[u] = ld_row_shared(S4q + list[e + u].row);
-        changed |= apply_four(x[0], x[1], x[2], x[3], list[e], list[e + 1], list[e + 2], list[e + 3], one, g);
-        changed |= apply_four(x[4], x[5], x[6], x[7], list[e + 4], list[e + 5], list[e + 6], list[e + 7], one, g);
+        changed |= apply_four(x[0], x[1], x[2], x[3], list[e], list[e + 1], list[e + 2], list[e + 3], g);
+        changed |= apply_four(x[4], x[5], x[6], x[7], list[e + 4], list[e + 5], list[e + 6], list[e + 7], g);
     }
 #pragma unroll 1
     for (; e < n; e += 4) {
@@ -421,7 +414,7 @@ __device__ __forceinline__ bool correct_piece(const int4 *S4q, const Raised *lis
             r[u] = entry_or_none(list, e + u, n);
             x[u] = ld_row_shared(S4q + r[u].row);
         }
-        changed |= apply_four(x[0], x[1], x[2], x[3], r[0], r[1], r[2], r[3], one, g);
+        changed |= apply_four(x[0], x[1], x[2], x[3], r[0], r[1], r[2], r[3], g);
     }
     return changed != 0;
 }
@@ -435,7 +428,7 @@ __device__ __forceinline__ bool correct_piece(const int4 *S4q, const Raised *lis
 template <int P> struct RowRing { static constexpr bool byRow = P <= 3; };
 constexpr int kRowStages = 8, kPieceStages = 16;
 template <int P, int kT>
-__device__ __forceinline__ void apply_list(const TeamView &t, int n, uint32_t one, unsigned long long (&g)[P][4])
+__device__ __forceinline__ void apply_list(const TeamView &t, int n, unsigned long long (&g)[P][4])
 {
     const int first = t.warpIn * 32 + t.lane, step = (kT ? kT : t.T) * 32;
     int4 *const ring = t.rowBuf + first;
@@ -475,7 +468,7 @@ __device__ __forceinline__ void apply_list(const TeamView &t, int n, uint32_t on
 #pragma unroll
             for (int p = 0; p < P; ++p)
                 if (p * step + first < t.ld4)
-                    apply_four(x[p * step], x[p * step + stride], x[p * step + 2 * stride], x[p * step + 3 * stride], r[0], r[1], r[2], r[3], one, g[p]);
+                    apply_four(x[p * step], x[p * step + stride], x[p * step + 2 * stride], x[p * step + 3 * stride], r[0], r[1], r[2], r[3], g[p]);
         }
     } else {
         int fq = first, fe = 0, fs = 0, at = 0;
@@ -507,12 +500,12 @@ __device__ __forceinline__ void apply_list(const TeamView &t, int n, uint32_t on
                     const int4 x0 = x[0], x1 = x[step], x2 = x[2 * step], x3 = x[3 * step];
                     fetch();
                     if (e + 4 <= n) {
-                        apply_four(x0, x1, x2, x3, list[e], list[e + 1], list[e + 2], list[e + 3], one, g[p]);
+                        apply_four(x0, x1, x2, x3, list[e], list[e + 1], list[e + 2], list[e + 3], g[p]);
                     } else {
                         Raised r[4];
 #pragma unroll
                         for (int u = 0; u < 4; ++u) r[u] = entry_or_none(list, e + u, n);
-                        apply_four(x0, x1, x2, x3, r[0], r[1], r[2], r[3], one, g[p]);
+                        apply_four(x0, x1, x2, x3, r[0], r[1], r[2], r[3], g[p]);
                     }
                 }
             }
@@ -674,7 +667,7 @@ __device__ __forceinline__ void team_of_one(const ClusterParams &prm, const Clas
             lead_init(best);
             sum = Summary{0, 0, 0};
             dirty = true;
-            apply_list<P, kT>(t, n, prm.one, g);
+            apply_list<P, kT>(t, n, g);
         };
         if ((int)what - 1 != v || all > room) {
             // another sample than foreseen, or more raised columns than one list holds
@@ -829,7 +822,7 @@ __device__ void list_candidates(const ClusterParams &prm, const uint32_t *bits, 
 // A team with several blocks, coverage and stored gains in memory (shared memory where they fit).  Its commands come
 // through a ring, in the order given.
 template <bool kCut, typename Where>
-__device__ __forceinline__ void team_of_many(const ClusterParams &prm, int l, const ClassDesc &c, const TeamView &t, int mine, int shift,
+__device__ __forceinline__ void team_of_many(const ClusterParams &prm, const ClassDesc &c, const TeamView &t, int mine, int shift,
                                              unsigned long long bias, uint32_t cmds, Where where, unsigned &corrected, unsigned &rows)
 {
     const int lane = t.lane, T = t.T, tid = t.warpIn * 32 + lane, step = T * 32;
@@ -859,13 +852,12 @@ __device__ __forceinline__ void team_of_many(const ClusterParams &prm, int l, co
     if (tid == 0) t.tm->count[0] = t.tm->count[1] = 0;
     int par = 0;
     for (int i = 0; i < mine; ++i) {
-        const int j = where(i, cov, gains, noteAddr, barAddr, told);
+        where(i, cov, gains, noteAddr, barAddr, told);
         for (int q = tid; q < t.ld4; q += step) {
             if (!kCut) cov[q] = make_int4(0, 0, 0, 0);
 #pragma unroll
             for (int u = 0; u < 4; ++u) gains[4 * q + u] = 4 * q + u < c.M ? (unsigned long long)__ldcg(prm.g0 + c.row0 + 4 * q + u) + bias : 0ull;
         }
-        (void)j;
     }
     team_barrier(t.team, T);
     for (uint32_t n = 1;; ++n) {
@@ -909,7 +901,7 @@ __device__ __forceinline__ void team_of_many(const ClusterParams &prm, int l, co
                     ulonglong2 *p = reinterpret_cast<ulonglong2 *>(gains) + 2 * q;
                     const ulonglong2 k0 = p[0], k1 = p[1];
                     unsigned long long k[4] = {k0.x, k0.y, k1.x, k1.y};
-                    if (correct_piece(t.S4 + q, t.list, m, prm.one, k)) {
+                    if (correct_piece(t.S4 + q, t.list, m, k)) {
                         p[0] = make_ulonglong2(k[0], k[1]);
                         p[1] = make_ulonglong2(k[2], k[3]);
                     }
@@ -1265,7 +1257,7 @@ __global__ void __launch_bounds__((P == 0 ? kMaxWarps + 1 + kListers : team_warp
                                                        base + prm.offCmd + team * prm.ring * 8, notes0 + j * (uint32_t)layout.words() * 8, bars0 + j * 8, corrected, rows);
             } else {
                 // the i-th block of the team
-                auto where = [&](int i, int4 *&cov, unsigned long long *&gains, uint32_t &noteAddr, uint32_t &barAddr, volatile uint32_t *&told) -> int {
+                auto where = [&](int i, int4 *&cov, unsigned long long *&gains, uint32_t &noteAddr, uint32_t &barAddr, volatile uint32_t *&told) {
                     const int slot = team + i * nTeams, j = slot * (int)C + (int)rank;
                     if (kSmemState) {
                         cov = reinterpret_cast<int4 *>(shared + prm.offCover) + (size_t)slot * (prm.maxLd >> 2);
@@ -1277,11 +1269,10 @@ __global__ void __launch_bounds__((P == 0 ? kMaxWarps + 1 + kListers : team_warp
                     noteAddr = notes0 + j * (uint32_t)layout.words() * 8;
                     told = told0 + slot;
                     barAddr = bars0 + j * 8;
-                    return j;
                 };
                 int mine = 0;
                 while (team + mine * nTeams < prm.slots && (team + mine * nTeams) * (int)C + (int)rank < W) ++mine;
-                if (mine > 0) team_of_many<kCut>(prm, l, c, t, mine, shift, bias, base + prm.offCmd + team * prm.ring * 8, where, corrected, rows);
+                if (mine > 0) team_of_many<kCut>(prm, c, t, mine, shift, bias, base + prm.offCmd + team * prm.ring * 8, where, corrected, rows);
             }
             if (lane == 0 && t.warpIn == 0 && corrected) {
                 atomicAdd(prm.stats + 15, (unsigned long long)corrected);
