@@ -205,7 +205,11 @@ RCD_API rcd_status rcd_similarity_gaussian(rcd_ctx *ctx, const void *X_dev, rcd_
 
 /* Upper bound of the workspace rcd_partition needs for N samples of width d in L classes none
  * larger than M_max, W blocks.  (rcd_partition recomputes the exact need from the label counts
- * and returns RCD_ERR_WORKSPACE_TOO_SMALL if a class was larger than promised.) */
+ * and returns RCD_ERR_WORKSPACE_TOO_SMALL if a class was larger than promised.)
+ * Its largest parts: the similarity matrices (4 bytes x M_l x M_l rounded up to 8, all classes), coverage and stored
+ * gains (4 + 8 bytes per sample and block: gains are 64-bit for either feature type, since sums of floating-point
+ * similarities are kept in fixed point), the sorted features, and the class split's table of chunks x labels
+ * (4 bytes x L x N / 256 while that is at most 64 MB and N at most 131072, else 4 bytes x L x N / 1024). */
 RCD_API rcd_status rcd_partition_workspace_bytes(rcd_ctx *ctx, rcd_feat_dtype dtype, int64_t N, int64_t d,
                                          int32_t L, int64_t M_max, int32_t W, size_t *bytes_out);
 

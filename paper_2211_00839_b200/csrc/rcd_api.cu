@@ -143,7 +143,7 @@ size_t layout_workspace(void *base, rcd_feat_dtype dtype, const Sizes &sz, Works
     return w.bytes;
 }
 
-static int32_t chunks_for(int64_t N) { return (int32_t)((N + group_chunk(N) - 1) / group_chunk(N)); }
+static int32_t chunks_for(int64_t N, int64_t labels) { return (int32_t)((N + group_chunk(N, labels) - 1) / group_chunk(N, labels)); }
 
 // Sizes for the promise "no class larger than Mmax".
 static bool float_arith(const rcd_ctx *ctx, rcd_feat_dtype dtype)
@@ -168,7 +168,7 @@ static Sizes bound_sizes(const rcd_ctx *ctx, rcd_feat_dtype dtype, int64_t N, in
     sz.maxM = Mmax;
     sz.sElems = N * (int64_t)pad_row(Mmax);               // sum M_l * ld_l <= N * pad_row(Mmax)
     sz.vElems = (int64_t)W * (N + 7LL * L);               // sum W * ld_l,  ld_l <= M_l + 7
-    sz.nChunks = chunks_for(N);
+    sz.nChunks = chunks_for(N, L);
     sz.pitch = features_pitch(ctx, dtype, d);
     return sz;
 }
@@ -246,7 +246,7 @@ static rcd_status prepare(rcd_ctx *ctx, const void *features, rcd_feat_dtype dty
     if (((uintptr_t)workspace) % kAlign != 0) return fail(ctx, RCD_ERR_INVALID_ARG, "workspace must be 256-byte aligned");
     // head of the workspace: status, counts, what the host will send, the split's tables
     Sizes head{};
-    head.N = N; head.d = d; head.L = L; head.W = W; head.nChunks = chunks_for(N);
+    head.N = N; head.d = d; head.L = L; head.W = W; head.nChunks = chunks_for(N, L);
     head.floatArith = float_arith(ctx, dtype);
     head.graphCut = ctx->cfg.objective == RCD_OBJ_GRAPH_CUT;
     head.pitch = features_pitch(ctx, dtype, d);
@@ -541,7 +541,7 @@ static size_t layout_lists(void *base, int64_t N, int32_t W, ListsWorkspace *out
     const size_t Wn = (size_t)std::max<int32_t>(W, 1);
     w.status = c.take<int32_t>(4);
     w.counts = c.take<int32_t>(Wn);
-    w.chunkHist = c.take<int32_t>((size_t)std::max<int32_t>(chunks_for(N), 1) * Wn);
+    w.chunkHist = c.take<int32_t>((size_t)std::max<int32_t>(chunks_for(N, W), 1) * Wn);
     w.bytes = align_up(c.off);
     if (out) *out = w;
     return w.bytes;

@@ -9,7 +9,7 @@
 namespace rcd {
 
 // ---- stable split ---------------------------------------------------------------------------
-// Chunks of consecutive samples (group_chunk(N) of them).  Three launches:
+// Chunks of consecutive samples (group_chunk samples each).  Three launches:
 //   histogram  a CTA per chunk counts its labels in shared memory, writes chunkHist[chunk][label] and adds to counts[label];
 //   scan       per label, exclusive running sum over the chunks, started at the class offset;
 //   place      position = chunk base + rank inside the chunk; the CTA then copies its feature rows to their places.
@@ -18,7 +18,7 @@ namespace rcd {
 // 1155 -> 40 us).  More labels than that take the kernels at the end of this section.
 constexpr int kGroupThreads = 256;
 constexpr int kGroupWarps = kGroupThreads / 32;
-constexpr int kMaxSharedLabels = 6000;      // kGroupWarps counters per label: 192 KB
+static_assert(kGroupWarps * kMaxSharedLabels * 4 <= 192 * 1024, "counters in shared memory");
 
 __global__ void __launch_bounds__(kGroupThreads) label_hist_kernel(const int32_t *__restrict__ labels, int64_t N, int32_t L, int32_t chunk,
                                                                   int32_t *__restrict__ chunkHist, int32_t *__restrict__ counts,
@@ -259,7 +259,7 @@ rcd_status launch_label_hist(rcd_ctx *ctx, const int32_t *labels, int64_t N, int
         if (callStatus) RCD_CUDA(ctx, cudaMemsetAsync(callStatus, 0, sizeof(int32_t), st));
         return RCD_OK;
     }
-    const int chunk = group_chunk(N);
+    const int chunk = group_chunk(N, L);
     const unsigned nChunks = (unsigned)((N + chunk - 1) / chunk);
     if (shared_labels(L)) {
         const size_t smem = (size_t)L * 4;
@@ -287,7 +287,7 @@ rcd_status launch_stable_split(rcd_ctx *ctx, const int32_t *labels, int64_t N, i
         if (offsets) RCD_CUDA(ctx, cudaMemsetAsync(offsets, 0, (size_t)(L + 1) * sizeof(int64_t), st));
         return RCD_OK;
     }
-    const int chunk = group_chunk(N);
+    const int chunk = group_chunk(N, L);
     const int nChunks = (int)((N + chunk - 1) / chunk);
     label_scan_kernel<<<(L + 31) / 32, 1024, 0, st>>>(chunkHist, nChunks, L, descDev, counts, offsets, status);
     ctx->kernelLaunches++;

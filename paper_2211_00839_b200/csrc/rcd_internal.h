@@ -162,9 +162,12 @@ struct Sizes {
     bool graphCut;          // graph-cut objective: the gains array holds 8-byte ties
 };
 
-// Samples per chunk of the stable class split: small chunks while that is what fills the SMs, large ones where the
-// per-chunk tables (chunks x labels) would grow.
-inline int group_chunk(int64_t N) { return N <= 131072 ? 256 : 1024; }
+// Labels whose counters the class split keeps in shared memory: one per warp of a CTA and label, 192 KB.
+constexpr int kMaxSharedLabels = 6000;
+// Samples per chunk of the stable class split: small chunks while that is what fills the SMs, large ones where the table of
+// chunks x labels, which is cleared and summed up on every call, would pass 64 MB (lists of 131072 samples over 20000 labels,
+// 41 MB: 101 us, large chunks 126; over 100000, 205 MB: 923 us, large chunks 468).
+inline int group_chunk(int64_t N, int64_t labels) { return N <= 131072 && (N + 255) / 256 * labels <= 1 << 24 ? 256 : 1024; }
 // Bytes between the class-sorted feature rows: whole 16-byte pieces, at least one 128-byte slab, so that every width can
 // be loaded by the tensor-core kernel (the padding is zeros and adds nothing to a dot product).
 inline int64_t row_pitch(int64_t rowBytes) { return rowBytes <= 128 ? 128 : (rowBytes + 15) / 16 * 16; }

@@ -35,6 +35,19 @@ def test_worker_lists_match_the_definition(rcd, orc, N, W, seed):
     assert np.array_equal(idx, want_idx)
 
 
+@pytest.mark.parametrize("N,W", [(131072, 32768), (131072, 32769), (131073, 6001)])
+def test_worker_lists_at_the_edges_of_the_chunk_size(rcd, N, W):
+    """Chunks of 256 samples while the table of chunks x workers stays within 64 MB, else of 1024; the caller's workspace follows."""
+    import torch
+    a = np.random.default_rng(W).integers(0, W, size=N).astype(np.int32)
+    with rcd.Context(0) as ctx:
+        off, idx = rcd.rcd_worker_lists(ctx, torch.from_numpy(a).cuda(), W)
+        ctx.sync_status()
+        assert ctx._ws.numel() <= (1 << 26) + (1 << 20)
+        off, idx = off.cpu().numpy(), idx.cpu().numpy()
+    assert np.array_equal(idx, np.argsort(a, kind="stable")) and np.array_equal(off, np.concatenate([[0], np.cumsum(np.bincount(a, minlength=W))]))
+
+
 def test_worker_lists_of_a_partition(rcd, orc):
     """From rcd_partition's own output: list sizes are the quota sums over the classes."""
     import torch
