@@ -8,7 +8,7 @@
  *   - "dev" pointers are CUDA device pointers on the context's device; "host"
  *     pointers are ordinary host memory.  The caller owns every buffer,
  *     including the workspace; the library never frees them and reads nothing of them after the
- *     call's last kernel (the device-side status of a call is copied into the context).
+ *     call's last kernel (the kernels report their status to a word that the context owns).
  *   - `cuda_stream` is a cudaStream_t passed as void* (NULL = default stream).
  *     Unless stated otherwise a call only enqueues work on that stream and
  *     returns; outputs are valid once the stream has been synchronised.
@@ -53,7 +53,9 @@ typedef enum {
 /* Feature element type.  It also fixes the arithmetic of everything downstream:
  *   RCD_FEAT_I8   int8 features, S = dot product in int32 (exact), gains and f in int64 (exact);
  *   RCD_FEAT_BF16 bfloat16 features (rows L2-normalised by the caller, so the dot product is the
- *                 cosine), S accumulated and stored in fp32, gains in fp32, f tracked in fp64.  */
+ *                 cosine), S accumulated and stored in fp32.  Gains and f: sums in 64-bit fixed point where the
+ *                 library chooses the cluster form (S rounded to 2^-30 of the class's largest squared norm; norms
+ *                 of a class within a factor of four), else gains in fp32 and f tracked in fp64.  */
 typedef enum { RCD_FEAT_I8 = 0, RCD_FEAT_BF16 = 1 } rcd_feat_dtype;
 
 /* Similarity sim(v, v') of Section 4 item 2.
@@ -140,7 +142,8 @@ typedef struct {
     int64_t async_visits;           /* asynchronous form: times the first sweep CTA went to a class and swept there */
     int64_t async_attempts;         /* ... and times it tried (an attempt fails when the tickets run out under way) */
     int64_t lazy_sweeps;            /* threshold passes that skipped rows below the blocks' floors */
-    int64_t lazy_misses;            /* picks whose best stored gain lay below its block's floor (answered by a pass over every row) */
+    int64_t lazy_misses;            /* picks whose best stored gain lay below its block's floor (answered by a pass over every row);
+                                       cluster form: times a block's leading candidates had all been taken (answered by a scan) */
     int64_t lazy_rows;              /* rows of S those passes did read */
     int64_t lazy_rows_skipped;      /* rows they did not */
     int64_t incremental_updates;    /* picks after which the block's stored gains were corrected in place (no pass needed) */

@@ -360,7 +360,7 @@ __device__ __forceinline__ int list_raised(const TeamView &t, int32_t *count, in
 }
 
 // Four listed columns taken off the stored gains of one piece.  Their losses (each below 2^30) add up in 32 bits, so that
-// widening and subtracting is paid once for four: 156 cycles of arithmetic per row of 20 KB and SM, 248 with two at a time.
+// widening and subtracting is paid once for four.
 __device__ __forceinline__ uint32_t apply_four(const int4 &x, const int4 &y, const int4 &z, const int4 &w, const Raised &a, const Raised &b,
                                                const Raised &c, const Raised &d, unsigned long long (&g)[4])
 {
@@ -382,9 +382,9 @@ __device__ __forceinline__ Raised entry_or_none(const Raised *list, int e, int n
     return r;
 }
 
-// The n listed columns taken off one piece, rows straight to registers, up to sixteen in flight
-// (a warp waits about 1100 cycles for a batch; with sixteen warps at it a row of 5 KB takes an SM about 140 cycles, the share
-// of the copy bandwidth that 148 SMs get).
+// The n listed columns taken off one piece, rows straight to registers, up to sixteen in flight: sixteen warps of an SM then
+// cover the trip to L2 or HBM (1000 classes of 1300 into 64 blocks, 148 SMs: 886 GB of rows in 160 ms, 0.85 of the copy
+// bandwidth; 100 of 500 into 32 blocks, S in L2: 6.9 GB to the SMs in 1.39 ms).
 __device__ __forceinline__ bool correct_piece(const int4 *S4q, const Raised *list, int n, unsigned long long (&g)[4])
 {
     uint32_t changed = 0;
@@ -422,9 +422,9 @@ __device__ __forceinline__ bool correct_piece(const int4 *S4q, const Raised *lis
 // The same for a team that keeps its P pieces per thread in registers.  The rows travel through asynchronous copies in
 // shared memory, each thread reading back only what it copied itself, so that loads in flight hold no registers.
 // Up to three pieces: row by row over all pieces (a list entry and a row's address serve them all), eight rows of room,
-// four under way while four are applied: 403 cycles per row of 20 KB and SM with 80 SMs at it, of which L2 and HBM take 350
-// (538 with two rows at a time).  More pieces, or less room: piece by piece through a ring of sixteen 16-byte slots per
-// thread, twelve under way (530 cycles; 620 with eight).
+// four under way while four are applied (10 classes of 5000 into 8 blocks, 80 SMs: 20.5 GB to the SMs in 7.5 ms, of which the
+// first thousand picks of a class draw most).  More pieces, or less room: piece by piece through a ring of sixteen 16-byte
+// slots per thread, twelve under way.
 template <int P> struct RowRing { static constexpr bool byRow = P <= 3; };
 constexpr int kRowStages = 8, kPieceStages = 16;
 template <int P, int kT>

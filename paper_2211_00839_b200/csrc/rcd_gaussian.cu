@@ -70,8 +70,9 @@ __device__ __forceinline__ double root_fp64(float v)
     return v > 0.f && v < INFINITY ? s : d;
 }
 
-// Both passes over S below give a CTA 64 rows of a class and its warps 128 columns at a time, four per lane: the norms of a
-// lane's columns stay in registers down the 64 rows, those of the rows sit in shared memory, and S moves in 128-bit pieces.
+// Both passes over S below give a CTA some rows of a class (sums 64, values 16) and its warps 128 columns at a time, four per
+// lane: the norms of a lane's columns stay in registers down the rows, those of the rows sit in shared memory, and S moves in
+// 128-bit pieces.
 
 // Sums of distances.  They are symmetric, so only the columns right of the diagonal are read and rooted (sigma counts each
 // pair twice).  Bound by the square roots in fp64: 212 us at 10 classes of 5000, 1 GB of S (338 with one row in flight per

@@ -191,8 +191,8 @@ inline int64_t sim_tiles(int64_t M, bool pairs)
     return n;
 }
 // Units of work on pairs of SMs: tiles, as long as they fill rounds of one per pair; those left over are cut into 2, 4 or 8
-// strips of columns, which share the last round out to more pairs (100 classes of 500 x 2048: 300 tiles on 74 pairs leave 4;
-// 85 -> 82 us).
+// strips of columns, which share the last round out to more pairs (100 classes of 500 x 2048: 300 tiles on 74 pairs leave 4, a
+// round of a quarter of a tile each instead of a whole one).
 struct PairUnits { int whole, strips, count; };
 __host__ __device__ inline PairUnits pair_units(int tiles, int pairs)
 {

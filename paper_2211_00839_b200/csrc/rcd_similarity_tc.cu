@@ -398,9 +398,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) sim_tc_kernel(const __grid_cons
 // Long rows: a pair of SMs per 256 x 256 tile (cta_group::2).  Each CTA holds 128 of the tile's rows (A and the accumulator)
 // and half of its columns (B), so every operand row comes in once: 32 KB per SM and k-slab, 16 on the diagonal, where both
 // operands are the same rows, against 48 and 32 above.  CTA 0 issues the MMAs of both.  Tiles on the diagonal are computed
-// whole and stored as they are, the others stored twice.  Bound by the tensor cores: a slab takes 0.43 us where its MMAs
-// alone take 0.37 at the rate of a large cuBLAS product.  100 classes of 500 x 2048 bf16: 92 -> 82 us (67 GFLOP, at least
-// 40 us; writing S and reading X, 47), 300 of 200 x 1024: 55 -> 48.
+// whole and stored as they are, the others stored twice.  Bound by the tensor cores: their pipe is active 60 % of the time an SM
+// has work.  100 classes of 500 x 2048 bf16: 78.7 us, the 128 x 256 kernel above 85.0 (both under the profiler; 67 GFLOP, at
+// least 40 us; writing S and reading X, 47).
 constexpr int kPairStages = 6;
 constexpr int kPairStageBytes = 2 * kOperandBytes;
 constexpr int kPairTile = 256;
