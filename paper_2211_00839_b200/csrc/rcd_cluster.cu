@@ -1587,6 +1587,9 @@ rcd_status launch_greedy_cluster(rcd_ctx *ctx, ClusterPlan &plan, const Sizes &s
     volatile int32_t *const left = ctx->hostStage + ctx->hostStageInts + kStageLeft;
     const bool toFix = sz.floatArith && ctx->cfg.similarity_kind != RCD_SIM_GAUSSIAN;     // (the Gaussian kernel writes fixed point itself)
     if (toFix) {
+        // (a class may have to be left to the forms with passes: whether a call is refused is not to depend on its features)
+        const rcd_status fits = check_coverage_fits(ctx, prm.maxLd);
+        if (fits != RCD_OK) return fits;
         *left = 0;
         fixed_exponent_kernel<<<sz.L, 256, 0, st>>>(ws.desc, (const float *)ws.S, ws.fixedExp, ws.sizesLeft, left);
         RCD_CUDA(ctx, cudaEventRecord(ctx->evCounts, st));

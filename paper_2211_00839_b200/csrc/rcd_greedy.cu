@@ -2419,6 +2419,14 @@ static cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
 
+static int64_t pass_smem_cap(const rcd_ctx *ctx) { return (int64_t)ctx->maxSmemOptin - 24 * 1024; }     // static shared of the kernels + margin
+rcd_status check_coverage_fits(rcd_ctx *ctx, int maxLd)
+{
+    if ((int64_t)maxLd * 4 <= pass_smem_cap(ctx)) return RCD_OK;
+    return fail(ctx, RCD_ERR_UNSUPPORTED, "class of %d samples: one coverage vector (%lld bytes) exceeds the %lld bytes of shared memory",
+                maxLd, (long long)maxLd * 4, (long long)pass_smem_cap(ctx));
+}
+
 template <typename SV>
 static rcd_status run_greedy(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws,
                              const std::vector<ClassDesc> &descHost, int32_t *assignment, int32_t *order,
@@ -2497,7 +2505,7 @@ static rcd_status run_greedy(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws,
     }
     int maxLd = 0;
     for (const auto &c : descHost) if (c.ld > maxLd) maxLd = c.ld;
-    const int64_t smemCap = (int64_t)ctx->maxSmemOptin - 24 * 1024;  // static shared of the kernels + margin
+    const int64_t smemCap = pass_smem_cap(ctx);
     int64_t smem = (int64_t)batch * maxLd * (int64_t)sizeof(SV);
     if (prm.sparseMinMembers >= 0)                                   // threshold pass: one vector + the warps' rings and queues
         smem = std::max<int64_t>(smem, (int64_t)thr_bytes_aligned(maxLd * (int)sizeof(SV)) + kSparseQueueBytes);
@@ -2509,10 +2517,8 @@ static rcd_status run_greedy(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws,
     }
     if (only) smem = std::max<int64_t>(smem, (int64_t)sizeof(PlanShared<FV>));       // (the owner kernel sets its classes up there)
     if (smem > smemCap) smem = smemCap;
-    if ((int64_t)maxLd * (int64_t)sizeof(SV) > smem)
-        return fail(ctx, RCD_ERR_UNSUPPORTED,
-                    "class of %d samples: one coverage vector (%lld bytes) exceeds the %lld bytes of shared memory",
-                    maxLd, (long long)maxLd * (long long)sizeof(SV), (long long)smem);
+    const rcd_status fits = check_coverage_fits(ctx, maxLd);
+    if (fits != RCD_OK) return fits;
     if (smem < 16) smem = 16;
     prm.smemBytes = (int32_t)smem;
     // 32-bit partial sums take terms below 16384*d each, four per chunk iteration

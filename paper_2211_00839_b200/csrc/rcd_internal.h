@@ -288,6 +288,9 @@ rcd_status launch_greedy(rcd_ctx *ctx, rcd_feat_dtype dtype, const Sizes &sz, co
                          const std::vector<ClassDesc> &descHost, int32_t *assignment, int32_t *order,
                          cudaStream_t st);
 
+// whether the forms with passes over S hold a class's coverage vector of one block in shared memory
+rcd_status check_coverage_fits(rcd_ctx *ctx, int maxLd);
+
 // the floating-point classes that the cluster form left (ws.fixedExp[l] == kNotFixed)
 rcd_status launch_greedy_not_fixed(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, const std::vector<ClassDesc> &descHost,
                                    int32_t *assignment, int32_t *order, void *partValues, cudaStream_t st);

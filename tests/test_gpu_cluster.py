@@ -91,6 +91,17 @@ def test_float_norms_far_apart(rcd, orc):
     check_float(rcd, orc, wl)
 
 
+def test_float_class_beyond_the_passes_is_refused(rcd):
+    """Bf16 classes that the forms with passes cannot hold are refused whatever their norms, although the cluster form could run
+    one whose norms lie close together (zero rows here)."""
+    import torch
+    X = torch.zeros((51976, 64), dtype=torch.bfloat16, device="cuda")
+    y = torch.zeros(51976, dtype=torch.int32, device="cuda")
+    with rcd.Context(0) as ctx:
+        with pytest.raises(rcd.RcdError, match="coverage vector"):
+            ctx.rcd_partition(X, y, [1.0, 2.0], 1)
+
+
 @pytest.mark.parametrize("sizes,W,apart", [([900, 700], 6, 2), ([1200, 33, 700], 24, 3), ([600, 300, 1, 500], 100, 2)])
 def test_float_norms_far_apart_on_all_sms(rcd, orc, sizes, W, apart):
     """Few classes left in floating point are swept by every SM, as they are when the asynchronous form is asked for; the first
