@@ -33,7 +33,8 @@ if ROOT not in sys.path:
 
 
 # DRAM bytes (read + write) of one launch of the dominant kernel under ncu, by (configuration, kernel).
-MEASURED_TRAFFIC = {("C2", "greedy_async_kernel"): 41.62e9}     # profiles/greedy_async_kernel_C2.md, capture A
+MEASURED_TRAFFIC = {("C2", "greedy_async_kernel"): 41.62e9,     # profiles/greedy_async_kernel_C2.md, capture A
+                    ("C2", "greedy_cluster_kernel"): 11.47e9}   # profiles/greedy_cluster_kernel.md
 
 
 def load_peaks():
@@ -322,9 +323,11 @@ def run_ours(args):
         yard = box[0]
     default_setup = args.classes == 0 and args.sweep_batch in (0, 8) and args.async_group == 0 and args.async_help_min == 0 and args.similarity == "dot"
     loop_s = prof["greedy_ms"] * 1e-3
-    # The cluster form makes no sweeps: it reads the row of S of every pick and one per column that the pick raised.
-    clustered = prof["sweep_bytes"] == 0 and prof["incremental_rows"] > 0
-    loop_bytes = 4 * ((M + 7) // 8 * 8) * (prof["incremental_rows"] + prof["incremental_updates"]) if clustered else prof["sweep_bytes"]
+    # The cluster form makes no sweeps: it reads every row of S once for the gains of empty blocks, then the row of S of every
+    # pick and one per column that the pick raised.  (Rows fetched on foresight whose sample another block received are not
+    # counted: see the traffic of the capture.)
+    clustered = prof["sweep_bytes"] == 0 and prof["incremental_updates"] > 0
+    loop_bytes = 4 * ((M + 7) // 8 * 8) * (wl.N + prof["incremental_rows"] + prof["incremental_updates"]) if clustered else prof["sweep_bytes"]
     achieved = loop_bytes / loop_s / 1e9 if loop_s > 0 else 0.0
     sms = torch.cuda.get_device_properties(local).multi_processor_count
     path = args.greedy_path if args.greedy_path else (3 if wl.L * 4 <= sms else 4)
