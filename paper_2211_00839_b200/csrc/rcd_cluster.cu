@@ -383,7 +383,7 @@ __device__ __forceinline__ Raised entry_or_none(const Raised *list, int e, int n
 }
 
 // The n listed columns taken off one piece, rows straight to registers, up to sixteen in flight: sixteen warps of an SM then
-// cover the trip to L2 or HBM (1000 classes of 1300 into 64 blocks, 148 SMs: 886 GB of rows in 160 ms, 0.85 of the copy
+// cover the trip to L2 or HBM (1000 classes of 1300 into 64 blocks, 148 SMs: 895 GB of rows in 162 ms, 0.85 of the copy
 // bandwidth; 100 of 500 into 32 blocks, S in L2: 6.9 GB to the SMs in 1.39 ms).
 __device__ __forceinline__ bool correct_piece(const int4 *S4q, const Raised *list, int n, unsigned long long (&g)[4])
 {

@@ -58,7 +58,7 @@ __device__ __forceinline__ float squared_distance(uint32_t ni, uint32_t nj, uint
     }
 }
 
-// Square root to the last bits of fp64: Heron's step s += (v - s s) / (2 s) twice, with the fp32 reciprocal root standing in for
+// Square root within a unit in the last place of fp64: Heron's step s += (v - s s) / (2 s) twice, with the fp32 reciprocal root standing in for
 // 1 / s: 22 bits right, then 44, then all that the format holds.  No branches (zeros and infinities are their own roots).
 __device__ __forceinline__ double root_fp64(float v)
 {
