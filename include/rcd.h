@@ -63,8 +63,8 @@ typedef enum { RCD_FEAT_I8 = 0, RCD_FEAT_BF16 = 1 } rcd_feat_dtype;
  *   RCD_SIM_GAUSSIAN  exp(-||v - v'||^2 / (2 sigma^2)) with sigma = the mean of ||v - v'||_2 over all ordered
  *                     pairs of the class (the paper's Gaussian kernel; exponent and the range of the mean are
  *                     readings, the paper gives neither).  S is then fp32 in (0, 1] for either feature type,
- *                     and everything downstream uses the floating-point arithmetic of RCD_FEAT_BF16
- *                     (gains fp32, tracked f and all objective outputs double).  */
+ *                     and everything downstream uses the arithmetic of RCD_FEAT_BF16 (tracked f and all
+ *                     objective outputs double).  */
 typedef enum { RCD_SIM_DOT = 0, RCD_SIM_GAUSSIAN = 1 } rcd_similarity_kind;
 
 /* Submodular function f used by GreedyStep and by the argmin over blocks (Section 4 item 2).
