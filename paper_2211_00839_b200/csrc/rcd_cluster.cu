@@ -1,5 +1,6 @@
 // The greedy loop of Algorithm 1 with the facility-location objective, one thread-block cluster per class: the form
-// the library chooses by itself (the pass-based forms of rcd_greedy.cu serve explicit configurations).
+// the library chooses by itself, except where classes run in rounds (rcd_rounds.cu: enough classes to fill the SMs one by one,
+// and many blocks).  The pass-based forms of rcd_greedy.cu serve explicit configurations.
 //
 // What bounds it.  A pick of block j depends on the previous pick of block j (its coverage and gains change), but on
 // picks of OTHER blocks only through two things: the tracked values f (which block is next) and the set of unassigned
@@ -16,7 +17,7 @@
 // Stored gains are always exact: a pick corrects those of its block from one row of S per column whose coverage it
 // raised (S is symmetric).  All arithmetic is int64 on int32 similarities, hence independent of the order in which
 // anything happens: results do not depend on timing.
-#include "rcd_internal.h"
+#include "rcd_exact.cuh"
 
 #include <limits.h>
 #include <algorithm>
@@ -62,12 +63,6 @@ struct NoteLayout {
     __host__ __device__ uint32_t tracked() const { return (uint32_t)(1 + entries() + T) * 8; }   // bytes a new note brings
 };
 
-struct __align__(16) Raised {
-    int32_t row;                          // a column whose coverage rose: its row of S, in 16-byte pieces from the class's first
-    int32_t minusOld, by;                 // - old coverage, new - old
-    int32_t pad_;
-};
-
 struct Team {
     unsigned long long best[kMaxWarps];
     int32_t count[4];                     // lengths of its lists: foreseen samples (in turn), others
@@ -105,7 +100,6 @@ struct ClusterParams {
 };
 
 namespace {
-__device__ __forceinline__ uint32_t smem32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ uint32_t remote(uint32_t addr, uint32_t rank)
 {
     uint32_t r;
@@ -171,76 +165,12 @@ __device__ __forceinline__ void team_barrier(int team, int T)
     else asm volatile("bar.sync %0, %1;" :: "r"(1 + team), "r"(T * 32) : "memory");
 }
 
-__device__ __forceinline__ int4 ld_row_shared(const int4 *p)       // (other teams of the CTA read the same rows: L1 may serve them)
-{
-    int4 v;
-    asm volatile("ld.global.nc.v4.s32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
-    return v;
-}
-__device__ __forceinline__ int4 ld_row_once(const int4 *p)
-{
-    int4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.s32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
-    return v;
-}
-
-// acc + x on the multiply-add pipe (the maxima occupy the other one)
-__device__ __forceinline__ unsigned long long add_wide(int x, uint32_t one, unsigned long long acc)
-{
-    unsigned long long r;
-    asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(r) : "r"((uint32_t)x), "r"(one), "l"(acc));
-    return r;
-}
-
 // g - l (one multiply-add)
 __device__ __forceinline__ unsigned long long take_off(unsigned long long g, int l)
 {
     unsigned long long r;
     asm("mad.wide.s32 %0, %1, -1, %2;" : "=l"(r) : "r"(l), "l"(g));
     return r;
-}
-
-// Sum of a value below 2^43 per lane over the warp.
-__device__ __forceinline__ unsigned long long warp_sum(unsigned long long x)
-{
-    const uint32_t lo = __reduce_add_sync(0xffffffffu, (uint32_t)(x & 0xffffffu));
-    const uint32_t hi = __reduce_add_sync(0xffffffffu, (uint32_t)(x >> 24));
-    return ((unsigned long long)hi << 24) + lo;
-}
-
-// A gain and a sample as one key: greater gain first, lower sample among equals.  Gains stay below 2^47 (at most 2^16
-// samples, similarities below 2^31).
-__device__ __forceinline__ unsigned long long make_key(unsigned long long g, int v) { return (g << 16) | (unsigned long long)(65535 - v); }
-__device__ __forceinline__ int key_sample(unsigned long long k) { return 65535 - (int)(k & 0xffffull); }
-
-__device__ __forceinline__ unsigned long long umax(unsigned long long a, unsigned long long b) { return a > b ? a : b; }
-__device__ __forceinline__ unsigned long long umin(unsigned long long a, unsigned long long b) { return a < b ? a : b; }
-
-// A row's contribution by one warp: sum_i max(0, S[v][i]), or for the graph cut sum_i S[v][i] and sum_i |S[v][i]|.
-template <bool kCut>
-__device__ __forceinline__ unsigned long long row_value(const int4 *row, int ld4, int lane, uint32_t one, unsigned long long &negative)
-{
-    unsigned long long acc = 0, neg = 0;
-    for (int q = lane; q < ld4; q += 8 * 32) {
-        int4 x[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) x[u] = q + u * 32 < ld4 ? ld_row_once(row + q + u * 32) : make_int4(0, 0, 0, 0);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            acc = add_wide(max(x[u].x, 0), one, acc);
-            acc = add_wide(max(x[u].y, 0), one, acc);
-            acc = add_wide(max(x[u].z, 0), one, acc);
-            acc = add_wide(max(x[u].w, 0), one, acc);
-            if (kCut) {
-                neg = add_wide(max(-x[u].x, 0), one, neg);
-                neg = add_wide(max(-x[u].y, 0), one, neg);
-                neg = add_wide(max(-x[u].z, 0), one, neg);
-                neg = add_wide(max(-x[u].w, 0), one, neg);
-            }
-        }
-    }
-    negative = kCut ? warp_sum(neg) : 0ull;
-    return warp_sum(acc);
 }
 
 // The team of a warp, and what it knows while it works on a class.
@@ -254,14 +184,6 @@ struct TeamView {
     const uint32_t *bits;      // assigned samples (and everything from M on)
 };
 
-// 16 bytes global -> shared without passing through registers
-__device__ __forceinline__ void copy16(int4 *dst, const int4 *src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(smem32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N> __device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_group %0;" :: "n"(N) : "memory"); }
-
 // Starts copying the team's pieces of row v into its row buffer.
 __device__ __forceinline__ void fetch_row(const TeamView &t, int v)
 {
@@ -269,10 +191,6 @@ __device__ __forceinline__ void fetch_row(const TeamView &t, int v)
     for (int q = t.warpIn * 32 + t.lane; q < t.ld4; q += t.T * 32) copy16(t.rowBuf + q, row + q);
     copies_commit();
 }
-
-// What a candidate loses for one raised column: min(max(x, old), new) - old, as one instruction.  Similarities stay
-// below 2^30 either way, so x - old does not wrap, and two losses fit an int.
-__device__ __forceinline__ int loss(int x, const Raised &e) { return __viaddmin_s32_relu(x, e.minusOld, e.by); }
 
 // The leading candidates among a thread's columns.  64-bit comparisons cost five instructions at half rate, so gains are
 // compared by their leading 32 bits first (gain >> shift, with shift such that the block's largest gain fits) and, among
@@ -1406,6 +1324,7 @@ struct ClusterPlan {
     int C, clusters, P;        // CTAs per cluster, clusters, pieces per thread (0: several blocks per warp)
     bool smemState;
     size_t smem;
+    std::shared_ptr<RoundsPlan> rounds;   // not null: the classes run in rounds instead, one CTA each
     ClusterParams prm;         // teamWarps, slots, maxLd, rowPieces and the offsets are set
 };
 static size_t cluster_layout(const Sizes &sz, int maxLd, int C, bool state, size_t cap, ClusterPlan &plan)
@@ -1501,6 +1420,9 @@ static bool cluster_plan(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassD
     }
     const size_t cap = (size_t)ctx->maxSmemOptin - 1024;
     plan.prm = ClusterParams{};
+    plan.prm.maxLd = maxLd;
+    plan.rounds = plan_greedy_rounds(ctx, sz, descHost);
+    if (plan.rounds) return true;
     for (int i = 0; i < 5; ++i)
         if (ctx->maxClusters[i] < 0) {
             int active = 0;
@@ -1599,11 +1521,16 @@ rcd_status launch_greedy_cluster(rcd_ctx *ctx, ClusterPlan &plan, const Sizes &s
         ctx->kernelLaunches += 2;
         RCD_CUDA(ctx, cudaGetLastError());
     }
-    ClusterKernel kernel = sz.graphCut ? (sz.W <= 32 ? pick_kernel<1, true>(plan.P, prm.teamWarps, plan.smemState) : pick_kernel<4, true>(plan.P, prm.teamWarps, plan.smemState))
-                                       : (sz.W <= 32 ? pick_kernel<1, false>(plan.P, prm.teamWarps, plan.smemState)
-                                          : sz.W <= 64 ? pick_kernel<2, false>(plan.P, prm.teamWarps, plan.smemState) : pick_kernel<4, false>(plan.P, prm.teamWarps, plan.smemState));
-    const rcd_status rs = launch_cluster(ctx, kernel, prm, (plan.P == 0 ? kMaxWarps + 1 + kListers : team_warps(prm.teamWarps) + 1) * 32, plan.C, plan.clusters, plan.smem, st, nullptr);
-    if (rs != RCD_OK) return rs;
+    if (plan.rounds) {
+        const rcd_status rs = launch_greedy_rounds(ctx, *plan.rounds, sz, ws, assignment, order, partValues, st);
+        if (rs != RCD_OK) return rs;
+    } else {
+        ClusterKernel kernel = sz.graphCut ? (sz.W <= 32 ? pick_kernel<1, true>(plan.P, prm.teamWarps, plan.smemState) : pick_kernel<4, true>(plan.P, prm.teamWarps, plan.smemState))
+                                           : (sz.W <= 32 ? pick_kernel<1, false>(plan.P, prm.teamWarps, plan.smemState)
+                                              : sz.W <= 64 ? pick_kernel<2, false>(plan.P, prm.teamWarps, plan.smemState) : pick_kernel<4, false>(plan.P, prm.teamWarps, plan.smemState));
+        const rcd_status rs = launch_cluster(ctx, kernel, prm, (plan.P == 0 ? kMaxWarps + 1 + kListers : team_warps(prm.teamWarps) + 1) * 32, plan.C, plan.clusters, plan.smem, st, nullptr);
+        if (rs != RCD_OK) return rs;
+    }
     ctx->steps = sz.maxM;
     ctx->phaseNsDev = ws.phaseNs;
     if (toFix) RCD_CUDA(ctx, cudaEventSynchronize(ctx->evCounts));

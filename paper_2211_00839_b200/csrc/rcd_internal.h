@@ -301,6 +301,12 @@ std::shared_ptr<ClusterPlan> plan_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, 
 rcd_status launch_greedy_cluster(rcd_ctx *ctx, ClusterPlan &plan, const Sizes &sz, const Workspace &ws, const std::vector<ClassDesc> &descHost,
                                  int32_t *assignment, int32_t *order, void *partValues, cudaStream_t st);
 
+// greedy loop in rounds, one CTA per class (null: it does not take the problem)
+struct RoundsPlan;
+std::shared_ptr<RoundsPlan> plan_greedy_rounds(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost);
+rcd_status launch_greedy_rounds(rcd_ctx *ctx, RoundsPlan &plan, const Sizes &sz, const Workspace &ws, int32_t *assignment, int32_t *order,
+                                void *partValues, cudaStream_t st);
+
 rcd_status launch_bounded_wait_selftest(rcd_ctx *ctx, unsigned *counter, int32_t *status, cudaStream_t st);
 
 // graph-cut objective: the whole greedy loop, and f from an assignment

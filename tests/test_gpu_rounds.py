@@ -1,0 +1,48 @@
+"""The greedy loop in rounds (taken where classes of about one size fill the SMs one by one and blocks are many) at the edges of its
+tiles, batches, lists and shared memory, against the oracle or the pass-based form."""
+import numpy as np
+import pytest
+
+import test_gpu_cluster as cluster
+from test_gpu_parity import check_exact, check_float, rcd, orc  # noqa: F401  (fixtures)
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("sizes,d,W", [
+    ([37] * 97, 16, 64),                          # fewer samples than blocks; batches of fewer blocks than wait (narrow features)
+    ([129, 128, 127, 126] * 25, 40, 48),          # edges of 128 columns
+    ([257] * 60, 75, 100),                        # more than 64 blocks: two batches a round
+    ([64] * 450, 24, 56),                         # two CTAs per SM
+    ([90] * 60 + [0, 1, 0], 16, 128),             # the most blocks; empty classes and one of a sample
+    ([333] * 98, 520, 61),                        # a last group of three columns, a number of blocks that is no multiple of four
+])
+@pytest.mark.parametrize("copies", [0, 30])
+def test_int8_exact(rcd, orc, sizes, d, W, copies):
+    check_exact(rcd, orc, cluster.workload(sizes, d, W, W + copies, copies=copies))
+
+
+@pytest.mark.parametrize("sizes,d,W", [([1000] * 148, 32, 16), ([1003] * 148, 256, 40), ([1610] * 140, 64, 49)])
+def test_int8_like_the_passes(rcd, sizes, d, W):
+    import torch
+    wl = cluster.workload(sizes, d, W, W)
+    X, y = rcd.features_to_torch(wl.features, device="cuda"), torch.from_numpy(wl.labels).cuda()
+    results = []
+    for path in (0, 4):
+        with rcd.Context(0, greedy_path=path) as ctx:
+            results.append(ctx.rcd_partition(X, y, wl.capacities, wl.L, M_max=max(sizes)))
+            ctx.sync_status()
+    for got, want in zip(*results):
+        assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("similarity", ["gaussian", "dot"])
+@pytest.mark.parametrize("sizes,W", [([101] * 98, 57), ([66] * 60, 70)])
+def test_float_is_exact_in_fixed_point(rcd, orc, similarity, sizes, W):
+    cluster.test_float_is_exact_in_fixed_point(rcd, orc, similarity, sizes, W)
+
+
+def test_float_norms_far_apart(rcd, orc):
+    """A class left in floating point beside those that run in rounds."""
+    wl = cluster.workload([141] + [140] * 99, 32, 60, 1, dtype="bf16", scale=lambda rng, M: 10.0 ** rng.uniform(-1.5 if M == 141 else 0.0, 1.5 if M == 141 else 0.1, M))
+    check_float(rcd, orc, wl)
