@@ -235,12 +235,14 @@ struct Prepared {
     Sizes sz{};
     Workspace ws{};
     std::vector<ClassDesc> desc;
+    bool covered = false;
     std::shared_ptr<ClusterPlan> cluster;   // null: another form of the greedy loop, or none
 };
 
-// capacities null: no quotas wanted.
+// capacities null: no quotas wanted.  blocks not null: the value of this assignment is wanted, and where S need not exist for that
+// (`covered`) the blocks' coverage is computed in its place.
 static rcd_status prepare(rcd_ctx *ctx, const void *features, rcd_feat_dtype dtype, int64_t N, int64_t d,
-                          const int32_t *labels, int32_t L, int32_t W, const double *capacities, void *workspace, size_t workspaceBytes,
+                          const int32_t *labels, int32_t L, int32_t W, const double *capacities, const int32_t *blocks, void *workspace, size_t workspaceBytes,
                           cudaStream_t st, Prepared *out)
 {
     if (((uintptr_t)workspace) % kAlign != 0) return fail(ctx, RCD_ERR_INVALID_ARG, "workspace must be 256-byte aligned");
@@ -311,7 +313,8 @@ static rcd_status prepare(rcd_ctx *ctx, const void *features, rcd_feat_dtype dty
         tiles += sim_tiles(P.desc[(size_t)l].M, false);
         pairTiles += sim_tiles(P.desc[(size_t)l].M, true);
     }
-    cls.pairs = sim_pairs(sz.pitch, maxM, tiles, pairTiles, ctx->smCount);
+    P.covered = blocks && !sz.graphCut && ctx->cfg.similarity_kind == RCD_SIM_DOT && ctx->cfg.similarity_path != 2;
+    cls.pairs = !P.covered && sim_pairs(sz.pitch, maxM, tiles, pairTiles, ctx->smCount);
     for (int32_t l = 0; l < L; ++l) {
         prefix[l] = (int32_t)cls.upperTiles;
         cls.upperTiles += sim_tiles(P.desc[(size_t)l].M, cls.pairs);
@@ -338,8 +341,15 @@ static rcd_status prepare(rcd_ctx *ctx, const void *features, rcd_feat_dtype dty
     const size_t firstBytes = early ? blobBytes : (size_t)((unsigned char *)hw.quota - (unsigned char *)hw.desc);
     RCD_CUDA(ctx, cudaMemcpyAsync(P.ws.desc, blob, firstBytes, cudaMemcpyHostToDevice, st));
     rs = launch_stable_split(ctx, labels, N, L, P.ws.chunkHist, P.ws.desc, nullptr, nullptr, nullptr, P.ws.perm,
-                             features, d * (int64_t)feat_bytes(dtype), sz.pitch, P.ws.Xs, st);
+                             P.covered ? nullptr : features, d * (int64_t)feat_bytes(dtype), sz.pitch, P.covered ? nullptr : P.ws.Xs, st);
     if (rs != RCD_OK) return rs;
+    if (P.covered) {
+        rs = launch_objective_order(ctx, sz, P.ws, blocks, st);
+        if (rs != RCD_OK) return rs;
+        rs = launch_gather_rows(ctx, features, P.ws.cand, N, d * (int64_t)feat_bytes(dtype), sz.pitch, P.ws.Xs, st);
+        if (rs != RCD_OK) return rs;
+        return launch_similarity_maxima(ctx, P.ws.Xs, dtype, N, sz.pitch / (int64_t)feat_bytes(dtype), cls, P.ws.pos, (int32_t *)P.ws.cover, st);
+    }
     if (ctx->cfg.profile >= 1) RCD_CUDA(ctx, cudaEventRecord(ctx->evPhase[1], st));
     const int64_t dPitch = sz.pitch / (int64_t)feat_bytes(dtype);
     rs = launch_similarity(ctx, P.ws.Xs, dtype, N, dPitch, cls, P.ws.S, st);
@@ -719,7 +729,7 @@ rcd_status rcd_partition(rcd_ctx *ctx, const void *features_dev, rcd_feat_dtype 
     if (prof) RCD_CUDA(ctx, cudaEventRecord(ctx->evPhase[0], st));
 
     Prepared P;
-    rs = prepare(ctx, features_dev, dtype, N, d, labels_dev, L, W, capacities_host, workspace_dev, workspace_bytes, st, &P);
+    rs = prepare(ctx, features_dev, dtype, N, d, labels_dev, L, W, capacities_host, nullptr, workspace_dev, workspace_bytes, st, &P);
     if (rs != RCD_OK) return rs;
 
     const bool valuesWritten = P.cluster != nullptr;
@@ -839,7 +849,7 @@ rcd_status rcd_objective(rcd_ctx *ctx, const void *features_dev, rcd_feat_dtype 
     const int savedProfile = ctx->cfg.profile;
     ctx->cfg.profile = 0;
     Prepared P;
-    rs = prepare(ctx, features_dev, dtype, N, d, labels_dev, L, W, nullptr, workspace_dev, workspace_bytes, st, &P);
+    rs = prepare(ctx, features_dev, dtype, N, d, labels_dev, L, W, nullptr, assignment_dev, workspace_dev, workspace_bytes, st, &P);
     ctx->cfg.profile = savedProfile;
     if (rs != RCD_OK) return rs;
     if (P.sz.graphCut) {
@@ -849,7 +859,7 @@ rcd_status rcd_objective(rcd_ctx *ctx, const void *features_dev, rcd_feat_dtype 
         rs = launch_cut_objective(ctx, P.sz, P.ws.desc, P.ws.S, P.ws.perm, assignment_dev, part_values_dev, total_dev,
                                   (unsigned char *)workspace_dev + P.ws.bytes, st);
     } else {
-        rs = launch_objective(ctx, P.sz.floatArith ? RCD_FEAT_BF16 : RCD_FEAT_I8, P.sz, P.ws, assignment_dev, part_values_dev, total_dev, st);
+        rs = launch_objective(ctx, P.sz.floatArith ? RCD_FEAT_BF16 : RCD_FEAT_I8, P.sz, P.ws, assignment_dev, P.covered, part_values_dev, total_dev, st);
     }
     return rs;
 }

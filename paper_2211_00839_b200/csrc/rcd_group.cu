@@ -277,6 +277,16 @@ rcd_status launch_label_hist(rcd_ctx *ctx, const int32_t *labels, int64_t N, int
     return RCD_OK;
 }
 
+rcd_status launch_gather_rows(rcd_ctx *ctx, const void *X, const int32_t *perm, int64_t N, int64_t rowBytes, int64_t pitch, void *dst, cudaStream_t st)
+{
+    if (N == 0) return RCD_OK;
+    const unsigned blocks = (unsigned)std::min<int64_t>((N + 7) / 8, 32LL * ctx->smCount);
+    gather_rows_kernel<<<blocks, 256, 0, st>>>((const uint8_t *)X, perm, N, rowBytes, pitch, (uint8_t *)dst);
+    ctx->kernelLaunches++;
+    RCD_CUDA(ctx, cudaGetLastError());
+    return RCD_OK;
+}
+
 // Stable split after launch_label_hist: perm, and with X the rows in split order (Xs, `pitch` bytes apart, zero-filled
 // beyond rowBytes).  desc null: label l starts after the counts of the labels below it; the starts go to offsets[L + 1].
 rcd_status launch_stable_split(rcd_ctx *ctx, const int32_t *labels, int64_t N, int32_t L, int32_t *chunkHist, const ClassDesc *descDev,
@@ -302,11 +312,7 @@ rcd_status launch_stable_split(rcd_ctx *ctx, const int32_t *labels, int64_t N, i
     } else {
         chunk_rank_kernel<false><<<nChunks, 1024, 0, st>>>(labels, N, L, chunk, chunkHist, perm, status);
         ctx->kernelLaunches++;
-        if (Xs) {
-            const unsigned blocks = (unsigned)std::min<int64_t>((N + 7) / 8, 32LL * ctx->smCount);
-            gather_rows_kernel<<<blocks, 256, 0, st>>>((const uint8_t *)X, perm, N, rowBytes, pitch, (uint8_t *)Xs);
-            ctx->kernelLaunches++;
-        }
+        if (Xs) return launch_gather_rows(ctx, X, perm, N, rowBytes, pitch, Xs, st);
     }
     RCD_CUDA(ctx, cudaGetLastError());
     return RCD_OK;

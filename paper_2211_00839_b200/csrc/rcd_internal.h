@@ -277,6 +277,11 @@ rcd_status launch_stable_split(rcd_ctx *ctx, const int32_t *labels, int64_t N, i
 rcd_status launch_similarity(rcd_ctx *ctx, const void *Xs, rcd_feat_dtype dtype, int64_t Ntot, int64_t d,
                              const SimClasses &cls, void *S, cudaStream_t st);
 
+// In place of S, the coverage of every block: rows in block order within their class (blockOf[Ntot], -1: no block), cover[block][row]
+// of a class at its vOff, zero at the start.  Tensor-core rows and cls.pairs false only.
+rcd_status launch_similarity_maxima(rcd_ctx *ctx, const void *Xs, rcd_feat_dtype dtype, int64_t Ntot, int64_t d,
+                                    const SimClasses &cls, const int32_t *blockOf, int32_t *cover, cudaStream_t st);
+
 // Gaussian-kernel similarity: transforms the dot products in S in place, to fp32 or (fixedExp not null) to the fixed-point
 // integers of the cluster form, whose scale it writes to fixedExp[l]
 rcd_status launch_gaussian(rcd_ctx *ctx, const void *Xs, rcd_feat_dtype dtype, int64_t N, int64_t d, const SimClasses &cls,
@@ -315,8 +320,13 @@ rcd_status launch_cut_objective(rcd_ctx *ctx, const Sizes &sz, const ClassDesc *
                                 const int32_t *assignment, void *partValues, void *total, void *scratch, cudaStream_t st);
 
 // objective from an assignment
+// covered: the coverage is there already (launch_similarity_maxima), else it is taken from S
 rcd_status launch_objective(rcd_ctx *ctx, rcd_feat_dtype dtype, const Sizes &sz, const Workspace &ws, const int32_t *assignment,
-                            void *partValues, void *total, cudaStream_t st);
+                            bool covered, void *partValues, void *total, cudaStream_t st);
+// class-sorted positions in block order: ws.cand the dataset index, ws.pos the block (-1: none); ws.cover cleared
+rcd_status launch_objective_order(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, const int32_t *assignment, cudaStream_t st);
+// dst row r = row perm[r] of X, `pitch` bytes apart, zero-filled beyond rowBytes
+rcd_status launch_gather_rows(rcd_ctx *ctx, const void *X, const int32_t *perm, int64_t N, int64_t rowBytes, int64_t pitch, void *dst, cudaStream_t st);
 
 
 #ifdef __CUDACC__

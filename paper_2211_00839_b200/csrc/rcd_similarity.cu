@@ -151,19 +151,28 @@ static rcd_status launch_similarity_generic(rcd_ctx *ctx, const void *Xs, rcd_fe
 }
 
 rcd_status launch_similarity_tc(rcd_ctx *ctx, const void *Xs, rcd_feat_dtype dtype, int64_t Ntot, int64_t d,
-                                const SimClasses &cls, void *S, cudaStream_t st, bool *handled);
+                                const SimClasses &cls, void *S, const int32_t *blockOf, int32_t *cover, cudaStream_t st, bool *handled);
 
 rcd_status launch_similarity(rcd_ctx *ctx, const void *Xs, rcd_feat_dtype dtype, int64_t Ntot, int64_t d,
                              const SimClasses &cls, void *S, cudaStream_t st)
 {
     if (ctx->cfg.similarity_path != 2) {
         bool handled = false;
-        rcd_status rs = launch_similarity_tc(ctx, Xs, dtype, Ntot, d, cls, S, st, &handled);
+        rcd_status rs = launch_similarity_tc(ctx, Xs, dtype, Ntot, d, cls, S, nullptr, nullptr, st, &handled);
         if (rs != RCD_OK) return rs;
         if (handled) return RCD_OK;
     }
     if (cls.clearStatus) RCD_CUDA(ctx, cudaMemsetAsync(const_cast<int32_t *>(ctx->statusDev), 0, sizeof(int32_t), st));
     return launch_similarity_generic(ctx, Xs, dtype, d, cls, S, st);
+}
+
+rcd_status launch_similarity_maxima(rcd_ctx *ctx, const void *Xs, rcd_feat_dtype dtype, int64_t Ntot, int64_t d,
+                                    const SimClasses &cls, const int32_t *blockOf, int32_t *cover, cudaStream_t st)
+{
+    bool handled = false;
+    const rcd_status rs = launch_similarity_tc(ctx, Xs, dtype, Ntot, d, cls, nullptr, blockOf, cover, st, &handled);
+    if (rs != RCD_OK || handled) return rs;
+    return fail(ctx, RCD_ERR_INTERNAL, "objective: rows of %lld elements", (long long)d);
 }
 
 }  // namespace rcd

@@ -42,6 +42,12 @@ constexpr int kTcThreads = 64 + 32 * kEpiWarps;
 constexpr int kTmemCols = 512;                           // two accumulator buffers of 256 columns
 constexpr uint32_t kSpinLimit = 1u << 22;               // polls of ~64 ns: a quarter of a second
 
+struct TileCoord { int l, tm, sn, skip, n; };         // n: columns computed, from column sn * 256 + skip on
+struct __align__(8) TileSlot {                          // a tile the producer has drawn
+    TileCoord t;                                        // (t.l < 0: no more)
+    ClassDesc c;
+};
+
 struct __align__(8) TcShared {
     uint64_t full[kStages];
     uint64_t empty[kStages];
@@ -49,7 +55,7 @@ struct __align__(8) TcShared {
     uint64_t accEmpty[2];
     uint64_t tileFull[kTileSlots];
     uint64_t tileEmpty[kTileSlots];
-    int32_t tile[kTileSlots];                           // tiles this CTA has drawn (-1: no more)
+    TileSlot tile[kTileSlots];
     uint32_t tmemBase;
     int32_t abort;
 };
@@ -150,7 +156,6 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
 // those with sn >= tm / 2, which contain a 128 x 128 block on or above the diagonal.  skip = 128 when the left half of the
 // tile lies below the diagonal (tm odd, sn = tm / 2): that half is the mirror image of a block another tile computes, so
 // only the right half is computed.
-struct TileCoord { int l, tm, sn, skip, n; };         // n: columns computed, from column sn * 256 + skip on
 __device__ __forceinline__ TileCoord decode_tile(const DescSource &src, const int32_t *__restrict__ prefix, int L, int uniTiles, int idx)
 {
     TileCoord t;
@@ -238,17 +243,154 @@ __device__ __forceinline__ void write_columns(uint32_t (*stage)[33], uint32_t *S
     }
 }
 
+// Where a tile's columns or rows belong, for the maxima: lane j holds the block of column (row) j of 32, -1: none.  The 32 are in block
+// order, so that a run of equal blocks is one maximum; `starts` has a bit where a run starts behind the first.
+__device__ __forceinline__ uint32_t run_starts(int block)
+{
+    const int before = __shfl_up_sync(0xffffffffu, block, 1);
+    return __ballot_sync(0xffffffffu, (threadIdx.x & 31) > 0 && before != block);
+}
+// The greater of a maximum so far, not below zero, and an entry.  (fmaxf passes a NaN over, as a comparison does; positive floats
+// order like their bit patterns.)
 template <bool kInt8>
+__device__ __forceinline__ uint32_t greater(uint32_t m, uint32_t x)
+{
+    if constexpr (kInt8) return (uint32_t)max((int32_t)m, (int32_t)x);
+    else return __float_as_uint(fmaxf(__uint_as_float(m), __uint_as_float(x)));
+}
+
+constexpr int kFewRuns = 4;                                     // runs of 32 up to which each is gone through by itself
+
+constexpr int kWarpCols = kTileN / 32 / (kEpiWarps / 4);       // column blocks of a tile that one epilogue warp takes
+
+// An epilogue warp's column blocks of a tile of rows in block order -> the blocks' coverage: cover[b][i] = max(0, max over the columns
+// of block b), row i per lane, and for blocks above the diagonal the same with rows and columns exchanged (through shared memory).  A
+// maximum leaves the registers where the block changes: the rows' at the end of a run that may span the tile, the columns' once per
+// 32 rows at least.  colBlock: the blocks of the warp's columns, looked up before the tile was ready.
+// Bound by this epilogue's own instructions and then by the operands' way from L2 (10 classes of 5000 x 512 int8 into 8 blocks: 189 us
+// with a test for every column and row, which 32 of them unrolled pay for even where no run ends; 115 with a pass per run; 95 with no
+// epilogue at all.  Writing S took 200 us and reading it back 200 more).  With more runs than kFewRuns in 32 the tests are cheaper.
+template <bool kInt8, typename Mirrored>
+__device__ __forceinline__ void keep_maxima(uint32_t (*stage)[33], int32_t *cover, const ClassDesc &c, int row0, int colB, uint32_t tmemRow,
+                                            int half, int nCb, uint32_t (&v)[32], int rowBlock, const int (&colBlock)[kWarpCols], Mirrored mirrored)
+{
+    const int lane = threadIdx.x & 31;
+    uint4 *const block4 = reinterpret_cast<uint4 *>(stage);
+    const uint32_t rowStarts = run_starts(rowBlock);
+    auto join = [&](int block, int i, uint32_t m) {
+        if (block >= 0 && i < c.M && (int32_t)m > 0) atomicMax(cover + (int64_t)block * c.ld + i, (int32_t)m);
+    };
+    uint32_t m = 0;
+    int block = -1;
+#pragma unroll
+    for (int k = 0; k < kWarpCols; ++k) {
+        const int cb = half + k * (kEpiWarps / 4), col0 = colB + cb * 32;
+        if (cb >= nCb) break;
+        const uint32_t colStarts = run_starts(colBlock[k]);
+        const int firstBlock = __shfl_sync(0xffffffffu, colBlock[k], 0);
+        const bool mirror = mirrored(cb);
+        tmem_load_wait();
+        if (firstBlock != block) {
+            join(block, row0 + lane, m);
+            m = 0;
+            block = firstBlock;
+        }
+        if (colStarts == 0) {                              // one block, as almost always where blocks are large
+            uint32_t part[4] = {m, 0, 0, 0};
+#pragma unroll
+            for (int j = 0; j < 32; ++j) part[j & 3] = greater<kInt8>(part[j & 3], v[j]);
+            m = greater<kInt8>(greater<kInt8>(part[0], part[1]), greater<kInt8>(part[2], part[3]));
+        } else if (__popc(colStarts) < kFewRuns) {
+            for (uint32_t left = colStarts | 1u; left; left &= left - 1) {
+                const uint32_t later = left & (left - 1), run = (later & (0u - later)) - (left & (0u - left));   // the run's columns
+                const int of = __shfl_sync(0xffffffffu, colBlock[k], __ffs((int)left) - 1);
+                if (of != block) {
+                    join(block, row0 + lane, m);
+                    m = 0;
+                    block = of;
+                }
+                uint32_t part[4] = {m, 0, 0, 0};
+#pragma unroll
+                for (int j = 0; j < 32; ++j) part[j & 3] = greater<kInt8>(part[j & 3], run >> j & 1 ? v[j] : 0u);
+                m = greater<kInt8>(greater<kInt8>(part[0], part[1]), greater<kInt8>(part[2], part[3]));
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+                if (colStarts >> j & 1) {
+                    join(block, row0 + lane, m);
+                    m = 0;
+                    block = __shfl_sync(0xffffffffu, colBlock[k], j);
+                }
+                m = greater<kInt8>(m, v[j]);
+            }
+        }
+        // (16-byte pieces, each row's turned by the row's number: neither side meets a bank twice)
+        if (mirror) {
+#pragma unroll
+            for (int g = 0; g < 8; ++g) block4[lane * 8 + (g ^ (lane & 7))] = make_uint4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
+        }
+        __syncwarp();
+        if (cb + kEpiWarps / 4 < nCb) tmem_load_32cols(tmemRow + (uint32_t)((cb + kEpiWarps / 4) * 32), v);
+        if (mirror) {
+            if (__popc(rowStarts) < kFewRuns) {
+                for (uint32_t left = rowStarts | 1u; left; left &= left - 1) {
+                    const uint32_t later = left & (left - 1);
+                    const int from = __ffs((int)left) - 1, to = later ? __ffs((int)later) - 1 : 32;
+                    // four columns per lane, every fourth row; then the four lanes of a piece
+                    uint4 n = make_uint4(0, 0, 0, 0);
+#pragma unroll
+                    for (int k8 = 0; k8 < 8; ++k8) {
+                        const int r = 4 * k8 + (lane >> 3);
+                        const uint4 x = block4[r * 8 + ((lane & 7) ^ (r & 7))];
+                        const bool in = r >= from && r < to;
+                        n.x = greater<kInt8>(n.x, in ? x.x : 0u);
+                        n.y = greater<kInt8>(n.y, in ? x.y : 0u);
+                        n.z = greater<kInt8>(n.z, in ? x.z : 0u);
+                        n.w = greater<kInt8>(n.w, in ? x.w : 0u);
+                    }
+#pragma unroll
+                    for (int off = 8; off < 32; off <<= 1) {
+                        n.x = greater<kInt8>(n.x, __shfl_xor_sync(0xffffffffu, n.x, off));
+                        n.y = greater<kInt8>(n.y, __shfl_xor_sync(0xffffffffu, n.y, off));
+                        n.z = greater<kInt8>(n.z, __shfl_xor_sync(0xffffffffu, n.z, off));
+                        n.w = greater<kInt8>(n.w, __shfl_xor_sync(0xffffffffu, n.w, off));
+                    }
+                    join(__shfl_sync(0xffffffffu, rowBlock, from), col0 + 4 * (lane & 7) + (lane >> 3),
+                         lane < 16 ? (lane < 8 ? n.x : n.y) : (lane < 24 ? n.z : n.w));
+                }
+            } else {
+                uint32_t n = 0;
+                int run = __shfl_sync(0xffffffffu, rowBlock, 0);
+#pragma unroll 4
+                for (int r = 0; r < 32; ++r) {
+                    if (rowStarts >> r & 1) {
+                        join(run, col0 + lane, n);
+                        n = 0;
+                        run = __shfl_sync(0xffffffffu, rowBlock, r);
+                    }
+                    n = greater<kInt8>(n, reinterpret_cast<const uint32_t *>(block4)[r * 32 + (((lane >> 2) ^ (r & 7)) << 2 | (lane & 3))]);
+                }
+                join(run, col0 + lane, n);
+            }
+        }
+        __syncwarp();
+    }
+    join(block, row0 + lane, m);
+}
+
+// kMaxima: rows are in block order within their class (blockOf), and instead of S the blocks' coverage is written.
+template <bool kInt8, bool kMaxima>
 __global__ void __launch_bounds__(kTcThreads, 1) sim_tc_kernel(const __grid_constant__ CUtensorMap map, DescSource src, int32_t L,
                                                               const int32_t *__restrict__ tilePrefix, int32_t uniTiles,
                                                               int32_t *ticket, int32_t totalTiles, int32_t numSlabs, uint32_t *__restrict__ S,
-                                                              int32_t *status, bool clearStatus)
+                                                              const int32_t *__restrict__ blockOf, int32_t *cover, int32_t *status, bool clearStatus)
 {
     extern __shared__ unsigned char smemRaw[];
     // operand stages need 1024-byte alignment for the 128-byte swizzle pattern
     unsigned char *tiles = reinterpret_cast<unsigned char *>(((uintptr_t)smemRaw + 1023) & ~(uintptr_t)1023);
     __shared__ TcShared sh;
-    __shared__ uint32_t stage32[kEpiWarps][32][33];             // per epilogue warp: one 32 x 32 block, padded
+    __shared__ __align__(16) uint32_t stage32[kEpiWarps][32][33];             // per epilogue warp: one 32 x 32 block, padded
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (clearStatus && blockIdx.x == 0 && threadIdx.x == 0) *(volatile int32_t *)status = 0;    // (no wait runs out for a quarter of a second)
@@ -284,12 +426,19 @@ __global__ void __launch_bounds__(kTcThreads, 1) sim_tc_kernel(const __grid_cons
             for (uint32_t nt = 0; ok; ++nt) {
                 const int slot = nt % kTileSlots;
                 if (!mbar_wait(&sh.tileEmpty[slot], ((nt / kTileSlots) & 1) ^ 1, &sh)) break;
-                *(volatile int32_t *)&sh.tile[slot] = idx;
-                mbar_arrive(&sh.tileFull[slot]);
-                if (idx < 0) break;
+                if (idx < 0) {
+                    sh.tile[slot].t.l = -1;
+                    mbar_arrive(&sh.tileFull[slot]);
+                    break;
+                }
                 int next = -1;
+                // (once for all roles: a search in the prefixes and a walk along the row blocks, which the epilogue would wait for
+                // tile by tile)
                 const TileCoord t = decode_tile(src, tilePrefix, L, uniTiles, idx);
                 const ClassDesc c = src.get(t.l);
+                sh.tile[slot].t = t;
+                sh.tile[slot].c = c;
+                mbar_arrive(&sh.tileFull[slot]);
                 const int rowA = c.row0 + t.tm * kTileM, rowB = c.row0 + t.sn * kTileN + t.skip;
                 const int halves = (t.n + kTileM - 1) / kTileM;         // 128-row pieces of B to bring in: 2, or 1
                 const bool shared = t.sn == t.tm / 2;                   // on the diagonal the first of them is A
@@ -327,10 +476,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) sim_tc_kernel(const __grid_cons
             for (; ok; ++nt) {
                 const int slot = nt % kTileSlots;
                 if (!mbar_wait(&sh.tileFull[slot], (nt / kTileSlots) & 1, &sh)) break;
-                const int idx = *(volatile int32_t *)&sh.tile[slot];
+                const TileCoord t = sh.tile[slot].t;
                 mbar_arrive(&sh.tileEmpty[slot]);
-                if (idx < 0) break;
-                const TileCoord t = decode_tile(src, tilePrefix, L, uniTiles, idx);
+                if (t.l < 0) break;
                 const uint32_t idesc = idescBase | ((uint32_t)(t.n >> 3) << 17);   // N = 256, less for a half tile or at the class's edge
                 const uint32_t buf = nt & 1;
                 // the epilogue must have drained this accumulator buffer (two tiles ago)
@@ -361,24 +509,35 @@ __global__ void __launch_bounds__(kTcThreads, 1) sim_tc_kernel(const __grid_cons
         for (;; ++nt) {
             const int slot = nt % kTileSlots;
             if (!mbar_wait(&sh.tileFull[slot], (nt / kTileSlots) & 1, &sh)) break;
-            const int idx = *(volatile int32_t *)&sh.tile[slot];
+            const TileCoord t = sh.tile[slot].t;
+            const ClassDesc c = sh.tile[slot].c;
             __syncwarp();
             if (lane == 0) mbar_arrive(&sh.tileEmpty[slot]);
-            if (idx < 0) break;
-            const TileCoord t = decode_tile(src, tilePrefix, L, uniTiles, idx);
-            const ClassDesc c = src.get(t.l);
+            if (t.l < 0) break;
             const int rowA = t.tm * kTileM, colB = t.sn * kTileN + t.skip;   // class-local: first row, first column computed
             const uint32_t buf = nt & 1;
+            [[maybe_unused]] int rowBlock = -1, colBlock[kWarpCols];
+            if constexpr (kMaxima) {
+                const int32_t *const of = blockOf + c.row0;
+                if (rowA + q * 32 + lane < c.M) rowBlock = of[rowA + q * 32 + lane];
+#pragma unroll
+                for (int k = 0; k < kWarpCols; ++k) {
+                    const int col = colB + (half + k * (kEpiWarps / 4)) * 32 + lane;
+                    colBlock[k] = col < c.M ? of[col] : -1;
+                }
+            }
             if (!mbar_wait(&sh.accFull[buf], (nt >> 1) & 1, &sh)) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             if (*(volatile int32_t *)&sh.abort) break;
-            uint32_t *Sl = S + c.sOff;
+            [[maybe_unused]] uint32_t *Sl = S + c.sOff;
             const int nCb = t.n / 32;
             const uint32_t tmemRow = tmemBase + buf * kTileN + ((uint32_t)(q * 32) << 16);
             uint32_t v[32];
             if (half < nCb) tmem_load_32cols(tmemRow + (uint32_t)(half * 32), v);
             // a 128 x 128 block lies on the diagonal (stored once) or above it (stored twice: itself and its mirror image)
-            write_columns(stage32[ew], Sl, c, rowA + q * 32, colB, tmemRow, half, nCb, v, [&](int cb) { return (colB + cb * 32) / kTileM != t.tm; });
+            auto mirrored = [&](int cb) { return (colB + cb * 32) / kTileM != t.tm; };
+            if constexpr (kMaxima) keep_maxima<kInt8>(stage32[ew], cover + c.vOff, c, rowA + q * 32, colB, tmemRow, half, nCb, v, rowBlock, colBlock, mirrored);
+            else write_columns(stage32[ew], Sl, c, rowA + q * 32, colB, tmemRow, half, nCb, v, mirrored);
             // hand the accumulator buffer back to the MMA warp
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
@@ -635,7 +794,7 @@ EncodeTiledFn encode_tiled_fn()
 }  // namespace
 
 rcd_status launch_similarity_tc(rcd_ctx *ctx, const void *Xs, rcd_feat_dtype dtype, int64_t Ntot, int64_t d,
-                                const SimClasses &cls, void *S, cudaStream_t st, bool *handled)
+                                const SimClasses &cls, void *S, const int32_t *blockOf, int32_t *cover, cudaStream_t st, bool *handled)
 {
     *handled = false;
     const int64_t rowBytes = d * (int64_t)feat_bytes(dtype);
@@ -684,10 +843,11 @@ rcd_status launch_similarity_tc(rcd_ctx *ctx, const void *Xs, rcd_feat_dtype dty
         // tiles up to three ahead of their turn (200 of 257 x 256 int8: 29 -> 34 us).  A ticket of its own for every launch
         // that can be under way at once: calls may overlap on several streams.
         int32_t *ticket = totalTiles <= 8LL * cls.L && numSlabs < 8 ? nullptr : ctx->statusOwn + kFirstTicket + ctx->simTurn++ % (kStatusWords - kFirstTicket);
-        auto *kernel = isInt8 ? sim_tc_kernel<true> : sim_tc_kernel<false>;
-        RCD_CUDA(ctx, allow(kernel, isInt8 ? 1 : 0, smem));
+        auto *kernel = blockOf ? (isInt8 ? sim_tc_kernel<true, true> : sim_tc_kernel<false, true>)
+                               : (isInt8 ? sim_tc_kernel<true, false> : sim_tc_kernel<false, false>);
+        RCD_CUDA(ctx, allow(kernel, (isInt8 ? 1 : 0) + (blockOf ? 4 : 0), smem));
         kernel<<<grid, kTcThreads, smem, st>>>(map, cls.src, cls.L, cls.tilePrefixDev, cls.uniTiles, ticket, totalTiles,
-                                               numSlabs, (uint32_t *)S, status, cls.clearStatus);
+                                               numSlabs, (uint32_t *)S, blockOf, cover, status, cls.clearStatus);
     }
     ctx->kernelLaunches++;
     ctx->tcLaunches++;
