@@ -310,7 +310,7 @@ def run_ours(args):
     h2d = Xh.numel() * Xh.element_size() + yh.numel() * 4
     d2h = sum(t.numel() * t.element_size() for t in host_out)
 
-    # Roofline of the dominant kernel.  The whole greedy loop is ONE launch (greedy_cluster_kernel, or, where a form with
+    # Roofline of the dominant kernel.  The whole greedy loop is ONE launch (greedy_cluster_kernel or greedy_rounds_kernel, or, where a form with
     # passes over S is asked for or needed: greedy_async_kernel when classes are few, greedy_owner_kernel when they are
     # many).  For the forms with passes: algorithmic bytes = for every sweep of a class, the rows of S of its unassigned samples
     # plus the coverage vectors of the blocks refreshed (4*ld*(n_R + n) bytes), summed on the device.
@@ -332,7 +332,8 @@ def run_ours(args):
     sms = torch.cuda.get_device_properties(local).multi_processor_count
     path = args.greedy_path if args.greedy_path else (3 if wl.L * 4 <= sms else 4)
     if clustered:
-        kernel_name = "greedy_cluster_kernel"
+        # (of the configurations only 1000 classes into 64 blocks run in rounds, where a round's rows count once for all blocks)
+        kernel_name = "greedy_rounds_kernel" if args.objective == "facility" and wl.W >= 48 and wl.L >= sms else "greedy_cluster_kernel"
     elif args.objective != "facility":
         kernel_name = "cut_chain_kernel"
     else:

@@ -15,8 +15,8 @@
 // What bounds it (1000 classes of 1300 int8 into 64 blocks: 165 ms in the cluster form, 81 here; per class, one CTA of 16 warps per SM):
 // 4.6 of 13 ms are the sums of `tile_rows`, a saturating subtraction (half rate) and a multiply-add (its own pipe) per loss, 13 cycles
 // per row, 4 blocks and 128 columns where the pipes would allow 10; 2.1 ms rows that few blocks need, straight from memory; the rest
-// trips to L2 and barriers of 110 rounds (lists 1.0, looks 1.3, decisions 0.7, looks asked for in between 0.8).  74 GB cross HBM
-// instead of 895.
+// trips to L2 and barriers of 110 rounds (lists 1.0, looks 1.3, decisions 0.7, looks asked for in between 0.8).  148 MB per class
+// cross HBM instead of 895.
 //
 // Results are those of the cluster form bit for bit: stored gains are exact integers, decisions are made in the same order.
 #include "rcd_exact.cuh"
