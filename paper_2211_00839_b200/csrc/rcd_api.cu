@@ -467,7 +467,8 @@ rcd_status rcd_selftest_bounded_wait(rcd_ctx *ctx, void *cuda_stream)
     RCD_CUDA(ctx, cudaSetDevice(ctx->device));
     RCD_CUDA(ctx, cudaMemsetAsync(ctx->statusOwn, 0, 64, st));
     ctx->statusDev = ctx->statusOwn;
-    return launch_bounded_wait_selftest(ctx, (unsigned *)(ctx->statusOwn + 8), ctx->statusOwn, st);
+    const rcd_status rs = launch_bounded_wait_selftest(ctx, (unsigned *)(ctx->statusOwn + 8), ctx->statusOwn, st);
+    return rs == RCD_OK ? launch_step_wait_selftest(ctx, ctx->statusOwn, st) : rs;
 }
 
 rcd_status rcd_get_profile(rcd_ctx *ctx, rcd_profile *out)

@@ -313,6 +313,7 @@ rcd_status launch_greedy_rounds(rcd_ctx *ctx, RoundsPlan &plan, const Sizes &sz,
                                 void *partValues, cudaStream_t st);
 
 rcd_status launch_bounded_wait_selftest(rcd_ctx *ctx, unsigned *counter, int32_t *status, cudaStream_t st);
+rcd_status launch_step_wait_selftest(rcd_ctx *ctx, int32_t *status, cudaStream_t st);
 
 // graph-cut objective: the whole greedy loop, and f from an assignment
 rcd_status launch_cut(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, int32_t *assignment, int32_t *order, cudaStream_t st);

@@ -60,7 +60,7 @@ constexpr int kStages = 3;                // of the ring of tiles
 constexpr int kGroup = 4;                 // blocks per warp of a tile
 constexpr int kMaxWarps = 16;             // of a CTA; blocks corrected together: kGroup each
 constexpr int kRoundBlocks = 128;
-constexpr unsigned kCopyLimit = 1u << 24; // looks at a stage's barrier before the copies count as lost
+constexpr unsigned kCopyLimit = 1u << 22; // looks at a stage's barrier, 64 ns apart, before the copies count as lost: a quarter of a second
 
 struct Pending { int32_t block, sample, first; };   // a pick whose correction is outstanding; first: its block was empty
 
@@ -158,6 +158,24 @@ __device__ __forceinline__ bool bar_done(uint32_t bar, uint32_t parity)
                  : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
+__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, unsigned limit)
+{
+    for (int k = 0; k < 64; ++k)
+        if (bar_done(bar, parity)) return true;
+    for (unsigned k = 0; k < limit; ++k) {
+        if (bar_done(bar, parity)) return true;
+        __nanosleep(64);
+    }
+    return false;
+}
+// Waits for the copies of a step, and for all threads.  Where a thread gives up, all of them learn of it at this very step (lostAt: the
+// first step without its copies; a thread that is ahead can only have put down a later one), so that they leave together.
+__device__ __forceinline__ bool step_arrived(uint32_t bar, uint32_t parity, int step, int *lostAt, unsigned limit)
+{
+    if (!bar_wait(bar, parity, limit)) atomicMin(lostAt, step);
+    __syncthreads();
+    return *(volatile int *)lostAt > step;
+}
 // (16-byte aligned on both sides, a multiple of 16 bytes)
 __device__ __forceinline__ void copy_bulk(uint32_t to, const void *from, uint32_t bytes, uint32_t bar)
 {
@@ -209,7 +227,7 @@ __global__ void __launch_bounds__(kWarps * 32, kMaxWarps / kWarps) greedy_rounds
     __shared__ int shRoom[kRoundBlocks];
     __shared__ uint8_t shHas[kRoundBlocks];
     __shared__ __align__(8) unsigned long long shBars[kStages];
-    __shared__ int shMostBy, shMade, shClass, shCommand, shListed, shNeeded, shFailed;
+    __shared__ int shMostBy, shMade, shClass, shCommand, shListed, shNeeded, shFailed, shLostAt;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int W = prm.W;
     unsigned char *const ring = shared + prm.offRing;
@@ -227,12 +245,14 @@ __global__ void __launch_bounds__(kWarps * 32, kMaxWarps / kWarps) greedy_rounds
     uint32_t parities = 0;                    // of the stages' barriers
     unsigned rescans = 0;
     unsigned long long rowsRead = 0, corrected = 0;
+    bool lost = false;                        // (in all threads or in none) copies did not arrive: nothing more is written, the kernel ends
 
     if (threadIdx.x == 0) {
+        shLostAt = INT_MAX;
         for (int k = 0; k < kStages; ++k) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(bars + 8 * k) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    for (;;) {
+    while (!lost) {
         if (threadIdx.x == 0) {
             const int k = atomicAdd(prm.counter, 1);
             shClass = (k < prm.L && *(volatile int32_t *)prm.status == 0) ? prm.classOrder[k] : -1;
@@ -273,7 +293,7 @@ __global__ void __launch_bounds__(kWarps * 32, kMaxWarps / kWarps) greedy_rounds
         look_part<true>(g0, ld4, bits, scratch, warp, kWarps, lane);
         __syncthreads();
         if (warp == 0) look_join(scratch, kWarps, keys + W * kListed, bounds + W, lane);
-        for (;;) {
+        while (!lost) {
             if (warp == 0) {
                 int n = 0, made = shMade;
                 unsigned long long f[KW];
@@ -387,7 +407,7 @@ __global__ void __launch_bounds__(kWarps * 32, kMaxWarps / kWarps) greedy_rounds
 
             const int perBlock = M * 8 + 32;       // scratch of a block: its part of the table
             const int most = (int)min((int64_t)min(nPending, kBatchBlocks), prm.scratchBytes / perBlock / kGroup * kGroup);
-            for (int p0 = 0; p0 < nPending; p0 += most) {
+            for (int p0 = 0; p0 < nPending && !lost; p0 += most) {
                 const int nP = min(most, nPending - p0), nP4 = (nP + kGroup - 1) / kGroup * kGroup;
                 const Pending *const pend = pending + p0;
                 int2 *const table = reinterpret_cast<int2 *>(prm.scratch + (int64_t)blockIdx.x * prm.scratchBytes);   // [rows needed][nP4]: - old coverage, new - old
@@ -585,11 +605,14 @@ __global__ void __launch_bounds__(kWarps * 32, kMaxWarps / kWarps) greedy_rounds
                     for (int k = 0; k < kStages - 1; ++k) fetch(k);
                     for (int step = 0; step < steps; ++step) {
                         const int stage = step % kStages;
-                        unsigned spin = 0;
-                        while (!bar_done(bars + 8 * stage, parities >> stage & 1) && ++spin < kCopyLimit) { }
-                        if (spin >= kCopyLimit) atomicOr(prm.status, kDevTimeout);
+                        // (and everybody is through with the stage before)
+                        if (!step_arrived(bars + 8 * stage, parities >> stage & 1, step, &shLostAt, kCopyLimit)) {
+                            // what is under way lands before shared memory is given up, if it lands at all
+                            for (int k = step; k < min(steps, step + kStages - 1); ++k) bar_wait(bars + 8 * (k % kStages), parities >> (k % kStages) & 1, kCopyLimit);
+                            lost = true;
+                            break;
+                        }
                         parities ^= 1u << stage;
-                        __syncthreads();                   // (everybody is through with the stage before)
                         fetch(step + kStages - 1);
                         const int tile = step / stages, part = step - tile * stages, n = min(perStage, need4 - part * perStage);
                         if (!works || tile * colGroups + colGroup >= G) continue;
@@ -621,6 +644,7 @@ __global__ void __launch_bounds__(kWarps * 32, kMaxWarps / kWarps) greedy_rounds
                 __threadfence();
                 __syncthreads();
             }
+            if (lost) break;
             if (threadIdx.x == 0) corrected += nPending;
             // the next notes: a warp per block, several for each of few
             int parts = 1;
@@ -641,6 +665,7 @@ __global__ void __launch_bounds__(kWarps * 32, kMaxWarps / kWarps) greedy_rounds
             }
             __syncthreads();
         }
+        if (lost) break;
         for (int p = threadIdx.x; p < W; p += kThreads) {
             const long long value = (long long)(shValue[p] >> 7);
             prm.fval[(int64_t)l * W + p] = prm.fixedExp ? __double_as_longlong(ldexp((double)value, -prm.fixedExp[l])) : value;
@@ -655,6 +680,7 @@ __global__ void __launch_bounds__(kWarps * 32, kMaxWarps / kWarps) greedy_rounds
         __syncthreads();
     }
     if (threadIdx.x == 0) {
+        if (lost) atomicOr(prm.status, kDevTimeout);
         if (rescans) atomicAdd(prm.stats + 9, (unsigned long long)rescans);
         if (corrected) {
             atomicAdd(prm.stats + 15, corrected);
@@ -663,7 +689,35 @@ __global__ void __launch_bounds__(kWarps * 32, kMaxWarps / kWarps) greedy_rounds
     }
 }
 
+// A step whose copies have arrived, then one whose copies never do, which half of the threads takes for arrived: all of them stay for
+// the first and leave at the second.  (After the grid barrier's test, which leaves the timeout's bit: kept only if this goes right too.)
+__global__ void step_wait_selftest_kernel(int32_t *status)
+{
+    __shared__ __align__(8) unsigned long long shBars[2];
+    __shared__ int shLostAt;
+    const uint32_t bars = smem32(shBars);
+    if (threadIdx.x == 0) {
+        shLostAt = INT_MAX;
+        for (int k = 0; k < 2; ++k) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(bars + 8 * k) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        bar_expect(bars, 0);
+    }
+    __syncthreads();
+    const bool first = step_arrived(bars, 0, 0, &shLostAt, 1u << 12);
+    const bool second = step_arrived(threadIdx.x < blockDim.x / 2 ? bars : bars + 8, 0, 1, &shLostAt, 1u << 12);
+    const bool right = __syncthreads_and(first && !second);
+    if (threadIdx.x == 0 && !right) *(volatile int32_t *)status = kDevBadState;
+}
+
 }  // namespace
+
+rcd_status launch_step_wait_selftest(rcd_ctx *ctx, int32_t *status, cudaStream_t st)
+{
+    step_wait_selftest_kernel<<<1, 128, 0, st>>>(status);
+    ctx->kernelLaunches++;
+    RCD_CUDA(ctx, cudaGetLastError());
+    return RCD_OK;
+}
 
 struct RoundsPlan {
     RoundsParams prm;

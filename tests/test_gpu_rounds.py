@@ -46,3 +46,15 @@ def test_float_norms_far_apart(rcd, orc):
     """A class left in floating point beside those that run in rounds."""
     wl = cluster.workload([141] + [140] * 99, 32, 60, 1, dtype="bf16", scale=lambda rng, M: 10.0 ** rng.uniform(-1.5 if M == 141 else 0.0, 1.5 if M == 141 else 0.1, M))
     check_float(rcd, orc, wl)
+
+
+def test_copies_that_never_arrive(rcd, orc):
+    """The wait for a step's copies runs out for half of the threads only: all of them leave at that step (another status than the
+    timeout's where they do not), and the context goes on."""
+    wl = cluster.workload([37] * 97, 16, 64, 64)
+    with rcd.Context(0) as ctx:
+        ctx.selftest_bounded_wait()
+        with pytest.raises(rcd.RcdError) as e:
+            ctx.sync_status()
+        assert e.value.status == 5          # RCD_ERR_TIMEOUT
+    check_exact(rcd, orc, wl)
