@@ -259,7 +259,7 @@ __device__ __forceinline__ uint32_t greater(uint32_t m, uint32_t x)
     else return __float_as_uint(fmaxf(__uint_as_float(m), __uint_as_float(x)));
 }
 
-constexpr int kFewRuns = 4;                                     // runs of 32 up to which each is gone through by itself
+constexpr int kFewRuns = 6;                                     // runs of 32 up to which each is gone through by itself
 
 constexpr int kWarpCols = kTileN / 32 / (kEpiWarps / 4);       // column blocks of a tile that one epilogue warp takes
 
@@ -267,9 +267,14 @@ constexpr int kWarpCols = kTileN / 32 / (kEpiWarps / 4);       // column blocks 
 // of block b), row i per lane, and for blocks above the diagonal the same with rows and columns exchanged (through shared memory).  A
 // maximum leaves the registers where the block changes: the rows' at the end of a run that may span the tile, the columns' once per
 // 32 rows at least.  colBlock: the blocks of the warp's columns, looked up before the tile was ready.
-// Bound by this epilogue's own instructions and then by the operands' way from L2 (10 classes of 5000 x 512 int8 into 8 blocks: 189 us
-// with a test for every column and row, which 32 of them unrolled pay for even where no run ends; 115 with a pass per run; 95 with no
-// epilogue at all.  Writing S took 200 us and reading it back 200 more).  With more runs than kFewRuns in 32 the tests are cheaper.
+// Bound by this epilogue's own instructions and then by the operands' way from L2 (10 classes of 5000 x 512 int8 into 8 blocks: 95 us
+// with no epilogue at all; writing S took 200 us and reading it back 200 more).  A pass per run of columns as long as they are few; with
+// more runs in 32 than kFewRuns a test per column is cheaper, four columns at a time from shared memory.  The code has to stay short:
+// with that test unrolled for 32 columns in registers, and all of it for each of a warp's column blocks, a warp spent 37 % of its time
+// waiting for instructions.  The whole call in us, through S : that code : as it is, by samples of a class per block (int8, 64 elements):
+//   1000 classes of 400   2 samples 766 : 871 : 737   6  564 : 759 : 531   8  537 : 792 : 485   16  498 : 466 : 353   128  477 : 318 : 275
+//   20 of 2500            4         385 : 385 : 363   6  334 : 386 : 318   8  312 : 439 : 279   16  287 : 238 : 210   625  264 : 151 : 128
+// Runs gone through by themselves up to 3 : 4 : 6 : 8 in 32 (1000 x 400, 8 samples): 521 : 517 : 485 : 475; (4 samples) 638 : 611 : 609 : 620.
 template <bool kInt8, typename Mirrored>
 __device__ __forceinline__ void keep_maxima(uint32_t (*stage)[33], int32_t *cover, const ClassDesc &c, int row0, int colB, uint32_t tmemRow,
                                             int half, int nCb, uint32_t (&v)[32], int rowBlock, const int (&colBlock)[kWarpCols], Mirrored mirrored)
@@ -282,12 +287,15 @@ __device__ __forceinline__ void keep_maxima(uint32_t (*stage)[33], int32_t *cove
     };
     uint32_t m = 0;
     int block = -1;
-#pragma unroll
+#pragma unroll 1
     for (int k = 0; k < kWarpCols; ++k) {
         const int cb = half + k * (kEpiWarps / 4), col0 = colB + cb * 32;
         if (cb >= nCb) break;
-        const uint32_t colStarts = run_starts(colBlock[k]);
-        const int firstBlock = __shfl_sync(0xffffffffu, colBlock[k], 0);
+        int mine = colBlock[0];
+#pragma unroll
+        for (int x = 1; x < kWarpCols; ++x) mine = k == x ? colBlock[x] : mine;
+        const uint32_t colStarts = run_starts(mine);
+        const int firstBlock = __shfl_sync(0xffffffffu, mine, 0);
         const bool mirror = mirrored(cb);
         tmem_load_wait();
         if (firstBlock != block) {
@@ -303,7 +311,7 @@ __device__ __forceinline__ void keep_maxima(uint32_t (*stage)[33], int32_t *cove
         } else if (__popc(colStarts) < kFewRuns) {
             for (uint32_t left = colStarts | 1u; left; left &= left - 1) {
                 const uint32_t later = left & (left - 1), run = (later & (0u - later)) - (left & (0u - left));   // the run's columns
-                const int of = __shfl_sync(0xffffffffu, colBlock[k], __ffs((int)left) - 1);
+                const int of = __shfl_sync(0xffffffffu, mine, __ffs((int)left) - 1);
                 if (of != block) {
                     join(block, row0 + lane, m);
                     m = 0;
@@ -314,21 +322,28 @@ __device__ __forceinline__ void keep_maxima(uint32_t (*stage)[33], int32_t *cove
                 for (int j = 0; j < 32; ++j) part[j & 3] = greater<kInt8>(part[j & 3], run >> j & 1 ? v[j] : 0u);
                 m = greater<kInt8>(greater<kInt8>(part[0], part[1]), greater<kInt8>(part[2], part[3]));
             }
-        } else {
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                if (colStarts >> j & 1) {
-                    join(block, row0 + lane, m);
-                    m = 0;
-                    block = __shfl_sync(0xffffffffu, colBlock[k], j);
-                }
-                m = greater<kInt8>(m, v[j]);
-            }
         }
         // (16-byte pieces, each row's turned by the row's number: neither side meets a bank twice)
-        if (mirror) {
+        const bool manyRuns = __popc(colStarts) >= kFewRuns;
+        if (mirror || manyRuns) {
 #pragma unroll
             for (int g = 0; g < 8; ++g) block4[lane * 8 + (g ^ (lane & 7))] = make_uint4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
+        }
+        if (manyRuns) {
+#pragma unroll 1
+            for (int g = 0; g < 8; ++g) {
+                const uint4 x = block4[lane * 8 + (g ^ (lane & 7))];   // (the lane's own)
+                const uint32_t y[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (colStarts >> (4 * g + j) & 1) {
+                        join(block, row0 + lane, m);
+                        m = 0;
+                        block = __shfl_sync(0xffffffffu, mine, 4 * g + j);
+                    }
+                    m = greater<kInt8>(m, y[j]);
+                }
+            }
         }
         __syncwarp();
         if (cb + kEpiWarps / 4 < nCb) tmem_load_32cols(tmemRow + (uint32_t)((cb + kEpiWarps / 4) * 32), v);

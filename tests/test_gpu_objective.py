@@ -29,6 +29,7 @@ def maxima(S, blocks, W):
     ([127, 128, 129, 255, 257], 96, 2),   # edges of both sides of a tile; runs longer than a row block
     ([300, 40], 64, 150),                 # runs of one or two samples, blocks without any
     ([520, 700], 144, 20),                # two to four runs in 32 rows
+    ([520, 700], 72, 95),                 # five to eight: about as many as are gone through by themselves
     ([900], 200, 1024),                   # the most blocks
 ])
 def test_objective_by_tiles(rcd, orc, sizes, d, W, dtype):
