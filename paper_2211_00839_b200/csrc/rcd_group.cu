@@ -240,11 +240,29 @@ __global__ void __launch_bounds__(1024, 1) chunk_rank_kernel(const int32_t *__re
     }
 }
 
+// Rows of up to 512 bytes are moved eight at a time by a warp, which then reads eight indices at once and has a piece of a row on its way
+// per lane (130000 rows of 64 bytes: 23.6 us a row at a time, 9.9 so).  Wider ones keep a warp busy by themselves.
+constexpr int kGatherRows = 8, kNarrowRow = 512;
 __global__ void __launch_bounds__(256) gather_rows_kernel(const uint8_t *__restrict__ X, const int32_t *__restrict__ perm, int64_t N,
                                                           int64_t rowBytes, int64_t pitch, uint8_t *__restrict__ Xs)
 {
     const int lane = threadIdx.x & 31;
     const bool vec = rowBytes % 16 == 0 && pitch % 16 == 0 && ((uintptr_t)X) % 16 == 0 && ((uintptr_t)Xs) % 16 == 0;
+    if (vec && pitch <= kNarrowRow) {
+        const int np = (int)(pitch >> 4), nx = (int)(rowBytes >> 4);
+        for (int64_t r0 = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * kGatherRows; r0 < N; r0 += (int64_t)gridDim.x * 8 * kGatherRows) {
+            const int pieces = (int)min((int64_t)kGatherRows, N - r0) * np;
+            const int32_t mine = lane < kGatherRows && r0 + lane < N ? perm[r0 + lane] : 0;
+            int4 *const to = reinterpret_cast<int4 *>(Xs + r0 * pitch);
+#pragma unroll 4
+            for (int q0 = 0; q0 < pieces; q0 += 32) {
+                const int q = q0 + lane, row = q / np, piece = q - row * np;
+                const int64_t from = __shfl_sync(0xffffffffu, mine, row & (kGatherRows - 1));
+                if (q < pieces) to[q] = piece < nx ? __ldg(reinterpret_cast<const int4 *>(X + from * rowBytes) + piece) : make_int4(0, 0, 0, 0);
+            }
+        }
+        return;
+    }
     for (int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); r < N; r += (int64_t)gridDim.x * 8)
         copy_row(X + (int64_t)perm[r] * rowBytes, Xs + r * pitch, rowBytes, pitch, vec, lane);
 }

@@ -31,6 +31,7 @@ def maxima(S, blocks, W):
     ([520, 700], 144, 20),                # two to four runs in 32 rows
     ([520, 700], 72, 95),                 # five to eight: about as many as are gone through by themselves
     ([900], 200, 1024),                   # the most blocks
+    ([65, 130], 520, 3),                  # rows of more than 512 bytes
 ])
 def test_objective_by_tiles(rcd, orc, sizes, d, W, dtype):
     wl = cluster.workload(sizes, d, W, 3 + W, dtype=dtype)
