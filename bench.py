@@ -324,20 +324,14 @@ def run_ours(args):
     default_setup = args.classes == 0 and args.sweep_batch in (0, 8) and args.async_group == 0 and args.async_help_min == 0 and args.similarity == "dot"
     loop_s = prof["greedy_ms"] * 1e-3
     # The cluster form makes no sweeps: it reads every row of S once for the gains of empty blocks, then the row of S of every
-    # pick and one per column that the pick raised.  (Rows fetched on foresight whose sample another block received are not
-    # counted: see the traffic of the capture.)
+    # pick and one per column that the pick raised (in rounds: a row read once for several blocks counts once).  (Rows fetched on
+    # foresight whose sample another block received are not counted: see the traffic of the capture.)
     clustered = prof["sweep_bytes"] == 0 and prof["incremental_updates"] > 0
     loop_bytes = 4 * ((M + 7) // 8 * 8) * (wl.N + prof["incremental_rows"] + prof["incremental_updates"]) if clustered else prof["sweep_bytes"]
     achieved = loop_bytes / loop_s / 1e9 if loop_s > 0 else 0.0
-    sms = torch.cuda.get_device_properties(local).multi_processor_count
-    path = args.greedy_path if args.greedy_path else (3 if wl.L * 4 <= sms else 4)
-    if clustered:
-        # (of the configurations only 1000 classes into 64 blocks run in rounds, where a round's rows count once for all blocks)
-        kernel_name = "greedy_rounds_kernel" if args.objective == "facility" and wl.W >= 48 and wl.L >= sms else "greedy_cluster_kernel"
-    elif args.objective != "facility":
-        kernel_name = "cut_chain_kernel"
-    else:
-        kernel_name = {1: "sweep_kernel", 2: "greedy_persistent_kernel", 3: "greedy_async_kernel", 4: "greedy_owner_kernel"}[path]
+    kernel_name = {rcd.RCD_FORM_LAUNCHES: "sweep_kernel", rcd.RCD_FORM_BARRIERS: "greedy_persistent_kernel", rcd.RCD_FORM_ASYNC: "greedy_async_kernel",
+                   rcd.RCD_FORM_CLASS_PER_CTA: "greedy_owner_kernel", rcd.RCD_FORM_CLUSTER: "greedy_cluster_kernel",
+                   rcd.RCD_FORM_ROUNDS: "greedy_rounds_kernel", rcd.RCD_FORM_CUT_CHAIN: "cut_chain_kernel"}[int(prof["greedy_form"])]
     # S larger than L2: the sweeps stream from HBM (peak: the measured copy bandwidth); S inside L2: they stream from
     # L2 (peak: this library's read-only sweep yardstick over an L2-resident buffer, measured in this run)
     bound = "l2" if fits_l2 else "hbm"

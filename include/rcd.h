@@ -79,8 +79,10 @@ typedef struct {
     int32_t sweep_batch_max;   /* blocks whose gains one pass over S may refresh: 1,2,4 or 8; 0 = default (8) */
     int32_t similarity_path;   /* 0 = tensor-core kernel when the shape allows, 2 = always the generic kernel */
     int32_t profile;           /* 0 off; 1 time the phases of rcd_partition; 2 also time every sweep launch */
-    int32_t greedy_path;       /* form of the greedy loop.  0 = choose: one thread-block cluster per class (at most 128 blocks,
-                                  none of the options below set), else asynchronous classes (3) when there are at most a quarter
+    int32_t greedy_path;       /* form of the greedy loop.  0 = choose: one thread-block cluster per class, or one CTA per class in
+                                  rounds of picks and corrections where classes of about one size fill the SMs and blocks are
+                                  many (both: at most 128 blocks, none of the options below set; rcd_profile.greedy_form tells
+                                  which ran), else asynchronous classes (3) when there are at most a quarter
                                   as many classes as SMs, else one CTA per class (4);  1 = two launches per round (always
                                   used with profile 2);  2 = one cooperative launch, rounds of a sweep phase and a pick phase
                                   separated by grid barriers;  3 = one cooperative launch, every class cycles between sweep and
@@ -118,7 +120,17 @@ typedef struct {
                                   path 3, where a pass is served by the whole GPU; 64 for path 4); at most 128 */
 } rcd_config;
 
-/* Timings and counters of the last rcd_partition / rcd_partition_host on a context (profile >= 1). */
+/* Forms of the greedy loop: 1 to 4 are those of rcd_config.greedy_path, the others are only chosen by the library.  (Classes that
+ * the cluster form or rounds leave in floating point run in 3 or 4 beside it.) */
+typedef enum {
+    RCD_FORM_LAUNCHES = 1, RCD_FORM_BARRIERS = 2, RCD_FORM_ASYNC = 3, RCD_FORM_CLASS_PER_CTA = 4,
+    RCD_FORM_CLUSTER = 5,      /* a thread-block cluster per class */
+    RCD_FORM_ROUNDS = 6,       /* a CTA per class, in rounds */
+    RCD_FORM_CUT_CHAIN = 7     /* graph cut, a CTA per class */
+} rcd_greedy_form;
+
+/* Timings and counters of the last rcd_partition / rcd_partition_host on a context (profile >= 1).  New ones are added at the end:
+ * build a program with the header of the library it runs with. */
 typedef struct {
     double  total_ms;          /* whole call, first to last kernel, on the call's stream */
     double  group_ms;          /* class split + feature gather */
@@ -143,14 +155,18 @@ typedef struct {
     int64_t async_attempts;         /* ... and times it tried (an attempt fails when the tickets run out under way) */
     int64_t lazy_sweeps;            /* threshold passes that skipped rows below the blocks' floors */
     int64_t lazy_misses;            /* picks whose best stored gain lay below its block's floor (answered by a pass over every row);
-                                       cluster form: times a block's leading candidates had all been taken (answered by a scan) */
+                                       cluster form and rounds: times a block's leading candidates had all been taken (answered by a scan) */
     int64_t lazy_rows;              /* rows of S those passes did read */
     int64_t lazy_rows_skipped;      /* rows they did not */
     int64_t incremental_updates;    /* picks after which the block's stored gains were corrected in place (no pass needed) */
-    int64_t incremental_rows;       /* rows of S those corrections read (one per column whose coverage rose) */
+    int64_t incremental_rows;       /* rows of S those corrections read: one per column whose coverage rose, but in rounds a row that
+                                       several blocks of a batch need counts once where it was read once for all of them */
     int64_t threshold_pass_ns;      /* one CTA per class: time the first CTA spent in threshold passes (part of persistent_sweep_ns) */
     int64_t threshold_pass_bytes;   /* bytes of S and threshold vectors the (row-visiting) threshold passes had to read (part of sweep_bytes) */
     int64_t noted_picks;            /* picks whose v* was noted when the block's stored gains were last corrected (no argmax over stored gains) */
+    int64_t greedy_form;            /* rcd_greedy_form of the last rcd_partition (0: no class had a sample); profile 0 too */
+    int64_t round_lists;            /* rounds: batches of picks corrected from one row of S per raised column ... */
+    int64_t round_tiles;            /* ... and from every row that any pick of the batch raised, once for all its blocks */
 } rcd_profile;
 
 typedef struct rcd_ctx rcd_ctx;

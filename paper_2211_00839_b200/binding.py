@@ -26,6 +26,7 @@ RCD_SIM_DOT = 0
 RCD_SIM_GAUSSIAN = 1
 RCD_OBJ_FACILITY = 0
 RCD_OBJ_GRAPH_CUT = 1
+RCD_FORM_LAUNCHES, RCD_FORM_BARRIERS, RCD_FORM_ASYNC, RCD_FORM_CLASS_PER_CTA, RCD_FORM_CLUSTER, RCD_FORM_ROUNDS, RCD_FORM_CUT_CHAIN = range(1, 8)
 
 STATUS_NAMES = {0: "RCD_OK", 1: "RCD_ERR_INVALID_ARG", 2: "RCD_ERR_UNSUPPORTED", 3: "RCD_ERR_WORKSPACE_TOO_SMALL",
                 4: "RCD_ERR_CUDA", 5: "RCD_ERR_TIMEOUT", 6: "RCD_ERR_INTERNAL"}
@@ -62,7 +63,8 @@ class RcdProfile(C.Structure):
                 ("threshold_elems", C.c_int64), ("threshold_max_blocks", C.c_int64),
                 ("async_lull_ns", C.c_int64), ("async_visits", C.c_int64), ("async_attempts", C.c_int64),
                 ("lazy_sweeps", C.c_int64), ("lazy_misses", C.c_int64), ("lazy_rows", C.c_int64),
-                ("lazy_rows_skipped", C.c_int64), ("incremental_updates", C.c_int64), ("incremental_rows", C.c_int64), ("threshold_pass_ns", C.c_int64), ("threshold_pass_bytes", C.c_int64), ("noted_picks", C.c_int64)]
+                ("lazy_rows_skipped", C.c_int64), ("incremental_updates", C.c_int64), ("incremental_rows", C.c_int64), ("threshold_pass_ns", C.c_int64), ("threshold_pass_bytes", C.c_int64), ("noted_picks", C.c_int64),
+                ("greedy_form", C.c_int64), ("round_lists", C.c_int64), ("round_tiles", C.c_int64)]
 
 
 def _load() -> C.CDLL:

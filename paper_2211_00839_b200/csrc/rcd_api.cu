@@ -478,6 +478,7 @@ rcd_status rcd_get_profile(rcd_ctx *ctx, rcd_profile *out)
     out->kernel_launches = ctx->kernelLaunches;
     out->steps = ctx->steps;
     out->similarity_tc_launches = ctx->tcLaunches;
+    out->greedy_form = ctx->greedyForm;
     if (!ctx->phaseValid) return RCD_OK;
     RCD_CUDA(ctx, cudaEventSynchronize(ctx->evPhase[4]));
     float ms = 0.f;
@@ -497,6 +498,8 @@ rcd_status rcd_get_profile(rcd_ctx *ctx, rcd_profile *out)
         out->incremental_updates = (int64_t)ns[15];
         out->incremental_rows = (int64_t)ns[16];
         out->noted_picks = (int64_t)ns[17];
+        out->round_lists = (int64_t)ns[18];
+        out->round_tiles = (int64_t)ns[19];
         out->threshold_pass_ns = (int64_t)ns[13];
         out->threshold_pass_bytes = (int64_t)ns[14];
         out->persistent_sweep_ns = (int64_t)ns[0];
@@ -720,6 +723,7 @@ rcd_status rcd_partition(rcd_ctx *ctx, const void *features_dev, rcd_feat_dtype 
     ctx->kernelLaunches = 0;
     ctx->tcLaunches = 0;
     ctx->steps = 0;
+    ctx->greedyForm = 0;
     ctx->passes = 0;
     ctx->phaseValid = false;
     ctx->stepBytesDev = nullptr;

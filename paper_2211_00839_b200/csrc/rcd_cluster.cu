@@ -1532,6 +1532,7 @@ rcd_status launch_greedy_cluster(rcd_ctx *ctx, ClusterPlan &plan, const Sizes &s
         if (rs != RCD_OK) return rs;
     }
     ctx->steps = sz.maxM;
+    ctx->greedyForm = plan.rounds ? RCD_FORM_ROUNDS : RCD_FORM_CLUSTER;
     ctx->phaseNsDev = ws.phaseNs;
     if (toFix) RCD_CUDA(ctx, cudaEventSynchronize(ctx->evCounts));
     if (toFix && *left) return launch_greedy_not_fixed(ctx, sz, ws, descHost, assignment, order, partValues, st);

@@ -242,6 +242,7 @@ static rcd_status run_cut(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, in
 rcd_status launch_cut(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, int32_t *assignment, int32_t *order, cudaStream_t st)
 {
     if (sz.L == 0 || sz.maxM == 0) return RCD_OK;
+    ctx->greedyForm = RCD_FORM_CUT_CHAIN;
     if (sz.floatArith) return run_cut<float>(ctx, sz, ws, assignment, order, st);
     return run_cut<int32_t>(ctx, sz, ws, assignment, order, st);
 }

@@ -2558,6 +2558,7 @@ static rcd_status run_greedy(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws,
         }
         if (perSm < 1) path = only ? 4 : 1;
     }
+    if (!only) ctx->greedyForm = path;
     if (path == 4) {
         RCD_CUDA(ctx, cudaFuncSetAttribute(ownerKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         // (in-place correction of stored gains: a class's passes are made by one SM here, so their cost grows with the

@@ -245,6 +245,7 @@ struct rcd_ctx {
     int64_t kernelLaunches = 0;
     int64_t tcLaunches = 0;
     int64_t steps = 0;
+    int64_t greedyForm = 0;             // rcd_greedy_form of the last rcd_partition
     int64_t passes = 0;                 // entries of stepBytes / stepOps that count
     const unsigned long long *stepBytesDev = nullptr;
     const unsigned long long *stepOpsDev = nullptr;

@@ -228,6 +228,7 @@ __global__ void __launch_bounds__(kWarps * 32, kMaxWarps / kWarps) greedy_rounds
     __shared__ uint8_t shHas[kRoundBlocks];
     __shared__ __align__(8) unsigned long long shBars[kStages];
     __shared__ int shMostBy, shMade, shClass, shCommand, shListed, shNeeded, shFailed, shLostAt;
+    __shared__ unsigned shLists, shTiles;     // batches corrected either way
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int W = prm.W;
     unsigned char *const ring = shared + prm.offRing;
@@ -249,6 +250,7 @@ __global__ void __launch_bounds__(kWarps * 32, kMaxWarps / kWarps) greedy_rounds
 
     if (threadIdx.x == 0) {
         shLostAt = INT_MAX;
+        shLists = shTiles = 0;
         for (int k = 0; k < kStages; ++k) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(bars + 8 * k) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -506,7 +508,10 @@ __global__ void __launch_bounds__(kWarps * 32, kMaxWarps / kWarps) greedy_rounds
                 // One row from memory per raised column, or every row once and all blocks against it.  In cycles per 128 columns: a row
                 // from memory 14, a row against a block 2.3, and what a table costs.
                 if (total <= prm.listShared && total * 16 <= need * max(2 * nP4, 14) + 3000) {
-                    if (threadIdx.x == 0) rowsRead += total;
+                    if (threadIdx.x == 0) {
+                        rowsRead += total;
+                        ++shLists;
+                    }
                     // (by blocks)
                     for (int i = threadIdx.x; i < total; i += kThreads) {
                         const int4 e = listShared[i];
@@ -542,7 +547,10 @@ __global__ void __launch_bounds__(kWarps * 32, kMaxWarps / kWarps) greedy_rounds
                         }
                     }
                 } else {
-                    if (threadIdx.x == 0) rowsRead += need;
+                    if (threadIdx.x == 0) {
+                        rowsRead += need;
+                        ++shTiles;
+                    }
                     const int need4 = (need + 3) & ~3;
                     for (int i = threadIdx.x; i < need * (nP4 - nP); i += kThreads) table[i / (nP4 - nP) * nP4 + nP + i % (nP4 - nP)] = make_int2(0, 0);
                     for (int i = threadIdx.x; i < (need4 - need) * nP4; i += kThreads) table[need * nP4 + i] = make_int2(0, 0);
@@ -685,6 +693,8 @@ __global__ void __launch_bounds__(kWarps * 32, kMaxWarps / kWarps) greedy_rounds
         if (corrected) {
             atomicAdd(prm.stats + 15, corrected);
             atomicAdd(prm.stats + 16, rowsRead);
+            atomicAdd(prm.stats + 18, (unsigned long long)shLists);
+            atomicAdd(prm.stats + 19, (unsigned long long)shTiles);
         }
     }
 }

@@ -9,6 +9,20 @@ from test_gpu_parity import check_exact, check_float, rcd, orc  # noqa: F401  (f
 pytestmark = pytest.mark.gpu
 
 
+def ran_in_rounds(rcd, wl, lists=None, tiles=None, **cfg):
+    """Whether the library takes the problem in rounds, and whether it corrects by lists and by tiles (None: either will do)."""
+    import torch
+    with rcd.Context(0, profile=1, **cfg) as ctx:
+        ctx.rcd_partition(rcd.features_to_torch(wl.features, device="cuda"), torch.from_numpy(wl.labels).cuda(), wl.capacities, wl.L,
+                          M_max=int(np.bincount(wl.labels).max()))
+        ctx.sync_status()
+        prof = ctx.profile()
+    print("form %d, lists %d, tiles %d" % (prof["greedy_form"], prof["round_lists"], prof["round_tiles"]))
+    assert prof["greedy_form"] == rcd.RCD_FORM_ROUNDS
+    assert lists is None or (prof["round_lists"] > 0) == lists
+    assert tiles is None or (prof["round_tiles"] > 0) == tiles
+
+
 @pytest.mark.parametrize("sizes,d,W", [
     ([37] * 97, 16, 64),                          # fewer samples than blocks; batches of fewer blocks than wait (narrow features)
     ([129, 128, 127, 126] * 25, 40, 48),          # edges of 128 columns
@@ -19,7 +33,17 @@ pytestmark = pytest.mark.gpu
 ])
 @pytest.mark.parametrize("copies", [0, 30])
 def test_int8_exact(rcd, orc, sizes, d, W, copies):
-    check_exact(rcd, orc, cluster.workload(sizes, d, W, W + copies, copies=copies))
+    wl = cluster.workload(sizes, d, W, W + copies, copies=copies)
+    check_exact(rcd, orc, wl)
+    ran_in_rounds(rcd, wl)
+
+
+def test_int8_sums_beyond_32_bits(rcd, orc):
+    """The losses of a column add up to more than 2^32 (300 rows, each of up to 2048 x 127^2): they are widened on the way."""
+    wl = cluster.workload([300] * 98, 2048, 60, 7)
+    wl.features = np.random.default_rng(7).integers(90, 128, size=wl.features.shape).astype(np.int8)
+    check_exact(rcd, orc, wl)
+    ran_in_rounds(rcd, wl, tiles=True)
 
 
 @pytest.mark.parametrize("sizes,d,W", [([1000] * 148, 32, 16), ([1003] * 148, 256, 40), ([1610] * 140, 64, 49)])
@@ -34,18 +58,22 @@ def test_int8_like_the_passes(rcd, sizes, d, W):
             ctx.sync_status()
     for got, want in zip(*results):
         assert torch.equal(got, want)
+    ran_in_rounds(rcd, wl, lists=True, tiles=True)
 
 
 @pytest.mark.parametrize("similarity", ["gaussian", "dot"])
 @pytest.mark.parametrize("sizes,W", [([101] * 98, 57), ([66] * 60, 70)])
 def test_float_is_exact_in_fixed_point(rcd, orc, similarity, sizes, W):
     cluster.test_float_is_exact_in_fixed_point(rcd, orc, similarity, sizes, W)
+    ran_in_rounds(rcd, cluster.workload(sizes, 64, W, 5 * W, dtype="bf16"),
+                  similarity_kind=rcd.RCD_SIM_GAUSSIAN if similarity == "gaussian" else rcd.RCD_SIM_DOT)
 
 
 def test_float_norms_far_apart(rcd, orc):
     """A class left in floating point beside those that run in rounds."""
     wl = cluster.workload([141] + [140] * 99, 32, 60, 1, dtype="bf16", scale=lambda rng, M: 10.0 ** rng.uniform(-1.5 if M == 141 else 0.0, 1.5 if M == 141 else 0.1, M))
     check_float(rcd, orc, wl)
+    ran_in_rounds(rcd, wl)
 
 
 def test_copies_that_never_arrive(rcd, orc):
@@ -58,3 +86,4 @@ def test_copies_that_never_arrive(rcd, orc):
             ctx.sync_status()
         assert e.value.status == 5          # RCD_ERR_TIMEOUT
     check_exact(rcd, orc, wl)
+    ran_in_rounds(rcd, wl)
