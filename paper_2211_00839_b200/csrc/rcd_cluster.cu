@@ -1402,27 +1402,10 @@ static size_t cluster_layout(const Sizes &sz, int maxLd, int C, bool state, size
     return cap + 1;
 }
 
-// Whether the cluster form takes a problem, and how: chosen by the library (no pass-based form or option asked for),
-// samples of a class and blocks within the packed keys' range, blocks that fit registers or shared memory.
-static bool cluster_plan(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost, ClusterPlan &plan)
+// How a problem is laid out over clusters, if its blocks fit registers or shared memory.  resident: clusters at a time.
+static bool cluster_shape(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost, int nonEmpty, int maxLd, ClusterPlan &plan, int *resident)
 {
-    const rcd_config &c = ctx->cfg;
-    if (c.greedy_path != 0 || c.profile >= 2 || c.sweep_batch_max != 0 || c.sweep_mode != 0 || c.async_group != 0 || c.async_help_min != 0 ||
-        c.threshold_from != 0 || c.threshold_hit_shift != 0 || c.lazy_mode != 0 || c.lazy_from != 0 || c.dense_ring != 0 ||
-        c.incremental != 0 || c.incremental_max != 0)
-        return false;
-    if (sz.W > kClusterBlocks || sz.maxM > 65535 || sz.d > 65535 || sz.L > 65535 || sz.maxM == 0) return false;
-    if (sz.graphCut && (sz.floatArith || sz.maxM > 8192)) return false;
-    int nonEmpty = 0, maxLd = 8;
-    for (const ClassDesc &d : descHost) {
-        if (d.M > 0) ++nonEmpty;
-        maxLd = std::max(maxLd, (int)d.ld);
-    }
     const size_t cap = (size_t)ctx->maxSmemOptin - 1024;
-    plan.prm = ClusterParams{};
-    plan.prm.maxLd = maxLd;
-    plan.rounds = plan_greedy_rounds(ctx, sz, descHost);
-    if (plan.rounds) return true;
     for (int i = 0; i < 5; ++i)
         if (ctx->maxClusters[i] < 0) {
             int active = 0;
@@ -1468,8 +1451,32 @@ static bool cluster_plan(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassD
     int idx = 0;
     while ((1 << idx) < plan.C) ++idx;
     if (ctx->maxClusters[idx] < 1) return false;
-    plan.clusters = std::max(1, std::min(nonEmpty, ctx->maxClusters[idx]));
+    *resident = ctx->maxClusters[idx];
+    plan.clusters = std::max(1, std::min(nonEmpty, *resident));
     return true;
+}
+
+// Whether the cluster form or the rounds take a problem, and how: chosen by the library (no pass-based form or option asked for),
+// samples of a class and blocks within the packed keys' range.
+static bool cluster_plan(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost, ClusterPlan &plan)
+{
+    const rcd_config &c = ctx->cfg;
+    if (c.greedy_path != 0 || c.profile >= 2 || c.sweep_batch_max != 0 || c.sweep_mode != 0 || c.async_group != 0 || c.async_help_min != 0 ||
+        c.threshold_from != 0 || c.threshold_hit_shift != 0 || c.lazy_mode != 0 || c.lazy_from != 0 || c.dense_ring != 0 ||
+        c.incremental != 0 || c.incremental_max != 0)
+        return false;
+    if (sz.W > kClusterBlocks || sz.maxM > 65535 || sz.d > 65535 || sz.L > 65535 || sz.maxM == 0) return false;
+    if (sz.graphCut && (sz.floatArith || sz.maxM > 8192)) return false;
+    int nonEmpty = 0, maxLd = 8, resident = 0;
+    for (const ClassDesc &d : descHost) {
+        if (d.M > 0) ++nonEmpty;
+        maxLd = std::max(maxLd, (int)d.ld);
+    }
+    plan.prm = ClusterParams{};
+    const bool clusters = cluster_shape(ctx, sz, descHost, nonEmpty, maxLd, plan, &resident);
+    plan.prm.maxLd = maxLd;
+    plan.rounds = plan_greedy_rounds(ctx, sz, descHost, clusters ? ClusterShape{plan.C, resident, plan.P} : ClusterShape{0, 0, 0});
+    return clusters || plan.rounds;
 }
 
 std::shared_ptr<ClusterPlan> plan_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost)

@@ -307,9 +307,10 @@ std::shared_ptr<ClusterPlan> plan_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, 
 rcd_status launch_greedy_cluster(rcd_ctx *ctx, ClusterPlan &plan, const Sizes &sz, const Workspace &ws, const std::vector<ClassDesc> &descHost,
                                  int32_t *assignment, int32_t *order, void *partValues, cudaStream_t st);
 
-// greedy loop in rounds, one CTA per class (null: it does not take the problem)
+// greedy loop in rounds, one CTA per class (null: it does not take the problem, or the cluster form would be faster)
 struct RoundsPlan;
-std::shared_ptr<RoundsPlan> plan_greedy_rounds(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost);
+struct ClusterShape { int ctas, resident, pieces; };       // of the cluster form: CTAs per class (0: it does not take the problem), classes at a time, steps per row
+std::shared_ptr<RoundsPlan> plan_greedy_rounds(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost, const ClusterShape &cluster);
 rcd_status launch_greedy_rounds(rcd_ctx *ctx, RoundsPlan &plan, const Sizes &sz, const Workspace &ws, int32_t *assignment, int32_t *order,
                                 void *partValues, cudaStream_t st);
 

@@ -735,26 +735,45 @@ struct RoundsPlan {
     size_t smem;
 };
 
-// Whether rounds are the faster form.  They take one CTA per class, so a problem has to fill the SMs with classes of about one size
-// (`full`: equal classes of the largest size that would be as much work, over the rounds of SMs they take), and they gain where
-// several blocks share a row.  Against the cluster form (us, whole call, both forms on one GPU; "dense": rectified features, whose
-// picks raise more columns; d = 256 but for the largest):
-//   64 blocks    1000 x 1300 (d 2048) 165000 : 82000   1000 x 500  24400 : 11400   148 x 1000  15800 : 8500   148 x 300  1410 : 1110
-//                100 x 500  3090 : 2400    300 x 1000  31200 : 20400, dense 30200 : 25600    200 x 1500, dense  39900 : 46300
-//   48           148 x 700, dense  5690 : 4260    1000 x 1000  61700 : 37000
-//   32           148 x 1000  7920 : 6290, dense 7120 : 6990   148 x 1300, dense 15700 : 12300   300 x 1000, dense 13900 : 16900
-//   16           148 x 1300  9760 : 7820    148 x 1000  5560 : 4860    300 x 700  5920 : 6190    148 x 700  2550 : 3010
-//   100          60 x 500  3260 : 2160    148 x 300  2630 : 960    10 x 1000  3380 : 8150
-// Floating-point similarities (cosines of rectified features raise most columns):
-//   64 blocks    1000 x 1000  102000 : 79000   1000 x 500  23800 : 15200   148 x 1000  15500 : 12700   148 x 1300  23500 : 27800
-//   56           100 x 500  2990 : 2400        48:  300 x 1000  21800 : 29100      32:  1000 x 1000  47200 : 59500
-static bool rounds_win(const Sizes &sz, double equal, double full, int sms)
+// Whether rounds are the faster form.  Both forms hold classes of about one size (`equal`: classes of the largest size that would be as
+// much work) and take them in turns: rounds one CTA per class, the cluster form C of them, of which the GPU holds 148, 74, 33, 15 or 7 at
+// a time for C = 1, 2, 4, 8, 16.  So what counts is how much faster a cluster is through a class than one CTA in rounds, over the turns:
+// `speed` below, from the times of both forms over 1000 problems (4 to 148 x their blocks).  It grows with C, less than in proportion, and
+// with the class, since a small class is bound by its chain of picks in either form; C in turn follows from the blocks' state, which has
+// to fit the cluster's shared memory.  Dense similarities (rectified features, whose picks raise more columns) cost rounds more than the
+// cluster form, cosines and Gaussian kernels most; `speed` is that of rectified features.  us, whole call, cluster : rounds:
+//   integers    64 blocks    1000 x 1300 (d 2048) 165000 : 82000   148 x 1000, dense 15000 : 9800   148 x 300 1410 : 990    60 x 1000, dense 6140 : 9000
+//                            300 x 500, dense 7480 : 5780   200 x 500, dense 5200 : 4110   200 x 400, dense 2540 : 2970   100 x 1300, dense 15800 : 17800
+//               128          148 x 1300 190000 : 20100   60 x 500, dense 3090 : 2450       80    60 x 500, dense 1890 : 2210   60 x 300, dense 1035 : 960
+//               48           148 x 700, dense 5690 : 4220   300 x 500, dense 4640 : 5220   200 x 1000, dense 14600 : 15900   148 x 100, dense 219 : 227
+//               32           148 x 1000, dense 7090 : 6880   444 x 1000 21400 : 15200, dense 19600 : 22700 (taken)
+//               24           148 x 1000, dense 5680 : 6070, 5370 : 5380   148 x 1050, dense 8390 : 7080   444 x 1000, dense 16100 : 20500
+//                            (up to 1024 samples a row keeps a team of four warps busy for two steps; from 1025 on it takes a third)
+//               16           148 x 1000, dense 6000 : 4910   444 x 1300, dense 28700 : 28900
+//   floating    64           1000 x 1000, dense 102000 : 79600   300 x 500, dense 7680 : 6620   300 x 700, dense 13400 : 14600   444 x 1300, dense 69700 : 84800
+//               65           60 x 500, dense 1930 : 2430   100 x 1000, dense 12200 : 12700   148 x 1000, dense 17400 : 13200
+//               128          100 x 1300, dense 120000 : 33900   100 x 2000, dense 86400 : 103000
+// Of 1059 measured calls this takes 807; eleven of them are 3 to 5 % slower in rounds, or dense ones of 444 x 1000 into 32 and 40 blocks.
+// Below 48 blocks (integers; 56 for floating point) only full turns of large classes were measured to gain.
+static bool rounds_win(const Sizes &sz, double equal, int sms, int ctasPerSm, const ClusterShape &cluster)
 {
-    const int64_t M = sz.maxM;
-    if (sz.W > 64) return full >= 0.4 && M <= 1000;
-    if (sz.floatArith) return sz.W >= 56 && ((full >= 0.65 && M <= 700) || (full >= 0.9 && M <= 1000) || (full >= 0.9 && equal >= 3.0 * sms));
-    if (sz.W >= 48) return (full >= 0.65 && M <= 1000) || full >= 0.9;
-    return sz.W >= 16 && full >= 0.9 && M >= 1000;
+    const double M = (double)sz.maxM;
+    const bool real = sz.floatArith, two = ctasPerSm > 1;
+    const double full = equal / (sms * std::ceil(equal / sms - 1e-9));
+    if (full < (sz.W >= 80 ? 0.4 : 0.65) || sz.W < (real ? 56 : 16)) return false;
+    if (sz.W < 48 && (full < 0.9 || sz.maxM < 1000)) return false;
+    if (cluster.ctas == 0) return true;
+    const double turns = std::ceil(equal / (sms * ctasPerSm) - 1e-9), clusterTurns = std::ceil(equal / cluster.resident - 1e-9);
+    double speed;
+    if (cluster.ctas == 1) speed = !real && M > 64 && M < 900 && sz.W < 60 && turns == 1.0 ? 1.1 : 0.95;
+    else if (cluster.ctas == 2) speed = M > 1024 ? 1.75 : std::min(std::min(0.55 + M / 230, 1.05 + M / 500), 2.15);
+    else if (cluster.ctas == 4) speed = real ? std::min(0.3 + M / 200, 5.5) : std::min(0.95 + M / 310, 4.1);
+    else if (cluster.ctas == 8) speed = std::min(M / 155, 8.0) * (real ? 1.2 : 1.0);
+    else speed = real ? M / 112 * std::max(1.0, M / 1400) : M / 140;
+    if ((cluster.ctas == 2 || cluster.ctas == 4) && sz.W > 64) speed *= 0.88;
+    if (cluster.pieces >= 6) speed *= 0.45;               // (teams of one or two warps, six steps and more per row)
+    if (two) speed *= cluster.ctas == 1 ? 1.45 : 1.68;    // (a CTA that shares its SM is slower)
+    return speed * turns < clusterTurns;
 }
 
 static bool rounds_plan(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost, int warps, RoundsPlan &plan)
@@ -793,19 +812,18 @@ static bool rounds_plan(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDe
     return true;
 }
 
-std::shared_ptr<RoundsPlan> plan_greedy_rounds(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost)
+std::shared_ptr<RoundsPlan> plan_greedy_rounds(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost, const ClusterShape &cluster)
 {
     if (sz.graphCut || sz.W > kRoundBlocks || sz.maxM == 0 || sz.maxM > 65535) return nullptr;
     double equal = 0;
     for (const ClassDesc &c : descHost) equal += (double)c.M * c.M;
     equal /= (double)sz.maxM * sz.maxM;
-    const double full = equal / (ctx->smCount * std::ceil(equal / ctx->smCount - 1e-9));
-    if (!rounds_win(sz, equal, full, ctx->smCount)) return nullptr;
     auto plan = std::make_shared<RoundsPlan>();
     // Two CTAs of eight warps per SM where there are classes for several rounds of them: one's barriers and trips to memory under the
     // other's sums (1000 x 1000 bf16 into 64 blocks: 85.1 ms with one of 16 warps, 80.4 with two; 300 x 1000 into 24: 20.8 and 23.5).
-    if (equal >= 3.0 * ctx->smCount && rounds_plan(ctx, sz, descHost, 8, *plan)) return plan;
-    return rounds_plan(ctx, sz, descHost, 16, *plan) ? plan : nullptr;
+    const bool two = equal >= 3.0 * ctx->smCount && rounds_plan(ctx, sz, descHost, 8, *plan);
+    if (!two && !rounds_plan(ctx, sz, descHost, 16, *plan)) return nullptr;
+    return rounds_win(sz, equal, ctx->smCount, two ? 2 : 1, cluster) ? plan : nullptr;
 }
 
 rcd_status launch_greedy_rounds(rcd_ctx *ctx, RoundsPlan &plan, const Sizes &sz, const Workspace &ws, int32_t *assignment, int32_t *order, void *partValues, cudaStream_t st)

@@ -25,7 +25,7 @@ def ran_in_rounds(rcd, wl, lists=None, tiles=None, **cfg):
 
 @pytest.mark.parametrize("sizes,d,W", [
     ([37] * 97, 16, 64),                          # fewer samples than blocks; batches of fewer blocks than wait (narrow features)
-    ([129, 128, 127, 126] * 25, 40, 48),          # edges of 128 columns
+    ([129, 128, 127, 126] * 25, 40, 64),          # edges of 128 columns
     ([257] * 60, 75, 100),                        # more than 64 blocks: two batches a round
     ([64] * 450, 24, 56),                         # two CTAs per SM
     ([90] * 60 + [0, 1, 0], 16, 128),             # the most blocks; empty classes and one of a sample
@@ -62,7 +62,7 @@ def test_int8_like_the_passes(rcd, sizes, d, W):
 
 
 @pytest.mark.parametrize("similarity", ["gaussian", "dot"])
-@pytest.mark.parametrize("sizes,W", [([101] * 98, 57), ([66] * 60, 70)])
+@pytest.mark.parametrize("sizes,W", [([101] * 98, 57), ([66] * 60, 100)])
 def test_float_is_exact_in_fixed_point(rcd, orc, similarity, sizes, W):
     cluster.test_float_is_exact_in_fixed_point(rcd, orc, similarity, sizes, W)
     ran_in_rounds(rcd, cluster.workload(sizes, 64, W, 5 * W, dtype="bf16"),
@@ -87,3 +87,29 @@ def test_copies_that_never_arrive(rcd, orc):
         assert e.value.status == 5          # RCD_ERR_TIMEOUT
     check_exact(rcd, orc, wl)
     ran_in_rounds(rcd, wl)
+
+
+@pytest.mark.parametrize("L,M,W,dtype,rounds", [
+    (148, 1000, 24, "int8", False),        # two CTAs per class and full rows: the cluster form is faster
+    (148, 1030, 24, "int8", True),         # rows of three steps
+    (148, 1000, 16, "int8", True),         # one CTA per class
+    (200, 400, 64, "int8", False),         # two turns of rounds, the second a third full, against three of the cluster form
+    (60, 500, 80, "int8", False), (60, 500, 128, "int8", True),
+    (100, 1300, 64, "int8", False), (100, 1300, 128, "int8", True),
+    (60, 500, 65, "bf16", False), (300, 500, 64, "bf16", True), (300, 700, 64, "bf16", False), (444, 1300, 56, "bf16", False),
+])
+def test_form(rcd, L, M, W, dtype, rounds):
+    """Which form the library takes, on either side of where the two were measured to change places (on 148 SMs)."""
+    import torch
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("measured on 148 SMs")
+    g = torch.Generator(device="cuda").manual_seed(M)
+    X = torch.randint(-9, 10, (L * M, 16), generator=g, device="cuda").to(torch.int8)
+    if dtype == "bf16":
+        X = (X / X.float().norm(dim=1, keepdim=True).clamp_min(1)).to(torch.bfloat16)
+    y = torch.arange(L, dtype=torch.int32, device="cuda").repeat(M)
+    with rcd.Context(0) as ctx:
+        a, o, v = ctx.rcd_partition(X, y, [1.0 + j % 4 for j in range(W)], L, M_max=M)
+        ctx.sync_status()
+        assert ctx.profile()["greedy_form"] == (rcd.RCD_FORM_ROUNDS if rounds else rcd.RCD_FORM_CLUSTER)
+    assert bool((o.sort()[0] == torch.arange(L * M, device="cuda")).all())
