@@ -1421,19 +1421,32 @@ static bool cluster_shape(rcd_ctx *ctx, const Sizes &sz, const std::vector<Class
     std::vector<int> sizes;
     for (const ClassDesc &d : descHost) if (d.M > 0) sizes.push_back(d.M);
     std::sort(sizes.begin(), sizes.end(), std::greater<int>());
+    std::vector<double> busy;
     double bestTime = 0;
     plan.C = 0;
     for (int i = 0; (1 << i) <= most; ++i) {
         const int C = 1 << i, n = ctx->maxClusters[i];
         if (n < 1) continue;
         if (cluster_layout(sz, maxLd, C, true, cap, plan) > cap) continue;
+        const size_t held = std::min<size_t>((size_t)n, sizes.size());
+        auto cost = [&](int M) { return (double)M * ((double)M / C + 300.0); };
+        // (all clusters busy to the end: no sooner than that.  A call of many small classes waits for the host here, 874 of up to 253
+        // samples 225 us without this)
+        double work = 0;
+        for (int M : sizes) work += cost(M);
+        if (plan.C > 0 && work / (double)held * (1 - 1e-9) > bestTime) continue;
         double time = 0;
-        std::vector<double> busy((size_t)std::min<size_t>((size_t)n, sizes.size()), 0.0);      // (a heap of the clusters' finishing times)
+        busy.assign(held, 0.0);                            // a heap of the clusters' finishing times, the earliest first
         for (int M : sizes) {
-            std::pop_heap(busy.begin(), busy.end(), std::greater<double>());
-            busy.back() += (double)M * ((double)M / C + 300.0);
-            time = std::max(time, busy.back());
-            std::push_heap(busy.begin(), busy.end(), std::greater<double>());
+            const double done = busy[0] + cost(M);
+            time = std::max(time, done);
+            size_t at = 0;
+            for (size_t child; (child = 2 * at + 1) < held; at = child) {
+                if (child + 1 < held && busy[child + 1] < busy[child]) ++child;
+                if (busy[child] >= done) break;
+                busy[at] = busy[child];
+            }
+            busy[at] = done;
         }
         if (plan.C == 0 || time < bestTime) { plan.C = C; bestTime = time; }
     }

@@ -754,14 +754,12 @@ struct RoundsPlan {
 //               65           60 x 500, dense 1930 : 2430   100 x 1000, dense 12200 : 12700   148 x 1000, dense 17400 : 13200
 //               128          100 x 1300, dense 120000 : 33900   100 x 2000, dense 86400 : 103000
 // Of 1059 measured calls this takes 807; eleven of them are 3 to 5 % slower in rounds, or dense ones of 444 x 1000 into 32 and 40 blocks.
-// Below 48 blocks (integers; 56 for floating point) only full turns of large classes were measured to gain.
+// Below 48 blocks (integers; 56 for floating point) only full turns of large classes were measured to gain, and turns that leave
+// most SMs idle nowhere: plan_greedy_rounds does not ask there.
 static bool rounds_win(const Sizes &sz, double equal, int sms, int ctasPerSm, const ClusterShape &cluster)
 {
     const double M = (double)sz.maxM;
     const bool real = sz.floatArith, two = ctasPerSm > 1;
-    const double full = equal / (sms * std::ceil(equal / sms - 1e-9));
-    if (full < (sz.W >= 80 ? 0.4 : 0.65) || sz.W < (real ? 56 : 16)) return false;
-    if (sz.W < 48 && (full < 0.9 || sz.maxM < 1000)) return false;
     if (cluster.ctas == 0) return true;
     const double turns = std::ceil(equal / (sms * ctasPerSm) - 1e-9), clusterTurns = std::ceil(equal / cluster.resident - 1e-9);
     double speed;
@@ -815,9 +813,12 @@ static bool rounds_plan(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDe
 std::shared_ptr<RoundsPlan> plan_greedy_rounds(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost, const ClusterShape &cluster)
 {
     if (sz.graphCut || sz.W > kRoundBlocks || sz.maxM == 0 || sz.maxM > 65535) return nullptr;
+    if (sz.W < (sz.floatArith ? 56 : 16)) return nullptr;
     double equal = 0;
     for (const ClassDesc &c : descHost) equal += (double)c.M * c.M;
     equal /= (double)sz.maxM * sz.maxM;
+    const double full = equal / (ctx->smCount * std::ceil(equal / ctx->smCount - 1e-9));
+    if (full < (sz.W >= 80 ? 0.4 : 0.65) || (sz.W < 48 && (full < 0.9 || sz.maxM < 1000))) return nullptr;
     auto plan = std::make_shared<RoundsPlan>();
     // Two CTAs of eight warps per SM where there are classes for several rounds of them: one's barriers and trips to memory under the
     // other's sums (1000 x 1000 bf16 into 64 blocks: 85.1 ms with one of 16 warps, 80.4 with two; 300 x 1000 into 24: 20.8 and 23.5).
