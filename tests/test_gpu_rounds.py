@@ -26,6 +26,7 @@ def ran_in_rounds(rcd, wl, lists=None, tiles=None, **cfg):
 @pytest.mark.parametrize("sizes,d,W", [
     ([37] * 97, 16, 64),                          # fewer samples than blocks; batches of fewer blocks than wait (narrow features)
     ([129, 128, 127, 126] * 25, 40, 64),          # edges of 128 columns
+    ([129, 128, 127, 126] * 25, 40, 48),          # (as many blocks as the cluster form is still faster with)
     ([257] * 60, 75, 100),                        # more than 64 blocks: two batches a round
     ([64] * 450, 24, 56),                         # two CTAs per SM
     ([90] * 60 + [0, 1, 0], 16, 128),             # the most blocks; empty classes and one of a sample
@@ -35,7 +36,8 @@ def ran_in_rounds(rcd, wl, lists=None, tiles=None, **cfg):
 def test_int8_exact(rcd, orc, sizes, d, W, copies):
     wl = cluster.workload(sizes, d, W, W + copies, copies=copies)
     check_exact(rcd, orc, wl)
-    ran_in_rounds(rcd, wl)
+    if W != 48:
+        ran_in_rounds(rcd, wl)
 
 
 def test_int8_sums_beyond_32_bits(rcd, orc):
@@ -62,11 +64,12 @@ def test_int8_like_the_passes(rcd, sizes, d, W):
 
 
 @pytest.mark.parametrize("similarity", ["gaussian", "dot"])
-@pytest.mark.parametrize("sizes,W", [([101] * 98, 57), ([66] * 60, 100)])
+@pytest.mark.parametrize("sizes,W", [([101] * 98, 57), ([66] * 60, 100), ([66] * 60, 70)])
 def test_float_is_exact_in_fixed_point(rcd, orc, similarity, sizes, W):
     cluster.test_float_is_exact_in_fixed_point(rcd, orc, similarity, sizes, W)
-    ran_in_rounds(rcd, cluster.workload(sizes, 64, W, 5 * W, dtype="bf16"),
-                  similarity_kind=rcd.RCD_SIM_GAUSSIAN if similarity == "gaussian" else rcd.RCD_SIM_DOT)
+    if W != 70:                                       # (where the cluster form is still faster)
+        ran_in_rounds(rcd, cluster.workload(sizes, 64, W, 5 * W, dtype="bf16"),
+                      similarity_kind=rcd.RCD_SIM_GAUSSIAN if similarity == "gaussian" else rcd.RCD_SIM_DOT)
 
 
 def test_float_norms_far_apart(rcd, orc):
