@@ -4,7 +4,7 @@
 //
 // With dot products S is never written: the rows of every class are brought into block order (objective_order_kernel, gather), the
 // similarity kernel's epilogue keeps the maxima of its tiles (keep_maxima in rcd_similarity_tc.cu) and joins them to the blocks'
-// coverage, and only the sums are left (ten classes of 5000 into 8 blocks: 438 us through S, 188 without).
+// coverage, and only the sums are left (ten classes of 5000 into 8 blocks: 440 us through S, 172 without).
 //
 // Otherwise (Gaussian kernel, whose bandwidth needs all distances first, and the generic similarity kernel) the maxima are taken
 // from S.  S is symmetric, so the maximum over a block's members may be taken down the members' rows: a thread owns four columns

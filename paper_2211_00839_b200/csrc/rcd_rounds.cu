@@ -10,13 +10,14 @@
 //   list     all warps fold the picked samples' rows into their blocks' coverage and list the columns each pick raised;
 //   correct  every row of S that any of the picks needs is fetched once, for all blocks that raised it;
 //   look     the leading candidates of every corrected block, for the next round's decisions.
-// The rows that some pick of a round raises are 9 times a class's matrix over a run instead of 136 (the same problem).
+// So a class's rows are read 13 times over a run instead of 130 (the same problem; 10 times where one CTA's batch holds all blocks).
 //
-// What bounds it (1000 classes of 1300 int8 into 64 blocks: 165 ms in the cluster form, 81 here; per class, one CTA of 16 warps per SM):
-// 4.6 of 13 ms are the sums of `tile_rows`, a saturating subtraction (half rate) and a multiply-add (its own pipe) per loss, 13 cycles
-// per row, 4 blocks and 128 columns where the pipes would allow 10; 2.1 ms rows that few blocks need, straight from memory; the rest
-// trips to L2 and barriers of 110 rounds (lists 1.0, looks 1.3, decisions 0.7, looks asked for in between 0.8).  148 MB per class
-// cross HBM instead of 895.
+// What bounds it (1000 classes of 1300 int8 into 64 blocks: 165 ms in the cluster form, 81 here).  A class alone on an SM (16 warps) takes
+// 11.0 ms, of which 4.3 are the sums of `tile_rows`: a saturating subtraction (half rate) and a multiply-add (its own pipe) per loss, 13
+// cycles per row, 4 blocks and 128 columns where the pipes would allow 10.  2.0 ms are rows that few blocks need, straight from memory; the
+// rest is trips to L2 and barriers of 110 rounds: lists 1.05, looks 1.0, copies of tiles and waits for them 0.9, decisions 0.7, looks
+// asked for in between 0.45, tables 0.4, gains of empty blocks 0.2.  Two CTAs of 8 warps on an SM take 20 ms for two classes.  148 MB
+// per class cross HBM instead of 895: 13 matrices of 6.8 MB, those of the empty blocks' gains and of the picks, gains and coverage.
 //
 // Results are those of the cluster form bit for bit: stored gains are exact integers, decisions are made in the same order.
 #include "rcd_exact.cuh"

@@ -267,8 +267,8 @@ constexpr int kWarpCols = kTileN / 32 / (kEpiWarps / 4);       // column blocks 
 // of block b), row i per lane, and for blocks above the diagonal the same with rows and columns exchanged (through shared memory).  A
 // maximum leaves the registers where the block changes: the rows' at the end of a run that may span the tile, the columns' once per
 // 32 rows at least.  colBlock: the blocks of the warp's columns, looked up before the tile was ready.
-// Bound by this epilogue's own instructions and then by the operands' way from L2 (10 classes of 5000 x 512 int8 into 8 blocks: 95 us
-// with no epilogue at all; writing S took 200 us and reading it back 200 more).  A pass per run of columns as long as they are few; with
+// Bound by the operands' way from L2 and then by this epilogue's own instructions (10 classes of 5000 x 512 int8 into 8 blocks: 108 us,
+// 93 with no epilogue at all, where 0.8 GB come at 8.9 TB/s; writing S took 200 us and reading it back 200 more).  A pass per run of columns as long as they are few; with
 // more runs in 32 than kFewRuns a test per column is cheaper, four columns at a time from shared memory.  The code has to stay short:
 // with that test unrolled for 32 columns in registers, and all of it for each of a warp's column blocks, a warp spent 37 % of its time
 // waiting for instructions.  The whole call in us, through S : that code : as it is, by samples of a class per block (int8, 64 elements):
