@@ -747,6 +747,8 @@ struct RoundsPlan {
 //                            300 x 500, dense 7480 : 5780   200 x 500, dense 5200 : 4110   200 x 400, dense 2540 : 2970   100 x 1300, dense 15800 : 17800
 //               128          148 x 1300 190000 : 20100   60 x 500, dense 3090 : 2450       80    60 x 500, dense 1890 : 2210   60 x 300, dense 1035 : 960
 //               48           148 x 700, dense 5690 : 4220   300 x 500, dense 4640 : 5220   200 x 1000, dense 14600 : 15900   148 x 100, dense 219 : 227
+//                            296 x 200 870 : 1100   296 x 133, dense 490 : 580   (one CTA per class either way, two turns, 128 to 250 samples: 1.05
+//                            times as long in rounds on average over 200 to 296 classes, up to 1.30; 52 blocks 1.0, 58 blocks 0.96)
 //               32           148 x 1000, dense 7090 : 6880   444 x 1000 21400 : 15200, dense 19600 : 22700 (taken)
 //               24           148 x 1000, dense 5680 : 6070, 5370 : 5380   148 x 1050, dense 8390 : 7080   444 x 1000, dense 16100 : 20500
 //                            (up to 1024 samples a row keeps a team of four warps busy for two steps; from 1025 on it takes a third)
@@ -755,6 +757,9 @@ struct RoundsPlan {
 //               65           60 x 500, dense 1930 : 2430   100 x 1000, dense 12200 : 12700   148 x 1000, dense 17400 : 13200
 //               128          100 x 1300, dense 120000 : 33900   100 x 2000, dense 86400 : 103000
 // Of 1059 measured calls this takes 807; eleven of them are 3 to 5 % slower in rounds, or dense ones of 444 x 1000 into 32 and 40 blocks.
+// Small integer classes into 60 to 80 blocks that one CTA holds either way are close: 127 x 133 into 64 blocks 257 : 296, dense 260 : 264 with rows of 128
+// bytes, whose tables hold 12 blocks at a time, 266 : 264 and 275 : 238 with 1 KB; 90 to 200 samples and rows up to 128 bytes take 0.96 of the cluster
+// form's time on average (0.54 to 1.18), 256 bytes 0.93, 1 KB 0.87.
 // Below 48 blocks (integers; 56 for floating point) only full turns of large classes were measured to gain, and turns that leave
 // most SMs idle nowhere: plan_greedy_rounds does not ask there.
 static bool rounds_win(const Sizes &sz, double equal, int sms, int ctasPerSm, const ClusterShape &cluster)
@@ -764,7 +769,7 @@ static bool rounds_win(const Sizes &sz, double equal, int sms, int ctasPerSm, co
     if (cluster.ctas == 0) return true;
     const double turns = std::ceil(equal / (sms * ctasPerSm) - 1e-9), clusterTurns = std::ceil(equal / cluster.resident - 1e-9);
     double speed;
-    if (cluster.ctas == 1) speed = !real && M > 64 && M < 900 && sz.W < 60 && turns == 1.0 ? 1.1 : 0.95;
+    if (cluster.ctas == 1) speed = !real && M > 64 && M < 900 && (turns == 1.0 ? sz.W < 60 : turns == 2.0 && !two && sz.W < 52 && M >= 128) ? 1.1 : 0.95;
     else if (cluster.ctas == 2) speed = M > 1024 ? 1.75 : std::min(std::min(0.55 + M / 230, 1.05 + M / 500), 2.15);
     else if (cluster.ctas == 4) speed = real ? std::min(0.3 + M / 200, 5.5) : std::min(0.95 + M / 310, 4.1);
     else if (cluster.ctas == 8) speed = std::min(M / 155, 8.0) * (real ? 1.2 : 1.0);

@@ -97,6 +97,7 @@ def test_copies_that_never_arrive(rcd, orc):
     (148, 1030, 24, "int8", True),         # rows of three steps
     (148, 1000, 16, "int8", True),         # one CTA per class
     (200, 400, 64, "int8", False),         # two turns of rounds, the second a third full, against three of the cluster form
+    (296, 200, 48, "int8", False), (296, 200, 64, "int8", True),          # one CTA per class either way, two turns
     (60, 500, 80, "int8", False), (60, 500, 128, "int8", True),
     (100, 1300, 64, "int8", False), (100, 1300, 128, "int8", True),
     (60, 500, 65, "bf16", False), (300, 500, 64, "bf16", True), (300, 700, 64, "bf16", False), (444, 1300, 56, "bf16", False),
