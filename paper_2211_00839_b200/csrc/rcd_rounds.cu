@@ -748,7 +748,7 @@ struct RoundsPlan {
 //               128          148 x 1300 190000 : 20100   60 x 500, dense 3090 : 2450       80    60 x 500, dense 1890 : 2210   60 x 300, dense 1035 : 960
 //               48           148 x 700, dense 5690 : 4220   300 x 500, dense 4640 : 5220   200 x 1000, dense 14600 : 15900   148 x 100, dense 219 : 227
 //                            296 x 200 870 : 1100   296 x 133, dense 490 : 580   (one CTA per class either way, two turns, 128 to 250 samples: 1.05
-//                            times as long in rounds on average over 200 to 296 classes, up to 1.30; 52 blocks 1.0, 58 blocks 0.96)
+//                            times as long in rounds on average over 200 to 296 classes, up to 1.30; 52 blocks 1.0, up to 1.24; 58 blocks 0.96, up to 1.21)
 //               32           148 x 1000, dense 7090 : 6880   444 x 1000 21400 : 15200, dense 19600 : 22700 (taken)
 //               24           148 x 1000, dense 5680 : 6070, 5370 : 5380   148 x 1050, dense 8390 : 7080   444 x 1000, dense 16100 : 20500
 //                            (up to 1024 samples a row keeps a team of four warps busy for two steps; from 1025 on it takes a third)
