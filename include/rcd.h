@@ -126,7 +126,8 @@ typedef enum {
     RCD_FORM_LAUNCHES = 1, RCD_FORM_BARRIERS = 2, RCD_FORM_ASYNC = 3, RCD_FORM_CLASS_PER_CTA = 4,
     RCD_FORM_CLUSTER = 5,      /* a thread-block cluster per class */
     RCD_FORM_ROUNDS = 6,       /* a CTA per class, in rounds */
-    RCD_FORM_CUT_CHAIN = 7     /* graph cut, a CTA per class */
+    RCD_FORM_CUT_CHAIN = 7,    /* graph cut, a CTA per class */
+    RCD_FORM_SMALL = 8         /* small classes, a CTA per class with its similarities in shared memory */
 } rcd_greedy_form;
 
 /* Timings and counters of the last rcd_partition / rcd_partition_host on a context (profile >= 1).  New ones are added at the end:

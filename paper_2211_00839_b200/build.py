@@ -16,7 +16,7 @@ CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(ROOT, "_build")
 LIB = os.path.join(HERE, "librcd.so")
 
-SOURCES = ["rcd_api.cu", "rcd_group.cu", "rcd_similarity.cu", "rcd_similarity_tc.cu", "rcd_greedy.cu", "rcd_cluster.cu", "rcd_rounds.cu",
+SOURCES = ["rcd_api.cu", "rcd_group.cu", "rcd_similarity.cu", "rcd_similarity_tc.cu", "rcd_greedy.cu", "rcd_cluster.cu", "rcd_rounds.cu", "rcd_small.cu",
            "rcd_objective.cu", "rcd_objective_static.cu", "rcd_gaussian.cu", "rcd_cut.cu", "rcd_yardstick.cu"]
 HEADERS = [os.path.join(CSRC, "rcd_internal.h"), os.path.join(CSRC, "rcd_exact.cuh"), os.path.join(ROOT, "include", "rcd.h")]
 

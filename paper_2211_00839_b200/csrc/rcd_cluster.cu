@@ -1252,12 +1252,9 @@ __global__ void __launch_bounds__(256, 8) fixed_point_kernel(const ClassDesc *__
     const float scale = ldexpf(1.f, fixedExp[blockIdx.y]);
     float4 *p = reinterpret_cast<float4 *>(S + c.sOff);
     const int64_t n = (int64_t)c.M * (c.ld >> 2);
-    constexpr int kMost = (1 << 30) - 1;
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
         const float4 x = p[i];
-        const int4 y = make_int4(min(max(__float2int_rn(x.x * scale), -kMost), kMost), min(max(__float2int_rn(x.y * scale), -kMost), kMost),
-                                 min(max(__float2int_rn(x.z * scale), -kMost), kMost), min(max(__float2int_rn(x.w * scale), -kMost), kMost));
-        reinterpret_cast<int4 *>(p)[i] = y;
+        reinterpret_cast<int4 *>(p)[i] = make_int4(to_fixed(x.x, scale), to_fixed(x.y, scale), to_fixed(x.z, scale), to_fixed(x.w, scale));
     }
 }
 
@@ -1325,6 +1322,7 @@ struct ClusterPlan {
     bool smemState;
     size_t smem;
     std::shared_ptr<RoundsPlan> rounds;   // not null: the classes run in rounds instead, one CTA each
+    std::shared_ptr<SmallPlan> small;     // not null: one CTA each with the class's similarities in its shared memory
     ClusterParams prm;         // teamWarps, slots, maxLd, rowPieces and the offsets are set
 };
 static size_t cluster_layout(const Sizes &sz, int maxLd, int C, bool state, size_t cap, ClusterPlan &plan)
@@ -1469,7 +1467,7 @@ static bool cluster_shape(rcd_ctx *ctx, const Sizes &sz, const std::vector<Class
     return true;
 }
 
-// Whether the cluster form or the rounds take a problem, and how: chosen by the library (no pass-based form or option asked for),
+// Whether the cluster form, the rounds or the form for small classes take a problem, and how: chosen by the library (no pass-based form or option asked for),
 // samples of a class and blocks within the packed keys' range.
 static bool cluster_plan(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost, ClusterPlan &plan)
 {
@@ -1486,10 +1484,16 @@ static bool cluster_plan(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassD
         maxLd = std::max(maxLd, (int)d.ld);
     }
     plan.prm = ClusterParams{};
+    plan.prm.maxLd = maxLd;
+    // (small classes whenever they fit: faster than the cluster form in every case measured.  Rounds first: where those are faster than the
+    // cluster form was measured before, and they stay)
+    plan.small = plan_greedy_small(ctx, sz);
+    if (plan.small && !rounds_possible(ctx, sz, descHost)) return true;
     const bool clusters = cluster_shape(ctx, sz, descHost, nonEmpty, maxLd, plan, &resident);
     plan.prm.maxLd = maxLd;
     plan.rounds = plan_greedy_rounds(ctx, sz, descHost, clusters ? ClusterShape{plan.C, resident, plan.P} : ClusterShape{0, 0, 0});
-    return clusters || plan.rounds;
+    if (plan.rounds) plan.small = nullptr;
+    return clusters || plan.rounds || plan.small;
 }
 
 std::shared_ptr<ClusterPlan> plan_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost)
@@ -1535,14 +1539,20 @@ rcd_status launch_greedy_cluster(rcd_ctx *ctx, ClusterPlan &plan, const Sizes &s
         *left = 0;
         fixed_exponent_kernel<<<sz.L, 256, 0, st>>>(ws.desc, (const float *)ws.S, ws.fixedExp, ws.sizesLeft, left);
         RCD_CUDA(ctx, cudaEventRecord(ctx->evCounts, st));
-        const int64_t pieces = sz.maxM * (int64_t)(prm.maxLd / 4);
-        const dim3 grid((unsigned)std::min<int64_t>((pieces + 1023) / 1024, std::max(1, 16 * ctx->smCount / sz.L)), (unsigned)sz.L);
-        fixed_point_kernel<<<grid, 256, 0, st>>>(ws.desc, ws.fixedExp, (float *)ws.S);
-        ctx->kernelLaunches += 2;
+        ctx->kernelLaunches++;
+        if (!plan.small) {                                 // (that form rounds what it loads)
+            const int64_t pieces = sz.maxM * (int64_t)(prm.maxLd / 4);
+            const dim3 grid((unsigned)std::min<int64_t>((pieces + 1023) / 1024, std::max(1, 16 * ctx->smCount / sz.L)), (unsigned)sz.L);
+            fixed_point_kernel<<<grid, 256, 0, st>>>(ws.desc, ws.fixedExp, (float *)ws.S);
+            ctx->kernelLaunches++;
+        }
         RCD_CUDA(ctx, cudaGetLastError());
     }
     if (plan.rounds) {
         const rcd_status rs = launch_greedy_rounds(ctx, *plan.rounds, sz, ws, assignment, order, partValues, st);
+        if (rs != RCD_OK) return rs;
+    } else if (plan.small) {
+        const rcd_status rs = launch_greedy_small(ctx, *plan.small, sz, ws, toFix, assignment, order, partValues, st);
         if (rs != RCD_OK) return rs;
     } else {
         ClusterKernel kernel = sz.graphCut ? (sz.W <= 32 ? pick_kernel<1, true>(plan.P, prm.teamWarps, plan.smemState) : pick_kernel<4, true>(plan.P, prm.teamWarps, plan.smemState))
@@ -1552,7 +1562,7 @@ rcd_status launch_greedy_cluster(rcd_ctx *ctx, ClusterPlan &plan, const Sizes &s
         if (rs != RCD_OK) return rs;
     }
     ctx->steps = sz.maxM;
-    ctx->greedyForm = plan.rounds ? RCD_FORM_ROUNDS : RCD_FORM_CLUSTER;
+    ctx->greedyForm = plan.rounds ? RCD_FORM_ROUNDS : plan.small ? RCD_FORM_SMALL : RCD_FORM_CLUSTER;
     ctx->phaseNsDev = ws.phaseNs;
     if (toFix) RCD_CUDA(ctx, cudaEventSynchronize(ctx->evCounts));
     if (toFix && *left) return launch_greedy_not_fixed(ctx, sz, ws, descHost, assignment, order, partValues, st);

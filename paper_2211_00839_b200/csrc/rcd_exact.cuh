@@ -1,4 +1,4 @@
-// What the two forms of the greedy loop with exact stored gains (rcd_cluster.cu, rcd_rounds.cu) have in common: keys, losses, and
+// What the forms of the greedy loop with exact stored gains (rcd_cluster.cu, rcd_rounds.cu, rcd_small.cu) have in common: keys, losses, and
 // the loads of rows of S.
 #pragma once
 
@@ -81,6 +81,9 @@ __device__ __forceinline__ unsigned long long row_value(const int4 *row, int ld4
 // What a candidate loses for one raised column: min(max(x, old), new) - old, as one instruction.  Similarities stay
 // below 2^30 either way, so x - old does not wrap, and two losses fit an int.
 __device__ __forceinline__ int loss(int x, const Raised &e) { return __viaddmin_s32_relu(x, e.minusOld, e.by); }
+
+// A floating-point similarity as a fixed-point integer below 2^30.
+__device__ __forceinline__ int to_fixed(float x, float scale) { return min(max(__float2int_rn(x * scale), -((1 << 30) - 1)), (1 << 30) - 1); }
 
 // 16 bytes global -> shared without passing through registers
 __device__ __forceinline__ void copy16(int4 *dst, const int4 *src)

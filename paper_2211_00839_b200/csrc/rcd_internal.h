@@ -314,6 +314,15 @@ std::shared_ptr<RoundsPlan> plan_greedy_rounds(rcd_ctx *ctx, const Sizes &sz, co
 rcd_status launch_greedy_rounds(rcd_ctx *ctx, RoundsPlan &plan, const Sizes &sz, const Workspace &ws, int32_t *assignment, int32_t *order,
                                 void *partValues, cudaStream_t st);
 
+bool rounds_possible(const rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost);
+
+// greedy loop of small classes, one CTA per class with S in its shared memory (null: it does not take the problem; toFix: S holds
+// floating-point dot products)
+struct SmallPlan;
+std::shared_ptr<SmallPlan> plan_greedy_small(rcd_ctx *ctx, const Sizes &sz);
+rcd_status launch_greedy_small(rcd_ctx *ctx, SmallPlan &plan, const Sizes &sz, const Workspace &ws, bool toFix, int32_t *assignment, int32_t *order,
+                               void *partValues, cudaStream_t st);
+
 rcd_status launch_bounded_wait_selftest(rcd_ctx *ctx, unsigned *counter, int32_t *status, cudaStream_t st);
 rcd_status launch_step_wait_selftest(rcd_ctx *ctx, int32_t *status, cudaStream_t st);
 

@@ -816,15 +816,27 @@ static bool rounds_plan(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDe
     return true;
 }
 
-std::shared_ptr<RoundsPlan> plan_greedy_rounds(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost, const ClusterShape &cluster)
+// Classes of the largest size that make as many entries of S.
+static double equal_classes(const Sizes &sz, const std::vector<ClassDesc> &descHost)
 {
-    if (sz.graphCut || sz.W > kRoundBlocks || sz.maxM == 0 || sz.maxM > 65535) return nullptr;
-    if (sz.W < (sz.floatArith ? 56 : 16)) return nullptr;
     double equal = 0;
     for (const ClassDesc &c : descHost) equal += (double)c.M * c.M;
-    equal /= (double)sz.maxM * sz.maxM;
-    const double full = equal / (ctx->smCount * std::ceil(equal / ctx->smCount - 1e-9));
-    if (full < (sz.W >= 80 ? 0.4 : 0.65) || (sz.W < 48 && (full < 0.9 || sz.maxM < 1000))) return nullptr;
+    return equal / ((double)sz.maxM * sz.maxM);
+}
+
+// Whether rounds come into question: blocks enough, and classes that fill the SMs.
+bool rounds_possible(const rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost)
+{
+    if (sz.graphCut || sz.W > kRoundBlocks || sz.maxM == 0 || sz.maxM > 65535) return false;
+    if (sz.W < (sz.floatArith ? 56 : 16)) return false;
+    const double equal = equal_classes(sz, descHost), full = equal / (ctx->smCount * std::ceil(equal / ctx->smCount - 1e-9));
+    return full >= (sz.W >= 80 ? 0.4 : 0.65) && (sz.W >= 48 || (full >= 0.9 && sz.maxM >= 1000));
+}
+
+std::shared_ptr<RoundsPlan> plan_greedy_rounds(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost, const ClusterShape &cluster)
+{
+    if (!rounds_possible(ctx, sz, descHost)) return nullptr;
+    const double equal = equal_classes(sz, descHost);
     auto plan = std::make_shared<RoundsPlan>();
     // Two CTAs of eight warps per SM where there are classes for several rounds of them: one's barriers and trips to memory under the
     // other's sums (1000 x 1000 bf16 into 64 blocks: 85.1 ms with one of 16 warps, 80.4 with two; 300 x 1000 into 24: 20.8 and 23.5).
