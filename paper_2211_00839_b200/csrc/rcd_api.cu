@@ -143,7 +143,11 @@ size_t layout_workspace(void *base, rcd_feat_dtype dtype, const Sizes &sz, Works
     return w.bytes;
 }
 
-static int32_t chunks_for(int64_t N, int64_t labels) { return (int32_t)((N + group_chunk(N, labels) - 1) / group_chunk(N, labels)); }
+static int32_t chunks_for(int64_t N, int64_t labels, bool rows)
+{
+    const int chunk = group_shape(N, labels, rows).chunk;
+    return (int32_t)((N + chunk - 1) / chunk);
+}
 
 // Sizes for the promise "no class larger than Mmax".
 static bool float_arith(const rcd_ctx *ctx, rcd_feat_dtype dtype)
@@ -168,7 +172,7 @@ static Sizes bound_sizes(const rcd_ctx *ctx, rcd_feat_dtype dtype, int64_t N, in
     sz.maxM = Mmax;
     sz.sElems = N * (int64_t)pad_row(Mmax);               // sum M_l * ld_l <= N * pad_row(Mmax)
     sz.vElems = (int64_t)W * (N + 7LL * L);               // sum W * ld_l,  ld_l <= M_l + 7
-    sz.nChunks = chunks_for(N, L);
+    sz.nChunks = chunks_for(N, L, true);
     sz.pitch = features_pitch(ctx, dtype, d);
     return sz;
 }
@@ -248,7 +252,7 @@ static rcd_status prepare(rcd_ctx *ctx, const void *features, rcd_feat_dtype dty
     if (((uintptr_t)workspace) % kAlign != 0) return fail(ctx, RCD_ERR_INVALID_ARG, "workspace must be 256-byte aligned");
     // head of the workspace: status, counts, what the host will send, the split's tables
     Sizes head{};
-    head.N = N; head.d = d; head.L = L; head.W = W; head.nChunks = chunks_for(N, L);
+    head.N = N; head.d = d; head.L = L; head.W = W; head.nChunks = chunks_for(N, L, true);
     head.floatArith = float_arith(ctx, dtype);
     head.graphCut = ctx->cfg.objective == RCD_OBJ_GRAPH_CUT;
     head.pitch = features_pitch(ctx, dtype, d);
@@ -258,19 +262,33 @@ static rcd_status prepare(rcd_ctx *ctx, const void *features, rcd_feat_dtype dty
     if (workspaceBytes < headBytes) return fail(ctx, RCD_ERR_WORKSPACE_TOO_SMALL, "workspace smaller than its %zu-byte head", headBytes);
     if ((size_t)L > ctx->hostStageInts) return fail(ctx, RCD_ERR_UNSUPPORTED, "L=%d exceeds the %zu classes the context can stage", L, ctx->hostStageInts);
 
-    RCD_CUDA(ctx, cudaMemsetAsync(hw.topGain, 0, (size_t)((unsigned char *)(hw.counts + L) - (unsigned char *)hw.topGain), st));
-    rcd_status rs = launch_label_hist(ctx, labels, N, L, hw.chunkHist, hw.counts, hw.status, ctx->statusOwn, st);
-    if (rs != RCD_OK) return rs;
-    ctx->statusDev = ctx->statusOwn;
     // the class sizes come back together with the words before them (the label check's verdict is the first)
     const size_t statusInts = (size_t)(hw.counts - hw.status);
-    RCD_CUDA(ctx, cudaMemcpyAsync(ctx->hostStage, hw.status, (statusInts + L) * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    const GroupShape shape = group_shape(N, L, true);
+    const bool few = shape.few;
+    rcd_status rs;
+    if (few) {
+        rs = launch_label_hist_few(ctx, labels, N, L, shape, hw.chunkHist, hw.counts, hw.status, ctx->statusOwn, (int32_t *)hw.topGain, hw.counts - (int32_t *)hw.topGain,
+                                   ctx->hostStage, ctx->hostStage + statusInts, st);
+    } else {
+        RCD_CUDA(ctx, cudaMemsetAsync(hw.topGain, 0, (size_t)((unsigned char *)(hw.counts + L) - (unsigned char *)hw.topGain), st));
+        rs = launch_label_hist(ctx, labels, N, L, shape, hw.chunkHist, hw.counts, hw.status, ctx->statusOwn, st);
+        if (rs == RCD_OK) RCD_CUDA(ctx, cudaMemcpyAsync(ctx->hostStage, hw.status, (statusInts + L) * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    }
+    if (rs != RCD_OK) return rs;
+    ctx->statusDev = ctx->statusOwn;
     if (!ctx->evCounts) RCD_CUDA(ctx, cudaEventCreateWithFlags(&ctx->evCounts, cudaEventDisableTiming));
-    RCD_CUDA(ctx, cudaEventRecord(ctx->evCounts, st));
+    if (!few) RCD_CUDA(ctx, cudaEventRecord(ctx->evCounts, st));
     const size_t blobBytes = (size_t)((unsigned char *)(hw.quota + (size_t)L * W) - (unsigned char *)hw.desc);
     unsigned char *blob = nullptr;
     rs = blob_begin(ctx, blobBytes, statusInts + (size_t)L, &blob);
-    RCD_CUDA(ctx, cudaEventSynchronize(ctx->evCounts));     // (also where that failed: the sizes are on their way to the staging buffer)
+    // (also where that failed: the sizes are on their way to the staging buffer)
+    if (few) {
+        const rcd_status arrived = wait_few_counts(ctx, st);
+        if (arrived != RCD_OK) return arrived;
+    } else {
+        RCD_CUDA(ctx, cudaEventSynchronize(ctx->evCounts));
+    }
     if (rs != RCD_OK) return rs;
     if (ctx->hostStage[0] & kDevBadLabel) return fail(ctx, RCD_ERR_INVALID_ARG, "a label lies outside [0, %d)", L);
     const int32_t *counts = ctx->hostStage + statusInts;      // (behind the zeroed words that came along)
@@ -340,7 +358,7 @@ static rcd_status prepare(rcd_ctx *ctx, const void *features, rcd_feat_dtype dty
     const BlobInUse inUse{ctx, st};
     const size_t firstBytes = early ? blobBytes : (size_t)((unsigned char *)hw.quota - (unsigned char *)hw.desc);
     RCD_CUDA(ctx, cudaMemcpyAsync(P.ws.desc, blob, firstBytes, cudaMemcpyHostToDevice, st));
-    rs = launch_stable_split(ctx, labels, N, L, P.ws.chunkHist, P.ws.desc, nullptr, nullptr, nullptr, P.ws.perm,
+    rs = launch_stable_split(ctx, labels, N, L, shape, P.ws.chunkHist, P.ws.desc, nullptr, nullptr, nullptr, P.ws.perm,
                              P.covered ? nullptr : features, d * (int64_t)feat_bytes(dtype), sz.pitch, P.covered ? nullptr : P.ws.Xs, st);
     if (rs != RCD_OK) return rs;
     if (P.covered) {
@@ -422,6 +440,7 @@ rcd_status rcd_create(rcd_ctx **out, int cuda_device, const rcd_config *cfg)
         delete ctx;
         return RCD_ERR_CUDA;
     }
+    ctx->hostStage[ctx->hostStageInts + kStageArrived] = 0;
     if (cudaMalloc((void **)&ctx->statusOwn, kStatusWords * sizeof(int32_t)) != cudaSuccess ||
         cudaMemset(ctx->statusOwn, 0, kStatusWords * sizeof(int32_t)) != cudaSuccess) {
         rcd_destroy(ctx);
@@ -555,7 +574,7 @@ static size_t layout_lists(void *base, int64_t N, int32_t W, ListsWorkspace *out
     const size_t Wn = (size_t)std::max<int32_t>(W, 1);
     w.status = c.take<int32_t>(4);
     w.counts = c.take<int32_t>(Wn);
-    w.chunkHist = c.take<int32_t>((size_t)std::max<int32_t>(chunks_for(N, W), 1) * Wn);
+    w.chunkHist = c.take<int32_t>((size_t)std::max<int32_t>(chunks_for(N, W, false), 1) * Wn);
     w.bytes = align_up(c.off);
     if (out) *out = w;
     return w.bytes;
@@ -584,16 +603,30 @@ rcd_status rcd_worker_lists(rcd_ctx *ctx, const int32_t *assignment_dev, int64_t
     RCD_CUDA(ctx, cudaSetDevice(ctx->device));
     ctx->kernelLaunches = 0;
     ctx->statusDev = ctx->statusOwn;
-    RCD_CUDA(ctx, cudaMemsetAsync(ws.status, 0, (size_t)((unsigned char *)(ws.counts + W) - (unsigned char *)ws.status), st));
-    rcd_status rs = launch_label_hist(ctx, assignment_dev, N, W, ws.chunkHist, ws.counts, ws.status, ctx->statusOwn, st);
+    const GroupShape shape = group_shape(N, W, false);
+    const bool few = shape.few;
+    rcd_status rs;
+    if (few) {
+        rs = launch_label_hist_few(ctx, assignment_dev, N, W, shape, ws.chunkHist, ws.counts, ws.status, ctx->statusOwn, nullptr, 0, ctx->hostStage, nullptr, st);
+    } else {
+        RCD_CUDA(ctx, cudaMemsetAsync(ws.status, 0, (size_t)((unsigned char *)(ws.counts + W) - (unsigned char *)ws.status), st));
+        rs = launch_label_hist(ctx, assignment_dev, N, W, shape, ws.chunkHist, ws.counts, ws.status, ctx->statusOwn, st);
+        if (rs == RCD_OK) RCD_CUDA(ctx, cudaMemcpyAsync(ctx->hostStage, ws.status, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    }
     if (rs != RCD_OK) return rs;
-    RCD_CUDA(ctx, cudaMemcpyAsync(ctx->hostStage, ws.status, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-    if (!ctx->evCounts) RCD_CUDA(ctx, cudaEventCreateWithFlags(&ctx->evCounts, cudaEventDisableTiming));
-    RCD_CUDA(ctx, cudaEventRecord(ctx->evCounts, st));
+    if (!few) {
+        if (!ctx->evCounts) RCD_CUDA(ctx, cudaEventCreateWithFlags(&ctx->evCounts, cudaEventDisableTiming));
+        RCD_CUDA(ctx, cudaEventRecord(ctx->evCounts, st));
+    }
     // the list boundaries are sums of the sizes, and a stable split by block number fills the lists (inside a list the
     // dataset indices ascend): enqueued behind the check of the entries, whose verdict they read themselves
-    rs = launch_stable_split(ctx, assignment_dev, N, W, ws.chunkHist, nullptr, ws.counts, offsets_dev, ws.status, indices_dev, nullptr, 0, 0, nullptr, st);
-    RCD_CUDA(ctx, cudaEventSynchronize(ctx->evCounts));
+    rs = launch_stable_split(ctx, assignment_dev, N, W, shape, ws.chunkHist, nullptr, ws.counts, offsets_dev, ws.status, indices_dev, nullptr, 0, 0, nullptr, st);
+    if (few) {
+        const rcd_status arrived = wait_few_counts(ctx, st);
+        if (arrived != RCD_OK) return arrived;
+    } else {
+        RCD_CUDA(ctx, cudaEventSynchronize(ctx->evCounts));
+    }
     if (rs != RCD_OK) return rs;
     if (ctx->hostStage[0] & kDevBadLabel) return fail(ctx, RCD_ERR_INVALID_ARG, "an assignment entry lies outside [0, %d)", W);
     return RCD_OK;

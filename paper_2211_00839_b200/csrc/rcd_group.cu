@@ -5,17 +5,19 @@
 #include "rcd_internal.h"
 
 #include <algorithm>
+#include <atomic>
 
 namespace rcd {
 
 // ---- stable split ---------------------------------------------------------------------------
-// Chunks of consecutive samples (group_chunk samples each).  Three launches:
+// Chunks of consecutive samples (GroupShape says how large).  Three launches:
 //   histogram  a CTA per chunk counts its labels in shared memory, writes chunkHist[chunk][label] and adds to counts[label];
 //   scan       per label, exclusive running sum over the chunks, started at the class offset;
 //   place      position = chunk base + rank inside the chunk; the CTA then copies its feature rows to their places.
+// or two where few numbers come out: the histogram's last CTA hands the sizes to the host, and the placing CTAs add up for themselves.
 // Up to kMaxSharedLabels labels the counters of a chunk sit in shared memory (a sample costs one shared-memory atomic
-// and one warp match, against 1024 comparisons per sample and one global atomic before: 1.3 M samples over 64 labels
-// 1155 -> 40 us).  More labels than that take the kernels at the end of this section.
+// and a few warp votes, against 1024 comparisons per sample and one global atomic before: 1.3 M samples over 64 labels
+// 1155 -> 40 us, 27 in two launches).  More labels than that take the kernels at the end of this section.
 constexpr int kGroupThreads = 256;
 constexpr int kGroupWarps = kGroupThreads / 32;
 static_assert(kGroupWarps * kMaxSharedLabels * 4 <= 192 * 1024, "counters in shared memory");
@@ -42,6 +44,79 @@ __global__ void __launch_bounds__(kGroupThreads) label_hist_kernel(const int32_t
         const int32_t c = shCount[l];
         chunkHist[(int64_t)blockIdx.x * L + l] = c;
         if (c) atomicAdd(&counts[l], c);
+    }
+}
+
+// Adds the numbers of the first n chunks to sum[L] (shared memory): threads side by side take labels, and runs of chunks where labels are few.
+__device__ __forceinline__ void add_chunks(const int32_t *chunkHist, int n, int32_t L, int32_t *sum)
+{
+    int parts = 1;
+    while (2 * parts * L <= (int)blockDim.x) parts *= 2;
+    const int per = (n + parts - 1) / parts;
+    for (int i = threadIdx.x; i < parts * L; i += blockDim.x) {
+        const int part = i / L, l = i - part * L;
+        int32_t s = 0;
+#pragma unroll 8
+        for (int c = part * per; c < min(n, part * per + per); ++c) s += __ldcg(&chunkHist[(int64_t)c * L + l]);
+        if (s) atomicAdd(&sum[l], s);
+    }
+}
+
+// The same where few numbers come out (GroupShape::few): the CTA that is done last adds them up and writes the sizes and the verdict on the labels
+// straight to the host's memory, so that neither a memset goes before this kernel nor a copy after it (4 of 52 us of the smallest calls).
+// ticket: zero between launches (CTAs that are done, and from bit 16 on those that met a bad label).  zeros: words the later kernels
+// want cleared.
+__global__ void __launch_bounds__(1024) label_hist_few_kernel(const int32_t *__restrict__ labels, int64_t N, int32_t L, int32_t chunk,
+                                                                      int32_t *__restrict__ chunkHist, int32_t *__restrict__ counts, int32_t *__restrict__ status,
+                                                                      int32_t *__restrict__ callStatus, int32_t *__restrict__ zeros, int32_t nZeros,
+                                                                      uint32_t *__restrict__ ticket, volatile int32_t *hostStatus, volatile int32_t *hostCounts,
+                                                                      volatile int32_t *hostArrived, int32_t turn)
+{
+    extern __shared__ int32_t shCount[];
+    __shared__ uint32_t shDone;
+    if (blockIdx.x == 0) {
+        if (callStatus && threadIdx.x == 0) *callStatus = 0;
+        for (int i = threadIdx.x; i < nZeros; i += blockDim.x) zeros[i] = 0;
+    }
+    for (int l = threadIdx.x; l < L; l += blockDim.x) shCount[l] = 0;
+    __syncthreads();
+    const int64_t base = (int64_t)blockIdx.x * chunk;
+    const int n = (int)min((int64_t)chunk, N - base);
+    bool bad = false;
+#pragma unroll 8
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const int32_t lab = labels[base + i];
+        if (lab < 0 || lab >= L) bad = true;
+        else atomicAdd(&shCount[lab], 1);
+    }
+    bad = __syncthreads_or(bad);
+    for (int l = threadIdx.x; l < L; l += blockDim.x) __stcg(&chunkHist[(int64_t)blockIdx.x * L + l], shCount[l]);
+    if (gridDim.x > 1) {
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) shDone = atomicAdd(ticket, bad ? 0x10001u : 1u) + (bad ? 0x10001u : 1u);
+        __syncthreads();
+        if ((shDone & 0xffffu) != gridDim.x) return;
+        __threadfence();
+        bad = shDone >> 16 != 0;
+        for (int l = threadIdx.x; l < L; l += blockDim.x) shCount[l] = 0;
+        __syncthreads();
+        add_chunks(chunkHist, (int)gridDim.x, L, shCount);
+        __syncthreads();
+    }
+    for (int l = threadIdx.x; l < L; l += blockDim.x) {
+        counts[l] = shCount[l];
+        if (hostCounts) hostCounts[l] = shCount[l];
+    }
+    if (threadIdx.x == 0) {
+        *status = bad ? kDevBadLabel : 0;
+        *hostStatus = bad ? kDevBadLabel : 0;
+        if (gridDim.x > 1) *ticket = 0;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence_system();                            // (for what the others wrote, too)
+        *hostArrived = turn;
     }
 }
 
@@ -140,37 +215,83 @@ __device__ __forceinline__ void copy_row(const uint8_t *__restrict__ src, uint8_
     }
 }
 
-__global__ void __launch_bounds__(kGroupThreads) label_place_kernel(const int32_t *__restrict__ labels, int64_t N, int32_t L, int32_t chunk,
+// The lanes with the same label, by its bits from the lowest up (`bits` ballots of 24 cycles that overlap; __match_any_sync takes 375).
+__device__ __forceinline__ unsigned same_label(int lab, int bits)
+{
+    unsigned same = 0xffffffffu;
+    for (int k = 0; k < bits; ++k) {
+        const bool set = lab >> k & 1;
+        const unsigned votes = __ballot_sync(0xffffffffu, set);
+        same &= set ? votes : ~votes;
+    }
+    return same;
+}
+
+__global__ void __launch_bounds__(1024) label_place_kernel(const int32_t *__restrict__ labels, int64_t N, int32_t L, int32_t chunk,
                                                                    const int32_t *__restrict__ chunkBase, int32_t *__restrict__ perm,
                                                                    const uint8_t *__restrict__ X, int64_t rowBytes, int64_t pitch,
-                                                                   uint8_t *__restrict__ Xs, const int32_t *__restrict__ status)
+                                                                   uint8_t *__restrict__ Xs, const int32_t *__restrict__ status,
+                                                                   const ClassDesc *__restrict__ desc, const int32_t *__restrict__ counts, int64_t *__restrict__ offsets)
 {
-    extern __shared__ int32_t shWarp[];                 // [kGroupWarps][L] counters, then [chunk] positions
+    extern __shared__ int32_t shWarp[];                 // [warps][L] counters, then [chunk] positions
     if (status && (*status & kDevBadLabel)) return;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // (no launch of label_scan_kernel before: chunkBase holds the chunks' own numbers, and every CTA adds up those before its own)
+    const bool few = desc || counts;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     int32_t *mine = shWarp + (size_t)warp * L;
-    int32_t *shPos = shWarp + (size_t)kGroupWarps * L;
+    int32_t *shPos = shWarp + (size_t)warps * L;
     const int64_t base = (int64_t)blockIdx.x * chunk;
     const int n = (int)min((int64_t)chunk, N - base);
-    const int per = chunk / kGroupWarps;                // a warp's run of consecutive samples (a multiple of 32)
+    const int per = chunk / warps;                // a warp's run of consecutive samples (a multiple of 32)
     for (int l = lane; l < L; l += 32) mine[l] = 0;
     __syncwarp();
     const int i0 = warp * per, i1 = min(n, i0 + per);
+#pragma unroll 8
     for (int i = i0 + lane; i < i1; i += 32) atomicAdd(&mine[labels[base + i]], 1);
     __syncthreads();
-    for (int l = threadIdx.x; l < L; l += kGroupThreads) {
-        int32_t run = chunkBase[(int64_t)blockIdx.x * L + l];
-        for (int w = 0; w < kGroupWarps; ++w) {
+    int32_t *const shStart = shWarp + (size_t)warps * L + (Xs ? chunk : 0);      // [L] where a label begins (few), then where the chunk's part of it does
+    if (few && !desc) {
+        if (warp == 0) {
+            int32_t run = 0;
+            for (int l0 = 0; l0 < L; l0 += 32) {
+                const int32_t own = l0 + lane < L ? counts[l0 + lane] : 0;
+                int32_t sum = own;
+                for (int off = 1; off < 32; off <<= 1) {
+                    const int32_t up = __shfl_up_sync(0xffffffffu, sum, off);
+                    if (lane >= off) sum += up;
+                }
+                if (l0 + lane < L) {
+                    shStart[l0 + lane] = run + sum - own;
+                    if (offsets && blockIdx.x == 0 && blockIdx.y == 0) offsets[l0 + lane] = run + sum - own;
+                }
+                run += __shfl_sync(0xffffffffu, sum, 31);
+            }
+            if (offsets && blockIdx.x == 0 && blockIdx.y == 0 && lane == 0) offsets[L] = run;
+        }
+        __syncthreads();
+    }
+    if (few) {
+        if (desc) {
+            for (int l = threadIdx.x; l < L; l += blockDim.x) shStart[l] = desc[l].row0;
+            __syncthreads();
+        }
+        add_chunks(chunkBase, (int)blockIdx.x, L, shStart);
+        __syncthreads();
+    }
+    for (int l = threadIdx.x; l < L; l += blockDim.x) {
+        int32_t run = few ? shStart[l] : chunkBase[(int64_t)blockIdx.x * L + l];
+        for (int w = 0; w < warps; ++w) {
             const int32_t c = shWarp[(size_t)w * L + l];
             shWarp[(size_t)w * L + l] = run;
             run += c;
         }
     }
     __syncthreads();
+    const int labelBits = 32 - __clz(L);                // (-1 for lanes without a sample differs from every label there)
     for (int i = i0; i < i1; i += 32) {
         const bool in = i + lane < i1;
         const int32_t lab = in ? labels[base + i + lane] : -1;
-        const unsigned same = __match_any_sync(0xffffffffu, lab);
+        const unsigned same = same_label(lab, labelBits);
         const int rank = __popc(same & ((1u << lane) - 1u));
         int32_t pos = 0;
         if (in) pos = mine[lab] + rank;
@@ -185,7 +306,7 @@ __global__ void __launch_bounds__(kGroupThreads) label_place_kernel(const int32_
     if (!Xs) return;
     __syncthreads();
     const bool vec = rowBytes % 16 == 0 && pitch % 16 == 0 && ((uintptr_t)X) % 16 == 0 && ((uintptr_t)Xs) % 16 == 0;
-    for (int i = warp + blockIdx.y * kGroupWarps; i < n; i += kGroupWarps * gridDim.y)
+    for (int i = warp + blockIdx.y * warps; i < n; i += warps * gridDim.y)
         copy_row(X + (base + i) * rowBytes, Xs + (int64_t)shPos[i] * pitch, rowBytes, pitch, vec, lane);
 }
 
@@ -269,15 +390,43 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const uint8_t *__restr
 
 static bool shared_labels(int32_t L) { return L <= kMaxSharedLabels; }
 
+// Histogram of few numbers (GroupShape::few): the verdict on the labels and, unless null, the sizes arrive in pinned memory (wait_few_counts).
+rcd_status launch_label_hist_few(rcd_ctx *ctx, const int32_t *labels, int64_t N, int32_t L, const GroupShape &shape, int32_t *chunkHist, int32_t *counts, int32_t *status,
+                                 int32_t *callStatus, int32_t *zeros, int64_t nZeros, int32_t *hostStatus, int32_t *hostCounts, cudaStream_t st)
+{
+    const int chunk = shape.chunk;
+    const size_t smem = (size_t)L * 4;
+    label_hist_few_kernel<<<(unsigned)((N + chunk - 1) / chunk), shape.threads, smem, st>>>(labels, N, L, chunk, chunkHist, counts, status, callStatus, zeros, (int32_t)nZeros,
+                                                                                     (uint32_t *)(ctx->statusOwn + kHistTicket), hostStatus, hostCounts,
+                                                                                     ctx->hostStage + ctx->hostStageInts + kStageArrived, ++ctx->histTurn);
+    ctx->kernelLaunches++;
+    RCD_CUDA(ctx, cudaGetLastError());
+    return RCD_OK;
+}
+
+// Waits for them: the kernel's last word is looked at directly, which is some microseconds sooner than an event behind the kernel.
+rcd_status wait_few_counts(rcd_ctx *ctx, cudaStream_t st)
+{
+    volatile int32_t *const arrived = ctx->hostStage + ctx->hostStageInts + kStageArrived;
+    for (unsigned k = 1; *arrived != ctx->histTurn; ++k)
+        if (k % 65536 == 0) {                              // (a kernel that failed says nothing)
+            const cudaError_t e = cudaStreamQuery(st);
+            if (e == cudaSuccess && *arrived != ctx->histTurn) return fail(ctx, RCD_ERR_INTERNAL, "the class sizes did not arrive");
+            if (e != cudaSuccess && e != cudaErrorNotReady) return cuda_fail(ctx, e, "waiting for the class sizes");
+        }
+    std::atomic_thread_fence(std::memory_order_acquire);
+    return RCD_OK;
+}
+
 // Histogram of the labels: counts[L] (zeroed by the caller, like *status), and per chunk.
-rcd_status launch_label_hist(rcd_ctx *ctx, const int32_t *labels, int64_t N, int32_t L, int32_t *chunkHist, int32_t *counts,
+rcd_status launch_label_hist(rcd_ctx *ctx, const int32_t *labels, int64_t N, int32_t L, const GroupShape &shape, int32_t *chunkHist, int32_t *counts,
                              int32_t *status, int32_t *callStatus, cudaStream_t st)
 {
     if (N == 0) {
         if (callStatus) RCD_CUDA(ctx, cudaMemsetAsync(callStatus, 0, sizeof(int32_t), st));
         return RCD_OK;
     }
-    const int chunk = group_chunk(N, L);
+    const int chunk = shape.chunk;
     const unsigned nChunks = (unsigned)((N + chunk - 1) / chunk);
     if (shared_labels(L)) {
         const size_t smem = (size_t)L * 4;
@@ -307,7 +456,7 @@ rcd_status launch_gather_rows(rcd_ctx *ctx, const void *X, const int32_t *perm, 
 
 // Stable split after launch_label_hist: perm, and with X the rows in split order (Xs, `pitch` bytes apart, zero-filled
 // beyond rowBytes).  desc null: label l starts after the counts of the labels below it; the starts go to offsets[L + 1].
-rcd_status launch_stable_split(rcd_ctx *ctx, const int32_t *labels, int64_t N, int32_t L, int32_t *chunkHist, const ClassDesc *descDev,
+rcd_status launch_stable_split(rcd_ctx *ctx, const int32_t *labels, int64_t N, int32_t L, const GroupShape &shape, int32_t *chunkHist, const ClassDesc *descDev,
                                const int32_t *counts, int64_t *offsets, const int32_t *status, int32_t *perm,
                                const void *X, int64_t rowBytes, int64_t pitch, void *Xs, cudaStream_t st)
 {
@@ -315,17 +464,20 @@ rcd_status launch_stable_split(rcd_ctx *ctx, const int32_t *labels, int64_t N, i
         if (offsets) RCD_CUDA(ctx, cudaMemsetAsync(offsets, 0, (size_t)(L + 1) * sizeof(int64_t), st));
         return RCD_OK;
     }
-    const int chunk = group_chunk(N, L);
+    const int chunk = shape.chunk;
     const int nChunks = (int)((N + chunk - 1) / chunk);
-    label_scan_kernel<<<(L + 31) / 32, 1024, 0, st>>>(chunkHist, nChunks, L, descDev, counts, offsets, status);
-    ctx->kernelLaunches++;
+    const bool few = shape.few;
+    if (!few) {
+        label_scan_kernel<<<(L + 31) / 32, 1024, 0, st>>>(chunkHist, nChunks, L, descDev, counts, offsets, status);
+        ctx->kernelLaunches++;
+    }
     if (shared_labels(L)) {
-        const size_t smem = ((size_t)kGroupWarps * L + (Xs ? chunk : 0)) * 4;
+        const size_t smem = ((size_t)shape.threads / 32 * L + (Xs ? chunk : 0) + (few ? L : 0)) * 4;
         if (smem > 48 * 1024) RCD_CUDA(ctx, cudaFuncSetAttribute(label_place_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         // (few samples: several CTAs rank the same chunk and share its rows out, so that wide rows occupy more than a few SMs)
         const dim3 grid(nChunks, Xs ? std::max(1, std::min(16, 2 * ctx->smCount / nChunks)) : 1);
-        label_place_kernel<<<grid, kGroupThreads, smem, st>>>(labels, N, L, chunk, chunkHist, perm, (const uint8_t *)X, rowBytes, pitch,
-                                                                (uint8_t *)Xs, status);
+        label_place_kernel<<<grid, shape.threads, smem, st>>>(labels, N, L, chunk, chunkHist, perm, (const uint8_t *)X, rowBytes, pitch,
+                                                                (uint8_t *)Xs, status, few ? descDev : nullptr, few && !descDev ? counts : nullptr, few ? offsets : nullptr);
         ctx->kernelLaunches++;
     } else {
         chunk_rank_kernel<false><<<nChunks, 1024, 0, st>>>(labels, N, L, chunk, chunkHist, perm, status);

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <stddef.h>
+#include <algorithm>
 #include <memory>
 #include <string>
 #include <vector>
@@ -142,10 +143,11 @@ struct Workspace {
 
 // Words of rcd_ctx::statusOwn, and where the similarity kernel's tile tickets (zero between launches) begin.
 constexpr int kStatusWords = 1024;
+constexpr int kHistTicket = 32;            // label_hist_few_kernel's (zero between launches)
 constexpr int kFirstTicket = 64;
-// The staging buffer holds as many class sizes as a call may have, behind them the status words that come along, and last a word
-// that the device writes: a class was left in floating point.
-constexpr int kStageSpare = 1024, kStageLeft = kStageSpare - 1;
+// The staging buffer holds as many class sizes as a call may have, behind them the status words that come along, and last two words
+// that the device writes: a class was left in floating point; the number of the last histogram whose sizes have arrived.
+constexpr int kStageSpare = 1024, kStageLeft = kStageSpare - 1, kStageArrived = kStageSpare - 2;
 
 // A class whose samples' norms lie too far apart for one fixed-point scale (see fixed_exponent_kernel).
 constexpr int32_t kNotFixed = INT32_MIN;
@@ -168,6 +170,23 @@ constexpr int kMaxSharedLabels = 6000;
 // chunks x labels, which is cleared and summed up on every call, would pass 64 MB (lists of 131072 samples over 20000 labels,
 // 41 MB: 101 us, large chunks 126; over 100000, 205 MB: 923 us, large chunks 468).
 inline int group_chunk(int64_t N, int64_t labels) { return N <= 131072 && (N + 255) / 256 * labels <= 1 << 24 ? 256 : 1024; }
+// How a split goes about it: samples per chunk, threads per CTA, and whether every CTA adds up the numbers of all chunks by itself, which
+// saves a memset, the launch of a scan and a copy.  With rows to gather (rows) up to 32 chunks and 4096 numbers (2 classes of 200: 148 -> 138
+// us the whole call, 4 of 20 52 -> 40; with 9600 numbers, 300 classes of 27, the additions take longer than the scan, 79 us against 70).
+// Lists alone have no rows to share out: their chunks are as large as gives an SM one, up to 16384 samples (1.3 million over 64 workers:
+// 41 us with 1024 samples per chunk and a scan, 27 so; 80 samples 26 -> 20).
+struct GroupShape { int chunk, threads; bool few; };
+inline GroupShape group_shape(int64_t N, int64_t labels, bool rows)
+{
+    GroupShape g{group_chunk(N, labels), 256, false};
+    if (!rows && labels <= 1024 && N > 160 * 256) {
+        g.chunk = (int)std::min<int64_t>((N + 144 * 1024 - 1) / (144 * 1024), 16) * 1024;
+        g.threads = 1024;
+    }
+    const int64_t chunks = (N + g.chunk - 1) / g.chunk;
+    g.few = N > 0 && labels <= kMaxSharedLabels && (rows ? chunks <= 32 && chunks * labels <= 4096 : chunks <= 144 && chunks * labels <= 16384);
+    return g;
+}
 // Bytes between the class-sorted feature rows: whole 16-byte pieces, at least one 128-byte slab, so that every width can
 // be loaded by the tensor-core kernel (the padding is zeros and adds nothing to a dot product).
 inline int64_t row_pitch(int64_t rowBytes) { return rowBytes <= 128 ? 128 : (rowBytes + 15) / 16 * 16; }
@@ -230,6 +249,7 @@ struct rcd_ctx {
     std::string err;
     int32_t *hostStage = nullptr;       // pinned, counts / status read-back
     int32_t *statusOwn = nullptr;       // device status word for calls that take no workspace; from kFirstTicket on, tile tickets
+    int32_t histTurn = 0;               // histograms of few numbers so far
     unsigned simReady = 0;              // tensor-core similarity kernels whose shared memory has been asked for, a bit each
     unsigned simTurn = 0;               // similarity launches so far: each takes the next ticket
     size_t hostStageInts = 0;
@@ -268,9 +288,12 @@ rcd_status cuda_fail(rcd_ctx *ctx, cudaError_t e, const char *what);
 // ---- launchers implemented in the .cu files (all asynchronous on `st`) ----
 
 // class split
-rcd_status launch_label_hist(rcd_ctx *ctx, const int32_t *labels, int64_t N, int32_t L, int32_t *chunkHist, int32_t *counts,
+rcd_status launch_label_hist(rcd_ctx *ctx, const int32_t *labels, int64_t N, int32_t L, const GroupShape &shape, int32_t *chunkHist, int32_t *counts,
                              int32_t *status, int32_t *callStatus, cudaStream_t st);
-rcd_status launch_stable_split(rcd_ctx *ctx, const int32_t *labels, int64_t N, int32_t L, int32_t *chunkHist, const ClassDesc *descDev,
+rcd_status launch_label_hist_few(rcd_ctx *ctx, const int32_t *labels, int64_t N, int32_t L, const GroupShape &shape, int32_t *chunkHist, int32_t *counts, int32_t *status,
+                                 int32_t *callStatus, int32_t *zeros, int64_t nZeros, int32_t *hostStatus, int32_t *hostCounts, cudaStream_t st);
+rcd_status wait_few_counts(rcd_ctx *ctx, cudaStream_t st);
+rcd_status launch_stable_split(rcd_ctx *ctx, const int32_t *labels, int64_t N, int32_t L, const GroupShape &shape, int32_t *chunkHist, const ClassDesc *descDev,
                                const int32_t *counts, int64_t *offsets, const int32_t *status, int32_t *perm,
                                const void *X, int64_t rowBytes, int64_t pitch, void *Xs, cudaStream_t st);
 
