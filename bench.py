@@ -332,7 +332,7 @@ def run_ours(args):
     kernel_name = {rcd.RCD_FORM_LAUNCHES: "sweep_kernel", rcd.RCD_FORM_BARRIERS: "greedy_persistent_kernel", rcd.RCD_FORM_ASYNC: "greedy_async_kernel",
                    rcd.RCD_FORM_CLASS_PER_CTA: "greedy_owner_kernel", rcd.RCD_FORM_CLUSTER: "greedy_cluster_kernel",
                    rcd.RCD_FORM_ROUNDS: "greedy_rounds_kernel", rcd.RCD_FORM_CUT_CHAIN: "cut_chain_kernel",
-                   rcd.RCD_FORM_SMALL: "greedy_small_kernel"}[int(prof["greedy_form"])]
+                   rcd.RCD_FORM_SMALL: "greedy_small_kernel", rcd.RCD_FORM_CUT_STEPS: "cut_lockstep_kernel"}[int(prof["greedy_form"])]
     # S larger than L2: the sweeps stream from HBM (peak: the measured copy bandwidth); S inside L2: they stream from
     # L2 (peak: this library's read-only sweep yardstick over an L2-resident buffer, measured in this run)
     bound = "l2" if fits_l2 else "hbm"

@@ -127,7 +127,8 @@ typedef enum {
     RCD_FORM_CLUSTER = 5,      /* a thread-block cluster per class */
     RCD_FORM_ROUNDS = 6,       /* a CTA per class, in rounds */
     RCD_FORM_CUT_CHAIN = 7,    /* graph cut, a CTA per class */
-    RCD_FORM_SMALL = 8         /* small classes, a CTA per class with its similarities in shared memory */
+    RCD_FORM_SMALL = 8,        /* small classes, a CTA per class with its similarities in shared memory */
+    RCD_FORM_CUT_STEPS = 9     /* graph cut, a cluster per class in step */
 } rcd_greedy_form;
 
 /* Timings and counters of the last rcd_partition / rcd_partition_host on a context (profile >= 1).  New ones are added at the end:

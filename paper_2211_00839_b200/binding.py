@@ -26,7 +26,7 @@ RCD_SIM_DOT = 0
 RCD_SIM_GAUSSIAN = 1
 RCD_OBJ_FACILITY = 0
 RCD_OBJ_GRAPH_CUT = 1
-RCD_FORM_LAUNCHES, RCD_FORM_BARRIERS, RCD_FORM_ASYNC, RCD_FORM_CLASS_PER_CTA, RCD_FORM_CLUSTER, RCD_FORM_ROUNDS, RCD_FORM_CUT_CHAIN, RCD_FORM_SMALL = range(1, 9)
+RCD_FORM_LAUNCHES, RCD_FORM_BARRIERS, RCD_FORM_ASYNC, RCD_FORM_CLASS_PER_CTA, RCD_FORM_CLUSTER, RCD_FORM_ROUNDS, RCD_FORM_CUT_CHAIN, RCD_FORM_SMALL, RCD_FORM_CUT_STEPS = range(1, 10)
 
 STATUS_NAMES = {0: "RCD_OK", 1: "RCD_ERR_INVALID_ARG", 2: "RCD_ERR_UNSUPPORTED", 3: "RCD_ERR_WORKSPACE_TOO_SMALL",
                 4: "RCD_ERR_CUDA", 5: "RCD_ERR_TIMEOUT", 6: "RCD_ERR_INTERNAL"}

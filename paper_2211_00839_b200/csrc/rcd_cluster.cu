@@ -1489,6 +1489,7 @@ static bool cluster_plan(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassD
     // cluster form was measured before, and they stay)
     plan.small = plan_greedy_small(ctx, sz);
     if (plan.small && !rounds_possible(ctx, sz, descHost)) return true;
+    if (sz.graphCut && cut_in_step(ctx, sz)) return false;
     const bool clusters = cluster_shape(ctx, sz, descHost, nonEmpty, maxLd, plan, &resident);
     plan.prm.maxLd = maxLd;
     plan.rounds = plan_greedy_rounds(ctx, sz, descHost, clusters ? ClusterShape{plan.C, resident, plan.P} : ClusterShape{0, 0, 0});

@@ -7,9 +7,11 @@
 // costs O(M) per pick.  Values: int64 for int8 features (exact), double otherwise.
 // The objective is not monotone (a sample that joins A stops being cut), gains may be negative;
 // Algorithm 1 runs unchanged: least-f non-full block, argmax with lowest-index ties.
-#include "rcd_internal.h"
+#include "rcd_exact.cuh"
 
 #include <limits.h>
+#include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 namespace rcd {
@@ -139,6 +141,291 @@ __global__ void __launch_bounds__(kCutThreads, 2) cut_chain_kernel(CutParams<SV>
     for (int p = threadIdx.x; p < W; p += kCutThreads) prm.fval[(int64_t)l * W + p] = shF[p];
 }
 
+// ---- integer similarities: a cluster per class, all warps in step ------------------------------
+// What bounds the alternatives.  One CTA per class with everything in global memory (cut_chain_kernel) takes 7.6 us per pick.  In the
+// cluster form (rcd_cluster.cu) picks of different blocks overlap, but under this objective all blocks want the same samples, so half the
+// notes of 10 classes of 5000 into 8 blocks are stale when their block's turn comes, and a pick takes 1.8 us.  Here a thread keeps some
+// columns of the class, with their gains for every block in shared memory, and nothing goes stale: all warps post their best unassigned
+// candidate for the block that is next to every CTA, and after one barrier everybody knows the pick.  The sample's row of S is asked for
+// then, and taken off the block's gains two picks later (or where the block comes again before), so that the trip to memory passes under
+// other picks.  One more warp per CTA keeps the blocks' values and prepares the choice of the next block.
+//
+// What bounds it (10 classes of 5000 into 8 blocks, 8 CTAs each, 2900 cycles a pick): instructions of one warp after another, a third of
+// the cycles for the candidates and the row's loads, and the cluster's barrier.  Whole calls, before and now: 3 classes of 1300 into 20
+// blocks 2103 and 1340 us, 30 of 2500 into 8 blocks 5060 and 4104, 200 of 700 into 8 blocks 2886 and 1256.
+constexpr int kLockWarps = 8;             // with columns, at most
+constexpr int kLockColumns = 8;           // of a thread, at most
+constexpr int kLockBlocks = 128;
+constexpr int kLockCtas = 16;
+constexpr unsigned long long kLockZero = 1ull << 55;        // (tracked values can be negative)
+
+struct LockParams {
+    const ClassDesc *desc;
+    const int32_t *S;
+    long long *base;           // [N] column sum minus the diagonal entry, class-sorted order
+    unsigned long long *top;   // [L] zero at the start: largest sum of |S| over a row
+    long long *fval;           // [L][W]
+    const int32_t *quota;
+    const int32_t *perm;
+    const int32_t *classOrder;
+    uint32_t *picks;           // [N] sample | block << 16, in the order picked
+    int32_t *assignment;
+    int32_t *order;            // may be null
+    int32_t *status;
+    int32_t W;
+    int32_t columns;           // of a CTA (its gains: [W][columns])
+    uint32_t one;              // the value 1, opaque to the compiler
+};
+
+__device__ __forceinline__ void lock_barrier(bool alone)
+{
+    if (alone) __syncthreads();
+    else asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// K: columns per thread; KW: blocks per lane of the leader.
+template <int K, int KW>
+__global__ void __launch_bounds__((kLockWarps + 1) * 32) cut_lockstep_kernel(const __grid_constant__ LockParams prm)
+{
+    extern __shared__ __align__(16) unsigned char shared[];
+    __shared__ unsigned long long shBest[2][kLockCtas * kLockWarps];           // the warps' best candidates, for two picks in turn
+    __shared__ unsigned long long shOthers[2];             // the least value << 7 | block among the blocks with room but the next
+    __shared__ int shLeft[2];                              // room of the next block
+    uint32_t rank, C;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
+    const bool alone = C == 1;
+    const int l = prm.classOrder[blockIdx.x / C], W = prm.W, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int NW = (int)(blockDim.x >> 5) - 1, NT = NW * 32, entries = NW * (int)C;
+    const ClassDesc c = prm.desc[l];
+    const int M = c.M;
+    if (M == 0) {                                          // empty class: every block has value 0
+        if (rank == 0) for (int p = threadIdx.x; p < W; p += blockDim.x) prm.fval[(int64_t)l * W + p] = 0;
+        return;
+    }
+    const int32_t *const Sl = prm.S + c.sOff;
+    long long *const base = prm.base + c.row0;
+    unsigned long long *const gains = reinterpret_cast<unsigned long long *>(shared) + threadIdx.x;  // of block j, k-th column: [j * prm.columns + k * NT]
+    const int column = (int)rank * prm.columns + threadIdx.x;
+
+    if (warp < NW) {
+        unsigned long long top = 0;
+        for (int u = (int)rank * NW + warp; u < M; u += entries) {
+            unsigned long long neg;
+            const unsigned long long pos = row_value<true>(reinterpret_cast<const int4 *>(Sl + (int64_t)u * c.ld), c.ld >> 2, lane, prm.one, neg);
+            top = umax(top, pos + neg);
+            if (lane == 0) __stcg(base + u, (long long)(pos - neg) - (long long)Sl[(int64_t)u * c.ld + u]);
+        }
+        if (lane == 0 && top) atomicMax(prm.top + l, top);
+    }
+    unsigned long long f[KW], least;                       // value << 7 | block; least: of the block that is next
+    int room[KW];
+    auto least_but = [&](int but) {
+        unsigned long long m = ~0ull;
+#pragma unroll
+        for (int k = 0; k < KW; ++k) m = room[k] > 0 && lane + 32 * k != but ? umin(m, f[k]) : m;
+        return ~warp_max_u64(~m);
+    };
+#pragma unroll
+    for (int k = 0; k < KW; ++k) {                         // (every warp finds the first block; the leader goes on with these)
+        f[k] = (kLockZero << 7) | (unsigned long long)(lane + 32 * k);
+        room[k] = lane + 32 * k < W ? prm.quota[(int64_t)l * W + lane + 32 * k] : 0;
+    }
+    least = least_but(-1);
+    lock_barrier(alone);
+    // gains lie within three times the largest sum of |S| over a row, either way
+    const unsigned long long bias = 3 * __ldcg(prm.top + l) + 1;
+    unsigned gone = 0;                                     // columns that are assigned or beyond the class
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int u = column + k * NT;
+        const bool own = warp < NW && k * NT + (int)threadIdx.x < prm.columns;
+        const unsigned long long g = own && u < M ? (unsigned long long)__ldcg(base + u) + bias : 0ull;
+        if (own)
+            for (int p = 0; p < W; ++p) gains[p * prm.columns + k * NT] = g;
+        gone |= own && u < M ? 0u : 1u << k;
+    }
+    struct Owed {                                          // the row of a sample picked lately, for its block (-1: none)
+        int32_t row[K];
+        int block;
+    } even, odd;
+    even.block = odd.block = -1;
+    auto settle = [&](Owed &o) {
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+            if (k * NT + (int)threadIdx.x < prm.columns) gains[o.block * prm.columns + k * NT] -= 2ll * o.row[k];
+        o.block = -1;
+    };
+    // (mine: of the pick before the last, and then of this one; last: of the pick before)
+    auto make_pick = [&](int t, Owed &mine, Owed &last) {
+        const int j = (int)(least & 127);
+        if (warp < NW) {
+            if (last.block == j) settle(last);
+            if (mine.block == j) settle(mine);
+            unsigned long long best = 0;
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+                if (!(gone >> k & 1)) best = umax(best, make_key(gains[j * prm.columns + k * NT], column + k * NT));
+            best = warp_max_u64(best);
+            unsigned long long *const to = &shBest[t & 1][rank * NW + warp];
+            if (alone) {
+                if (lane == 0) *to = best;
+            } else if (lane < (int)C) {
+                uint32_t at;
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(smem32(to)), "r"(lane));
+                asm volatile("st.shared::cluster.u64 [%0], %1;" :: "r"(at), "l"(best) : "memory");
+            }
+            if (mine.block >= 0) settle(mine);
+        } else {
+            const unsigned long long others = least_but(j);
+            int left = room[0];
+#pragma unroll
+            for (int k = 1; k < KW; ++k) left ^= (left ^ room[k]) & (j >> 5 == k ? ~0 : 0);
+            left = __shfl_sync(0xffffffffu, left, j & 31);
+            if (lane == 0) {
+                shOthers[t & 1] = others;
+                shLeft[t & 1] = left;
+            }
+        }
+        lock_barrier(alone);
+        unsigned long long best = 0;
+        for (int i = lane; i < entries; i += 32) best = umax(best, shBest[t & 1][i]);
+        best = warp_max_u64(best);
+        const unsigned long long others = shOthers[t & 1], inc = ((best >> 16) - bias) << 7;
+        const bool more = shLeft[t & 1] > 1;
+        const int v = key_sample(best);
+        least = umin(others, more ? least + inc : ~0ull);
+        if (warp < NW) {
+            if (more) {                                    // (a full block needs no gains any more)
+                const int32_t *const from = Sl + (int64_t)v * c.ld + column;
+#pragma unroll
+                for (int k = 0; k < K; ++k) mine.row[k] = k * NT + (int)threadIdx.x < prm.columns && column + k * NT < M ? __ldg(from + k * NT) : 0;
+                mine.block = j;
+            }
+#pragma unroll
+            for (int k = 0; k < K; ++k) gone |= column + k * NT == v ? 1u << k : 0u;
+        } else {
+#pragma unroll
+            for (int k = 0; k < KW; ++k) {
+                f[k] += lane + 32 * k == j ? inc : 0ull;
+                room[k] -= lane + 32 * k == j ? 1 : 0;
+            }
+            // (a load in front of the stores that need it would hold up every pick)
+            if (rank == 0 && lane == 0) prm.picks[c.row0 + t] = (uint32_t)v | (uint32_t)j << 16;
+        }
+        if (best == 0 || (least == ~0ull && t + 1 < M)) {  // (cannot be: samples are left, and the quotas add up to M)
+            if (threadIdx.x == 0) atomicOr(prm.status, kDevNoCandidate);
+            return false;
+        }
+        return true;
+    };
+    for (int t = 0; t < M; t += 2) {
+        if (!make_pick(t, even, odd)) break;
+        if (t + 1 < M && !make_pick(t + 1, odd, even)) break;
+    }
+    if (rank == 0 && warp == NW) {
+#pragma unroll
+        for (int k = 0; k < KW; ++k)
+            if (lane + 32 * k < W) prm.fval[(int64_t)l * W + lane + 32 * k] = (long long)(f[k] >> 7) - (long long)kLockZero;
+    }
+    lock_barrier(alone);                                   // (and nobody writes to a CTA that has gone)
+    // class-local picks -> outputs
+    for (int t = (int)(rank * blockDim.x + threadIdx.x); t < M; t += (int)(C * blockDim.x)) {
+        const uint32_t p = __ldcg(prm.picks + c.row0 + t);
+        const int global = prm.perm[c.row0 + (p & 0xffff)];
+        prm.assignment[global] = (int)(p >> 16);
+        if (prm.order) prm.order[c.row0 + t] = global;
+    }
+}
+
+typedef void (*LockKernel)(LockParams);
+template <int KW>
+static LockKernel pick_lockstep(int K)
+{
+    return K == 1 ? cut_lockstep_kernel<1, KW> : K == 2 ? cut_lockstep_kernel<2, KW> : K == 3 ? cut_lockstep_kernel<3, KW> : K <= 4 ? cut_lockstep_kernel<4, KW> : cut_lockstep_kernel<kLockColumns, KW>;
+}
+
+struct LockPlan { int C, K, warps, columns; size_t smem; };
+
+// Whether the classes run in step, and on how many CTAs each: those with which they are through soonest.  A pick takes 1600 cycles with one
+// CTA, 2100 with several (a barrier over a cluster takes 400, over a CTA 30), and 260 more for every column of a thread (measured on 250 to
+// 5000 samples); clusters keep within a GPC.  Not with few blocks and classes, whose picks wait for the sample's row, while the cluster
+// form foresees it (3 or 30 classes of 700 to 2500: 0.6 to 0.9 times as fast with 2 and 4 blocks, 0.96 to 1.45 times with 8, 1.1 to 2.2 with
+// more; 200 classes: 1 to 2.8 times, whatever the blocks), and not where short classes come one to an SM and have to come again (200 of 400
+// into 50 blocks: 1014 us, the cluster form 874).
+static bool plan_lockstep(const rcd_ctx *ctx, const Sizes &sz, LockPlan &plan)
+{
+    if (sz.W > kLockBlocks || sz.maxM == 0 || sz.maxM > 65535 || sz.floatArith) return false;
+    if (sz.W < 6 && sz.L <= 64 && sz.maxM <= 8192) return false;
+    double best = 0;
+    plan.C = 0;
+    bool again = false;
+    for (int C = 1; C <= kLockCtas; C *= 2) {
+        LockPlan p;
+        p.C = C;
+        const int share = (int)((sz.maxM + C - 1) / C), words = (share + 31) / 32;
+        p.K = (words + kLockWarps - 1) / kLockWarps;
+        if (p.K > 4) p.K = kLockColumns;
+        p.warps = std::min(kLockWarps, (words + p.K - 1) / p.K);
+        p.columns = words * 32;
+        p.smem = (size_t)sz.W * p.columns * 8;
+        if (words > kLockWarps * kLockColumns || p.smem > (size_t)ctx->maxSmemOptin - 8192 || (C > 1 && share < 128)) continue;
+        const int perSm = (int)std::max<size_t>(1, std::min<size_t>(6, (size_t)ctx->maxSmemOptin / (p.smem + 4096)));
+        const double resident = C == 1 ? (double)ctx->smCount * perSm : C == 16 ? (double)(ctx->smCount / 20) : std::floor(0.9 * ctx->smCount / C);
+        const double turns = std::max(1.0, std::ceil(sz.L / resident - 1e-9));
+        const double time = turns * ((C == 1 ? 1570.0 : 2130.0) + 260.0 * p.K);
+        if (plan.C == 0 || time < best) {
+            plan = p;
+            best = time;
+            again = turns > 1 && perSm == 1 && sz.maxM < 512;
+        }
+    }
+    return plan.C > 0 && !again;
+}
+
+bool cut_in_step(const rcd_ctx *ctx, const Sizes &sz)
+{
+    LockPlan plan;
+    return plan_lockstep(ctx, sz, plan);
+}
+
+static rcd_status run_lockstep(rcd_ctx *ctx, const LockPlan &plan, const Sizes &sz, const Workspace &ws, int32_t *assignment, int32_t *order, cudaStream_t st)
+{
+    LockParams prm;
+    prm.desc = ws.desc;
+    prm.S = (const int32_t *)ws.S;
+    prm.base = (long long *)ws.cutBase;
+    prm.top = ws.topGain;
+    prm.fval = (long long *)ws.fval;
+    prm.quota = ws.quota;
+    prm.perm = ws.perm;
+    prm.classOrder = ws.classOrder;
+    prm.picks = (uint32_t *)ws.cand;
+    prm.assignment = assignment;
+    prm.order = order;
+    prm.status = ctx->statusOwn;
+    prm.W = sz.W;
+    prm.columns = plan.columns;
+    prm.one = 1u;
+    const LockKernel kernel = sz.W <= 32 ? pick_lockstep<1>(plan.K) : sz.W <= 64 ? pick_lockstep<2>(plan.K) : pick_lockstep<4>(plan.K);
+    RCD_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem));
+    RCD_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(sz.L * plan.C));
+    cfg.blockDim = dim3((unsigned)(plan.warps + 1) * 32);
+    cfg.dynamicSmemBytes = plan.smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)plan.C;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    RCD_CUDA(ctx, cudaLaunchKernelEx(&cfg, kernel, prm));
+    ctx->kernelLaunches++;
+    return RCD_OK;
+}
+
 // f(A_p) for every block from the definition: per row v the sums r_p(v) = sum_{a in A_p} S[v][a], then
 // f_p += r_p(v) for every block p that v is not in.  int64 sums are exact; fp64 sums inside a row are
 // accumulated with shared-memory atomics, so their last bits can differ from run to run.
@@ -243,6 +530,11 @@ rcd_status launch_cut(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, int32_
 {
     if (sz.L == 0 || sz.maxM == 0) return RCD_OK;
     ctx->greedyForm = RCD_FORM_CUT_CHAIN;
+    LockPlan plan;
+    if (plan_lockstep(ctx, sz, plan)) {
+        ctx->greedyForm = RCD_FORM_CUT_STEPS;
+        return run_lockstep(ctx, plan, sz, ws, assignment, order, st);
+    }
     if (sz.floatArith) return run_cut<float>(ctx, sz, ws, assignment, order, st);
     return run_cut<int32_t>(ctx, sz, ws, assignment, order, st);
 }

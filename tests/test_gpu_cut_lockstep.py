@@ -1,0 +1,43 @@
+"""The graph cut in step (integers, several blocks) at the edges of its columns per thread and of its clusters, against the oracle."""
+import numpy as np
+import pytest
+
+import test_gpu_cluster as cluster
+from test_gpu_parity import rcd, orc, run_partition  # noqa: F401  (fixtures)
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("sizes,W,copies", [
+    ([257, 31], 6, 0), ([300, 0, 1, 250], 9, 40),          # one or two columns per thread; an empty class, one of a sample, ties
+    ([513], 33, 0), ([770, 5], 65, 30),                    # two and four blocks per lane; a class that leaves most CTAs without columns
+    ([1300, 1281], 8, 60), ([2600], 50, 0),                # clusters
+    ([260] * 160, 2, 0), ([250] * 70, 5, 20),              # more classes than SMs, few blocks
+])
+def test_exact(rcd, orc, sizes, W, copies):
+    import torch
+    wl = cluster.workload(sizes, 32, W, W + len(sizes), copies=copies)
+    a, o, v = run_partition(rcd, wl, objective=rcd.RCD_OBJ_GRAPH_CUT)
+    ref = orc.partition(wl.features, wl.labels, wl.capacities, wl.L, variant="incremental", objective="cut")
+    assert np.array_equal(a, ref.assignment) and np.array_equal(o, ref.order) and np.array_equal(v, ref.part_values)
+    with rcd.Context(0, objective=rcd.RCD_OBJ_GRAPH_CUT) as ctx:
+        ctx.rcd_partition(rcd.features_to_torch(wl.features, device="cuda"), torch.from_numpy(wl.labels).cuda(), wl.capacities, wl.L)
+        ctx.sync_status()
+        assert ctx.profile()["greedy_form"] == rcd.RCD_FORM_CUT_STEPS
+
+
+def test_like_the_chain(rcd):
+    """A class over clusters of every size the plan takes, against one CTA with everything in global memory (more than 128 blocks)."""
+    import torch
+    for M, W in ((6000, 12), (3000, 100)):
+        wl = cluster.workload([M, 300], 48, W, W)
+        X, y = rcd.features_to_torch(wl.features, device="cuda"), torch.from_numpy(wl.labels).cuda()
+        out = []
+        for caps in (list(wl.capacities), list(wl.capacities) + [1e-9] * (129 - W)):       # (blocks that get nothing)
+            with rcd.Context(0, objective=rcd.RCD_OBJ_GRAPH_CUT) as ctx:
+                r = ctx.rcd_partition(X, y, caps, wl.L)
+                ctx.sync_status()
+                out.append((r[0].cpu().numpy(), r[1].cpu().numpy(), r[2].cpu().numpy()[:, :W], ctx.profile()["greedy_form"]))
+        assert out[0][3] == rcd.RCD_FORM_CUT_STEPS and out[1][3] == rcd.RCD_FORM_CUT_CHAIN
+        for got, want in zip(out[0][:3], out[1][:3]):
+            assert np.array_equal(got, want)
