@@ -146,13 +146,13 @@ __global__ void __launch_bounds__(kCutThreads, 2) cut_chain_kernel(CutParams<SV>
 // cluster form (rcd_cluster.cu) picks of different blocks overlap, but under this objective all blocks want the same samples, so half the
 // notes of 10 classes of 5000 into 8 blocks are stale when their block's turn comes, and a pick takes 1.8 us.  Here a thread keeps some
 // columns of the class, with their gains for every block in shared memory, and nothing goes stale: all warps post their best unassigned
-// candidate for the block that is next to every CTA, and after one barrier everybody knows the pick.  The sample's row of S is asked for
+// candidate for the block that is next to every CTA, and when all have arrived everybody knows the pick.  The sample's row of S is asked for
 // then, and taken off the block's gains two picks later (or where the block comes again before), so that the trip to memory passes under
 // other picks.  One more warp per CTA keeps the blocks' values and prepares the choice of the next block.
 //
-// What bounds it (10 classes of 5000 into 8 blocks, 8 CTAs each, 2900 cycles a pick): instructions of one warp after another, a third of
-// the cycles for the candidates and the row's loads, and the cluster's barrier.  Whole calls, before and now: 3 classes of 1300 into 20
-// blocks 2103 and 1340 us, 30 of 2500 into 8 blocks 5060 and 4104, 200 of 700 into 8 blocks 2886 and 1256.
+// What bounds it (10 classes of 5000 into 8 blocks, 8 CTAs each, 2700 cycles a pick): instructions of one warp after another, half of them
+// for the candidates and the row's loads.  Whole calls, before and now: 3 classes of 1300 into 20 blocks 2103 and 1120 us, 30 of 2500 into 8
+// blocks 5060 and 3644, 200 of 700 into 8 blocks 2886 and 1247.
 constexpr int kLockWarps = 8;             // with columns, at most
 constexpr int kLockColumns = 8;           // of a thread, at most
 constexpr int kLockBlocks = 128;
@@ -183,14 +183,42 @@ __device__ __forceinline__ void lock_barrier(bool alone)
     else asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
+// Over a cluster the candidates travel as asynchronous stores that count towards an mbarrier of the CTA they reach (phases of two picks in
+// turn).  A cluster's own barrier for every pick, whose release waits for the rows on their way, cost 700 cycles of 3200.
+__device__ __forceinline__ uint32_t lock_remote(uint32_t addr, uint32_t rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void lock_send(const unsigned long long *to, unsigned long long v, uint32_t bar, uint32_t rank)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" :: "r"(lock_remote(smem32(to), rank)), "l"(v), "r"(lock_remote(bar, rank)) : "memory");
+}
+__device__ __forceinline__ bool lock_wait(uint32_t bar, uint32_t parity)
+{
+    for (unsigned k = 0; k < (1u << 28); ++k) {
+        uint32_t ok;
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+        if (ok) {
+            // (what the stores brought is not read before this; only shared memory: an acquire of everything would drop the L1's lines)
+            asm volatile("fence.acquire.sync_restrict::shared::cluster.cluster;" ::: "memory");
+            return true;
+        }
+    }
+    return false;
+}
+
 // K: columns per thread; KW: blocks per lane of the leader.
 template <int K, int KW>
 __global__ void __launch_bounds__((kLockWarps + 1) * 32) cut_lockstep_kernel(const __grid_constant__ LockParams prm)
 {
     extern __shared__ __align__(16) unsigned char shared[];
     __shared__ unsigned long long shBest[2][kLockCtas * kLockWarps];           // the warps' best candidates, for two picks in turn
-    __shared__ unsigned long long shOthers[2];             // the least value << 7 | block among the blocks with room but the next
-    __shared__ int shLeft[2];                              // room of the next block
+    // by the leader of each CTA: the least value << 7 | block among the blocks with room but the next | 1 << 63: the next has room for one only
+    __shared__ unsigned long long shOthers[2][kLockCtas];
+    __shared__ __align__(8) unsigned long long shBars[2];
     uint32_t rank, C;
     asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
     asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
@@ -208,6 +236,11 @@ __global__ void __launch_bounds__((kLockWarps + 1) * 32) cut_lockstep_kernel(con
     unsigned long long *const gains = reinterpret_cast<unsigned long long *>(shared) + threadIdx.x;  // of block j, k-th column: [j * prm.columns + k * NT]
     const int column = (int)rank * prm.columns + threadIdx.x;
 
+    const uint32_t bars = smem32(shBars);
+    if (threadIdx.x == 0) {
+        for (int k = 0; k < 2; ++k) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(bars + 8 * k) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
     if (warp < NW) {
         unsigned long long top = 0;
         for (int u = (int)rank * NW + warp; u < M; u += entries) {
@@ -259,6 +292,9 @@ __global__ void __launch_bounds__((kLockWarps + 1) * 32) cut_lockstep_kernel(con
     // (mine: of the pick before the last, and then of this one; last: of the pick before)
     auto make_pick = [&](int t, Owed &mine, Owed &last) {
         const int j = (int)(least & 127);
+        const uint32_t bar = bars + 8 * (t & 1);
+        if (!alone && threadIdx.x == 0)
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(bar), "r"((uint32_t)((entries + (int)C) * 8)) : "memory");
         if (warp < NW) {
             if (last.block == j) settle(last);
             if (mine.block == j) settle(mine);
@@ -268,12 +304,10 @@ __global__ void __launch_bounds__((kLockWarps + 1) * 32) cut_lockstep_kernel(con
                 if (!(gone >> k & 1)) best = umax(best, make_key(gains[j * prm.columns + k * NT], column + k * NT));
             best = warp_max_u64(best);
             unsigned long long *const to = &shBest[t & 1][rank * NW + warp];
-            if (alone) {
-                if (lane == 0) *to = best;
-            } else if (lane < (int)C) {
-                uint32_t at;
-                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(smem32(to)), "r"(lane));
-                asm volatile("st.shared::cluster.u64 [%0], %1;" :: "r"(at), "l"(best) : "memory");
+            if (!alone) {
+                if (lane < (int)C) lock_send(to, best, bar, lane);
+            } else if (lane == 0) {
+                *to = best;
             }
             if (mine.block >= 0) settle(mine);
         } else {
@@ -282,17 +316,28 @@ __global__ void __launch_bounds__((kLockWarps + 1) * 32) cut_lockstep_kernel(con
 #pragma unroll
             for (int k = 1; k < KW; ++k) left ^= (left ^ room[k]) & (j >> 5 == k ? ~0 : 0);
             left = __shfl_sync(0xffffffffu, left, j & 31);
-            if (lane == 0) {
-                shOthers[t & 1] = others;
-                shLeft[t & 1] = left;
+            // (to every CTA: nobody writes to candidates that a leader may still be reading)
+            const unsigned long long word = others & ~(1ull << 63) | (left > 1 ? 0ull : 1ull << 63);
+            if (!alone) {
+                if (lane < (int)C) lock_send(&shOthers[t & 1][rank], word, bar, lane);
+            } else if (lane == 0) {
+                shOthers[t & 1][0] = word;
             }
         }
-        lock_barrier(alone);
+        if (alone) {
+            __syncthreads();
+        } else if (!lock_wait(bar, (uint32_t)t >> 1 & 1)) {
+            if (lane == 0) atomicOr(prm.status, kDevTimeout);
+            return false;
+        }
         unsigned long long best = 0;
         for (int i = lane; i < entries; i += 32) best = umax(best, shBest[t & 1][i]);
         best = warp_max_u64(best);
-        const unsigned long long others = shOthers[t & 1], inc = ((best >> 16) - bias) << 7;
-        const bool more = shLeft[t & 1] > 1;
+        unsigned long long others = shOthers[t & 1][rank];
+        const unsigned long long inc = ((best >> 16) - bias) << 7;
+        const bool more = !(others >> 63);
+        others &= ~(1ull << 63);
+        others = others == ~(1ull << 63) ? ~0ull : others;     // (none)
         const int v = key_sample(best);
         least = umin(others, more ? least + inc : ~0ull);
         if (warp < NW) {
@@ -348,15 +393,15 @@ static LockKernel pick_lockstep(int K)
 struct LockPlan { int C, K, warps, columns; size_t smem; };
 
 // Whether the classes run in step, and on how many CTAs each: those with which they are through soonest.  A pick takes 1600 cycles with one
-// CTA, 2100 with several (a barrier over a cluster takes 400, over a CTA 30), and 260 more for every column of a thread (measured on 250 to
-// 5000 samples); clusters keep within a GPC.  Not with few blocks and classes, whose picks wait for the sample's row, while the cluster
-// form foresees it (3 or 30 classes of 700 to 2500: 0.6 to 0.9 times as fast with 2 and 4 blocks, 0.96 to 1.45 times with 8, 1.1 to 2.2 with
-// more; 200 classes: 1 to 2.8 times, whatever the blocks), and not where short classes come one to an SM and have to come again (200 of 400
-// into 50 blocks: 1014 us, the cluster form 874).
+// CTA, 1700 with several, and 260 more for every column of a thread (measured on 250 to 5000 samples); clusters keep within a GPC.
+// Not with few blocks and classes, whose picks wait for the sample's row, while the cluster form foresees it (3 or 30 classes of 700 to
+// 2500: 0.6 to 0.9 times as fast with 2 and 4 blocks, 1.0 to 1.7 times with 8, 1.1 to 2.7 with more; 200 classes: 1.2 to 3 times, but 0.96
+// for 1300 samples into 2 blocks), and not where short classes come one to an SM and have to come again (200 of 400 into 50 blocks in one
+// CTA each 1014 us, the cluster form 874).
 static bool plan_lockstep(const rcd_ctx *ctx, const Sizes &sz, LockPlan &plan)
 {
     if (sz.W > kLockBlocks || sz.maxM == 0 || sz.maxM > 65535 || sz.floatArith) return false;
-    if (sz.W < 6 && sz.L <= 64 && sz.maxM <= 8192) return false;
+    if (sz.W < 6 && sz.maxM <= 8192 && (sz.L <= 64 || (sz.W < 4 && sz.maxM >= 1024))) return false;
     double best = 0;
     plan.C = 0;
     bool again = false;
@@ -373,7 +418,7 @@ static bool plan_lockstep(const rcd_ctx *ctx, const Sizes &sz, LockPlan &plan)
         const int perSm = (int)std::max<size_t>(1, std::min<size_t>(6, (size_t)ctx->maxSmemOptin / (p.smem + 4096)));
         const double resident = C == 1 ? (double)ctx->smCount * perSm : C == 16 ? (double)(ctx->smCount / 20) : std::floor(0.9 * ctx->smCount / C);
         const double turns = std::max(1.0, std::ceil(sz.L / resident - 1e-9));
-        const double time = turns * ((C == 1 ? 1570.0 : 2130.0) + 260.0 * p.K);
+        const double time = turns * ((C == 1 ? 1570.0 : 1700.0) + 260.0 * p.K);
         if (plan.C == 0 || time < best) {
             plan = p;
             best = time;
