@@ -1471,11 +1471,7 @@ static bool cluster_shape(rcd_ctx *ctx, const Sizes &sz, const std::vector<Class
 // samples of a class and blocks within the packed keys' range.
 static bool cluster_plan(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost, ClusterPlan &plan)
 {
-    const rcd_config &c = ctx->cfg;
-    if (c.greedy_path != 0 || c.profile >= 2 || c.sweep_batch_max != 0 || c.sweep_mode != 0 || c.async_group != 0 || c.async_help_min != 0 ||
-        c.threshold_from != 0 || c.threshold_hit_shift != 0 || c.lazy_mode != 0 || c.lazy_from != 0 || c.dense_ring != 0 ||
-        c.incremental != 0 || c.incremental_max != 0)
-        return false;
+    if (!library_chooses(ctx->cfg)) return false;
     if (sz.W > kClusterBlocks || sz.maxM > 65535 || sz.d > 65535 || sz.L > 65535 || sz.maxM == 0) return false;
     if (sz.graphCut && (sz.floatArith || sz.maxM > 8192)) return false;
     int nonEmpty = 0, maxLd = 8, resident = 0;

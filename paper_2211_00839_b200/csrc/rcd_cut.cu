@@ -400,7 +400,7 @@ struct LockPlan { int C, K, warps, columns; size_t smem; };
 // CTA each 1014 us, the cluster form 874).
 static bool plan_lockstep(const rcd_ctx *ctx, const Sizes &sz, LockPlan &plan)
 {
-    if (sz.W > kLockBlocks || sz.maxM == 0 || sz.maxM > 65535 || sz.floatArith) return false;
+    if (!library_chooses(ctx->cfg) || sz.W > kLockBlocks || sz.maxM == 0 || sz.maxM > 65535 || sz.floatArith) return false;
     if (sz.W < 6 && sz.maxM <= 8192 && (sz.L <= 64 || (sz.W < 4 && sz.maxM >= 1024))) return false;
     double best = 0;
     plan.C = 0;

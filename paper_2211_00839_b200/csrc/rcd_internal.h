@@ -276,6 +276,14 @@ struct rcd_ctx {
 
 namespace rcd {
 
+// Whether the library chooses the form of the greedy loop: no pass-based form and none of their options asked for.
+inline bool library_chooses(const rcd_config &c)
+{
+    return c.greedy_path == 0 && c.profile < 2 && c.sweep_batch_max == 0 && c.sweep_mode == 0 && c.async_group == 0 && c.async_help_min == 0 &&
+           c.threshold_from == 0 && c.threshold_hit_shift == 0 && c.lazy_mode == 0 && c.lazy_from == 0 && c.dense_ring == 0 &&
+           c.incremental == 0 && c.incremental_max == 0;
+}
+
 rcd_status fail(rcd_ctx *ctx, rcd_status st, const char *fmt, ...);
 rcd_status cuda_fail(rcd_ctx *ctx, cudaError_t e, const char *what);
 

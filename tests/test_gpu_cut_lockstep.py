@@ -41,3 +41,15 @@ def test_like_the_chain(rcd):
         assert out[0][3] == rcd.RCD_FORM_CUT_STEPS and out[1][3] == rcd.RCD_FORM_CUT_CHAIN
         for got, want in zip(out[0][:3], out[1][:3]):
             assert np.array_equal(got, want)
+
+
+def test_only_where_the_library_chooses(rcd, orc):
+    """An option of the pass-based forms keeps the chain, as before."""
+    import torch
+    wl = cluster.workload([300, 250], 32, 8, 3)
+    with rcd.Context(0, objective=rcd.RCD_OBJ_GRAPH_CUT, greedy_path=3) as ctx:
+        a, o, v = ctx.rcd_partition(rcd.features_to_torch(wl.features, device="cuda"), torch.from_numpy(wl.labels).cuda(), wl.capacities, wl.L)
+        ctx.sync_status()
+        assert ctx.profile()["greedy_form"] == rcd.RCD_FORM_CUT_CHAIN
+    ref = orc.partition(wl.features, wl.labels, wl.capacities, wl.L, variant="incremental", objective="cut")
+    assert np.array_equal(a.cpu().numpy(), ref.assignment) and np.array_equal(v.cpu().numpy(), ref.part_values)
