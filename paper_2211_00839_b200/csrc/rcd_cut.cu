@@ -390,6 +390,9 @@ static LockKernel pick_lockstep(int K)
     return K == 1 ? cut_lockstep_kernel<1, KW> : K == 2 ? cut_lockstep_kernel<2, KW> : K == 3 ? cut_lockstep_kernel<3, KW> : K <= 4 ? cut_lockstep_kernel<4, KW> : cut_lockstep_kernel<kLockColumns, KW>;
 }
 
+// (asked for in full by every launch: contexts of several threads share the kernel)
+static size_t lock_shared(const rcd_ctx *ctx) { return (size_t)ctx->maxSmemOptin - 8192; }
+
 struct LockPlan { int C, K, warps, columns; size_t smem; };
 
 // Whether the classes run in step, and on how many CTAs each: those with which they are through soonest.  A pick takes 1600 cycles with one
@@ -414,7 +417,7 @@ static bool plan_lockstep(const rcd_ctx *ctx, const Sizes &sz, LockPlan &plan)
         p.warps = std::min(kLockWarps, (words + p.K - 1) / p.K);
         p.columns = words * 32;
         p.smem = (size_t)sz.W * p.columns * 8;
-        if (words > kLockWarps * kLockColumns || p.smem > (size_t)ctx->maxSmemOptin - 8192 || (C > 1 && share < 128)) continue;
+        if (words > kLockWarps * kLockColumns || p.smem > lock_shared(ctx) || (C > 1 && share < 128)) continue;
         const int perSm = (int)std::max<size_t>(1, std::min<size_t>(6, (size_t)ctx->maxSmemOptin / (p.smem + 4096)));
         const double resident = C == 1 ? (double)ctx->smCount * perSm : C == 16 ? (double)(ctx->smCount / 20) : std::floor(0.9 * ctx->smCount / C);
         const double turns = std::max(1.0, std::ceil(sz.L / resident - 1e-9));
@@ -453,7 +456,7 @@ static rcd_status run_lockstep(rcd_ctx *ctx, const LockPlan &plan, const Sizes &
     prm.columns = plan.columns;
     prm.one = 1u;
     const LockKernel kernel = sz.W <= 32 ? pick_lockstep<1>(plan.K) : sz.W <= 64 ? pick_lockstep<2>(plan.K) : pick_lockstep<4>(plan.K);
-    RCD_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem));
+    RCD_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lock_shared(ctx)));
     RCD_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(sz.L * plan.C));

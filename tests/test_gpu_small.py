@@ -71,3 +71,32 @@ def test_graph_cut_int8_exact(rcd, orc, sizes, W, copies):
     ref = orc.partition(wl.features, wl.labels, wl.capacities, wl.L, variant="incremental", objective="cut")
     assert np.array_equal(a, ref.assignment) and np.array_equal(o, ref.order) and np.array_equal(v, ref.part_values)
     assert form(rcd, wl, objective=rcd.RCD_OBJ_GRAPH_CUT) == rcd.RCD_FORM_SMALL
+
+
+def test_threads_with_contexts_of_their_own(rcd):
+    """Four threads, each with a context and a stream, problems of very different shared memory at a time: each gets its own results."""
+    import threading
+    import torch
+    wls = [cluster.workload([n], 64, w, n) for n, w in ((210, 4), (60, 3), (140, 40), (100, 9))]
+    want = [run_partition(rcd, wl, greedy_path=4) for wl in wls]
+    bad = []
+
+    def work(wl, ref):
+        try:
+            st = torch.cuda.Stream()
+            with torch.cuda.stream(st), rcd.Context(0) as ctx:
+                X, y = rcd.features_to_torch(wl.features, device="cuda"), torch.from_numpy(wl.labels).cuda()
+                for _ in range(20):
+                    got = ctx.rcd_partition(X, y, wl.capacities, wl.L)
+                    ctx.sync_status()
+                    if not all(np.array_equal(g.cpu().numpy(), r) for g, r in zip(got, ref)):
+                        bad.append(len(wl.labels))
+        except Exception as e:      # noqa: BLE001
+            bad.append(repr(e))
+
+    threads = [threading.Thread(target=work, args=p) for p in zip(wls, want)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
