@@ -38,7 +38,6 @@ constexpr uint32_t kScanCmd = 0u;         // a command's low word: look again;
 constexpr uint32_t kStopCmd = 0xfffffu;   //   the class is done;  anything else: sample + 1 joins the block
 constexpr int kListers = 3;               // listing warps per CTA (17 warps would occupy the registers of 20 anyway)
 constexpr unsigned kPollLimit = 1u << 28;
-constexpr unsigned long long kZeroValue = 1ull << 55;   // (tracked values of the graph cut can be negative)
 
 // Candidates a warp of a team of T contributes to a note: a power of two, at most 16 in all.
 __host__ __device__ constexpr int entries_per_warp(int T) { return T <= 1 ? 16 : T <= 2 ? 8 : T <= 4 ? 4 : T <= 8 ? 2 : 1; }
@@ -852,7 +851,7 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
     volatile const unsigned long long *notes = reinterpret_cast<const unsigned long long *>(shared + prm.offNotes);
     volatile const unsigned long long *firsts = reinterpret_cast<const unsigned long long *>(shared + prm.offFirsts);
     const uint32_t bars = base + prm.offBars, notesAt = base + prm.offNotes;
-    unsigned long long f[KW];              // (value + kZeroValue) << 7 | block
+    unsigned long long f[KW];              // (value + kTrackedZero) << 7 | block
     int room[KW];
     uint32_t given[KW];                    // commands given to the block
     uint32_t cmdAddr[KW];
@@ -863,7 +862,7 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
 #pragma unroll
     for (int k = 0; k < KW; ++k) {
         const int p = lane + 32 * k;
-        f[k] = (kZeroValue << 7) | (unsigned long long)p;
+        f[k] = (kTrackedZero << 7) | (unsigned long long)p;
         given[k] = 0;
         room[k] = p < W ? prm.quota[(int64_t)l * W + p] : 0;
         const uint32_t owner = (uint32_t)(p < W ? p : 0) & (C - 1), slot = (uint32_t)(p < W ? p : 0) >> prm.logC;
@@ -1045,7 +1044,7 @@ __device__ void lead(const ClusterParams &prm, int l, const ClassDesc &c, unsign
         parities = (parities & ~(1u << k)) | (st & kParity ? 1u << k : 0u);
         if (p < W) {
             if (!kMany || p >> prm.logC < nTeams) command(k, kStopCmd);
-            const long long value = (long long)(f[k] >> 7) - (long long)kZeroValue;
+            const long long value = (long long)(f[k] >> 7) - (long long)kTrackedZero;
             prm.fval[(int64_t)l * W + p] = prm.fixedExp ? __double_as_longlong(ldexp((double)value, -prm.fixedExp[l])) : value;
         }
     }

@@ -157,7 +157,6 @@ constexpr int kLockWarps = 8;             // with columns, at most
 constexpr int kLockColumns = 8;           // of a thread, at most
 constexpr int kLockBlocks = 128;
 constexpr int kLockCtas = 16;
-constexpr unsigned long long kLockZero = 1ull << 55;        // (tracked values can be negative)
 
 struct LockParams {
     const ClassDesc *desc;
@@ -261,7 +260,7 @@ __global__ void __launch_bounds__((kLockWarps + 1) * 32) cut_lockstep_kernel(con
     };
 #pragma unroll
     for (int k = 0; k < KW; ++k) {                         // (every warp finds the first block; the leader goes on with these)
-        f[k] = (kLockZero << 7) | (unsigned long long)(lane + 32 * k);
+        f[k] = (kTrackedZero << 7) | (unsigned long long)(lane + 32 * k);
         room[k] = lane + 32 * k < W ? prm.quota[(int64_t)l * W + lane + 32 * k] : 0;
     }
     least = least_but(-1);
@@ -371,7 +370,7 @@ __global__ void __launch_bounds__((kLockWarps + 1) * 32) cut_lockstep_kernel(con
     if (rank == 0 && warp == NW) {
 #pragma unroll
         for (int k = 0; k < KW; ++k)
-            if (lane + 32 * k < W) prm.fval[(int64_t)l * W + lane + 32 * k] = (long long)(f[k] >> 7) - (long long)kLockZero;
+            if (lane + 32 * k < W) prm.fval[(int64_t)l * W + lane + 32 * k] = (long long)(f[k] >> 7) - (long long)kTrackedZero;
     }
     lock_barrier(alone);                                   // (and nobody writes to a CTA that has gone)
     // class-local picks -> outputs
@@ -403,7 +402,7 @@ struct LockPlan { int C, K, warps, columns; size_t smem; };
 // CTA each 1014 us, the cluster form 874).
 static bool plan_lockstep(const rcd_ctx *ctx, const Sizes &sz, LockPlan &plan)
 {
-    if (!library_chooses(ctx->cfg) || sz.W > kLockBlocks || sz.maxM == 0 || sz.maxM > 65535 || sz.floatArith) return false;
+    if (!library_chooses(ctx->cfg) || sz.W > kLockBlocks || sz.maxM == 0 || sz.maxM > 65535 || sz.floatArith || !cut_values_fit(sz.maxM, sz.d)) return false;
     if (sz.W < 6 && sz.maxM <= 8192 && (sz.L <= 64 || (sz.W < 4 && sz.maxM >= 1024))) return false;
     double best = 0;
     plan.C = 0;

@@ -235,6 +235,17 @@ inline bool sim_pairs(int64_t rowBytes, int64_t maxM, int64_t tiles, int64_t pai
     return (double)(u.whole / (sms / 2)) + last <= (double)((tiles + sms - 1) / sms);
 }
 
+// The forms that find the next block by a warp-wide minimum keep a block's value as (value + kTrackedZero) << 7 | block in 64 bits, the
+// topmost of which stays free: values have to lie below 2^55 either way.  Facility location does at any size these forms take (at most
+// 65535 samples with entries below 2^31).  The graph cut's f(A) is a sum over |A| (M - |A|) <= M^2 / 4 entries of at most 2^14 d:
+// what passes 2^55 (from 8193 samples of the largest width on, d = 131071, or 23171 of width 16384) is left to plain 64-bit integers.
+// (Within that bound the gains fit the 48 bits of a key, too: three times a row's sum of |S| either way, up to 32768 samples.)
+constexpr unsigned long long kTrackedZero = 1ull << 55;
+inline bool cut_values_fit(int64_t maxM, int64_t d)
+{
+    return (unsigned __int128)maxM * (unsigned __int128)maxM / 4 * 16384 * (unsigned __int128)d < kTrackedZero;
+}
+
 // Lays the workspace out at `base` (may be null to measure).  Returns total bytes.
 size_t layout_workspace(void *base, rcd_feat_dtype dtype, const Sizes &sz, Workspace *ws);
 

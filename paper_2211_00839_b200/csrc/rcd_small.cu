@@ -44,7 +44,6 @@ namespace {
 
 constexpr int kSmallWords = 8;            // of 32 samples at most
 constexpr int kSmallBlocks = 128;
-constexpr unsigned long long kSmallZero = 1ull << 55;   // (tracked values of the graph cut can be negative)
 
 // A class's similarities to shared memory, as they are or rounded to fixed point (as fixed_point_kernel does).
 __device__ __forceinline__ void load_similarities(int4 *to, const int4 *from, int n, bool toFix, int exponent)
@@ -213,13 +212,13 @@ __global__ void __launch_bounds__((NW + 1) * 32) greedy_small_kernel(const __gri
             }
         }
     } else {
-        unsigned long long f[KW];                          // (value + kSmallZero) << 7 | block
+        unsigned long long f[KW];                          // (value + kTrackedZero) << 7 | block
         int room[KW];
         uint32_t has[KW];                                  // blocks that are not empty
 #pragma unroll
         for (int k = 0; k < KW; ++k) {
             const int p = lane + 32 * k;
-            f[k] = (kSmallZero << 7) | (unsigned long long)p;
+            f[k] = (kTrackedZero << 7) | (unsigned long long)p;
             room[k] = p < W ? prm.quota[(int64_t)l * W + p] : 0;
             has[k] = 0;
         }
@@ -273,7 +272,7 @@ __global__ void __launch_bounds__((NW + 1) * 32) greedy_small_kernel(const __gri
 #pragma unroll
         for (int k = 0; k < KW; ++k) {
             const int p = lane + 32 * k;
-            const long long value = (long long)(f[k] >> 7) - (long long)kSmallZero;
+            const long long value = (long long)(f[k] >> 7) - (long long)kTrackedZero;
             if (p < W) prm.fval[(int64_t)l * W + p] = prm.fixedExp ? __double_as_longlong(ldexp((double)value, -exponent)) : value;
         }
         if (lane == 0) {

@@ -53,3 +53,16 @@ def test_only_where_the_library_chooses(rcd, orc):
         assert ctx.profile()["greedy_form"] == rcd.RCD_FORM_CUT_CHAIN
     ref = orc.partition(wl.features, wl.labels, wl.capacities, wl.L, variant="incremental", objective="cut")
     assert np.array_equal(a.cpu().numpy(), ref.assignment) and np.array_equal(v.cpu().numpy(), ref.part_values)
+
+
+@pytest.mark.parametrize("M,d", [(8400, 64), (14400, 131071)])
+def test_values_beyond_the_packed_word(rcd, M, d):
+    """Equal samples into two blocks: picks in index order, the blocks in turn, f = (M / 2)^2 x S.  The second class passes 3 x 2^55."""
+    import torch
+    X, y = torch.full((M, d), 127, dtype=torch.int8, device="cuda"), torch.zeros(M, dtype=torch.int32, device="cuda")
+    with rcd.Context(0, objective=rcd.RCD_OBJ_GRAPH_CUT) as ctx:
+        a, o, v = ctx.rcd_partition(X, y, [1.0, 1.0], 1, M_max=M)
+        ctx.sync_status()
+        assert ctx.profile()["greedy_form"] == (rcd.RCD_FORM_CUT_STEPS if d == 64 else rcd.RCD_FORM_CUT_CHAIN)
+    assert np.array_equal(o.cpu().numpy(), np.arange(M)) and np.array_equal(a.cpu().numpy(), np.arange(M) % 2)
+    assert v.cpu().numpy().tolist() == [[(M // 2) ** 2 * 127 * 127 * d] * 2]

@@ -57,3 +57,32 @@ def test_partition_bad_label(rcd):
         a, o, v = ctx.rcd_partition(X, y, [1.0, 1.0], 1)
         ctx.sync_status()
         assert np.bincount(a.cpu().numpy()).tolist() == [250, 250]
+
+
+def test_threads_with_lists_of_very_different_shared_memory(rcd):
+    """Two threads, a context and a stream each: one's counters take 131 KB of shared memory, the other's 51 KB."""
+    import threading
+    import torch
+    bad = []
+
+    def work(W):
+        try:
+            a = np.random.default_rng(W).integers(0, W, size=50000).astype(np.int32)
+            want = np.argsort(a, kind="stable")
+            st = torch.cuda.Stream()
+            with torch.cuda.stream(st), rcd.Context(0) as ctx:
+                t = torch.from_numpy(a).cuda()
+                for _ in range(2000):
+                    offsets, indices = rcd.rcd_worker_lists(ctx, t, W)
+                ctx.sync_status()
+                if not np.array_equal(indices.cpu().numpy(), want):
+                    bad.append(W)
+        except Exception as e:      # noqa: BLE001
+            bad.append(repr(e))
+
+    threads = [threading.Thread(target=work, args=(W,)) for W in (1024, 400)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
