@@ -1293,7 +1293,7 @@ static ClusterKernel pick_kernel(int P, int T, bool smemState)
 
 static rcd_status launch_cluster(rcd_ctx *ctx, ClusterKernel kernel, const ClusterParams &prm, int threads, int C, int clusters, size_t smem, cudaStream_t st, int *active)
 {
-    RCD_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    RCD_CUDA(ctx, allow_shared(kernel, whole_shared(ctx)));
     RCD_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(clusters * C));
@@ -1402,7 +1402,7 @@ static size_t cluster_layout(const Sizes &sz, int maxLd, int C, bool state, size
 // How a problem is laid out over clusters, if its blocks fit registers or shared memory.  resident: clusters at a time.
 static bool cluster_shape(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost, int nonEmpty, int maxLd, ClusterPlan &plan, int *resident)
 {
-    const size_t cap = (size_t)ctx->maxSmemOptin - 1024;
+    const size_t cap = (size_t)whole_shared(ctx);
     for (int i = 0; i < 5; ++i)
         if (ctx->maxClusters[i] < 0) {
             int active = 0;

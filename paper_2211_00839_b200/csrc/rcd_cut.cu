@@ -389,7 +389,6 @@ static LockKernel pick_lockstep(int K)
     return K == 1 ? cut_lockstep_kernel<1, KW> : K == 2 ? cut_lockstep_kernel<2, KW> : K == 3 ? cut_lockstep_kernel<3, KW> : K <= 4 ? cut_lockstep_kernel<4, KW> : cut_lockstep_kernel<kLockColumns, KW>;
 }
 
-// (asked for in full by every launch: contexts of several threads share the kernel)
 static size_t lock_shared(const rcd_ctx *ctx) { return (size_t)ctx->maxSmemOptin - 8192; }
 
 struct LockPlan { int C, K, warps, columns; size_t smem; };
@@ -455,7 +454,7 @@ static rcd_status run_lockstep(rcd_ctx *ctx, const LockPlan &plan, const Sizes &
     prm.columns = plan.columns;
     prm.one = 1u;
     const LockKernel kernel = sz.W <= 32 ? pick_lockstep<1>(plan.K) : sz.W <= 64 ? pick_lockstep<2>(plan.K) : pick_lockstep<4>(plan.K);
-    RCD_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lock_shared(ctx)));
+    RCD_CUDA(ctx, allow_shared(kernel, (int64_t)lock_shared(ctx)));
     RCD_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(sz.L * plan.C));
@@ -593,9 +592,9 @@ static rcd_status run_cut_objective(rcd_ctx *ctx, const Sizes &sz, const ClassDe
     using FV = typename CutArith<SV>::FV;
     const int maxBlocks = (int)((sz.maxM + 63) / 64);
     const size_t smem = (size_t)16 * sz.W * 8;
-    if ((int64_t)smem > ctx->maxSmemOptin - 1024) return fail(ctx, RCD_ERR_UNSUPPORTED, "W=%d too large for the cut objective kernel", sz.W);
+    if ((int64_t)smem > whole_shared(ctx)) return fail(ctx, RCD_ERR_UNSUPPORTED, "W=%d too large for the cut objective kernel", sz.W);
     if (sz.L > 65535) return fail(ctx, RCD_ERR_UNSUPPORTED, "objective: more than 65535 classes");
-    RCD_CUDA(ctx, cudaFuncSetAttribute(cut_objective_rows_kernel<SV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    RCD_CUDA(ctx, allow_shared(cut_objective_rows_kernel<SV>, whole_shared(ctx)));
     if (maxBlocks > 0) {
         dim3 grid(maxBlocks, sz.L);
         cut_objective_rows_kernel<SV><<<grid, 256, smem, st>>>(descDev, (const SV *)S, perm, assignment, sz.W, maxBlocks, (FV *)scratch);

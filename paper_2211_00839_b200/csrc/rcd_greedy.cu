@@ -2529,7 +2529,7 @@ static rcd_status run_greedy(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws,
         if (it > 1 << 20) it = 1 << 20;
         prm.segIters = (int32_t)it;
     }
-    RCD_CUDA(ctx, cudaFuncSetAttribute(sweep_kernel<SV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    RCD_CUDA(ctx, allow_shared(sweep_kernel<SV>, smemCap));
 
     // Which form of the loop: greedy_path 1 = two launches per round, 2 = one launch, rounds with grid
     // barriers, 3 = one launch, asynchronous classes, 0 = choose.  With few classes the pick phases of
@@ -2550,17 +2550,17 @@ static rcd_status run_greedy(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws,
         // one cooperative launch needs one CTA per SM resident at once
         int perSm = 0;
         if (path == 3) {
-            RCD_CUDA(ctx, cudaFuncSetAttribute(asyncKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            RCD_CUDA(ctx, allow_shared(asyncKernel, smemCap));
             RCD_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&perSm, asyncKernel, kSweepThreads, (size_t)smem));
         } else {
-            RCD_CUDA(ctx, cudaFuncSetAttribute(greedy_persistent_kernel<SV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            RCD_CUDA(ctx, allow_shared(greedy_persistent_kernel<SV>, smemCap));
             RCD_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&perSm, greedy_persistent_kernel<SV>, kSweepThreads, (size_t)smem));
         }
         if (perSm < 1) path = only ? 4 : 1;
     }
     if (!only) ctx->greedyForm = path;
     if (path == 4) {
-        RCD_CUDA(ctx, cudaFuncSetAttribute(ownerKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        RCD_CUDA(ctx, allow_shared(ownerKernel, smemCap));
         // (in-place correction of stored gains: a class's passes are made by one SM here, so their cost grows with the
         // square of the class size while a correction reads a few dozen rows; measured: it wins on 1300-sample classes
         // with 64 blocks (208 -> 183 ms) and loses on 500-sample classes with 32 (3.9 -> 5.0 ms))

@@ -20,7 +20,10 @@ namespace rcd {
 // 1155 -> 40 us, 27 in two launches).  More labels than that take the kernels at the end of this section.
 constexpr int kGroupThreads = 256;
 constexpr int kGroupWarps = kGroupThreads / 32;
-static_assert(kGroupWarps * kMaxSharedLabels * 4 <= 192 * 1024, "counters in shared memory");
+// (histogram: a counter per label.  Placement: one per warp and label, with 32 warps up to 1024 labels (GroupShape), the labels' starts, and
+// with rows the positions of up to 1024 samples)
+static_assert(kMaxSharedLabels * 4 <= 48 * 1024, "a histogram's counters in the shared memory that every launch has");
+static_assert((kGroupWarps + 1) * kMaxSharedLabels * 4 + 1024 * 4 <= 226 * 1024 && 33 * 1024 * 4 <= 226 * 1024, "counters in shared memory");
 
 __global__ void __launch_bounds__(kGroupThreads) label_hist_kernel(const int32_t *__restrict__ labels, int64_t N, int32_t L, int32_t chunk,
                                                                   int32_t *__restrict__ chunkHist, int32_t *__restrict__ counts,
@@ -430,7 +433,6 @@ rcd_status launch_label_hist(rcd_ctx *ctx, const int32_t *labels, int64_t N, int
     const unsigned nChunks = (unsigned)((N + chunk - 1) / chunk);
     if (shared_labels(L)) {
         const size_t smem = (size_t)L * 4;
-        if (smem > 48 * 1024) RCD_CUDA(ctx, cudaFuncSetAttribute(label_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         label_hist_kernel<<<nChunks, kGroupThreads, smem, st>>>(labels, N, L, chunk, chunkHist, counts, status, callStatus);
         ctx->kernelLaunches++;
     } else {
@@ -473,7 +475,7 @@ rcd_status launch_stable_split(rcd_ctx *ctx, const int32_t *labels, int64_t N, i
     }
     if (shared_labels(L)) {
         const size_t smem = ((size_t)shape.threads / 32 * L + (Xs ? chunk : 0) + (few ? L : 0)) * 4;
-        if (smem > 48 * 1024) RCD_CUDA(ctx, cudaFuncSetAttribute(label_place_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        if (smem > 48 * 1024) RCD_CUDA(ctx, allow_shared(label_place_kernel, whole_shared(ctx)));
         // (few samples: several CTAs rank the same chunk and share its rows out, so that wide rows occupy more than a few SMs)
         const dim3 grid(nChunks, Xs ? std::max(1, std::min(16, 2 * ctx->smCount / nChunks)) : 1);
         label_place_kernel<<<grid, shape.threads, smem, st>>>(labels, N, L, chunk, chunkHist, perm, (const uint8_t *)X, rowBytes, pitch,

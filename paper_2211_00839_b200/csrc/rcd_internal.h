@@ -304,6 +304,17 @@ rcd_status cuda_fail(rcd_ctx *ctx, cudaError_t e, const char *what);
         if (e__ != cudaSuccess) return ::rcd::cuda_fail(ctx, e__, #call); \
     } while (0)
 
+// Lets a kernel's launches take up to `most` bytes of dynamic shared memory: the most that any call may ask of it, which depends on the
+// device alone.  The limit belongs to the function and so to all contexts and threads of the process: set to a call's own size, it can be
+// lowered by another thread between this one's setting and its launch, which is then refused (lists for 1024 and 400 workers did that).
+template <typename Kernel>
+inline cudaError_t allow_shared(Kernel *kernel, int64_t most)
+{
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+// What a CTA with at most 1 KB of variables of its own in shared memory can be given besides.
+inline int64_t whole_shared(const rcd_ctx *ctx) { return (int64_t)ctx->maxSmemOptin - 1024; }
+
 // ---- launchers implemented in the .cu files (all asynchronous on `st`) ----
 
 // class split

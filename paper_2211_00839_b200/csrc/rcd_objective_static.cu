@@ -129,9 +129,9 @@ static rcd_status run_static(rcd_ctx *ctx, const void *S, int M, int ld, const i
 {
     const int nBlocks = (M + kStaticRowsPerCta - 1) / kStaticRowsPerCta;
     const size_t smem = (size_t)kStaticWarps * W * (sizeof(FV) + sizeof(int32_t));
-    if ((int64_t)smem > ctx->maxSmemOptin - 1024)
+    if ((int64_t)smem > whole_shared(ctx))
         return fail(ctx, RCD_ERR_UNSUPPORTED, "W=%d needs %zu bytes of shared memory", W, smem);
-    RCD_CUDA(ctx, cudaFuncSetAttribute(objective_class_rows_kernel<SV, FV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    RCD_CUDA(ctx, allow_shared(objective_class_rows_kernel<SV, FV>, whole_shared(ctx)));
     if (nBlocks > 0)
         objective_class_rows_kernel<SV, FV><<<nBlocks, kStaticWarps * 32, smem, st>>>((const SV *)S, M, ld, assignment, W, (FV *)scratch);
     objective_class_finish_kernel<FV><<<1, 256, 0, st>>>((const FV *)scratch, nBlocks, W, (FV *)partValues, (FV *)total);

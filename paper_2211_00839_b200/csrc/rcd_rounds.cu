@@ -61,6 +61,7 @@ constexpr int kStages = 3;                // of the ring of tiles
 constexpr int kGroup = 4;                 // blocks per warp of a tile
 constexpr int kMaxWarps = 16;             // of a CTA; blocks corrected together: kGroup each
 constexpr int kRoundBlocks = 128;
+constexpr int kRoundsOwnShared = 3072;     // bytes of shared memory the kernel's own variables take, at most
 constexpr unsigned kCopyLimit = 1u << 22; // looks at a stage's barrier, 64 ns apart, before the copies count as lost: a quarter of a second
 
 struct Pending { int32_t block, sample, first; };   // a pick whose correction is outstanding; first: its block was empty
@@ -795,8 +796,8 @@ static bool rounds_plan(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDe
     const int blocks = (std::min(sz.W, batch) + kGroup - 1) / kGroup * kGroup;
     if (prm.scratchBytes < perBlock * kGroup) return false;
     prm.scratchBytes = std::min<int64_t>(prm.scratchBytes, (perBlock * blocks + 255) / 256 * 256);
-    // (1 KB per CTA is the system's, and the kernel's own variables take less than 3)
-    const size_t cap = ((size_t)ctx->maxSmemOptin + 1024) / perSm - 1024 - 3072, words = (size_t)(pad_row(sz.maxM) + 31) / 32;
+    // (1 KB per CTA is the system's)
+    const size_t cap = ((size_t)ctx->maxSmemOptin + 1024) / perSm - 1024 - kRoundsOwnShared, words = (size_t)(pad_row(sz.maxM) + 31) / 32;
     size_t off = 0;
     auto take = [&](size_t bytes) { const size_t at = off; off = (off + bytes + 127) / 128 * 128; return (int32_t)at; };
     prm.offKeys = take((size_t)(sz.W + 1) * kListed * 8);
@@ -870,7 +871,7 @@ rcd_status launch_greedy_rounds(rcd_ctx *ctx, RoundsPlan &plan, const Sizes &sz,
     prm.one = 1u;
     auto kernel = plan.warps == 8 ? (sz.W <= 32 ? greedy_rounds_kernel<1, 8> : sz.W <= 64 ? greedy_rounds_kernel<2, 8> : greedy_rounds_kernel<4, 8>)
                                   : (sz.W <= 32 ? greedy_rounds_kernel<1, 16> : sz.W <= 64 ? greedy_rounds_kernel<2, 16> : greedy_rounds_kernel<4, 16>);
-    RCD_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem));
+    RCD_CUDA(ctx, allow_shared(kernel, ctx->maxSmemOptin - kRoundsOwnShared));
     kernel<<<plan.ctas, plan.warps * 32, plan.smem, st>>>(prm);
     RCD_CUDA(ctx, cudaGetLastError());
     ctx->kernelLaunches++;

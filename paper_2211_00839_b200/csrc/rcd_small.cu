@@ -312,9 +312,6 @@ static SmallKernel pick_small(int words, int W)
 
 }  // namespace
 
-// (asked for in full by every launch: contexts of several threads share the kernel)
-static size_t small_shared(const rcd_ctx *ctx) { return (size_t)ctx->maxSmemOptin - 1024; }
-
 struct SmallPlan {
     int words;
     size_t smem;
@@ -335,7 +332,7 @@ std::shared_ptr<SmallPlan> plan_greedy_small(rcd_ctx *ctx, const Sizes &sz)
     prm.offList = take(sz.graphCut ? 0 : ((size_t)plan.words * 32 + 8) * 16);
     prm.offPicks = take((size_t)sz.maxM * 4);
     plan.smem = off;
-    if (off > small_shared(ctx)) return nullptr;
+    if (off > (size_t)whole_shared(ctx)) return nullptr;
     return std::make_shared<SmallPlan>(plan);
 }
 
@@ -358,7 +355,7 @@ rcd_status launch_greedy_small(rcd_ctx *ctx, SmallPlan &plan, const Sizes &sz, c
     prm.toFix = toFix ? 1 : 0;
     prm.one = 1u;
     const SmallKernel kernel = sz.graphCut ? pick_small<true>(plan.words, sz.W) : pick_small<false>(plan.words, sz.W);
-    RCD_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)small_shared(ctx)));
+    RCD_CUDA(ctx, allow_shared(kernel, whole_shared(ctx)));
     kernel<<<sz.L, (plan.words + 1) * 32, plan.smem, st>>>(prm);
     RCD_CUDA(ctx, cudaGetLastError());
     ctx->kernelLaunches++;
