@@ -186,7 +186,9 @@ RCD_API const char *rcd_version(void);
 
 /* Waits for `cuda_stream` and returns the device-side status of the last call on the context. */
 RCD_API rcd_status rcd_sync_status(rcd_ctx *ctx, void *cuda_stream);
-/* Self-test of the bounded waits the kernels use: enqueues a one-CTA kernel that arrives at a grid barrier expecting two
+/* Self-test of the bounded waits the kernels use.  First the greedy loops that write their outputs last get a class whose
+ * quotas end before its samples: they have to record that and to write no outputs (RCD_ERR_INTERNAL otherwise; waits for
+ * the stream).  Then it enqueues a one-CTA kernel that arrives at a grid barrier expecting two
  * arrivals, and one whose threads wait for copies that nobody makes (the loop in rounds: all have to leave at the same
  * step).  The waits give up after a few thousand polls and record the timeout in the context's status word, so the next
  * rcd_sync_status returns RCD_ERR_TIMEOUT (RCD_ERR_INTERNAL if the threads did not leave together) and the context

@@ -243,6 +243,64 @@ struct Prepared {
     std::shared_ptr<ClusterPlan> cluster;   // null: another form of the greedy loop, or none
 };
 
+// A class whose quotas leave off before its samples do, as no call's can: the greedy loops that hand their picks over in memory have to
+// say so and to write none of them out: behind the last one is whatever that memory held.  Here that names a sample of the class and a
+// block, so that a loop that went on would do no harm.
+static rcd_status selftest_stopped(rcd_ctx *ctx, bool graphCut, cudaStream_t st)
+{
+    constexpr int M = 300;
+    Sizes sz{};
+    sz.N = sz.maxM = M; sz.d = 16; sz.L = 1; sz.W = 8; sz.graphCut = graphCut;
+    sz.sElems = (int64_t)M * pad_row(M); sz.vElems = (int64_t)sz.W * pad_row(M);
+    sz.nChunks = 2;
+    sz.pitch = 128;
+    const std::vector<ClassDesc> desc{ClassDesc{M, pad_row(M), 0, 0, 0, 0}};
+    const auto cluster = graphCut ? nullptr : plan_greedy_cluster(ctx, sz, desc);
+    if (!graphCut && !cluster) return RCD_OK;              // (a context with options of the other forms)
+    const size_t bytes = layout_workspace(nullptr, RCD_FEAT_I8, sz, nullptr);
+    std::vector<unsigned char> host(bytes + 2 * M * sizeof(int32_t), 0);
+    unsigned char *dev = nullptr;
+    RCD_CUDA(ctx, cudaMalloc((void **)&dev, host.size()));
+    Workspace ws{};
+    layout_workspace(dev, RCD_FEAT_I8, sz, &ws);
+    auto at = [&](void *p) { return (int32_t *)(host.data() + ((unsigned char *)p - dev)); };
+    memcpy(at(ws.desc), desc.data(), sizeof(ClassDesc));
+    std::fill(at(ws.S), at(ws.S) + sz.sElems, 1);
+    at(ws.quota)[2] = 10;
+    at(ws.quota)[5] = 5;
+    for (int i = 0; i < M; ++i) {
+        at(ws.perm)[i] = i;
+        at(ws.cand)[i] = M - 1 | 7 << 16;
+    }
+    int32_t *const assignment = (int32_t *)(dev + bytes), *const order = assignment + M;
+    std::fill(at(assignment), at(assignment) + 2 * M, -1);
+    // (what a profile reads belongs to the last partition)
+    const int64_t steps = ctx->steps;
+    const int form = ctx->greedyForm;
+    const auto phases = ctx->phaseNsDev;
+    int32_t word = 0;
+    auto run = [&]() -> rcd_status {
+        RCD_CUDA(ctx, cudaMemcpyAsync(dev, host.data(), host.size(), cudaMemcpyHostToDevice, st));
+        const rcd_status rs = graphCut ? launch_cut_stopped_selftest(ctx, sz, ws, assignment, order, st)
+                                       : launch_greedy_cluster(ctx, *cluster, sz, ws, desc, assignment, order, nullptr, st);
+        if (rs != RCD_OK) return rs;
+        RCD_CUDA(ctx, cudaMemcpyAsync(at(assignment), assignment, 2 * M * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+        RCD_CUDA(ctx, cudaMemcpyAsync(&word, ctx->statusOwn, sizeof word, cudaMemcpyDeviceToHost, st));
+        RCD_CUDA(ctx, cudaMemsetAsync(ctx->statusOwn, 0, sizeof(int32_t), st));
+        RCD_CUDA(ctx, cudaStreamSynchronize(st));
+        return RCD_OK;
+    };
+    const rcd_status rs = run();
+    ctx->steps = steps;
+    ctx->greedyForm = form;
+    ctx->phaseNsDev = phases;
+    cudaFree(dev);
+    if (rs != RCD_OK) return rs;
+    bool right = word == kDevNoCandidate;
+    for (int i = 0; i < 2 * M; ++i) right = right && at(assignment)[i] == -1;
+    return right ? RCD_OK : fail(ctx, RCD_ERR_INTERNAL, "a greedy loop that stopped early wrote outputs");
+}
+
 // capacities null: no quotas wanted.  blocks not null: the value of this assignment is wanted, and where S need not exist for that
 // (`covered`) the blocks' coverage is computed in its place.
 static rcd_status prepare(rcd_ctx *ctx, const void *features, rcd_feat_dtype dtype, int64_t N, int64_t d,
@@ -486,7 +544,10 @@ rcd_status rcd_selftest_bounded_wait(rcd_ctx *ctx, void *cuda_stream)
     RCD_CUDA(ctx, cudaSetDevice(ctx->device));
     RCD_CUDA(ctx, cudaMemsetAsync(ctx->statusOwn, 0, 64, st));
     ctx->statusDev = ctx->statusOwn;
-    const rcd_status rs = launch_bounded_wait_selftest(ctx, (unsigned *)(ctx->statusOwn + 8), ctx->statusOwn, st);
+    rcd_status rs = selftest_stopped(ctx, true, st);
+    if (rs == RCD_OK) rs = selftest_stopped(ctx, false, st);
+    if (rs != RCD_OK) return rs;
+    rs = launch_bounded_wait_selftest(ctx, (unsigned *)(ctx->statusOwn + 8), ctx->statusOwn, st);
     return rs == RCD_OK ? launch_step_wait_selftest(ctx, ctx->statusOwn, st) : rs;
 }
 

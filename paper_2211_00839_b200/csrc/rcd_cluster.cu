@@ -1197,9 +1197,11 @@ __global__ void __launch_bounds__((P == 0 ? kMaxWarps + 1 + kListers : team_warp
             }
         }
         cluster_barrier();
-        // class-local picks -> outputs
+        // class-local picks -> outputs (none where the loop stopped early: the words behind the last pick are whatever memory held)
+        const bool stopped = __ldcg(prm.status) != 0;
         for (int t = rank * blockDim.x + threadIdx.x; t < c.M; t += C * blockDim.x) {
             const uint32_t p = __ldcg(prm.picks + c.row0 + t);
+            if (stopped) break;
             const int global = prm.perm[c.row0 + (p & 0xffff)];
             prm.assignment[global] = (int)(p >> 16);
             if (prm.order) prm.order[c.row0 + t] = global;

@@ -373,9 +373,11 @@ __global__ void __launch_bounds__((kLockWarps + 1) * 32) cut_lockstep_kernel(con
             if (lane + 32 * k < W) prm.fval[(int64_t)l * W + lane + 32 * k] = (long long)(f[k] >> 7) - (long long)kTrackedZero;
     }
     lock_barrier(alone);                                   // (and nobody writes to a CTA that has gone)
-    // class-local picks -> outputs
+    // class-local picks -> outputs (none where the loop stopped early: the words behind the last pick are whatever memory held)
+    const bool stopped = __ldcg(prm.status) != 0;
     for (int t = (int)(rank * blockDim.x + threadIdx.x); t < M; t += (int)(C * blockDim.x)) {
         const uint32_t p = __ldcg(prm.picks + c.row0 + t);
+        if (stopped) break;
         const int global = prm.perm[c.row0 + (p & 0xffff)];
         prm.assignment[global] = (int)(p >> 16);
         if (prm.order) prm.order[c.row0 + t] = global;
@@ -470,6 +472,13 @@ static rcd_status run_lockstep(rcd_ctx *ctx, const LockPlan &plan, const Sizes &
     RCD_CUDA(ctx, cudaLaunchKernelEx(&cfg, kernel, prm));
     ctx->kernelLaunches++;
     return RCD_OK;
+}
+
+rcd_status launch_cut_stopped_selftest(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, int32_t *assignment, int32_t *order, cudaStream_t st)
+{
+    const int words = (int)(sz.maxM + 63) / 64;                          // of 32 columns, of each of two CTAs
+    const LockPlan plan{2, 1, std::min(kLockWarps, words), words * 32, (size_t)sz.W * words * 32 * 8};
+    return run_lockstep(ctx, plan, sz, ws, assignment, order, st);
 }
 
 // f(A_p) for every block from the definition: per row v the sums r_p(v) = sum_{a in A_p} S[v][a], then

@@ -379,7 +379,8 @@ rcd_status launch_greedy_small(rcd_ctx *ctx, SmallPlan &plan, const Sizes &sz, c
 rcd_status launch_bounded_wait_selftest(rcd_ctx *ctx, unsigned *counter, int32_t *status, cudaStream_t st);
 rcd_status launch_step_wait_selftest(rcd_ctx *ctx, int32_t *status, cudaStream_t st);
 
-// graph-cut objective: the whole greedy loop, and f from an assignment
+// graph-cut objective: the whole greedy loop, and f from an assignment (selftest: in step, on two CTAs, whatever the plan says)
+rcd_status launch_cut_stopped_selftest(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, int32_t *assignment, int32_t *order, cudaStream_t st);
 // (in step: integers, where that is faster than the cluster form)
 bool cut_in_step(const rcd_ctx *ctx, const Sizes &sz);
 rcd_status launch_cut(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, int32_t *assignment, int32_t *order, cudaStream_t st);

@@ -66,3 +66,13 @@ def test_values_beyond_the_packed_word(rcd, M, d):
         assert ctx.profile()["greedy_form"] == (rcd.RCD_FORM_CUT_STEPS if d == 64 else rcd.RCD_FORM_CUT_CHAIN)
     assert np.array_equal(o.cpu().numpy(), np.arange(M)) and np.array_equal(a.cpu().numpy(), np.arange(M) % 2)
     assert v.cpu().numpy().tolist() == [[(M // 2) ** 2 * 127 * 127 * d] * 2]
+
+
+def test_no_outputs_where_the_loop_stops_early(rcd):
+    """A class whose quotas end before its samples: the loop in step and the cluster form stop, say so, and leave the outputs alone
+    (the self-test fails with its own status where they do not)."""
+    with rcd.Context(0, objective=rcd.RCD_OBJ_GRAPH_CUT) as ctx:
+        ctx.selftest_bounded_wait()
+        with pytest.raises(rcd.RcdError) as e:
+            ctx.sync_status()
+        assert e.value.status == 5          # RCD_ERR_TIMEOUT, of the waits that follow
