@@ -230,7 +230,13 @@ __device__ __forceinline__ unsigned same_label(int lab, int bits)
     return same;
 }
 
-__global__ void __launch_bounds__(1024) label_place_kernel(const int32_t *__restrict__ labels, int64_t N, int32_t L, int32_t chunk,
+// kFew: no launch of label_scan_kernel before; chunkBase holds the chunks' own numbers, and every CTA adds up those before its own (null
+// desc: counts says where the labels begin).  The number of threads and kFew are fixed at compile time, and five CTAs of 256 have to fit an
+// SM: rows are copied by as many warps as there are.  One kernel for all of them, bounded by 1024 threads, took 64 registers instead of 48,
+// and the split of 1.3 million rows of 2 KB over 1000 labels 1085 us (now 940), that of 81920 rows of 130 bytes over 4096 labels 186 (160),
+// lists of 1.3 million samples over 5000 workers 156 (124).  (A run of 256 threads' samples has four per lane: counted all at once.)
+template <int kThreads, bool kFew>
+__global__ void __launch_bounds__(kThreads, kThreads == 1024 ? 1 : 5) label_place_kernel(const int32_t *__restrict__ labels, int64_t N, int32_t L, int32_t chunk,
                                                                    const int32_t *__restrict__ chunkBase, int32_t *__restrict__ perm,
                                                                    const uint8_t *__restrict__ X, int64_t rowBytes, int64_t pitch,
                                                                    uint8_t *__restrict__ Xs, const int32_t *__restrict__ status,
@@ -238,9 +244,8 @@ __global__ void __launch_bounds__(1024) label_place_kernel(const int32_t *__rest
 {
     extern __shared__ int32_t shWarp[];                 // [warps][L] counters, then [chunk] positions
     if (status && (*status & kDevBadLabel)) return;
-    // (no launch of label_scan_kernel before: chunkBase holds the chunks' own numbers, and every CTA adds up those before its own)
-    const bool few = desc || counts;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    constexpr int warps = kThreads / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int32_t *mine = shWarp + (size_t)warp * L;
     int32_t *shPos = shWarp + (size_t)warps * L;
     const int64_t base = (int64_t)blockIdx.x * chunk;
@@ -249,11 +254,11 @@ __global__ void __launch_bounds__(1024) label_place_kernel(const int32_t *__rest
     for (int l = lane; l < L; l += 32) mine[l] = 0;
     __syncwarp();
     const int i0 = warp * per, i1 = min(n, i0 + per);
-#pragma unroll 8
+#pragma unroll (kThreads == 1024 ? 8 : 4)
     for (int i = i0 + lane; i < i1; i += 32) atomicAdd(&mine[labels[base + i]], 1);
     __syncthreads();
-    int32_t *const shStart = shWarp + (size_t)warps * L + (Xs ? chunk : 0);      // [L] where a label begins (few), then where the chunk's part of it does
-    if (few && !desc) {
+    int32_t *const shStart = shWarp + (size_t)warps * L + (Xs ? chunk : 0);      // [L] where a label begins (kFew), then where the chunk's part of it does
+    if (kFew && !desc) {
         if (warp == 0) {
             int32_t run = 0;
             for (int l0 = 0; l0 < L; l0 += 32) {
@@ -273,16 +278,16 @@ __global__ void __launch_bounds__(1024) label_place_kernel(const int32_t *__rest
         }
         __syncthreads();
     }
-    if (few) {
+    if (kFew) {
         if (desc) {
-            for (int l = threadIdx.x; l < L; l += blockDim.x) shStart[l] = desc[l].row0;
+            for (int l = threadIdx.x; l < L; l += kThreads) shStart[l] = desc[l].row0;
             __syncthreads();
         }
         add_chunks(chunkBase, (int)blockIdx.x, L, shStart);
         __syncthreads();
     }
-    for (int l = threadIdx.x; l < L; l += blockDim.x) {
-        int32_t run = few ? shStart[l] : chunkBase[(int64_t)blockIdx.x * L + l];
+    for (int l = threadIdx.x; l < L; l += kThreads) {
+        int32_t run = kFew ? shStart[l] : chunkBase[(int64_t)blockIdx.x * L + l];
         for (int w = 0; w < warps; ++w) {
             const int32_t c = shWarp[(size_t)w * L + l];
             shWarp[(size_t)w * L + l] = run;
@@ -475,11 +480,13 @@ rcd_status launch_stable_split(rcd_ctx *ctx, const int32_t *labels, int64_t N, i
     }
     if (shared_labels(L)) {
         const size_t smem = ((size_t)shape.threads / 32 * L + (Xs ? chunk : 0) + (few ? L : 0)) * 4;
-        if (smem > 48 * 1024) RCD_CUDA(ctx, allow_shared(label_place_kernel, whole_shared(ctx)));
+        auto *const kernel = shape.threads == 1024 ? (few ? label_place_kernel<1024, true> : label_place_kernel<1024, false>)
+                                                   : (few ? label_place_kernel<kGroupThreads, true> : label_place_kernel<kGroupThreads, false>);
+        if (smem > 48 * 1024) RCD_CUDA(ctx, allow_shared(kernel, whole_shared(ctx)));
         // (few samples: several CTAs rank the same chunk and share its rows out, so that wide rows occupy more than a few SMs)
         const dim3 grid(nChunks, Xs ? std::max(1, std::min(16, 2 * ctx->smCount / nChunks)) : 1);
-        label_place_kernel<<<grid, shape.threads, smem, st>>>(labels, N, L, chunk, chunkHist, perm, (const uint8_t *)X, rowBytes, pitch,
-                                                                (uint8_t *)Xs, status, few ? descDev : nullptr, few && !descDev ? counts : nullptr, few ? offsets : nullptr);
+        kernel<<<grid, shape.threads, smem, st>>>(labels, N, L, chunk, chunkHist, perm, (const uint8_t *)X, rowBytes, pitch, (uint8_t *)Xs, status,
+                                                  descDev, counts, few ? offsets : nullptr);
         ctx->kernelLaunches++;
     } else {
         chunk_rank_kernel<false><<<nChunks, 1024, 0, st>>>(labels, N, L, chunk, chunkHist, perm, status);
