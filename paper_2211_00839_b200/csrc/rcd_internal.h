@@ -174,7 +174,10 @@ inline int group_chunk(int64_t N, int64_t labels) { return N <= 131072 && (N + 2
 // saves a memset, the launch of a scan and a copy.  With rows to gather (rows) up to 32 chunks and 4096 numbers (2 classes of 200: 148 -> 138
 // us the whole call, 4 of 20 52 -> 40; with 9600 numbers, 300 classes of 27, the additions take longer than the scan, 79 us against 70).
 // Lists alone have no rows to share out: their chunks are as large as gives an SM one, up to 16384 samples (1.3 million over 64 workers:
-// 41 us with 1024 samples per chunk and a scan, 27 so; 80 samples 26 -> 20).
+// 41 us with 1024 samples per chunk and a scan, 27 so; 80 samples 26 -> 20), and every CTA adds up where there are up to 1024 labels and
+// 16384 numbers, with small chunks 8192: one warp finds where the labels begin (100 samples over 1024 labels 28 us, with the scan 32; over
+// 2000 31 and 29, over 5000 63 and 31), and small CTAs take longer to add (4000 samples over 500 labels, 8000 numbers, 25.6 us, with the scan
+// 27.8; over 1000 35 and 29; 20000 over 100 26.6 and 27.8, over 200 28.8 and 27.7).
 struct GroupShape { int chunk, threads; bool few; };
 inline GroupShape group_shape(int64_t N, int64_t labels, bool rows)
 {
@@ -184,7 +187,8 @@ inline GroupShape group_shape(int64_t N, int64_t labels, bool rows)
         g.threads = 1024;
     }
     const int64_t chunks = (N + g.chunk - 1) / g.chunk;
-    g.few = N > 0 && labels <= kMaxSharedLabels && (rows ? chunks <= 32 && chunks * labels <= 4096 : chunks <= 144 && chunks * labels <= 16384);
+    g.few = N > 0 && labels <= kMaxSharedLabels && (rows ? chunks <= 32 && chunks * labels <= 4096
+                                                                : chunks <= 144 && labels <= 1024 && chunks * labels <= (g.threads == 1024 ? 16384 : 8192));
     return g;
 }
 // Bytes between the class-sorted feature rows: whole 16-byte pieces, at least one 128-byte slab, so that every width can

@@ -25,6 +25,12 @@ def test_lists(rcd, N, W):
         assert np.array_equal(indices.cpu().numpy(), np.argsort(a, kind="stable"))
 
 
+@pytest.mark.parametrize("N,W", [(2048, 1024), (2049, 1024), (4096, 512), (4097, 512), (8192, 256), (8200, 257), (45056, 372), (45057, 372), (300, 6000), (5000, 2048)])
+def test_lists_of_many_workers(rcd, N, W):
+    """On either side of 8192 numbers of small chunks, of 16384 of large ones, and of 1024 workers."""
+    test_lists(rcd, N, W)
+
+
 @pytest.mark.parametrize("N,W,at", [(300, 4, 299), (50000, 64, 0), (1000000, 64, 123456)])
 def test_lists_bad_entry(rcd, N, W, at):
     """An entry out of range is refused, and the next call is not disturbed."""
