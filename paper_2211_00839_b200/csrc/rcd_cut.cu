@@ -7,11 +7,11 @@
 // costs O(M) per pick.  Values: int64 for int8 features (exact), double otherwise.
 // The objective is not monotone (a sample that joins A stops being cut), gains may be negative;
 // Algorithm 1 runs unchanged: least-f non-full block, argmax with lowest-index ties.
+#include "rcd_cut_plan.h"
 #include "rcd_exact.cuh"
 
 #include <limits.h>
 #include <algorithm>
-#include <cmath>
 #include <type_traits>
 
 namespace rcd {
@@ -153,11 +153,6 @@ __global__ void __launch_bounds__(kCutThreads, 2) cut_chain_kernel(CutParams<SV>
 // What bounds it (10 classes of 5000 into 8 blocks, 8 CTAs each, 2700 cycles a pick): instructions of one warp after another, half of them
 // for the candidates and the row's loads.  Whole calls, before and now: 3 classes of 1300 into 20 blocks 2103 and 1120 us, 30 of 2500 into 8
 // blocks 5060 and 3644, 200 of 700 into 8 blocks 2886 and 1247.
-constexpr int kLockWarps = 8;             // with columns, at most
-constexpr int kLockColumns = 8;           // of a thread, at most
-constexpr int kLockBlocks = 128;
-constexpr int kLockCtas = 16;
-
 struct LockParams {
     const ClassDesc *desc;
     const int32_t *S;
@@ -391,47 +386,63 @@ static LockKernel pick_lockstep(int K)
     return K == 1 ? cut_lockstep_kernel<1, KW> : K == 2 ? cut_lockstep_kernel<2, KW> : K == 3 ? cut_lockstep_kernel<3, KW> : K <= 4 ? cut_lockstep_kernel<4, KW> : cut_lockstep_kernel<kLockColumns, KW>;
 }
 
-static size_t lock_shared(const rcd_ctx *ctx) { return (size_t)ctx->maxSmemOptin - 8192; }
-
-struct LockPlan { int C, K, warps, columns; size_t smem; };
-
-// Whether the classes run in step, and on how many CTAs each: those with which they are through soonest.  A pick takes 1600 cycles with one
-// CTA, 1700 with several, and 260 more for every column of a thread (measured on 250 to 5000 samples); clusters keep within a GPC.
-// Not with few blocks and classes, whose picks wait for the sample's row, while the cluster form foresees it (3 or 30 classes of 700 to
-// 2500: 0.6 to 0.9 times as fast with 2 and 4 blocks, 1.0 to 1.7 times with 8, 1.1 to 2.7 with more; 200 classes: 1.2 to 3 times, but 0.96
-// for 1300 samples into 2 blocks), and not where short classes come one to an SM and have to come again (200 of 400 into 50 blocks in one
-// CTA each 1014 us, the cluster form 874).
-static bool plan_lockstep(const rcd_ctx *ctx, const Sizes &sz, LockPlan &plan)
+static LockKernel lock_kernel(const Sizes &sz, const LockPlan &plan)
 {
-    if (!library_chooses(ctx->cfg) || sz.W > kLockBlocks || sz.maxM == 0 || sz.maxM > 65535 || sz.floatArith || !cut_values_fit(sz.maxM, sz.d)) return false;
-    if (sz.W < 6 && sz.maxM <= 8192 && (sz.L <= 64 || (sz.W < 4 && sz.maxM >= 1024))) return false;
-    double best = 0;
-    plan.C = 0;
-    bool again = false;
-    for (int C = 1; C <= kLockCtas; C *= 2) {
-        LockPlan p;
-        p.C = C;
-        const int share = (int)((sz.maxM + C - 1) / C), words = (share + 31) / 32;
-        p.K = (words + kLockWarps - 1) / kLockWarps;
-        if (p.K > 4) p.K = kLockColumns;
-        p.warps = std::min(kLockWarps, (words + p.K - 1) / p.K);
-        p.columns = words * 32;
-        p.smem = (size_t)sz.W * p.columns * 8;
-        if (words > kLockWarps * kLockColumns || p.smem > lock_shared(ctx) || (C > 1 && share < 128)) continue;
-        const int perSm = (int)std::max<size_t>(1, std::min<size_t>(6, (size_t)ctx->maxSmemOptin / (p.smem + 4096)));
-        const double resident = C == 1 ? (double)ctx->smCount * perSm : C == 16 ? (double)(ctx->smCount / 20) : std::floor(0.9 * ctx->smCount / C);
-        const double turns = std::max(1.0, std::ceil(sz.L / resident - 1e-9));
-        const double time = turns * ((C == 1 ? 1570.0 : 1700.0) + 260.0 * p.K);
-        if (plan.C == 0 || time < best) {
-            plan = p;
-            best = time;
-            again = turns > 1 && perSm == 1 && sz.maxM < 512;
-        }
-    }
-    return plan.C > 0 && !again;
+    return sz.W <= 32 ? pick_lockstep<1>(plan.K) : sz.W <= 64 ? pick_lockstep<2>(plan.K) : pick_lockstep<4>(plan.K);
 }
 
-bool cut_in_step(const rcd_ctx *ctx, const Sizes &sz)
+static cudaError_t allow_lockstep(const rcd_ctx *ctx, LockKernel kernel)
+{
+    const cudaError_t e = allow_shared(kernel, lock_shared(ctx->maxSmemOptin));
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+}
+
+static cudaLaunchConfig_t lock_launch(const LockPlan &plan, int threads, size_t smem, int clusters, cudaLaunchAttribute *attr, cudaStream_t st)
+{
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = (unsigned)plan.C;
+    attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(clusters * plan.C));
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+// Whether the GPU can place a cluster of that many CTAs, with all the shared memory that a plan may ask for (a partition of a GPU may
+// not: the launch would be refused).  Asked once per context and size.
+static bool lock_clusters_fit(rcd_ctx *ctx, const Sizes &sz, const LockPlan &plan)
+{
+    int idx = 0;
+    while ((1 << idx) < plan.C) ++idx;
+    int &fits = ctx->lockClusters[idx];
+    if (fits < 0) {
+        const LockKernel kernel = lock_kernel(sz, plan);
+        cudaLaunchAttribute attr[1];
+        const cudaLaunchConfig_t cfg = lock_launch(plan, (kLockWarps + 1) * 32, (size_t)lock_shared(ctx->maxSmemOptin), 1, attr, nullptr);
+        int active = 0;
+        if (allow_lockstep(ctx, kernel) != cudaSuccess || cudaOccupancyMaxActiveClusters(&active, kernel, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            active = 0;
+        }
+        fits = active;
+    }
+    return fits > 0;
+}
+
+static bool plan_lockstep(rcd_ctx *ctx, const Sizes &sz, LockPlan &plan)
+{
+    if (!library_chooses(ctx->cfg)) return false;
+    for (int most = kLockCtas;; most = plan.C / 2) {
+        if (!lock_plan(ctx->smCount, ctx->maxSmemOptin, most, sz, plan)) return false;
+        if (plan.C == 1 || lock_clusters_fit(ctx, sz, plan)) return true;
+    }
+}
+
+bool cut_in_step(rcd_ctx *ctx, const Sizes &sz)
 {
     LockPlan plan;
     return plan_lockstep(ctx, sz, plan);
@@ -455,20 +466,10 @@ static rcd_status run_lockstep(rcd_ctx *ctx, const LockPlan &plan, const Sizes &
     prm.W = sz.W;
     prm.columns = plan.columns;
     prm.one = 1u;
-    const LockKernel kernel = sz.W <= 32 ? pick_lockstep<1>(plan.K) : sz.W <= 64 ? pick_lockstep<2>(plan.K) : pick_lockstep<4>(plan.K);
-    RCD_CUDA(ctx, allow_shared(kernel, (int64_t)lock_shared(ctx)));
-    RCD_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(sz.L * plan.C));
-    cfg.blockDim = dim3((unsigned)(plan.warps + 1) * 32);
-    cfg.dynamicSmemBytes = plan.smem;
-    cfg.stream = st;
+    const LockKernel kernel = lock_kernel(sz, plan);
+    RCD_CUDA(ctx, allow_lockstep(ctx, kernel));
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)plan.C;
-    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    const cudaLaunchConfig_t cfg = lock_launch(plan, (plan.warps + 1) * 32, plan.smem, sz.L, attr, st);
     RCD_CUDA(ctx, cudaLaunchKernelEx(&cfg, kernel, prm));
     ctx->kernelLaunches++;
     return RCD_OK;

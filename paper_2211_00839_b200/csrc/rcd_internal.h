@@ -287,6 +287,7 @@ struct rcd_ctx {
     const unsigned long long *phaseNsDev = nullptr;
     const int32_t *statusDev = nullptr;
     int maxClusters[5] = {-1, -1, -1, -1, -1};   // clusters of 1, 2, 4, 8, 16 CTAs of the cluster form resident at once (-1: not asked yet)
+    int lockClusters[5] = {-1, -1, -1, -1, -1};  // the same of the graph cut in step
 };
 
 namespace rcd {
@@ -386,7 +387,7 @@ rcd_status launch_step_wait_selftest(rcd_ctx *ctx, int32_t *status, cudaStream_t
 // graph-cut objective: the whole greedy loop, and f from an assignment (selftest: in step, on two CTAs, whatever the plan says)
 rcd_status launch_cut_stopped_selftest(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, int32_t *assignment, int32_t *order, cudaStream_t st);
 // (in step: integers, where that is faster than the cluster form)
-bool cut_in_step(const rcd_ctx *ctx, const Sizes &sz);
+bool cut_in_step(rcd_ctx *ctx, const Sizes &sz);
 rcd_status launch_cut(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, int32_t *assignment, int32_t *order, cudaStream_t st);
 rcd_status launch_cut_objective(rcd_ctx *ctx, const Sizes &sz, const ClassDesc *descDev, const void *S, const int32_t *perm,
                                 const int32_t *assignment, void *partValues, void *total, void *scratch, cudaStream_t st);

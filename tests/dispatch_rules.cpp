@@ -2,7 +2,7 @@
 #include <iostream>
 #include <string>
 
-#include "rcd_internal.h"
+#include "rcd_cut_plan.h"
 
 int main()
 {
@@ -12,6 +12,13 @@ int main()
             int64_t M, d;
             std::cin >> M >> d;
             std::cout << rcd::cut_values_fit(M, d) << "\n";
+        } else if (what == "cut_plan") {
+            int sms, shared, most;
+            rcd::Sizes sz{};
+            std::cin >> sms >> shared >> most >> sz.L >> sz.maxM >> sz.d >> sz.W;
+            rcd::LockPlan p{};
+            if (rcd::lock_plan(sms, shared, most, sz, p)) std::cout << p.C << " " << p.K << " " << p.warps << " " << p.columns << " " << p.smem << "\n";
+            else std::cout << "0 0 0 0 0\n";
         } else {
             return 1;
         }

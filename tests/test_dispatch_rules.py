@@ -33,3 +33,31 @@ def test_graph_cut_values_fit_the_packed_word(rules):
         if fits and M <= 32768:
             # and the gains fit the 48 bits of a key: within three times the largest sum of a row, either way
             assert 6 * M * 16384 * d + 1 < 1 << 48, (M, d)
+
+
+B200 = (148, 232448)        # SMs, bytes of shared memory a CTA can ask for
+
+
+def test_graph_cut_in_step_covers_every_column(rules):
+    """Whatever the sizes and the largest cluster that the GPU can place (none at all on a slice of a few SMs)."""
+    import random
+    rng = random.Random(5)
+    log = lambda lo, hi: int(round(lo * (hi / lo) ** rng.random()))      # noqa: E731
+    questions = [("cut_plan", *rng.choice([B200, B200, (16, 232448), (1, 232448), (132, 101376)]), rng.choice([1, 2, 4, 8, 16]), log(1, 2000), log(1, 65535),
+                  log(1, 131071), log(1, 200)) for _ in range(20000)]
+    taken = 0
+    for (_, sms, shared, most, L, M, d, W), (C, K, warps, columns, smem) in zip(questions, rules(questions)):
+        if C == 0:
+            continue
+        taken += 1
+        assert C in (1, 2, 4, 8, 16) and C <= most and K in (1, 2, 3, 4, 8) and 1 <= warps <= 8
+        assert C * columns >= M and columns % 32 == 0 and warps * 32 * K >= columns and smem == W * columns * 8 <= shared - 8192
+        assert M * M // 4 * 16384 * d < 1 << 55 and W <= 128
+    assert taken > 2000
+
+
+def test_graph_cut_in_step_without_large_clusters(rules):
+    """A class that wants a cluster of 16 takes the largest there is, and another form where its gains do not fit that."""
+    ask = lambda most, M, W: rules([("cut_plan", *B200, most, 1, M, 64, W)])[0][0]      # noqa: E731
+    assert [ask(m, 6000, 12) for m in (16, 8, 4, 2, 1)] == [16, 8, 4, 0, 0]
+    assert [ask(m, 1300, 8) for m in (16, 8, 4, 2, 1)] == [8, 8, 4, 2, 1]
