@@ -166,6 +166,7 @@ struct LockParams {
     int32_t *assignment;
     int32_t *order;            // may be null
     int32_t *status;
+    unsigned long long *stats; // phase words
     int32_t W;
     int32_t columns;           // of a CTA (its gains: [W][columns])
     uint32_t one;              // the value 1, opaque to the compiler
@@ -366,6 +367,14 @@ __global__ void __launch_bounds__((kLockWarps + 1) * 32) cut_lockstep_kernel(con
 #pragma unroll
         for (int k = 0; k < KW; ++k)
             if (lane + 32 * k < W) prm.fval[(int64_t)l * W + lane + 32 * k] = (long long)(f[k] >> 7) - (long long)kTrackedZero;
+        // every pick but the last of a block takes one row off its gains
+        int blocks = 0;
+#pragma unroll
+        for (int k = 0; k < KW; ++k) blocks += __popc(__ballot_sync(0xffffffffu, lane + 32 * k < W && prm.quota[(int64_t)l * W + lane + 32 * k] > 0));
+        if (lane == 0) {
+            atomicAdd(prm.stats + 15, (unsigned long long)(M - blocks));
+            atomicAdd(prm.stats + 16, (unsigned long long)(M - blocks));
+        }
     }
     lock_barrier(alone);                                   // (and nobody writes to a CTA that has gone)
     // class-local picks -> outputs (none where the loop stopped early: the words behind the last pick are whatever memory held)
@@ -463,6 +472,7 @@ static rcd_status run_lockstep(rcd_ctx *ctx, const LockPlan &plan, const Sizes &
     prm.assignment = assignment;
     prm.order = order;
     prm.status = ctx->statusOwn;
+    prm.stats = ws.phaseNs;
     prm.W = sz.W;
     prm.columns = plan.columns;
     prm.one = 1u;
@@ -586,9 +596,11 @@ rcd_status launch_cut(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, int32_
 {
     if (sz.L == 0 || sz.maxM == 0) return RCD_OK;
     ctx->greedyForm = RCD_FORM_CUT_CHAIN;
+    ctx->steps = sz.maxM;
     LockPlan plan;
     if (plan_lockstep(ctx, sz, plan)) {
         ctx->greedyForm = RCD_FORM_CUT_STEPS;
+        ctx->phaseNsDev = ws.phaseNs;
         return run_lockstep(ctx, plan, sz, ws, assignment, order, st);
     }
     if (sz.floatArith) return run_cut<float>(ctx, sz, ws, assignment, order, st);

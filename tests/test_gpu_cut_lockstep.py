@@ -76,3 +76,20 @@ def test_no_outputs_where_the_loop_stops_early(rcd):
         with pytest.raises(rcd.RcdError) as e:
             ctx.sync_status()
         assert e.value.status == 5          # RCD_ERR_TIMEOUT, of the waits that follow
+
+
+def test_profile(rcd):
+    """Steps executed and rows taken off stored gains: every pick's but the last one's of each block that gets samples."""
+    import torch
+    wl = cluster.workload([400, 390], 16, 8, 1)
+    for caps, blocks in (([1.0] * 8, 8), ([1.0] * 8 + [1e-9] * 3, 8)):
+        with rcd.Context(0, objective=rcd.RCD_OBJ_GRAPH_CUT, profile=1) as ctx:
+            ctx.rcd_partition(rcd.features_to_torch(wl.features, device="cuda"), torch.from_numpy(wl.labels).cuda(), caps, wl.L)
+            ctx.sync_status()
+            p = ctx.profile()
+        assert p["greedy_form"] == rcd.RCD_FORM_CUT_STEPS and p["steps"] == 400
+        assert p["incremental_updates"] == p["incremental_rows"] == 400 + 390 - 2 * blocks
+    with rcd.Context(0, objective=rcd.RCD_OBJ_GRAPH_CUT, greedy_path=3) as ctx:
+        ctx.rcd_partition(rcd.features_to_torch(wl.features, device="cuda"), torch.from_numpy(wl.labels).cuda(), caps, wl.L)
+        ctx.sync_status()
+        assert ctx.profile()["steps"] == 400
