@@ -61,3 +61,11 @@ def test_graph_cut_in_step_without_large_clusters(rules):
     ask = lambda most, M, W: rules([("cut_plan", *B200, most, 1, M, 64, W)])[0][0]      # noqa: E731
     assert [ask(m, 6000, 12) for m in (16, 8, 4, 2, 1)] == [16, 8, 4, 0, 0]
     assert [ask(m, 1300, 8) for m in (16, 8, 4, 2, 1)] == [8, 8, 4, 2, 1]
+
+
+def test_shapes_compared_on_the_gpu_take_what_they_name(rules):
+    """The graph cut in step: every number of columns per thread, alone and in clusters."""
+    from test_gpu_cut_lockstep import SHAPES
+    got = rules([("cut_plan", *B200, 16, L + 1, M, 16, W) for L, M, W, _, _ in SHAPES])
+    assert [(C, K) for C, K, *_ in got] == [(C, K) for *_, C, K in SHAPES]
+    assert {K for *_, K in SHAPES} == {1, 3, 4, 8}          # (two: a class of 6000 into 12 blocks, beside them)

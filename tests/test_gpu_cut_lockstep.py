@@ -27,7 +27,7 @@ def test_exact(rcd, orc, sizes, W, copies):
 
 
 def test_like_the_chain(rcd):
-    """A class over clusters of every size the plan takes, against one CTA with everything in global memory (more than 128 blocks)."""
+    """A class over clusters of 16, one and two columns per thread, against one CTA with everything in global memory (more than 128 blocks)."""
     import torch
     for M, W in ((6000, 12), (3000, 100)):
         wl = cluster.workload([M, 300], 48, W, W)
@@ -41,6 +41,31 @@ def test_like_the_chain(rcd):
         assert out[0][3] == rcd.RCD_FORM_CUT_STEPS and out[1][3] == rcd.RCD_FORM_CUT_CHAIN
         for got, want in zip(out[0][:3], out[1][:3]):
             assert np.array_equal(got, want)
+
+
+# number and size of classes, blocks, and what the plan makes of them on 148 SMs (test_dispatch_rules.py): CTAs per class, columns per thread
+SHAPES = [
+    (200, 700, 8, 1, 3), (300, 900, 7, 1, 4), (160, 1100, 6, 1, 8),          # a CTA each; the last one's columns end before its threads' do
+    (2, 1300, 8, 8, 1), (10, 5000, 8, 8, 3), (40, 4000, 8, 2, 8), (75, 2100, 6, 4, 3),
+    (1, 16000, 6, 16, 4), (1, 17000, 4, 16, 8),
+]
+
+
+@pytest.mark.parametrize("L,M,W,C,K", SHAPES)
+def test_columns_per_thread(rcd, L, M, W, C, K):
+    """One to eight columns per thread, alone and in clusters, against the chain as above, with a smaller class beside the others."""
+    import torch
+    wl = cluster.workload([M] * L + [min(M - 1, 300)], 16, W, W, copies=20)
+    X, y = rcd.features_to_torch(wl.features, device="cuda"), torch.from_numpy(wl.labels).cuda()
+    out = []
+    for caps in (list(wl.capacities), list(wl.capacities) + [1e-9] * (129 - W)):       # (blocks that get nothing)
+        with rcd.Context(0, objective=rcd.RCD_OBJ_GRAPH_CUT) as ctx:
+            r = ctx.rcd_partition(X, y, caps, wl.L, M_max=M)
+            ctx.sync_status()
+            out.append((r[0].cpu().numpy(), r[1].cpu().numpy(), r[2].cpu().numpy()[:, :W], ctx.profile()["greedy_form"]))
+    assert out[0][3] == rcd.RCD_FORM_CUT_STEPS and out[1][3] == rcd.RCD_FORM_CUT_CHAIN
+    for got, want in zip(out[0][:3], out[1][:3]):
+        assert np.array_equal(got, want)
 
 
 def test_only_where_the_library_chooses(rcd, orc):
