@@ -367,14 +367,11 @@ __global__ void __launch_bounds__((kLockWarps + 1) * 32) cut_lockstep_kernel(con
 #pragma unroll
         for (int k = 0; k < KW; ++k)
             if (lane + 32 * k < W) prm.fval[(int64_t)l * W + lane + 32 * k] = (long long)(f[k] >> 7) - (long long)kTrackedZero;
-        // every pick but the last of a block takes one row off its gains
+        // every pick but the last of a block takes the sample's own row off its gains (no other: as the cluster form counts)
         int blocks = 0;
 #pragma unroll
         for (int k = 0; k < KW; ++k) blocks += __popc(__ballot_sync(0xffffffffu, lane + 32 * k < W && prm.quota[(int64_t)l * W + lane + 32 * k] > 0));
-        if (lane == 0) {
-            atomicAdd(prm.stats + 15, (unsigned long long)(M - blocks));
-            atomicAdd(prm.stats + 16, (unsigned long long)(M - blocks));
-        }
+        if (lane == 0) atomicAdd(prm.stats + 15, (unsigned long long)(M - blocks));
     }
     lock_barrier(alone);                                   // (and nobody writes to a CTA that has gone)
     // class-local picks -> outputs (none where the loop stopped early: the words behind the last pick are whatever memory held)

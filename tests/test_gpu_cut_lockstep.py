@@ -104,7 +104,7 @@ def test_no_outputs_where_the_loop_stops_early(rcd):
 
 
 def test_profile(rcd):
-    """Steps executed and rows taken off stored gains: every pick's but the last one's of each block that gets samples."""
+    """Steps executed, and picks that corrected stored gains: all but the last of each block that gets samples, by their own row only."""
     import torch
     wl = cluster.workload([400, 390], 16, 8, 1)
     for caps, blocks in (([1.0] * 8, 8), ([1.0] * 8 + [1e-9] * 3, 8)):
@@ -113,7 +113,7 @@ def test_profile(rcd):
             ctx.sync_status()
             p = ctx.profile()
         assert p["greedy_form"] == rcd.RCD_FORM_CUT_STEPS and p["steps"] == 400
-        assert p["incremental_updates"] == p["incremental_rows"] == 400 + 390 - 2 * blocks
+        assert p["incremental_updates"] == 400 + 390 - 2 * blocks and p["incremental_rows"] == 0
     with rcd.Context(0, objective=rcd.RCD_OBJ_GRAPH_CUT, greedy_path=3) as ctx:
         ctx.rcd_partition(rcd.features_to_torch(wl.features, device="cuda"), torch.from_numpy(wl.labels).cuda(), caps, wl.L)
         ctx.sync_status()
