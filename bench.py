@@ -325,9 +325,11 @@ def run_ours(args):
     loop_s = prof["greedy_ms"] * 1e-3
     # The cluster form makes no sweeps: it reads every row of S once for the gains of empty blocks, then the row of S of every
     # pick and one per column that the pick raised (in rounds: a row read once for several blocks counts once).  (Rows fetched on
-    # foresight whose sample another block received are not counted: see the traffic of the capture.)
+    # foresight whose sample another block received are not counted: see the traffic of the capture.)  The form for small classes
+    # reads S once, into shared memory: its later rows are no traffic.
     clustered = prof["sweep_bytes"] == 0 and prof["incremental_updates"] > 0
-    loop_bytes = 4 * ((M + 7) // 8 * 8) * (wl.N + prof["incremental_rows"] + prof["incremental_updates"]) if clustered else prof["sweep_bytes"]
+    later_rows = 0 if int(prof["greedy_form"]) == rcd.RCD_FORM_SMALL else prof["incremental_rows"] + prof["incremental_updates"]
+    loop_bytes = 4 * ((M + 7) // 8 * 8) * (wl.N + later_rows) if clustered else prof["sweep_bytes"]
     achieved = loop_bytes / loop_s / 1e9 if loop_s > 0 else 0.0
     kernel_name = {rcd.RCD_FORM_LAUNCHES: "sweep_kernel", rcd.RCD_FORM_BARRIERS: "greedy_persistent_kernel", rcd.RCD_FORM_ASYNC: "greedy_async_kernel",
                    rcd.RCD_FORM_CLASS_PER_CTA: "greedy_owner_kernel", rcd.RCD_FORM_CLUSTER: "greedy_cluster_kernel",
