@@ -113,7 +113,7 @@ __global__ void __launch_bounds__((NW + 1) * 32) greedy_small_kernel(const __gri
         if (kCut) {
             const unsigned long long top = warp_max_u64(v < M ? g0 + size : 0ull);
             if (lane == 0) shBest[warp] = top;
-            g0 = g0 - size - (long long)col[vs * ld];
+            g0 = g0 - size - (long long)col[min(vs, M - 1) * ld];       // (no row beyond the class's: with one block less than that follows S)
         }
     }
     if (kCut) {

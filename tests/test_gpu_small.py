@@ -73,6 +73,13 @@ def test_graph_cut_int8_exact(rcd, orc, sizes, W, copies):
     assert form(rcd, wl, objective=rcd.RCD_OBJ_GRAPH_CUT) == rcd.RCD_FORM_SMALL
 
 
+@pytest.mark.parametrize("M,W", [(155, 1), (233, 1), (9, 1), (33, 1), (97, 2), (129, 2), (217, 3)])
+def test_graph_cut_few_blocks_after_the_similarities(rcd, orc, M, W):
+    """Class sizes far below the next multiple of eight, with few blocks: threads beyond the class read no row beyond it (nothing that
+    large follows the similarities in shared memory)."""
+    test_graph_cut_int8_exact(rcd, orc, [M, M - 1], W, 0)
+
+
 def test_threads_with_contexts_of_their_own(rcd):
     """Four threads, each with a context and a stream, problems of very different shared memory at a time: each gets its own results."""
     import threading
