@@ -241,6 +241,7 @@ struct Prepared {
     std::vector<ClassDesc> desc;
     bool covered = false;
     std::shared_ptr<ClusterPlan> cluster;   // null: another form of the greedy loop, or none
+    bool cutInStep = false;
 };
 
 // A class whose quotas leave off before its samples do, as no call's can: the greedy loops that hand their picks over in memory have to
@@ -255,7 +256,8 @@ static rcd_status selftest_stopped(rcd_ctx *ctx, bool graphCut, cudaStream_t st)
     sz.nChunks = 2;
     sz.pitch = 128;
     const std::vector<ClassDesc> desc{ClassDesc{M, pad_row(M), 0, 0, 0, 0}};
-    const auto cluster = graphCut ? nullptr : plan_greedy_cluster(ctx, sz, desc);
+    bool inStep = false;
+    const auto cluster = graphCut ? nullptr : plan_greedy_cluster(ctx, sz, desc, &inStep);
     if (!graphCut && !cluster) return RCD_OK;              // (a context with options of the other forms)
     const size_t bytes = layout_workspace(nullptr, RCD_FEAT_I8, sz, nullptr);
     std::vector<unsigned char> host(bytes + 2 * M * sizeof(int32_t), 0);
@@ -430,7 +432,7 @@ static rcd_status prepare(rcd_ctx *ctx, const void *features, rcd_feat_dtype dty
     const int64_t dPitch = sz.pitch / (int64_t)feat_bytes(dtype);
     rs = launch_similarity(ctx, P.ws.Xs, dtype, N, dPitch, cls, P.ws.S, st);
     if (rs != RCD_OK) return rs;
-    if (capacities) P.cluster = plan_greedy_cluster(ctx, sz, P.desc);
+    if (capacities) P.cluster = plan_greedy_cluster(ctx, sz, P.desc, &P.cutInStep);
     if (ctx->cfg.similarity_kind == RCD_SIM_GAUSSIAN) {
         rs = launch_gaussian(ctx, P.ws.Xs, dtype, N, dPitch, cls, P.ws.S, P.ws.gaussNorms, P.ws.gaussPartial, P.ws.gaussSigma,
                              P.ws.gaussScale, P.cluster ? P.ws.fixedExp : nullptr, st);
@@ -835,7 +837,7 @@ rcd_status rcd_partition(rcd_ctx *ctx, const void *features_dev, rcd_feat_dtype 
     if (P.cluster) {
         rs = launch_greedy_cluster(ctx, *P.cluster, P.sz, P.ws, P.desc, assignment_dev, order_dev_or_null, part_values_dev_or_null, st);
     } else if (P.sz.graphCut) {
-        rs = launch_cut(ctx, P.sz, P.ws, assignment_dev, order_dev_or_null, st);
+        rs = launch_cut(ctx, P.sz, P.ws, P.cutInStep, assignment_dev, order_dev_or_null, st);
     } else {
         rs = launch_greedy(ctx, P.sz.floatArith ? RCD_FEAT_BF16 : RCD_FEAT_I8, P.sz, P.ws, P.desc, assignment_dev, order_dev_or_null, st);
     }

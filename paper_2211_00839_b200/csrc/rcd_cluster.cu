@@ -17,6 +17,7 @@
 // Stored gains are always exact: a pick corrects those of its block from one row of S per column whose coverage it
 // raised (S is symmetric).  All arithmetic is int64 on int32 similarities, hence independent of the order in which
 // anything happens: results do not depend on timing.
+#include "rcd_cut_plan.h"
 #include "rcd_exact.cuh"
 
 #include <limits.h>
@@ -1324,6 +1325,7 @@ struct ClusterPlan {
     size_t smem;
     std::shared_ptr<RoundsPlan> rounds;   // not null: the classes run in rounds instead, one CTA each
     std::shared_ptr<SmallPlan> small;     // not null: one CTA each with the class's similarities in its shared memory
+    double cutCycles = 0;      // graph cut: what the clusters are expected to take
     ClusterParams prm;         // teamWarps, slots, maxLd, rowPieces and the offsets are set
 };
 static size_t cluster_layout(const Sizes &sz, int maxLd, int C, bool state, size_t cap, ClusterPlan &plan)
@@ -1486,18 +1488,20 @@ static bool cluster_plan(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassD
     // cluster form was measured before, and they stay)
     plan.small = plan_greedy_small(ctx, sz);
     if (plan.small && !rounds_possible(ctx, sz, descHost)) return true;
-    if (sz.graphCut && cut_in_step(ctx, sz)) return false;
     const bool clusters = cluster_shape(ctx, sz, descHost, nonEmpty, maxLd, plan, &resident);
     plan.prm.maxLd = maxLd;
+    if (sz.graphCut && clusters) plan.cutCycles = cut_cluster_cycles(plan.C, resident, sz.W, descHost);
     plan.rounds = plan_greedy_rounds(ctx, sz, descHost, clusters ? ClusterShape{plan.C, resident, plan.P} : ClusterShape{0, 0, 0});
     if (plan.rounds) plan.small = nullptr;
     return clusters || plan.rounds || plan.small;
 }
 
-std::shared_ptr<ClusterPlan> plan_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost)
+std::shared_ptr<ClusterPlan> plan_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost, bool *cutInStep)
 {
     auto plan = std::make_shared<ClusterPlan>();
-    return cluster_plan(ctx, sz, descHost, *plan) ? plan : nullptr;
+    if (!cluster_plan(ctx, sz, descHost, *plan)) plan = nullptr;
+    *cutInStep = sz.graphCut && !(plan && plan->small) && cut_in_step(ctx, sz, descHost, plan ? plan->cutCycles : 0.0);
+    return *cutInStep ? nullptr : plan;
 }
 
 // Runs the greedy loop.  partValues (may be null) receives the tracked values.

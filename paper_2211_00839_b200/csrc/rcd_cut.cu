@@ -448,10 +448,12 @@ static bool plan_lockstep(rcd_ctx *ctx, const Sizes &sz, LockPlan &plan)
     }
 }
 
-bool cut_in_step(rcd_ctx *ctx, const Sizes &sz)
+bool cut_in_step(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost, double otherCycles)
 {
     LockPlan plan;
-    return plan_lockstep(ctx, sz, plan);
+    if (!plan_lockstep(ctx, sz, plan)) return false;
+    if (otherCycles <= 0) otherCycles = cut_chain_cycles(ctx->smCount, descHost);
+    return cut_steps_cycles(ctx->smCount, ctx->maxSmemOptin, plan, descHost) <= otherCycles;
 }
 
 static rcd_status run_lockstep(rcd_ctx *ctx, const LockPlan &plan, const Sizes &sz, const Workspace &ws, int32_t *assignment, int32_t *order, cudaStream_t st)
@@ -589,13 +591,13 @@ static rcd_status run_cut(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, in
     return RCD_OK;
 }
 
-rcd_status launch_cut(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, int32_t *assignment, int32_t *order, cudaStream_t st)
+rcd_status launch_cut(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, bool inStep, int32_t *assignment, int32_t *order, cudaStream_t st)
 {
     if (sz.L == 0 || sz.maxM == 0) return RCD_OK;
     ctx->greedyForm = RCD_FORM_CUT_CHAIN;
     ctx->steps = sz.maxM;
     LockPlan plan;
-    if (plan_lockstep(ctx, sz, plan)) {
+    if (inStep && plan_lockstep(ctx, sz, plan)) {
         ctx->greedyForm = RCD_FORM_CUT_STEPS;
         ctx->phaseNsDev = ws.phaseNs;
         return run_lockstep(ctx, plan, sz, ws, assignment, order, st);

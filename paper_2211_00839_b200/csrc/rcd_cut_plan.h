@@ -3,6 +3,8 @@
 
 #include <algorithm>
 #include <cmath>
+#include <functional>
+#include <vector>
 
 #include "rcd_internal.h"
 
@@ -52,6 +54,62 @@ inline bool lock_plan(int smCount, int maxSmemOptin, int mostCtas, const Sizes &
         }
     }
     return plan.C > 0 && !again;
+}
+
+// When the last of the classes is through, if `at` of them run at a time and the largest start first (cost: of a class of M samples).
+template <typename Cost>
+inline double cut_finish(const std::vector<ClassDesc> &classes, int at, Cost cost)
+{
+    std::vector<double> costs;
+    bool equal = true;
+    for (const ClassDesc &c : classes)
+        if (c.M > 0) {
+            costs.push_back(cost((double)c.M));
+            equal = equal && costs.back() == costs[0];
+        }
+    if (costs.empty()) return 0;
+    at = std::max(at, 1);
+    if (equal) return costs[0] * (double)((costs.size() + at - 1) / at);
+    std::sort(costs.begin(), costs.end(), std::greater<double>());
+    std::vector<double> busy(std::min<size_t>((size_t)at, costs.size()), 0.0);      // a heap, the earliest first
+    for (double c : costs) {
+        std::pop_heap(busy.begin(), busy.end(), std::greater<double>());
+        busy.back() += c;
+        std::push_heap(busy.begin(), busy.end(), std::greater<double>());
+    }
+    return *std::max_element(busy.begin(), busy.end());
+}
+
+// What the forms of the graph cut take, in cycles: in step, in clusters of C CTAs of which `resident` run at a time, and in one CTA per
+// class (two to an SM).  Fitted to 660 random problems of 260 to 6000 samples, 1 to 300 classes, a third of them of uneven sizes, 2 to
+// 128 blocks: a tenth off on average (the chain a fifth).  With 330 more: of some 720 that run in step two are slower than without that form
+// (5 and 13 %), and six that would be faster are left to another (by 6 to 20 %); by the largest class alone those of many classes and
+// blocks took up to 2.8 times as long (208 of 1383 into 111 blocks 20.7 ms in step, 7.4 in the chain), uneven ones up to 1.5 times (83 of up to 1051 into 6 2467 us,
+// in clusters 1644), equal ones up to 1.3 times (70 of 1941 into 7 4791 us, in clusters 3780).
+inline double cut_steps_cycles(int smCount, int maxSmemOptin, const LockPlan &plan, const std::vector<ClassDesc> &classes)
+{
+    // CTAs that share an SM slow one another down a little, and so do the many of the largest clusters
+    const int perSm = (int)std::max<size_t>(1, std::min<size_t>(6, (size_t)maxSmemOptin / (plan.smem + 4096)));
+    const int resident = plan.C == 1 ? smCount * perSm : plan.C == 16 ? smCount / 20 * perSm : (int)(0.9 * smCount * perSm / plan.C);
+    double samples = 0, largest = 1;
+    for (const ClassDesc &c : classes) {
+        samples += c.M;
+        largest = std::max(largest, (double)c.M);
+    }
+    const double share = std::min((double)perSm, std::max(1.0, std::ceil(samples / largest * plan.C / smCount - 1e-9)));
+    const double pick = (plan.C == 1 ? 1600.0 : plan.C == 16 ? 1800.0 : 1400.0) + 400.0 * plan.K;
+    return cut_finish(classes, resident, [&](double M) { return M * pick; }) * (1.0 + 0.15 * (share - 1.0));
+}
+inline double cut_cluster_cycles(int C, int resident, int W, const std::vector<ClassDesc> &classes)
+{
+    const double pick = 1200.0 + 300.0 * std::log2((double)W);
+    return cut_finish(classes, resident, [&](double M) { return M * (pick + 2.0 * M / C + 0.0003 * (M / C) * (M / C)); });
+}
+inline double cut_chain_cycles(int smCount, const std::vector<ClassDesc> &classes)
+{
+    int64_t some = 0;
+    for (const ClassDesc &c : classes) some += c.M > 0 ? 1 : 0;
+    return cut_finish(classes, some <= smCount ? smCount : 2 * smCount, [&](double M) { return M * (2000.0 + 3.0 * M); }) * (some <= smCount ? 1.0 : 1.4);
 }
 
 }  // namespace rcd

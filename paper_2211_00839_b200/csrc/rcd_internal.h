@@ -361,7 +361,8 @@ rcd_status launch_greedy_not_fixed(rcd_ctx *ctx, const Sizes &sz, const Workspac
 
 // greedy loop, one thread-block cluster per class: how it takes a problem (null: it does not), and the loop
 struct ClusterPlan;
-std::shared_ptr<ClusterPlan> plan_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost);
+// (null: another form takes the problem; cutInStep: the graph cut in step does)
+std::shared_ptr<ClusterPlan> plan_greedy_cluster(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost, bool *cutInStep);
 rcd_status launch_greedy_cluster(rcd_ctx *ctx, ClusterPlan &plan, const Sizes &sz, const Workspace &ws, const std::vector<ClassDesc> &descHost,
                                  int32_t *assignment, int32_t *order, void *partValues, cudaStream_t st);
 
@@ -386,9 +387,9 @@ rcd_status launch_step_wait_selftest(rcd_ctx *ctx, int32_t *status, cudaStream_t
 
 // graph-cut objective: the whole greedy loop, and f from an assignment (selftest: in step, on two CTAs, whatever the plan says)
 rcd_status launch_cut_stopped_selftest(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, int32_t *assignment, int32_t *order, cudaStream_t st);
-// (in step: integers, where that is faster than the cluster form)
-bool cut_in_step(rcd_ctx *ctx, const Sizes &sz);
-rcd_status launch_cut(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, int32_t *assignment, int32_t *order, cudaStream_t st);
+// (in step: integers, where that is faster than another form, which takes otherCycles; 0: one CTA per class)
+bool cut_in_step(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassDesc> &descHost, double otherCycles);
+rcd_status launch_cut(rcd_ctx *ctx, const Sizes &sz, const Workspace &ws, bool inStep, int32_t *assignment, int32_t *order, cudaStream_t st);
 rcd_status launch_cut_objective(rcd_ctx *ctx, const Sizes &sz, const ClassDesc *descDev, const void *S, const int32_t *perm,
                                 const int32_t *assignment, void *partValues, void *total, void *scratch, cudaStream_t st);
 

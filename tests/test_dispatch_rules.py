@@ -69,3 +69,33 @@ def test_shapes_compared_on_the_gpu_take_what_they_name(rules):
     got = rules([("cut_plan", *B200, 16, L + 1, M, 16, W) for L, M, W, _, _ in SHAPES])
     assert [(C, K) for C, K, *_ in got] == [(C, K) for *_, C, K in SHAPES]
     assert {K for *_, K in SHAPES} == {1, 3, 4, 8}          # (two: a class of 6000 into 12 blocks, beside them)
+
+
+def test_graph_cut_in_step_where_it_is_the_faster_form(rules):
+    """Either side of the choice as measured (ms on a B200): in step against clusters of C CTAs, or against a CTA per class."""
+    uneven = lambda L, M: [M] + [round(M * (l + 0.5) / L) for l in range(L - 1)]       # noqa: E731
+    faster, slower = [
+        ("clusters", 8, 8, 16, [5000] * 10),        # 7.2, 8.7
+        ("clusters", 8, 4, 33, [2500] * 30),        # 3.6, 5.1
+        ("clusters", 8, 1, 148, [700] * 200),       # 1.2, 2.9
+        ("chain", 100, 0, 0, [3000] * 2),           # 3.0, 11.7
+        ("chain", 65, 0, 0, [770, 5]),
+    ], [
+        ("clusters", 7, 2, 74, [1941] * 70),        # 4.8, 3.8
+        ("clusters", 6, 2, 74, [609] * 67),         # 0.90, 0.85
+        ("clusters", 6, 4, 33, uneven(83, 1051)),   # 2.5, 1.6
+        ("clusters", 9, 4, 33, uneven(86, 1068)),   # 2.5, 2.1
+        ("chain", 111, 0, 0, [1383] * 208),         # 20.7, 7.4
+        ("chain", 124, 0, 0, [2955] * 92),          # 46.4, 20.4
+        ("chain", 107, 0, 0, uneven(183, 1633)),    # 10.8, 8.8
+    ]
+    got = rules([("cut_cycles", W, max(C, 1), max(at, 1), len(sizes), *sizes) for _, W, C, at, sizes in faster + slower])
+    for k, ((other, *_, sizes), (steps, clusters, chain)) in enumerate(zip(faster + slower, got)):
+        assert steps > 0
+        assert (steps <= (clusters if other == "clusters" else chain)) == (k < len(faster)), (other, sizes[0], len(sizes))
+
+
+def test_finish_time_of_uneven_classes(rules):
+    """Largest first on the machine that is free first: two clusters take 9 + 2 and 7 + 6, costs by the number of samples alone."""
+    (_, two, _), (_, one, _) = rules([("cut_cycles", 1, 1 << 20, 2, 4, 9, 7, 6, 2), ("cut_cycles", 1, 1 << 20, 1, 4, 9, 7, 6, 2)])
+    assert two == 13 * 1200 and one == 24 * 1200

@@ -118,3 +118,14 @@ def test_profile(rcd):
         ctx.rcd_partition(rcd.features_to_torch(wl.features, device="cuda"), torch.from_numpy(wl.labels).cuda(), caps, wl.L)
         ctx.sync_status()
         assert ctx.profile()["steps"] == 400
+
+
+@pytest.mark.parametrize("L,M,W,form", [(67, 609, 6, "RCD_FORM_CLUSTER"), (118, 1138, 126, "RCD_FORM_CUT_CHAIN"), (3, 700, 126, "RCD_FORM_CUT_STEPS")])
+def test_where_another_form_is_faster(rcd, L, M, W, form):
+    import torch
+    X = torch.randint(-9, 10, (L * M, 16), dtype=torch.int8, device="cuda")
+    y = torch.arange(L * M, dtype=torch.int32, device="cuda") % L
+    with rcd.Context(0, objective=rcd.RCD_OBJ_GRAPH_CUT) as ctx:
+        ctx.rcd_partition(X, y, [1.0] * W, L, M_max=M)
+        ctx.sync_status()
+        assert ctx.profile()["greedy_form"] == getattr(rcd, form)
