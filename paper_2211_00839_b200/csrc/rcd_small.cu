@@ -12,7 +12,7 @@
 //
 // What bounds it: the chain of a pick, 900 to 1100 cycles, of which 340 go into the candidates (two warp-wide maxima of 64 bits, 56 cycles
 // each, and 25 of a barrier), as much into the row and its list, and 12 cycles per raised column once more than a few rise.  Whole calls, in us, the
-// cluster form and this one: 2 classes of 200 int8 into 4 blocks 236 and 153; 10 of 160 into 32 blocks 332 and 215; 1000 of 100 into 8 blocks
+// cluster form and this one: 2 classes of 200 int8 into 4 blocks 236 and 153 (138 with the class split in two launches); 10 of 160 into 32 blocks 332 and 215; 1000 of 100 into 8 blocks
 // 896 and 294; 35 of 128 bf16 into 22 blocks 300 and 211; graph cut, 60 of 180 into 12 blocks 255 and 103.
 //
 // Results are those of the other forms bit for bit: gains are exact integers, decisions are made in the same order.
