@@ -1486,7 +1486,7 @@ static bool cluster_plan(rcd_ctx *ctx, const Sizes &sz, const std::vector<ClassD
     plan.prm.maxLd = maxLd;
     // (small classes whenever they fit: on mixtures of Gaussians 0.5 to 0.9 times the cluster form's time.  What a pick costs grows with the
     // columns it raises, which only the features tell: rectified ones 0.6 to 1.0 times, with 200 and more bf16 samples into 7 to 12 blocks
-    // up to 1.1 for a few classes and 1.2 for one; features without any classes in them, where a pick raises a third of the columns, up
+    // up to 1.1 for a few classes and 1.2 for one; independent normal ones, whose picks raise many, up
     // to 1.3 from 200 samples and 8 blocks on.  Rounds first: where those are faster than the cluster form was measured before, and they
     // stay)
     plan.small = plan_greedy_small(ctx, sz);
